@@ -416,10 +416,11 @@ __device__ __forceinline__ long long nbr(const Dev &d, int x, int y, int z, int 
 }
 
 __device__ __forceinline__ void coords(const Dev &d, long long idx, int &x, int &y, int &z) {
-    x = (int)(idx % d.nx);
-    long long r = idx / d.nx;
-    y = (int)(r % d.ny);
-    z = (int)(r / d.ny);
+    // every cell index is below 2^32 (checked at create): 32-bit divisions
+    const uint32_t i = (uint32_t)idx, r = i / (uint32_t)d.nx;
+    x = (int)(i - r * (uint32_t)d.nx);
+    z = (int)(r / (uint32_t)d.ny);
+    y = (int)(r - (uint32_t)z * (uint32_t)d.ny);
 }
 
 // class of cell i (the flag byte without the neighbour-obstacle bit); walls
@@ -568,13 +569,20 @@ __device__ __forceinline__ void body_velocity_at(const Dev &d, const Body &b, co
     uw[2] = b.v[2] + c2;
 }
 
+// (c_x u_0 + c_y u_1) + c_z u_2 without the products by the zeros of c_q
+__device__ __forceinline__ double dot_c(int q, const double *u) {
+    double s = cx(q) ? cx(q) * u[0] : 0.0;
+    if (cy(q)) s = cx(q) ? s + cy(q) * u[1] : cy(q) * u[1];
+    if (cz(q)) s = (cx(q) || cy(q)) ? s + cz(q) * u[2] : cz(q) * u[2];
+    return s;
+}
 // c_q . u_w with u_w at the midpoint x_c + c_qbar / 2 of the link (x, q)
 __device__ __forceinline__ double link_cuw(const Dev &d, const Body &b, int x, int y, int z, int q) {
     int qb = opp(q);
     double p[3] = {(x + 0.5) + 0.5 * cx(qb), (y + 0.5) + 0.5 * cy(qb), (z + 0.5) + 0.5 * cz(qb)};
     double uw[3];
     body_velocity_at(d, b, p, uw);
-    return (cx(q) * uw[0] + cy(q) * uw[1]) + cz(q) * uw[2];
+    return dot_c(q, uw);
 }
 
 // the same in float for the float storages: the body state is rounded once
@@ -677,24 +685,91 @@ __device__ __forceinline__ double cell_rho_u(const Dev &d, const void *g, long l
     return r;
 }
 
-// double BGK collision of the post-stream cell fp -> fnew (Eq. lbgk, R1 order)
+// Double BGK collision of the post-stream cell fp -> fnew (Eq. lbgk with Eq.
+// forceterm).  GB300 executes 2 double operations per SM and cycle, so the
+// double storage's kernels are bound by their number of double operations, and
+// the collision is written with as few as keep the oracle's roundings: each
+// result is the oracle's expression
+//   rho, j = sums in q order; u = j / rho;
+//   t = ((1 + 3 cu) + (4.5 cu) cu) - 1.5 u.u,  fe = (w rho) t,
+//   F = (w rho) ((tx + ty) + tz),  tx = (3 (cx - ux) + (9 cu) cx) ax, ...
+//   f = (f' - omega (f' - fe)) + F
+// without its products by the zeros of c_q (x + 0 y = x) and with every value
+// that directions share computed once: c_qbar . u = -(c_q . u) exactly, so the
+// pair shares 3 cu, 9 cu and (4.5 cu) cu, and a component with c = 0
+// contributes (-3 u) a to every such direction.  ZG (ax = ay = 0, gravity
+// along z alone, chosen per launch from the uniform parameters) also drops the
+// products by those zero accelerations.  612 double operations per liquid cell
+// before, about 330 with ZG and 420 without.
+template <bool ZG> __device__ __forceinline__ void collide_d_t(const Dev &d, const double *fp, double *fnew) {
+    double rho = fp[0], j0 = 0.0, j1 = 0.0, j2 = 0.0;
+#pragma unroll
+    for (int q = 1; q < Q; ++q) rho += fp[q];
+#pragma unroll
+    for (int q = 1; q < Q; ++q) {
+        if (cx(q) > 0) j0 += fp[q];
+        if (cx(q) < 0) j0 -= fp[q];
+        if (cy(q) > 0) j1 += fp[q];
+        if (cy(q) < 0) j1 -= fp[q];
+        if (cz(q) > 0) j2 += fp[q];
+        if (cz(q) < 0) j2 -= fp[q];
+    }
+    const double u[3] = {j0 / rho, j1 / rho, j2 / rho};
+    const double us15 = 1.5 * ((u[0] * u[0] + u[1] * u[1]) + u[2] * u[2]);
+    const double om = d.omega;
+    // per component: 3 (1 - u), 3 (-1 - u), and the term of a direction with c = 0
+    double fpos[3], fneg[3], fzero[3];
+#pragma unroll
+    for (int k = 0; k < 3; ++k) {
+        fzero[k] = (3.0 * -u[k]) * d.a[k];
+        fpos[k] = 3.0 * (1.0 - u[k]);
+        fneg[k] = 3.0 * (-1.0 - u[k]);
+    }
+    // weight classes: w rho, and with ZG the force of a direction with c_z = 0
+    const double wr0 = wd(0) * rho, wr1 = wd(1) * rho, wr2 = wd(7) * rho;
+    {
+        const double fe = wr0 * (1.0 - us15);
+        const double fq = wr0 * (ZG ? fzero[2] : (fzero[0] + fzero[1]) + fzero[2]);
+        fnew[0] = (fp[0] - om * (fp[0] - fe)) + fq;
+    }
+    const double fz1 = wr1 * fzero[2], fz2 = wr2 * fzero[2];
+#pragma unroll
+    for (int q = 1; q < Q; ++q) {
+        const int qb = opp(q);
+        if (qb < q) continue;  // each pair once
+        const double wr = q <= 6 ? wr1 : wr2;
+        double cu = 0.0;
+        bool first = true;
+        if (cx(q)) {
+            cu = cx(q) > 0 ? u[0] : -u[0];
+            first = false;
+        }
+        if (cy(q)) {
+            cu = first ? (cy(q) > 0 ? u[1] : -u[1]) : (cy(q) > 0 ? cu + u[1] : cu - u[1]);
+            first = false;
+        }
+        if (cz(q)) cu = first ? (cz(q) > 0 ? u[2] : -u[2]) : (cz(q) > 0 ? cu + u[2] : cu - u[2]);
+        const double c3 = 3.0 * cu, c9 = 9.0 * cu, s = (4.5 * cu) * cu;
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+            const int p = h ? qb : q;
+            const double t = ((h ? 1.0 - c3 : 1.0 + c3) + s) - us15;
+            const double fe = wr * t;
+            // (9 cu_p) c_p,k = (9 cu) c_q,k for both members of the pair
+            double f0 = fzero[0], f1 = fzero[1], f2 = fzero[2];
+            if (!ZG && cx(p)) f0 = ((cx(p) > 0 ? fpos[0] : fneg[0]) + (cx(q) > 0 ? c9 : -c9)) * d.a[0];
+            if (!ZG && cy(p)) f1 = ((cy(p) > 0 ? fpos[1] : fneg[1]) + (cy(q) > 0 ? c9 : -c9)) * d.a[1];
+            if (cz(p)) f2 = ((cz(p) > 0 ? fpos[2] : fneg[2]) + (cz(q) > 0 ? c9 : -c9)) * d.a[2];
+            double fq;
+            if (ZG) fq = cz(p) ? wr * f2 : (q <= 6 ? fz1 : fz2);
+            else fq = wr * ((f0 + f1) + f2);
+            fnew[p] = (fp[p] - om * (fp[p] - fe)) + fq;
+        }
+    }
+}
 __device__ __forceinline__ void collide_d(const Dev &d, const double *fp, double *fnew) {
-    double rho = 0.0, j0 = 0.0, j1 = 0.0, j2 = 0.0;
-#pragma unroll
-    for (int q = 0; q < Q; ++q) rho += fp[q];
-#pragma unroll
-    for (int q = 0; q < Q; ++q) {
-        j0 += cx(q) * fp[q];
-        j1 += cy(q) * fp[q];
-        j2 += cz(q) * fp[q];
-    }
-    double u[3] = {j0 / rho, j1 / rho, j2 / rho};
-#pragma unroll
-    for (int q = 0; q < Q; ++q) {
-        double fe = feq_d(q, rho, u);
-        double fq = force_d(q, rho, u, d.a);
-        fnew[q] = (fp[q] - d.omega * (fp[q] - fe)) + fq;
-    }
+    if (d.a[0] == 0.0 && d.a[1] == 0.0) collide_d_t<true>(d, fp, fnew);
+    else collide_d_t<false>(d, fp, fnew);
 }
 
 // ----------------------------------------- float arithmetic on deviations
@@ -884,14 +959,15 @@ __device__ __forceinline__ long long range_count(const int *lo, const int *hi) {
 }
 __device__ __forceinline__ void range_cell(const Dev &d, const int *lo, const int *hi, long long k, int &x, int &y,
                                            int &z) {
-    int lx = hi[0] - lo[0], ly = hi[1] - lo[1];
-    x = lo[0] + (int)(k % lx);
-    long long r = k / lx;
-    y = lo[1] + (int)(r % ly);
-    z = lo[2] + (int)(r / ly);
-    x = ((x % d.nx) + d.nx) % d.nx;  // only periodic axes can leave [0, n)
-    y = ((y % d.ny) + d.ny) % d.ny;
-    z = ((z % d.nz) + d.nz) % d.nz;
+    // a range holds at most the grid's cells (fewer than 2^32)
+    const uint32_t lx = (uint32_t)(hi[0] - lo[0]), ly = (uint32_t)(hi[1] - lo[1]);
+    const uint32_t kk = (uint32_t)k, r = kk / lx, rz = r / ly;
+    x = lo[0] + (int)(kk - r * lx);
+    y = lo[1] + (int)(r - rz * ly);
+    z = lo[2] + (int)rz;
+    if (x < 0 || x >= d.nx) x = ((x % d.nx) + d.nx) % d.nx;  // only periodic axes can leave [0, n)
+    if (y < 0 || y >= d.ny) y = ((y % d.ny) + d.ny) % d.ny;
+    if (z < 0 || z >= d.nz) z = ((z % d.nz) + d.nz) % d.nz;
 }
 
 // mapping of a newly added body (Sec. 2.3); book_mass: charge the covered mass
@@ -921,10 +997,23 @@ struct VB {
 };
 __device__ __forceinline__ VB vb_own() { return VB{blockIdx.x, blockIdx.y, blockIdx.z, gridDim.x, gridDim.y, gridDim.z}; }
 
+// A worklist's items spread over a launch's blocks, a warp's worth (`per` items)
+// at a time: as few warps of each block as hold the list, so that a short list
+// gets an SM per warp (its latency chains, and in double arithmetic the 2
+// operations per SM and cycle, don't queue behind one another) and a long list
+// keeps neighbouring items in one block.  First item of the calling warp and
+// the stride; a warp without items starts at n.
+__device__ __forceinline__ void list_span(const VB &vb, uint32_t n, uint32_t per, uint32_t &first, uint32_t &stride) {
+    const uint32_t wpb = blockDim.x >> 5, warp = threadIdx.x >> 5;
+    const uint32_t groups = (n + per - 1) / per, used = min(wpb, (groups + vb.nx - 1) / vb.nx);
+    first = warp < used ? (vb.x * used + warp) * per : n;
+    stride = vb.nx * used * per;
+}
 #define LIST_LOOP(L, var)                                                                                     \
-    uint32_t n_##var = wl_count(d, L);                                                                         \
-    for (uint32_t it_##var = vb.x * blockDim.x + threadIdx.x; it_##var < n_##var;                              \
-         it_##var += vb.nx * blockDim.x)
+    const uint32_t n_##var = wl_count(d, L);                                                                   \
+    uint32_t f_##var, s_##var;                                                                                 \
+    list_span(vb, n_##var, 32u, f_##var, s_##var);                                                             \
+    for (uint32_t it_##var = f_##var + (threadIdx.x & 31u); it_##var < n_##var; it_##var += s_##var)
 
 // neighbour-obstacle bit: set when any of the 18 neighbours is an obstacle
 // (the bulk kernel then lists the cell for k_general; walls and periodic
@@ -1076,58 +1165,86 @@ __device__ __forceinline__ void forces_f64_body(const Dev &d, const VB &vb) {
         }
     }
     unsigned __int128 acc[7] = {0, 0, 0, 0, 0, 0, 0};
-    // the cells of the box around the body spread over all the body's blocks;
-    // only cells next to an obstacle (neighbour-obstacle bit) can hold links
-    const long long ncell = range_count(lo, hi);
-    const int tidf = threadIdx.x + blockDim.x * threadIdx.y, nthr = blockDim.x * blockDim.y;
-    for (long long kk = (long long)vb.x * nthr + tidf; kk < ncell; kk += (long long)vb.nx * nthr) {
+    // the cells of the box around the body, 32 consecutive cells per warp, the
+    // warps' groups dealt out block by block (the double unit serves one SM:
+    // with the groups of a small body in consecutive warps of a few blocks
+    // those SMs' units held the kernel up); only cells next to an obstacle
+    // (neighbour-obstacle bit) can hold links
+    const uint32_t ncell = (uint32_t)range_count(lo, hi);
+    const int tidf = threadIdx.x + blockDim.x * threadIdx.y, nwarp = (blockDim.x * blockDim.y) >> 5;
+    const long long sy = d.nx, sz = (long long)d.nx * d.ny;
+    for (uint32_t kk = ((uint32_t)(tidf >> 5) * vb.nx + vb.x) * 32u + (uint32_t)(tidf & 31); kk < ncell;
+         kk += (uint32_t)nwarp * vb.nx * 32u) {
         int x, y, z;
         range_cell(d, lo, hi, kk, x, y, z);
-        long long i = x + (long long)d.nx * (y + (long long)d.ny * z);
-        int fb = d.flags[i];
-        int cl = fb & CL_MASK;
+        const long long i = x + sy * (y + (long long)d.ny * z);
+        const int fb = d.flags[i];
+        const int cl = fb & CL_MASK;
         if (!(fb & NB_OBST) || cl == CL_O) continue;
-        {
-            // double, in the order of the plain restatement
-            const double phi_x = cl == CL_L ? 1.0 : (cl == CL_I ? d.phisrc[i] : 0.0);
-            const double r[3] = {min_image(d, (x + 0.5) - b.o[0], 0), min_image(d, (y + 0.5) - b.o[1], 1),
-                                 min_image(d, (z + 0.5) - b.o[2], 2)};
-            bool have_rho = false;
-            double rho_x = 0.0;
-#pragma unroll 1
-            for (int q = 1; q < Q; ++q) {
-                long long si = nbr(d, x, y, z, -cx(q), -cy(q), -cz(q));
-                if (si < 0 || clsv(d, si) != CL_O || d.bid[si] != bi) continue;
-                double cuw = link_cuw(d, b, x, y, z, q);
-                int qb = opp(q);
-                double inner;
-                if (cl == CL_G) {
-                    inner = wd(q) * d.rho_g;
-                } else {
-                    double A = phi_x * Sto<S>::ldf(d.fsrc, qb, i, d.N);
-                    double B = (1.0 - phi_x) * (wd(q) * d.rho_g);
-                    double C;
-                    if (cuw == 0.0) {
-                        C = phi_x * 0.0;
-                    } else {
-                        if (!have_rho) {
-                            rho_x = cell_density<S>(d, d.fsrc, i);
-                            have_rho = true;
-                        }
-                        C = phi_x * (((3.0 * wd(q)) * rho_x) * cuw);
-                    }
-                    inner = (A + B) + C;
+        // directions into body bi and the cell's populations, requested at once
+        const bool inner = x > 0 && x < d.nx - 1 && y > 0 && y < d.ny - 1 && z > 0 && z < d.nz - 1;
+        const bool fluid = cl != CL_G;
+        double f[Q];
+#pragma unroll
+        for (int q = 0; q < Q; ++q) f[q] = fluid ? Sto<S>::ldf(d.fsrc, q, i, d.N) : 0.0;
+        const double phi_x = cl == CL_L ? 1.0 : (cl == CL_I ? d.phisrc[i] : 0.0);
+        unsigned lm = 0;
+#pragma unroll
+        for (int q = 1; q < Q; ++q) {
+            const long long si = inner ? i - (cx(q) + cy(q) * sy + cz(q) * sz) : nbr(d, x, y, z, -cx(q), -cy(q), -cz(q));
+            if (si >= 0 && clsv(d, si) == CL_O) lm |= 1u << q;
+        }
+        if (d.nb > 1) {
+            unsigned om = lm;
+            lm = 0;
+#pragma unroll
+            for (int q = 1; q < Q; ++q)
+                if (om & (1u << q)) {
+                    const long long si =
+                        inner ? i - (cx(q) + cy(q) * sy + cz(q) * sz) : nbr(d, x, y, z, -cx(q), -cy(q), -cz(q));
+                    if (d.bid[si] == bi) lm |= 1u << q;
                 }
-                double g = 2.0 * inner;
-                double F0 = cx(qb) * g, F1 = cy(qb) * g, F2 = cz(qb) * g;
-                acc[0] += fixed96(F0);
-                acc[1] += fixed96(F1);
-                acc[2] += fixed96(F2);
-                acc[3] += fixed96(r[1] * F2 - r[2] * F1);
-                acc[4] += fixed96(r[2] * F0 - r[0] * F2);
-                acc[5] += fixed96(r[0] * F1 - r[1] * F0);
-                acc[6] += fixed96(fabs(g));
+        }
+        if (!lm) continue;
+        // double, each value in the order of the plain restatement; the
+        // direction is a constant of each unrolled term, so products by its
+        // zeros are left out (x + 0 y = x)
+        const double r[3] = {min_image(d, (x + 0.5) - b.o[0], 0), min_image(d, (y + 0.5) - b.o[1], 1),
+                             min_image(d, (z + 0.5) - b.o[2], 2)};
+        double rho_x = 0.0;
+#pragma unroll
+        for (int q = 0; q < Q; ++q) rho_x += f[q];
+        const double pg = 1.0 - phi_x;
+#pragma unroll
+        for (int q = 1; q < Q; ++q) {
+            if (!(lm & (1u << q))) continue;
+            const int qb = opp(q);
+            double inr = wd(q) * d.rho_g;
+            if (fluid) {
+                const double cuw = link_cuw(d, b, x, y, z, q);
+                const double A = phi_x * f[qb], B = pg * inr;
+                const double C = cuw == 0.0 ? 0.0 : phi_x * (((3.0 * wd(q)) * rho_x) * cuw);
+                inr = (A + B) + C;
             }
+            const double g = 2.0 * inr;
+            // the integer of +-g: floor(-t) = -floor(t) where t 2^96 is an
+            // integer, which holds from |g| = 2^-43 up
+            const unsigned __int128 pos = fixed96(g);
+            const unsigned __int128 neg = fabs(g) >= 1.1368683772161603e-13 ? (unsigned __int128)0 - pos : fixed96(-g);
+            if (cx(qb)) acc[0] += cx(qb) > 0 ? pos : neg;
+            if (cy(qb)) acc[1] += cy(qb) > 0 ? pos : neg;
+            if (cz(qb)) acc[2] += cz(qb) > 0 ? pos : neg;
+            const double F0 = cx(qb) > 0 ? g : -g, F1 = cy(qb) > 0 ? g : -g, F2 = cz(qb) > 0 ? g : -g;
+            if (cy(qb) && cz(qb)) acc[3] += fixed96(r[1] * F2 - r[2] * F1);
+            else if (cz(qb)) acc[3] += fixed96(r[1] * F2);
+            else if (cy(qb)) acc[3] += fixed96(-(r[2] * F1));
+            if (cx(qb) && cz(qb)) acc[4] += fixed96(r[2] * F0 - r[0] * F2);
+            else if (cx(qb)) acc[4] += fixed96(r[2] * F0);
+            else if (cz(qb)) acc[4] += fixed96(-(r[0] * F2));
+            if (cx(qb) && cy(qb)) acc[5] += fixed96(r[0] * F1 - r[1] * F0);
+            else if (cy(qb)) acc[5] += fixed96(r[0] * F1);
+            else if (cx(qb)) acc[5] += fixed96(-(r[1] * F0));
+            acc[6] += g >= 0.0 ? pos : neg;
         }
     }
     // block reduction of the exact integer sums (any order gives the same
@@ -1414,10 +1531,10 @@ __device__ __forceinline__ void bulk_body(const Dev &d, const VB &vb, int zb) {
     else if (d.pair_ok) liquid_body_pair<S, ZBMAX>(d, vb, zb);
     else liquid_body<S, ZBMAX>(d, vb, zb);
 }
-template <int S>
+template <int S, int ZB>
 __global__ void __launch_bounds__(BULK_THREADS, S == 0 ? 1 : (LBMFS_BULK_PAIR ? LBMFS_PAIR_MINB : LBMFS_BULK_MINB))
     k_liquid(const __grid_constant__ Dev d) {
-    bulk_body<S, LBMFS_BULK_ZB>(d, vb_own(), LBMFS_BULK_ZB);
+    bulk_body<S, ZB>(d, vb_own(), ZB);
 }
 
 template <int S>
@@ -2158,8 +2275,9 @@ __device__ __forceinline__ void interface_trio(const Dev &d, const VB &vb) {
 #define TRIO_POS(k) ((pk[k] >> 16) & 1u)
     const float ax = d.a_f[0], ay = d.a_f[1], az = d.a_f[2];
     const uint32_t n = wl_count(d, WL_IFACE);
-    const uint32_t wpb = blockDim.x >> 5;
-    for (uint32_t w0 = (vb.x * wpb + (threadIdx.x >> 5)) * 10u; w0 < n; w0 += vb.nx * wpb * 10u) {
+    uint32_t first, stride;
+    list_span(vb, n, 10u, first, stride);
+    for (uint32_t w0 = first; w0 < n; w0 += stride) {
         const uint32_t it = w0 + (uint32_t)g;
         const bool valid = lane_ok && it < n;
         const long long i = d.list[WL_IFACE][valid ? it : w0];
@@ -2366,9 +2484,8 @@ __device__ __forceinline__ void interface_d(const Dev &d, const VB &vb) {
     // the bulk kernel has read this step's fluid top: clear the slot for the
     // next step to record into
     if (vb.x == 0 && threadIdx.x == 0) *d.ztop_rd = -1;
-    uint32_t n = wl_count(d, WL_IFACE);
-    for (uint32_t it = vb.x * blockDim.x + threadIdx.x; it < n; it += vb.nx * blockDim.x) {
-        long long i = d.list[WL_IFACE][it];
+    LIST_LOOP(WL_IFACE, f) {
+        long long i = d.list[WL_IFACE][it_f];
         int x, y, z;
         coords(d, i, x, y, z);
         double own_phi = d.phisrc[i];
@@ -2404,9 +2521,9 @@ __device__ __forceinline__ void interface_d(const Dev &d, const VB &vb) {
         double j0 = 0.0, j1 = 0.0, j2 = 0.0;
 #pragma unroll
         for (int q = 0; q < Q; ++q) {
-            j0 += cx(q) * fo[q];
-            j1 += cy(q) * fo[q];
-            j2 += cz(q) * fo[q];
+            if (cx(q)) j0 += cx(q) * fo[q];
+            if (cy(q)) j1 += cy(q) * fo[q];
+            if (cz(q)) j2 += cz(q) * fo[q];
         }
         double ux[3] = {j0 / rho_x - d.a[0], j1 / rho_x - d.a[1], j2 / rho_x - d.a[2]};
         // gas density of the boundary condition, raised by the Laplace pressure
@@ -2416,39 +2533,65 @@ __device__ __forceinline__ void interface_d(const Dev &d, const VB &vb) {
             unit_vec_d(nv, nc);
             rg = d.rho_g + (6.0 * d.sigma) * curvature_d(d, x, y, z, nc[0], nc[1], nc[2]);
         }
+        // the equilibrium sum f_eq,q + f_eq,qbar of the reconstruction is the
+        // same for both members of a pair: once per pair, with the
+        // collision's shared terms (collide_d_t), instead of up to four
+        // evaluations per direction
+        const double us15 = 1.5 * ((ux[0] * ux[0] + ux[1] * ux[1]) + ux[2] * ux[2]);
+        const double wg1 = wd(1) * rg, wg2 = wd(7) * rg;
+        double pull[Q], feb[Q];
+#pragma unroll
+        for (int q = 1; q < Q; ++q) pull[q] = (scl[q] == CL_L || scl[q] == CL_I) ? P::ld(d.fsrc, q, src[q], N) : 0.0;
+#pragma unroll
+        for (int q = 1; q < Q; ++q) {
+            if (opp(q) < q) continue;
+            double cu = 0.0, cn = 0.0;
+            bool first = true;
+            if (cx(q)) {
+                cu = cx(q) > 0 ? ux[0] : -ux[0];
+                cn = cx(q) > 0 ? nv[0] : -nv[0];
+                first = false;
+            }
+            if (cy(q)) {
+                cu = first ? (cy(q) > 0 ? ux[1] : -ux[1]) : (cy(q) > 0 ? cu + ux[1] : cu - ux[1]);
+                cn = first ? (cy(q) > 0 ? nv[1] : -nv[1]) : (cy(q) > 0 ? cn + nv[1] : cn - nv[1]);
+                first = false;
+            }
+            if (cz(q)) {
+                cu = first ? (cz(q) > 0 ? ux[2] : -ux[2]) : (cz(q) > 0 ? cu + ux[2] : cu - ux[2]);
+                cn = first ? (cz(q) > 0 ? nv[2] : -nv[2]) : (cz(q) > 0 ? cn + nv[2] : cn - nv[2]);
+            }
+            const double c3 = 3.0 * cu, s = (4.5 * cu) * cu, wg = q <= 6 ? wg1 : wg2;
+            feb[q] = wg * (((1.0 + c3) + s) - us15) + wg * (((1.0 - c3) + s) - us15);
+            feb[opp(q)] = cn;  // the pair's second slot carries c_q . n
+        }
         fp[0] = fo[0];
 #pragma unroll
         for (int q = 1; q < Q; ++q) {
-            int qb = opp(q);
+            const int qb = opp(q);
+            const bool lead = qb > q;
+            const double fe2 = lead ? feb[q] : feb[qb], cn = lead ? feb[qb] : -feb[q];
             if (scl[q] == CL_WALL || scl[q] == CL_O) {
                 double cuw = scl[q] == CL_O ? link_cuw(d, d.bodies[d.bid[src[q]]], x, y, z, q)
                                             : (d.walls_move ? wall_cuw(d, x, y, z, q) : 0.0);
                 fp[q] = fo[qb] + ((6.0 * wd(q)) * rho_x) * cuw;
-            } else if (scl[q] == CL_G) {
-                fp[q] = (feq_d(q, rg, ux) + feq_d(qb, rg, ux)) - fo[qb];
+            } else if (scl[q] == CL_G || cn < -d.deadband) {
+                fp[q] = fe2 - fo[qb];
             } else {
-                fp[q] = P::ld(d.fsrc, q, src[q], N);
+                fp[q] = pull[q];
             }
         }
-#pragma unroll
-        for (int q = 1; q < Q; ++q) {
-            double cn = (cx(q) * nv[0] + cy(q) * nv[1]) + cz(q) * nv[2];
-            if (cn < -d.deadband && scl[q] != CL_O && scl[q] != CL_WALL) {
-                int qb = opp(q);
-                fp[q] = (feq_d(q, rg, ux) + feq_d(qb, rg, ux)) - fo[qb];
-            }
-        }
+        // mass exchange with the neighbour x + c_q: the source of qbar, whose
+        // class and population are at hand
         double dm = 0.0;
 #pragma unroll
         for (int q = 1; q < Q; ++q) {
-            int qb = opp(q);
-            long long yi = nbr(d, x, y, z, cx(q), cy(q), cz(q));
-            int yc = cls(d, yi);
-            if (yc == CL_L) {
-                dm += P::ld(d.fsrc, qb, yi, N) - fo[q];
-            } else if (yc == CL_I) {
-                double wgt = 0.5 * (own_phi + d.phisrc[yi]);
-                dm += wgt * (P::ld(d.fsrc, qb, yi, N) - fo[q]);
+            const int qb = opp(q);
+            if (scl[qb] == CL_L) {
+                dm += pull[qb] - fo[q];
+            } else if (scl[qb] == CL_I) {
+                const double wgt = 0.5 * (own_phi + d.phisrc[src[qb]]);
+                dm += wgt * (pull[qb] - fo[q]);
             }
         }
         const double m_new = d.m[i] + dm;
@@ -2478,7 +2621,7 @@ template <int S> __device__ __forceinline__ void interface_body(const Dev &d, co
     else interface_trio<S>(d, vb);
 }
 template <int S>
-__global__ void __launch_bounds__(128, LBMFS_IFACE_MINB) k_interface(const __grid_constant__ Dev d) {
+__global__ void __launch_bounds__(128, S == 0 ? 2 : LBMFS_IFACE_MINB) k_interface(const __grid_constant__ Dev d) {
     interface_body<S>(d, vb_own());
 }
 
@@ -3175,7 +3318,7 @@ LBMFS_BATCH_BODY(BkLiquid, BULK_THREADS, S == 0 ? 1 : (LBMFS_BULK_PAIR ? LBMFS_P
 // the batch's listed cells are spread over many more blocks: 4 resident per SM
 // (128 registers) beat 1 there, not on the single tank
 template <int S> LBMFS_BATCH_BODY(BkGeneral, GEN_THREADS, 4, general_body<S>(d, vb))
-template <int S> LBMFS_BATCH_BODY(BkInterface, 128, LBMFS_IFACE_MINB, interface_body<S>(d, vb))
+template <int S> LBMFS_BATCH_BODY(BkInterface, 128, S == 0 ? 2 : LBMFS_IFACE_MINB, interface_body<S>(d, vb))
 LBMFS_BATCH_BODY(BkConvFilled, LIST_THREADS, 1, conv_filled_body(d, vb))
 LBMFS_BATCH_BODY(BkConvEmptied, LIST_THREADS, 1, conv_emptied_body(d, vb))
 template <int S> LBMFS_BATCH_BODY(BkConvInit, LIST_THREADS, 1, conv_init_body<S>(d, vb))
@@ -3204,6 +3347,21 @@ template <int S> void batch_bulk_launch(const BatchLaunch &b, cudaStream_t st) {
     }
 }
 
+// z-planes per block of the single-tank bulk kernel.  A thread steps its planes
+// one after another, so blocks of 8 planes suit only grids whose blocks still
+// fill the GPU several times over; on smaller ones a few threads would walk 8
+// dependent cells while SMs idle.  Measured (bulk kernel, us at 8 / 4 / 2 / 1
+// planes): 32^3 FP64 111 / 60 / 34 / 21, 96^3 FP64 308 / 304 / 304 / 288;
+// 96x32x32 FP32 27 / 17 / 12 / 10, 128^3 FP32 42 / 39 / 39 / 49, 385x190x127
+// FP16S 141 / 124 / 136 / 199; the 768x384x256 tank 2 % faster at 8 than at 4.
+inline int bulk_planes(int storage, unsigned gx, int nz) {
+    auto blocks = [&](int zb) { return (long long)gx * ((nz + zb - 1) / zb); };
+    if (storage == 0) return 1;  // bound by the double unit: the most even spread
+    if (blocks(8) >= 12000) return 8;
+    if (blocks(4) >= 12000) return 4;
+    return blocks(2) >= 2000 ? 2 : 1;
+}
+
 template <int S> struct Launch {
     static void init_cells(const Dev &d, const uint8_t *flags, const double *fill, const double *rho, const double *vel,
                            cudaStream_t st) {
@@ -3227,6 +3385,21 @@ template <int S> struct Launch {
             (mask & 4u) ? (double *)dst[2] : nullptr, (mask & 8u) ? (double *)dst[3] : nullptr,
             (mask & 16u) ? (double *)dst[4] : nullptr, (mask & 32u) ? (double *)dst[5] : nullptr);
     }
+    template <int ZB> static void bulk_zb(const Dev &d, unsigned gx, cudaStream_t st) {
+        k_liquid<S, ZB><<<dim3(gx, 1, (d.nz + ZB - 1) / ZB), BULK_THREADS, 0, st>>>(d);
+    }
+    // the bulk kernel with the z-planes per block of bulk_planes
+    static void bulk(const Dev &d, cudaStream_t st) {
+        const int bc = bulk_cells(S, d);
+        const unsigned gx = (unsigned)(((long long)d.nx * d.ny + bc - 1) / bc);
+        const int zb = bulk_planes(S, gx, d.nz);
+        if (zb == 1) bulk_zb<1>(d, gx, st);
+        if constexpr (S != 0) {
+            if (zb == 2) bulk_zb<2>(d, gx, st);
+            if (zb == 4) bulk_zb<4>(d, gx, st);
+            if (zb == 8) bulk_zb<8>(d, gx, st);
+        }
+    }
     // one time step; with ev != nullptr, event k is recorded before kernel k
     // and ev[count] after the last one
     static int step(const Dev &d, cudaStream_t st, float *, cudaEvent_t *ev) {
@@ -3241,18 +3414,15 @@ template <int S> struct Launch {
         if (d.nb > 0) k_forces<S><<<dim3(FORCE_BLOCKS, d.nb), dim3(32, 8), 0, st>>>(d);
         mark();
         {
-            const long long nxy = (long long)d.nx * d.ny;
-            const int bc = bulk_cells(S, d);
-            dim3 grid((unsigned)((nxy + bc - 1) / bc), 1, (d.nz + LBMFS_BULK_ZB - 1) / LBMFS_BULK_ZB);
             if constexpr (S != 0) {
                 // the staged variants tile rows: (ceil(nx / BULK_THREADS), ny, z-blocks)
                 dim3 rgrid((d.nx + BULK_THREADS - 1) / BULK_THREADS, d.ny, (d.nz + LBMFS_BULK_ZB - 1) / LBMFS_BULK_ZB);
                 dim3 pgrid(rgrid.x, rgrid.y, (d.nz + LBMFS_BULK_PIPE_ZB - 1) / LBMFS_BULK_PIPE_ZB);
                 if (d.bulk == BULK_TMA) k_liquid_tma<S><<<rgrid, BULK_THREADS, 128 + 2 * Stage<S>::BYTES, st>>>(d);
                 else if (d.bulk == BULK_PIPE) k_liquid_pipe<S><<<pgrid, BULK_THREADS, 0, st>>>(d);
-                else k_liquid<S><<<grid, BULK_THREADS, 0, st>>>(d);
+                else bulk(d, st);
             } else {
-                k_liquid<S><<<grid, BULK_THREADS, 0, st>>>(d);
+                bulk(d, st);
             }
         }
         mark();
