@@ -60,6 +60,27 @@ lbm_fs_status status_bits(uint32_t st) {
     return LBM_FS_OK;
 }
 
+cudaError_t Sides::create() {
+    int lo = 0, hi = 0;
+    cudaError_t e = cudaDeviceGetStreamPriorityRange(&lo, &hi);
+    for (int k = 0; k < SIDE_STREAMS && e == cudaSuccess; ++k) {
+        e = cudaStreamCreateWithPriority(&st[k], cudaStreamNonBlocking, hi);
+        if (e == cudaSuccess) e = cudaEventCreateWithFlags(&join[k], cudaEventDisableTiming);
+    }
+    if (e == cudaSuccess) e = cudaEventCreateWithFlags(&fork, cudaEventDisableTiming);
+    return e;
+}
+void Sides::destroy() {
+    for (int k = 0; k < SIDE_STREAMS; ++k) {
+        if (st[k]) cudaStreamDestroy(st[k]);
+        if (join[k]) cudaEventDestroy(join[k]);
+        st[k] = nullptr;
+        join[k] = nullptr;
+    }
+    if (fork) cudaEventDestroy(fork);
+    fork = nullptr;
+}
+
 void begin_mass(lbm_fs *h) {
     if (h->started) return;
     h->ks.liquid_mass(h->d[h->cur], h->st);
@@ -82,7 +103,7 @@ lbm_fs_status capture_graphs(lbm_fs *h) {
     for (int k = 0; k < 2; ++k) {
         cudaGraph_t g = nullptr;
         CK(cudaStreamBeginCapture(h->cap_st, cudaStreamCaptureModeThreadLocal));
-        h->per_step = h->ks.step(h->d[k], h->cap_st, nullptr, nullptr);
+        h->per_step = h->ks.step(h->d[k], h->cap_st, &h->sides, nullptr);
         cudaError_t e = cudaStreamEndCapture(h->cap_st, &g);
         if (e != cudaSuccess) return cuda_fail(e, "cudaStreamEndCapture");
         e = cudaGraphInstantiate(&h->gexec[k], g, 0);
@@ -170,6 +191,7 @@ lbm_fs_status lbm_fs_create(const lbm_fs_params *p, lbm_fs **out) {
         return s;
     };
     cudaError_t e = cudaStreamCreateWithFlags(&h->cap_st, cudaStreamNonBlocking);
+    if (e == cudaSuccess && p->use_graphs) e = h->sides.create();
     if (e != cudaSuccess) return bail(cuda_fail(e, "cudaStreamCreate"));
 
     Dev d{};
@@ -224,12 +246,18 @@ lbm_fs_status lbm_fs_create(const lbm_fs_params *p, lbm_fs **out) {
     double *pA = (double *)h->alloc(N * 8), *pB = (double *)h->alloc(N * 8);
     d.m = (double *)h->alloc(N * 8);
     for (int k = 0; k < WL_COUNT; ++k) d.list[k] = (uint32_t *)h->alloc(N * 4);
-    d.cnt = (uint32_t *)h->alloc(WL_COUNT * 4);
-    d.bodies = (Body *)h->alloc(sizeof(Body) * MAX_BODIES);
+    // what a step reads of the one before it: second copies of some lists, of
+    // the counters and of the body records
+    uint32_t *list2[PREV_LISTS];
+    for (int k = 0; k < PREV_LISTS; ++k) list2[k] = (uint32_t *)h->alloc(N * 4);
+    d.cnt = (uint32_t *)h->alloc(2 * CN_COUNT * 4);
+    d.bodies = (Body *)h->alloc(2 * sizeof(Body) * MAX_BODIES);
+    const size_t pfb = p->storage == LBM_FS_F64 ? 0 : (size_t)N * 4;
+    float *pfA = (float *)h->alloc(pfb), *pfB = (float *)h->alloc(pfb);
     d.part = (double *)h->alloc(2 * sizeof(double) * MAX_BODIES * FORCE_BLOCKS * 7);
     d.part128 = p->storage == LBM_FS_F64;
     d.ledger = (double *)h->alloc(sizeof(double) * LG_COUNT);
-    d.status = (uint32_t *)h->alloc(4);
+    d.status = (uint32_t *)h->alloc(16);
     d.rdec = (uint8_t *)h->alloc(nb4);
     d.rrho = (double *)h->alloc(N * 8);
     d.rphi = (double *)h->alloc(N * 8);
@@ -239,7 +267,7 @@ lbm_fs_status lbm_fs_create(const lbm_fs_params *p, lbm_fs **out) {
     int *ztop = (int *)h->alloc(sizeof(int) * 2);
     for (void *ptr : h->allocs)
         if (!ptr) return bail(fail(LBM_FS_ENOMEM, "device allocation failed%s"));
-    if (h->allocs.size() != 19 + WL_COUNT) return bail(fail(LBM_FS_ENOMEM, "device allocation failed%s"));
+    if (h->allocs.size() != 21 + WL_COUNT + PREV_LISTS) return bail(fail(LBM_FS_ENOMEM, "device allocation failed%s"));
     if (h->misaligned) return bail(fail(LBM_FS_EINVAL, "dev_alloc must return 16-byte aligned memory%s"));
     d.walls_move = 0;
     for (int f = 0; f < 6; ++f)
@@ -257,9 +285,12 @@ lbm_fs_status lbm_fs_create(const lbm_fs_params *p, lbm_fs **out) {
     CKB(cudaMemsetAsync(pA, 0, N * 8, st));
     CKB(cudaMemsetAsync(pB, 0, N * 8, st));
     CKB(cudaMemsetAsync(d.m, 0, N * 8, st));
-    CKB(cudaMemsetAsync(d.cnt, 0, WL_COUNT * 4, st));
+    CKB(cudaMemsetAsync(pfA, 0, pfb, st));
+    CKB(cudaMemsetAsync(pfB, 0, pfb, st));
+    CKB(cudaMemsetAsync(d.cnt, 0, 2 * CN_COUNT * 4, st));
+    CKB(cudaMemsetAsync(d.bodies, 0, 2 * sizeof(Body) * MAX_BODIES, st));
     CKB(cudaMemsetAsync(d.ledger, 0, sizeof(double) * LG_COUNT, st));
-    CKB(cudaMemsetAsync(d.status, 0, 4, st));
+    CKB(cudaMemsetAsync(d.status, 0, 16, st));
     CKB(cudaMemsetAsync(d.part, 0, 2 * sizeof(double) * MAX_BODIES * FORCE_BLOCKS * 7, st));
     CKB(cudaMemcpyAsync(wallv, &p->wall_vel[0][0], sizeof(double) * 18, cudaMemcpyHostToDevice, st));
     // the first step visits every tile (its read slot: nz) and records the top
@@ -268,6 +299,19 @@ lbm_fs_status lbm_fs_create(const lbm_fs_params *p, lbm_fs **out) {
     h->d[0] = d;
     h->d[1] = d;
     set_grids(h, fA, fB, pA, pB);
+    for (int k = 0; k < 2; ++k) {
+        Dev &e = h->d[k];
+        e.phifsrc = k ? pfB : pfA;
+        e.phifdst = k ? pfA : pfB;
+        e.bodies = d.bodies + k * MAX_BODIES;
+        e.bodies_new = d.bodies + (k ^ 1) * MAX_BODIES;
+        e.cnt = d.cnt + k * CN_COUNT;
+        e.pcnt = d.cnt + (k ^ 1) * CN_COUNT;
+        for (int j = 0; j < PREV_LISTS; ++j) {
+            if (k) e.list[prev_wl(j)] = list2[j];
+            e.plist[j] = k ? d.list[prev_wl(j)] : list2[j];
+        }
+    }
     h->d[0].ztop_rd = ztop;
     h->d[0].ztop_wr = ztop + 1;
     h->d[1].ztop_rd = ztop + 1;
@@ -342,7 +386,7 @@ lbm_fs_status lbm_fs_add_box(lbm_fs *h, const lbm_fs_box *b, int32_t *out_id) {
     hb.shape = b->shape;
     int id = h->nb;
     cudaStream_t st = h->st;
-    CK(cudaMemcpyAsync(h->d[0].bodies + id, &hb, sizeof hb, cudaMemcpyHostToDevice, st));
+    CK(cudaMemcpyAsync(h->d[h->cur].bodies + id, &hb, sizeof hb, cudaMemcpyHostToDevice, st));
     CK(cudaStreamSynchronize(st));
     h->nb++;
     for (int k = 0; k < 2; ++k) h->d[k].nb = h->nb;
@@ -392,7 +436,7 @@ lbm_fs_status lbm_fs_body_state(lbm_fs *h, int32_t id, lbm_fs_body_state_t *out)
     if (id < 0 || id >= h->nb || !out) return fail(LBM_FS_EINVAL, "bad body id%s");
     CK(cudaStreamSynchronize(h->st));
     Body hb;
-    CK(cudaMemcpy(&hb, h->d[0].bodies + id, sizeof hb, cudaMemcpyDeviceToHost));
+    CK(cudaMemcpy(&hb, h->d[h->cur].bodies + id, sizeof hb, cudaMemcpyDeviceToHost));
     for (int k = 0; k < 3; ++k) {
         out->F[k] = hb.F[k];
         out->T[k] = hb.T[k];
@@ -413,7 +457,7 @@ lbm_fs_status lbm_fs_body_states(lbm_fs *h, int32_t first, int32_t count, lbm_fs
     if (count == 0) return read_status(h);
     std::vector<Body> hb(count);
     uint32_t st = 0;  // the status word comes with the bodies: one synchronisation
-    CK(cudaMemcpyAsync(hb.data(), h->d[0].bodies + first, sizeof(Body) * count, cudaMemcpyDeviceToHost, h->st));
+    CK(cudaMemcpyAsync(hb.data(), h->d[h->cur].bodies + first, sizeof(Body) * count, cudaMemcpyDeviceToHost, h->st));
     CK(cudaMemcpyAsync(&st, h->d[0].status, sizeof st, cudaMemcpyDeviceToHost, h->st));
     CK(cudaStreamSynchronize(h->st));
     for (int32_t b = 0; b < count; ++b) {
@@ -489,9 +533,10 @@ lbm_fs_status lbm_fs_stats(lbm_fs *h, lbm_fs_stats_t *out) {
     CK(cudaGetLastError());
     CK(cudaStreamSynchronize(st));
     double lg[LG_COUNT];
-    uint32_t cnt[WL_COUNT], status;
+    uint32_t cnt[CN_COUNT], status;
     CK(cudaMemcpy(lg, h->d[0].ledger, sizeof lg, cudaMemcpyDeviceToHost));
-    CK(cudaMemcpy(cnt, h->d[0].cnt, sizeof cnt, cudaMemcpyDeviceToHost));
+    memset(cnt, 0, sizeof cnt);
+    if (h->step > 0) CK(cudaMemcpy(cnt, h->d[h->cur ^ 1].cnt, sizeof cnt, cudaMemcpyDeviceToHost));  // of the last step
     CK(cudaMemcpy(&status, h->d[0].status, sizeof status, cudaMemcpyDeviceToHost));
     memset(out, 0, sizeof *out);
     out->step = h->step;
@@ -509,7 +554,7 @@ lbm_fs_status lbm_fs_stats(lbm_fs *h, lbm_fs_stats_t *out) {
     out->status = status;
     out->kernel_launches = h->launches;
     out->wall_source = lg[LG_WALL];
-    out->n_general = cnt[WL_GEN];
+    out->n_general = cnt[CN_NEAR];
     return read_status(h);
 }
 

@@ -47,6 +47,7 @@ struct lbm_fs_batch {
     int bulk_blocks = 0;  // 0: one block per bulk tile
     int list_cells = LIST_CELLS_DEFAULT;
     int lanes = 1;  // groups of tanks whose step chains run concurrently
+    Sides sides;    // one lane: the kernels that run beside the bulk kernel
     cudaStream_t lane_st[MAX_LANES] = {};
     cudaEvent_t fork_ev = nullptr, join_ev[MAX_LANES] = {};
     std::vector<std::unique_ptr<Chunk>> chunks;
@@ -107,7 +108,7 @@ Tile tile(int tank, int x, int y, int z, int nx, int ny, int nz) {
     t.nx = (uint16_t)nx;
     t.ny = (uint16_t)ny;
     t.nz = (uint16_t)nz;
-    t.pad = 0;
+    t.kind = 0;
     return t;
 }
 
@@ -143,6 +144,15 @@ lbm_fs_status build(lbm_fs_batch *b) {
             for (int x = 0; x < lb; ++x) tb[SH_LIST].push_back(tile(j, x, 0, 0, lb, 1, 1));
             for (int x = 0; x < nb; ++x) tb[SH_BODY].push_back(tile(j, x, 0, 0, nb, 1, 1));
             if (nb > 0) tb[SH_ONE].push_back(tile(j, 0, 0, 0, 1, 1, 1));
+            for (int y = 0; y < nb; ++y)
+                for (int x = 0; x < FORCE_BLOCKS; ++x) tb[SH_GEN].push_back(tile(j, x, y, 0, FORCE_BLOCKS, nb, 1));
+            if (d.walls_move) {
+                for (int x = 0; x < 2 * lb; ++x) {
+                    Tile t2 = tile(j, x, 0, 0, 2 * lb, 1, 1);
+                    t2.kind = 1;
+                    tb[SH_GEN].push_back(t2);
+                }
+            }
         }
         for (int s = 0; s < SH_COUNT; ++s) {
             offs.push_back(all.size());
@@ -215,20 +225,22 @@ void make_chunks(lbm_fs_batch *b) {
     b->built = false;
 }
 
-// One step of every tank.  With several lanes the lanes' launch chains fork
-// from st and join back into it, so their kernels may run at the same time
-// (one lane's short list kernels beside another's bulk kernel).
-int enqueue_step(lbm_fs_batch *b, int parity, cudaStream_t st) {
+// One step of every tank.  With one lane and `sides`, the kernels that do not
+// depend on the bulk kernel run beside it.  With several lanes the lanes'
+// launch chains fork from st and join back into it, so their kernels may run
+// at the same time (one lane's short list kernels beside another's bulk
+// kernel).
+int enqueue_step(lbm_fs_batch *b, int parity, cudaStream_t st, const Sides *sides) {
     int n = 0;
     if (b->lanes == 1) {
-        for (auto &cp : b->chunks) n += b->ks.batch_step(launch_of(b, *cp, parity), st, nullptr);
+        for (auto &cp : b->chunks) n += b->ks.batch_step(launch_of(b, *cp, parity), st, sides, nullptr);
         return n;
     }
     cudaEventRecord(b->fork_ev, st);
     for (int l = 0; l < b->lanes; ++l) {
         cudaStreamWaitEvent(b->lane_st[l], b->fork_ev, 0);
         for (auto &cp : b->chunks)
-            if (cp->lane == l) n += b->ks.batch_step(launch_of(b, *cp, parity), b->lane_st[l], nullptr);
+            if (cp->lane == l) n += b->ks.batch_step(launch_of(b, *cp, parity), b->lane_st[l], nullptr, nullptr);
         cudaEventRecord(b->join_ev[l], b->lane_st[l]);
         cudaStreamWaitEvent(st, b->join_ev[l], 0);
     }
@@ -240,7 +252,7 @@ lbm_fs_status capture(lbm_fs_batch *b) {
     for (int k = 0; k < 2; ++k) {
         cudaGraph_t g = nullptr;
         CK(cudaStreamBeginCapture(b->cap_st, cudaStreamCaptureModeThreadLocal));
-        b->per_step = enqueue_step(b, k, b->cap_st);
+        b->per_step = enqueue_step(b, k, b->cap_st, &b->sides);
         cudaError_t e = cudaStreamEndCapture(b->cap_st, &g);
         if (e != cudaSuccess) return cuda_fail(e, "cudaStreamEndCapture (batch)");
         e = cudaGraphInstantiate(&b->gexec[k], g, 0);
@@ -286,6 +298,7 @@ void destroy_all(lbm_fs_batch *b) {
         if (b->join_ev[l]) cudaEventDestroy(b->join_ev[l]);
     }
     if (b->fork_ev) cudaEventDestroy(b->fork_ev);
+    b->sides.destroy();
     delete b;
 }
 
@@ -315,6 +328,7 @@ lbm_fs_status lbm_fs_batch_create(const lbm_fs_params *params, int32_t count, lb
         if (e == cudaSuccess) e = cudaEventCreateWithFlags(&b->join_ev[l], cudaEventDisableTiming);
     }
     if (e == cudaSuccess) e = cudaEventCreateWithFlags(&b->fork_ev, cudaEventDisableTiming);
+    if (e == cudaSuccess && b->use_graphs) e = b->sides.create();
     if (e != cudaSuccess) {
         destroy_all(b);
         return cuda_fail(e, "cudaStreamCreate (batch)");
@@ -376,7 +390,7 @@ lbm_fs_status lbm_fs_batch_step(lbm_fs_batch *b, int32_t nsteps) {
         if (b->use_graphs) {
             CK(cudaGraphLaunch(b->gexec[b->cur], b->st));
         } else {
-            n = enqueue_step(b, b->cur, b->st);
+            n = enqueue_step(b, b->cur, b->st, nullptr);
             CK(cudaGetLastError());
         }
         advance(b, n);
@@ -443,12 +457,12 @@ lbm_fs_status lbm_fs_batch_autotune(lbm_fs_batch *b, lbm_fs_batch_config_t *out)
     // the timed launches append interface cells and may book moving-wall
     // mass: keep the counters and ledgers and put them back afterwards
     std::vector<double> ledgers((size_t)nt * LG_COUNT);
-    std::vector<uint32_t> counters((size_t)nt * WL_COUNT);
+    std::vector<uint32_t> counters((size_t)nt * 2 * CN_COUNT);
     CK(cudaStreamSynchronize(b->st));
     for (int k = 0; k < nt; ++k) {
         CK(cudaMemcpy(&ledgers[(size_t)k * LG_COUNT], b->tanks[k]->d[0].ledger, sizeof(double) * LG_COUNT,
                       cudaMemcpyDeviceToHost));
-        CK(cudaMemcpy(&counters[(size_t)k * WL_COUNT], b->tanks[k]->d[0].cnt, sizeof(uint32_t) * WL_COUNT,
+        CK(cudaMemcpy(&counters[(size_t)k * 2 * CN_COUNT], b->tanks[k]->d[0].cnt, sizeof(uint32_t) * 2 * CN_COUNT,
                       cudaMemcpyDeviceToHost));
     }
     const int keep_zb = b->zb, keep_blocks = b->bulk_blocks;
@@ -472,7 +486,7 @@ lbm_fs_status lbm_fs_batch_autotune(lbm_fs_batch *b, lbm_fs_batch_config_t *out)
             if (err) break;
             // one warm-up and five timed launches append at most six times a
             // tank's interface cells to its list (capacity: one entry per cell)
-            for (lbm_fs *t : b->tanks) cudaMemsetAsync(t->d[0].cnt, 0, sizeof(uint32_t) * WL_COUNT, b->st);
+            for (lbm_fs *t : b->tanks) cudaMemsetAsync(t->d[b->cur].cnt, 0, sizeof(uint32_t) * CN_COUNT, b->st);
             const int reps = 5;
             for (auto &cp : b->chunks) b->ks.batch_bulk(launch_of(b, *cp, b->cur), b->st);
             cudaEventRecord(e0, b->st);
@@ -500,7 +514,7 @@ lbm_fs_status lbm_fs_batch_autotune(lbm_fs_batch *b, lbm_fs_batch_config_t *out)
     for (int k = 0; k < nt; ++k) {
         CK(cudaMemcpyAsync(b->tanks[k]->d[0].ledger, &ledgers[(size_t)k * LG_COUNT], sizeof(double) * LG_COUNT,
                            cudaMemcpyHostToDevice, b->st));
-        CK(cudaMemcpyAsync(b->tanks[k]->d[0].cnt, &counters[(size_t)k * WL_COUNT], sizeof(uint32_t) * WL_COUNT,
+        CK(cudaMemcpyAsync(b->tanks[k]->d[0].cnt, &counters[(size_t)k * 2 * CN_COUNT], sizeof(uint32_t) * 2 * CN_COUNT,
                            cudaMemcpyHostToDevice, b->st));
     }
     CK(cudaStreamSynchronize(b->st));
@@ -527,14 +541,14 @@ lbm_fs_status lbm_fs_batch_kernel_times(lbm_fs_batch *b, int32_t nsteps, double 
     if (nsteps <= 0 || !ms || cap <= 0) return fail(LBM_FS_EINVAL, "bad arguments%s");
     s = prepare(b);
     if (s) return s;
-    const int K = b->ks.nkernels;
+    const int K = b->ks.batch_kernels;
     std::vector<cudaEvent_t> ev(K + 1);
     for (auto &x : ev) CK(cudaEventCreate(&x));
     std::vector<double> acc(K, 0.0);
     for (int32_t it = 0; it < nsteps; ++it) {
         int n = 0;
         for (auto &cp : b->chunks) {
-            n += b->ks.batch_step(launch_of(b, *cp, b->cur), b->st, ev.data());
+            n += b->ks.batch_step(launch_of(b, *cp, b->cur), b->st, nullptr, ev.data());
             CK(cudaGetLastError());
             CK(cudaEventSynchronize(ev[K]));
             for (int k = 0; k < K; ++k) {
@@ -549,7 +563,7 @@ lbm_fs_status lbm_fs_batch_kernel_times(lbm_fs_batch *b, int32_t nsteps, double 
     int m = K < cap ? K : cap;
     for (int k = 0; k < m; ++k) {
         ms[k] = acc[k];
-        if (names) names[k] = b->ks.names[k];
+        if (names) names[k] = b->ks.batch_names[k];
     }
     if (nk) *nk = K;
     return lbm_fs_batch_sync(b);

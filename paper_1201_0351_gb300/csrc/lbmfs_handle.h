@@ -15,6 +15,7 @@ struct lbm_fs {
     int cur = 0;
     cudaStream_t st = nullptr;
     cudaStream_t cap_st = nullptr;
+    lbmfs::Sides sides;
     std::vector<void *> allocs;
     int nb = 0;
     bool started = false;
@@ -49,6 +50,7 @@ struct lbm_fs {
         }
         allocs.clear();
         if (cap_st) cudaStreamDestroy(cap_st);
+        sides.destroy();
     }
 };
 

@@ -27,8 +27,9 @@ constexpr int BULK_THREADS = LBMFS_BULK_THREADS;  // x extent of a bulk-kernel b
 #endif
 
 // cell classes (as in the C ABI) in the low nibble of the flag byte; bit 4
-// marks a cell with an obstacle or a wall among its 18 neighbours
-enum : uint8_t { CL_L = 1, CL_I = 2, CL_G = 4, CL_O = 8, CL_MASK = 15, NB_OBST = 16 };
+// marks a cell with an obstacle among its 18 neighbours, bit 5 a cell on a face
+// of a grid with moving walls
+enum : uint8_t { CL_L = 1, CL_I = 2, CL_G = 4, CL_O = 8, CL_MASK = 15, NB_OBST = 16, MOVING_FACE = 32 };
 // per-cell conversion marks (separate byte array, zero between steps)
 enum : uint8_t {
     MK_FILLED = 1, MK_EMPTIED = 2, MK_NEWG = 4, MK_NEWL = 8, MK_RECV = 16, MK_PEND = 32, MK_FRESH = 64
@@ -40,7 +41,17 @@ enum : uint32_t { ST_LIQUID_GAS = 1, ST_NONFINITE = 2, ST_OVERFLOW = 4, ST_TIMEO
 constexpr int ZTOP_MARGIN = 4;
 
 // worklists
-enum { WL_IFACE = 0, WL_FILLED, WL_EMPTIED, WL_NEWG, WL_NEWL, WL_RECV, WL_PEND, WL_COVER, WL_GEN, WL_COUNT };
+enum { WL_IFACE = 0, WL_FILLED, WL_EMPTIED, WL_NEWG, WL_NEWL, WL_RECV, WL_PEND, WL_COVER, WL_COUNT };
+// counters of a step: one per worklist, then the liquid cells next to a body or
+// on a moving wall
+enum { CN_NEAR = WL_COUNT, CN_COUNT = 16 };
+// lists of the previous step that hold every cell that may be interface now:
+// the interface cells its bulk pass met and those its conversions and its
+// remap may have added
+constexpr int PREV_LISTS = 4;
+__host__ __device__ constexpr int prev_wl(int k) {
+    return k == 0 ? WL_IFACE : (k == 1 ? WL_NEWG : (k == 2 ? WL_NEWL : WL_PEND));
+}
 // ledger slots (double)
 enum { LG_COVERED = 0, LG_UNCOVERED, LG_LOST, LG_MASS0, LG_MASS, LG_WALL, LG_COUNT };
 
@@ -69,15 +80,18 @@ struct Dev {
     uint8_t *flags, *bid, *cmark;
     void *fsrc, *fdst;
     double *phisrc, *phidst, *m;
+    float *phifsrc, *phifdst;  // the fill levels rounded to float (float storages: no double conversion per read)
     uint32_t *list[WL_COUNT];
-    uint32_t *cnt;  // WL_COUNT counters
+    uint32_t *cnt;   // CN_COUNT counters of this step
+    const uint32_t *plist[PREV_LISTS];  // the previous step's lists prev_wl(k)
+    uint32_t *pcnt;  // and its counters
     uint32_t cap;
-    Body *bodies;
+    Body *bodies, *bodies_new;  // body states before and after this step's rigid-body update
     int nb;
     double *part;   // force partials: MAX_BODIES * FORCE_BLOCKS * 7 slots of 16 bytes
     int part128;    // partials are exact 128-bit fixed-point sums (double storage)
     double *ledger; // LG_COUNT
-    uint32_t *status;
+    uint32_t *status;  // [0] sticky bits, [1], [2] the tail kernel's grid barrier
     uint8_t *rdec;  // remap scratch: decision per pending item
     double *rrho, *rphi;
     double *red;    // reduction scratch
@@ -118,7 +132,7 @@ struct TankSet {
 static_assert(sizeof(TankSet) + 64 <= 32764, "tank descriptors must fit the kernel parameter space");
 
 struct Tile {
-    uint16_t tank, x, y, z, nx, ny, nz, pad;  // tank; block (x, y, z) of a (nx, ny, nz) grid
+    uint16_t tank, x, y, z, nx, ny, nz, kind;  // tank; block (x, y, z) of a (nx, ny, nz) grid; see SH_GEN
 };
 
 // block tables by launch shape
@@ -130,6 +144,7 @@ enum {
     SH_BODY,       // (bodies): rigid-body step
     SH_ONE,        // (1) per tank with bodies: remap resolution
     SH_TANK,       // (1) per tank: counter reset
+    SH_GEN,        // liquid cells next to bodies: (FORCE_BLOCKS, bodies), kind 0; on moving walls: (2 lb), kind 1
     SH_COUNT
 };
 struct Shape {
@@ -142,6 +157,17 @@ struct BatchLaunch {
     Shape sh[SH_COUNT];
     int zb;             // z-planes per bulk tile
 };
+// Streams (and events to fork to and join from them) on which a step's kernels
+// that do not depend on the bulk kernel run beside it.  They are created with
+// the highest priority: the bulk kernel fills every SM, and its thousands of
+// waiting blocks would otherwise all go first.
+constexpr int SIDE_STREAMS = 3;
+struct Sides {
+    cudaStream_t st[SIDE_STREAMS] = {};
+    cudaEvent_t fork = nullptr, join[SIDE_STREAMS] = {};
+    cudaError_t create();
+    void destroy();
+};
 
 struct KernelSet {
     void (*init_cells)(const Dev &, const uint8_t *flags, const double *fill, const double *rho, const double *vel,
@@ -149,17 +175,20 @@ struct KernelSet {
     void (*body_prepare)(const Dev &, int b, cudaStream_t);
     void (*map_body)(const Dev &, int b, int book_mass, cudaStream_t);
     // one time step, in order; returns the number of kernels launched
-    int (*step)(const Dev &, cudaStream_t, float *ev_ms, cudaEvent_t *ev);
+    // (with sides: as a fork and join of independent chains, else in one chain)
+    int (*step)(const Dev &, cudaStream_t, const Sides *sides, cudaEvent_t *ev);
     void (*liquid_mass)(const Dev &, cudaStream_t);  // -> ledger[LG_MASS]
     void (*read_fields)(const Dev &, unsigned mask, void *const *dst, cudaStream_t);
-    // one time step of every tank of a batch chunk; same event protocol and
-    // kernel slots as step
-    int (*batch_step)(const BatchLaunch &, cudaStream_t, cudaEvent_t *ev);
+    // one time step of every tank of a batch chunk; same event protocol, with
+    // the batch's kernel slots
+    int (*batch_step)(const BatchLaunch &, cudaStream_t, const Sides *sides, cudaEvent_t *ev);
     // the bulk kernel alone over a chunk (autotuning), and its occupancy
     void (*batch_bulk)(const BatchLaunch &, cudaStream_t);
     int (*bulk_blocks_per_sm)();
-    int nkernels;
+    int nkernels;              // slots of step, and their names
     const char *const *names;
+    int batch_kernels;         // slots of batch_step
+    const char *const *batch_names;
 };
 
 // cells of an xy-plane per bulk-kernel block: two per thread for the float

@@ -428,7 +428,7 @@ __device__ __forceinline__ void coords(const Dev &d, long long idx, int &x, int 
 __device__ __forceinline__ int clsv(const Dev &d, long long i) { return (int)(d.flags[i] & CL_MASK); }
 __device__ __forceinline__ int cls(const Dev &d, long long i) { return i < 0 ? CL_WALL : clsv(d, i); }
 __device__ __forceinline__ void set_cls(const Dev &d, long long i, int c) {
-    d.flags[i] = (uint8_t)((d.flags[i] & NB_OBST) | c);
+    d.flags[i] = (uint8_t)((d.flags[i] & ~CL_MASK) | c);
 }
 
 // warp-aggregated append of val to a worklist
@@ -449,6 +449,46 @@ __device__ __forceinline__ void wl_append(const Dev &d, bool pred, int list, uin
 __device__ __forceinline__ uint32_t wl_count(const Dev &d, int list) {
     uint32_t c = *reinterpret_cast<volatile uint32_t *>(&d.cnt[list]);
     return c < d.cap ? c : d.cap;
+}
+
+// components of a direction known at run time only (a lane's), 2 bits each
+__host__ __device__ constexpr unsigned long long dir_bits(int axis) {
+    unsigned long long b = 0;
+    for (int q = 0; q < Q; ++q)
+        b |= (unsigned long long)((axis == 0 ? cx(q) : (axis == 1 ? cy(q) : cz(q))) + 1) << (2 * q);
+    return b;
+}
+__device__ __forceinline__ int dir_x(int q) { return (int)((dir_bits(0) >> (2 * q)) & 3u) - 1; }
+__device__ __forceinline__ int dir_y(int q) { return (int)((dir_bits(1) >> (2 * q)) & 3u) - 1; }
+__device__ __forceinline__ int dir_z(int q) { return (int)((dir_bits(2) >> (2 * q)) & 3u) - 1; }
+
+// The cells that may be interface in this step: the interface cells that the
+// previous step's bulk pass met, then those its conversions (from gas, from
+// liquid) and its remap may have added, as one sequence.  The sets are
+// disjoint (a cell was interface, gas, liquid or obstacle at the start of that
+// step); an entry whose class is no longer interface is passed over.  So the
+// interface kernel needs no list from this step's bulk pass and runs beside
+// it.
+struct IfaceSeq {
+    uint32_t e[PREV_LISTS];  // ends of the parts
+};
+__device__ __forceinline__ IfaceSeq iface_seq(const Dev &d) {
+    IfaceSeq r;
+    uint32_t t = 0;
+#pragma unroll
+    for (int k = 0; k < PREV_LISTS; ++k) {
+        const uint32_t c = d.pcnt[prev_wl(k)];
+        t += c < d.cap ? c : d.cap;
+        r.e[k] = t;
+    }
+    return r;
+}
+__device__ __forceinline__ uint32_t iface_cell(const Dev &d, const IfaceSeq &r, uint32_t it) {
+    const uint32_t *p = d.plist[0] + it;
+#pragma unroll
+    for (int k = 1; k < PREV_LISTS; ++k)
+        if (it >= r.e[k - 1]) p = d.plist[k] + (it - r.e[k - 1]);
+    return *p;
 }
 
 // atomic OR / AND on one byte of the mark array; returns the old byte
@@ -892,8 +932,11 @@ template <int S>
 __global__ void k_init(Dev d, const uint8_t *flags, const double *fill, const double *rho, const double *vel) {
     long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x;
     if (i >= d.N) return;
-    int c = flags[i];
-    d.flags[i] = (uint8_t)c;
+    const int c = flags[i] & CL_MASK;
+    int x, y, z;
+    coords(d, i, x, y, z);
+    const bool face = x == 0 || x == d.nx - 1 || y == 0 || y == d.ny - 1 || z == 0 || z == d.nz - 1;
+    d.flags[i] = (uint8_t)(c | (face && d.walls_move ? MOVING_FACE : 0));
     d.bid[i] = 0;
     d.cmark[i] = 0;
     if (c != CL_L && c != CL_I) return;
@@ -912,7 +955,15 @@ __global__ void k_init(Dev d, const uint8_t *flags, const double *fill, const do
         double m = fill[i] * r;
         d.m[i] = m;
         d.phisrc[i] = m / r;
+        if constexpr (S != 0) d.phifsrc[i] = (float)(m / r);
     }
+}
+
+// the initial interface cells as the first step's list (d.list, d.cnt: those
+// of the step before the first)
+__global__ void k_list_interface(Dev d) {
+    const long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x;
+    wl_append(d, i < d.N && clsv(d, i) == CL_I, WL_IFACE, (uint32_t)i);
 }
 
 // rotation matrix and the cell range that may lie inside the body
@@ -970,6 +1021,24 @@ __device__ __forceinline__ void range_cell(const Dev &d, const int *lo, const in
     if (z < 0 || z >= d.nz) z = ((z % d.nz) + d.nz) % d.nz;
 }
 
+// the cells of the body's range and one beyond it (all that may have an
+// obstacle of the body among their neighbours)
+__device__ __forceinline__ void near_range(const Dev &d, const Body &b, int *lo, int *hi) {
+    const int n3[3] = {d.nx, d.ny, d.nz};
+#pragma unroll
+    for (int k = 0; k < 3; ++k) {
+        lo[k] = b.lo[k] - 1;
+        hi[k] = b.hi[k] + 1;
+        if (!(d.periodic & (1u << k))) {
+            lo[k] = lo[k] < 0 ? 0 : lo[k];
+            hi[k] = hi[k] > n3[k] ? n3[k] : hi[k];
+        } else if (hi[k] - lo[k] > n3[k]) {
+            hi[k] = lo[k] + n3[k];
+        }
+        if (hi[k] < lo[k]) hi[k] = lo[k];  // a body that has left the grid through a wall has no cells
+    }
+}
+
 // mapping of a newly added body (Sec. 2.3); book_mass: charge the covered mass
 template <int S>
 __global__ void k_map_body(Dev d, int bi, int book_mass) {
@@ -993,19 +1062,22 @@ __global__ void k_map_body(Dev d, int bi, int book_mass) {
 // Coordinates a kernel body runs at: its launch's own block, or one entry of
 // a packed block table when a single launch serves many tanks
 struct VB {
-    unsigned x, y, z, nx, ny, nz;
+    unsigned x, y, z, nx, ny, nz, kind;
 };
-__device__ __forceinline__ VB vb_own() { return VB{blockIdx.x, blockIdx.y, blockIdx.z, gridDim.x, gridDim.y, gridDim.z}; }
+__device__ __forceinline__ VB vb_own() {
+    return VB{blockIdx.x, blockIdx.y, blockIdx.z, gridDim.x, gridDim.y, gridDim.z, 0};
+}
 
 // A worklist's items spread over a launch's blocks, a warp's worth (`per` items)
-// at a time: as few warps of each block as hold the list, so that a short list
-// gets an SM per warp (its latency chains, and in double arithmetic the 2
-// operations per SM and cycle, don't queue behind one another) and a long list
-// keeps neighbouring items in one block.  First item of the calling warp and
+// at a time.  A short list goes to as many blocks (SMs) as possible: its
+// latency chains and its double operations, each of which holds a scheduler
+// for 64 cycles, don't queue behind one another.  From a group per SM up the
+// blocks fill their warps, so that a long list's blocks are few and full and
+// keep neighbouring items together.  First item of the calling warp and
 // the stride; a warp without items starts at n.
 __device__ __forceinline__ void list_span(const VB &vb, uint32_t n, uint32_t per, uint32_t &first, uint32_t &stride) {
     const uint32_t wpb = blockDim.x >> 5, warp = threadIdx.x >> 5;
-    const uint32_t groups = (n + per - 1) / per, used = min(wpb, (groups + vb.nx - 1) / vb.nx);
+    const uint32_t groups = (n + per - 1) / per, wide = min(vb.nx, 152u), used = min(wpb, (groups + wide - 1) / wide);
     first = warp < used ? (vb.x * used + warp) * per : n;
     stride = vb.nx * used * per;
 }
@@ -1014,6 +1086,72 @@ __device__ __forceinline__ void list_span(const VB &vb, uint32_t n, uint32_t per
     uint32_t f_##var, s_##var;                                                                                 \
     list_span(vb, n_##var, 32u, f_##var, s_##var);                                                             \
     for (uint32_t it_##var = f_##var + (threadIdx.x & 31u); it_##var < n_##var; it_##var += s_##var)
+
+// Walk over the cells around a body (its range of ncell cells, lo .. hi) that
+// satisfy `want(flag byte)`, by `blocks` blocks.  Few cells of the range are
+// next to the body's surface, and those come in whole rows and planes: groups
+// of G cells are dealt out to the blocks in turn, and a block first looks
+// through the flags of its groups (CHUNK cells at a time) and packs the cells
+// it wants into shared memory, then works on them with full warps
+// (`work(x, y, z, i)`).
+constexpr uint32_t CHUNK = 1024;
+template <uint32_t G, class Want, class Work>
+__device__ __forceinline__ void walk_near(const Dev &d, const int *lo, const int *hi, uint32_t ncell, const VB &vb,
+                                          uint32_t blocks, Want want, Work work) {
+    __shared__ uint32_t s_cell[CHUNK];
+    __shared__ uint32_t s_n;
+    if (vb.x >= blocks) return;
+    const uint32_t nthr = blockDim.x * blockDim.y, tid = threadIdx.x + blockDim.x * threadIdx.y, lane = tid & 31u;
+    const uint32_t groups = (ncell + G - 1) / G;
+    const uint32_t mine = groups > vb.x ? (groups - vb.x + blocks - 1) / blocks * G : 0;  // cells of this block
+    constexpr int U = 4;  // flag loads in flight per thread
+    for (uint32_t c0 = 0; c0 < mine; c0 += CHUNK) {
+        const uint32_t c1 = min(c0 + CHUNK, mine);
+        if (tid == 0) s_n = 0;
+        __syncthreads();
+        for (uint32_t l0 = c0 + tid - lane; l0 < c1; l0 += U * nthr) {  // warp-uniform
+            uint32_t k[U];
+            int fb[U];
+#pragma unroll
+            for (int u = 0; u < U; ++u) {
+                const uint32_t l = l0 + u * nthr;
+                k[u] = (l / G * blocks + vb.x) * G + l % G + lane;  // l: a multiple of 32
+                fb[u] = 0;
+                if (l < c1 && k[u] < ncell) {
+                    int x, y, z;
+                    range_cell(d, lo, hi, k[u], x, y, z);
+                    fb[u] = d.flags[x + (long long)d.nx * (y + (long long)d.ny * z)];
+                }
+            }
+#pragma unroll
+            for (int u = 0; u < U; ++u) {
+                const bool on = want(fb[u]);
+                const unsigned m = __ballot_sync(0xffffffffu, on);
+                uint32_t at = 0;
+                if (lane == 0 && m) at = atomicAdd(&s_n, (uint32_t)__popc(m));
+                at = __shfl_sync(0xffffffffu, at, 0);
+                if (on) s_cell[at + __popc(m & ((1u << lane) - 1u))] = k[u];
+            }
+        }
+        __syncthreads();
+        const uint32_t n = s_n;
+        for (uint32_t j = tid; j < n; j += nthr) {
+            int x, y, z;
+            range_cell(d, lo, hi, s_cell[j], x, y, z);
+            work(x, y, z, x + (long long)d.nx * (y + (long long)d.ny * z));
+        }
+        __syncthreads();
+    }
+}
+
+// Blocks for a body's cells when the blocks' sums do not matter: in a batch
+// (dense), whose tanks fill the GPU, as many as have CHUNK cells each, so that
+// the packed warps are full; for a single tank all that fit the GPU with the
+// other bodies' (two per SM), so that the work of a small body spreads.
+__device__ __forceinline__ uint32_t near_blocks(const Dev &d, const VB &vb, uint32_t ncell, bool dense) {
+    const uint32_t full = (ncell + CHUNK - 1) / CHUNK;
+    return min(vb.nx, dense ? full : max(full, 304u / (uint32_t)d.nb));
+}
 
 // neighbour-obstacle bit: set when any of the 18 neighbours is an obstacle
 // (the bulk kernel then lists the cell for k_general; walls and periodic
@@ -1027,7 +1165,7 @@ __device__ __forceinline__ void nb_refresh(const Dev &d, long long i) {
         int c = cls(d, nbr(d, x, y, z, cx(q), cy(q), cz(q)));
         nb = nb || c == CL_O;
     }
-    d.flags[i] = (uint8_t)((d.flags[i] & CL_MASK) | (nb ? NB_OBST : 0));
+    d.flags[i] = (uint8_t)((d.flags[i] & ~NB_OBST) | (nb ? NB_OBST : 0));
 }
 
 // neighbour-obstacle bits of the cells x0 <= x < x1 (grid (x-tiles, ny, nz))
@@ -1041,7 +1179,7 @@ __global__ void k_nb_all(Dev d) {
         int c = cls(d, nbr(d, x, y, z, cx(q), cy(q), cz(q)));
         nb = nb || c == CL_O;
     }
-    d.flags[i] = (uint8_t)((d.flags[i] & CL_MASK) | (nb ? NB_OBST : 0));
+    d.flags[i] = (uint8_t)((d.flags[i] & ~NB_OBST) | (nb ? NB_OBST : 0));
 }
 
 // the same over the cells around body bi (its range widened by one cell)
@@ -1143,44 +1281,30 @@ __device__ __forceinline__ double fixed96_value(unsigned __int128 v) {
     const unsigned long long L = (unsigned long long)v;
     return (double)H * 2.3283064365386962890625e-10 + (double)L * 1.2621774483536188886587657044524580e-29;
 }
+__device__ __forceinline__ unsigned __int128 shfl_xor_128(unsigned __int128 v, int off) {
+    const unsigned long long lo = __shfl_xor_sync(0xffffffffu, (unsigned long long)v, off);
+    const unsigned long long hi = __shfl_xor_sync(0xffffffffu, (unsigned long long)(v >> 64), off);
+    return ((unsigned __int128)hi << 64) | (unsigned __int128)lo;
+}
 __device__ __forceinline__ unsigned __int128 shfl_down_128(unsigned __int128 v, int off) {
     const unsigned long long lo = __shfl_down_sync(0xffffffffu, (unsigned long long)v, off);
     const unsigned long long hi = __shfl_down_sync(0xffffffffu, (unsigned long long)(v >> 64), off);
     return ((unsigned __int128)hi << 64) | (unsigned __int128)lo;
 }
 
-template <int S>
+template <int S, bool DENSE>
 __device__ __forceinline__ void forces_f64_body(const Dev &d, const VB &vb) {
-    int bi = vb.y;
+    const int bi = vb.y;
     const Body &b = d.bodies[bi];
-    int lo[3] = {b.lo[0] - 1, b.lo[1] - 1, b.lo[2] - 1};
-    int hi[3] = {b.hi[0] + 1, b.hi[1] + 1, b.hi[2] + 1};
-    int n3[3] = {d.nx, d.ny, d.nz};
-    for (int k = 0; k < 3; ++k) {
-        if (!(d.periodic & (1u << k))) {
-            lo[k] = lo[k] < 0 ? 0 : lo[k];
-            hi[k] = hi[k] > n3[k] ? n3[k] : hi[k];
-        } else if (hi[k] - lo[k] > n3[k]) {
-            hi[k] = lo[k] + n3[k];
-        }
-    }
     unsigned __int128 acc[7] = {0, 0, 0, 0, 0, 0, 0};
-    // the cells of the box around the body, 32 consecutive cells per warp, the
-    // warps' groups dealt out block by block (the double unit serves one SM:
-    // with the groups of a small body in consecutive warps of a few blocks
-    // those SMs' units held the kernel up); only cells next to an obstacle
-    // (neighbour-obstacle bit) can hold links
-    const uint32_t ncell = (uint32_t)range_count(lo, hi);
-    const int tidf = threadIdx.x + blockDim.x * threadIdx.y, nwarp = (blockDim.x * blockDim.y) >> 5;
+    // only cells next to an obstacle (neighbour-obstacle bit) can hold links
     const long long sy = d.nx, sz = (long long)d.nx * d.ny;
-    for (uint32_t kk = ((uint32_t)(tidf >> 5) * vb.nx + vb.x) * 32u + (uint32_t)(tidf & 31); kk < ncell;
-         kk += (uint32_t)nwarp * vb.nx * 32u) {
-        int x, y, z;
-        range_cell(d, lo, hi, kk, x, y, z);
-        const long long i = x + sy * (y + (long long)d.ny * z);
-        const int fb = d.flags[i];
-        const int cl = fb & CL_MASK;
-        if (!(fb & NB_OBST) || cl == CL_O) continue;
+    int lo[3], hi[3];
+    near_range(d, b, lo, hi);
+    const uint32_t ncell = (uint32_t)range_count(lo, hi);
+    walk_near<32>(d, lo, hi, ncell, vb, near_blocks(d, vb, ncell, DENSE), [](int fb) { return (fb & NB_OBST) && (fb & CL_MASK) != CL_O; },
+                  [&](int x, int y, int z, long long i) {
+        const int cl = clsv(d, i);
         // directions into body bi and the cell's populations, requested at once
         const bool inner = x > 0 && x < d.nx - 1 && y > 0 && y < d.ny - 1 && z > 0 && z < d.nz - 1;
         const bool fluid = cl != CL_G;
@@ -1205,7 +1329,7 @@ __device__ __forceinline__ void forces_f64_body(const Dev &d, const VB &vb) {
                     if (d.bid[si] == bi) lm |= 1u << q;
                 }
         }
-        if (!lm) continue;
+        if (!lm) return;
         // double, each value in the order of the plain restatement; the
         // direction is a constant of each unrolled term, so products by its
         // zeros are left out (x + 0 y = x)
@@ -1246,12 +1370,12 @@ __device__ __forceinline__ void forces_f64_body(const Dev &d, const VB &vb) {
             else if (cx(qb)) acc[5] += fixed96(-(r[1] * F0));
             acc[6] += g >= 0.0 ? pos : neg;
         }
-    }
+    });
     // block reduction of the exact integer sums (any order gives the same
     // bits); a warp without any link skips the tree (its sums are zeros).
     // The block's partials go out as 128-bit integers (low, high word).
     __shared__ unsigned __int128 sh[8][7];
-    int tid = threadIdx.x + blockDim.x * threadIdx.y;
+    const int tid = threadIdx.x + blockDim.x * threadIdx.y;
     int lane = tid & 31, wid = tid >> 5;
     const bool any = __any_sync(0xffffffffu, (acc[6] | acc[0] | acc[1] | acc[2]) != 0);
 #pragma unroll
@@ -1283,30 +1407,22 @@ __device__ __forceinline__ long long warp_sum64(long long v) {
     return (long long)sa * (1ll << 42) + (long long)sb * (1ll << 21) + (long long)sc;
 }
 
-// Float storages.  The rows (y, z) of the cell range around the body are
-// spread over the body's warps, lanes along x (coalesced flag loads, no
-// per-cell division); every sum is an integer, so the totals do not depend
-// on that mapping.  The link term is split into the uniform gas-pressure part
-// 2 w_q rho_G (exact integer sums of 36 (2 w_q) c_qbar and of the lever arm
-// twice the cell centre) and the small remainder 2 (phi (f_qbar - w_q rho_G)
-// + moving-wall part), computed in float from the stored deviations f - w and
-// summed in fixed point.  The lever arm r is the cell's, so each part is
-// summed over the cell's links first and its torque is r x that sum.
-template <int S>
+// Float storages.  Every sum within a block is an integer, so a block's totals
+// do not depend on the cell-to-thread map; which cells a block sums is fixed
+// (FORCE_GROUP consecutive cells of the range, dealt out to as many blocks as
+// there are groups), so the totals are the same in every launch form.  The
+// link term is split into the uniform gas-pressure part 2 w_q rho_G (exact
+// integer sums of 36 (2 w_q) c_qbar and of the lever arm twice the cell centre)
+// and the small remainder 2 (phi (f_qbar - w_q rho_G) + moving-wall part),
+// computed in float from the stored deviations f - w and summed in fixed point.
+// The lever arm r is the cell's, so each part is summed over the cell's links
+// first and its torque is r x that sum.
+constexpr uint32_t FORCE_GROUP = 256;
+template <int S, bool DENSE>
 __device__ __forceinline__ void forces_float_body(const Dev &d, const VB &vb) {
     const int bi = vb.y;
     const Body &b = d.bodies[bi];
-    int lo[3] = {b.lo[0] - 1, b.lo[1] - 1, b.lo[2] - 1};
-    int hi[3] = {b.hi[0] + 1, b.hi[1] + 1, b.hi[2] + 1};
     const int n3[3] = {d.nx, d.ny, d.nz};
-    for (int k = 0; k < 3; ++k) {
-        if (!(d.periodic & (1u << k))) {
-            lo[k] = lo[k] < 0 ? 0 : lo[k];
-            hi[k] = hi[k] > n3[k] ? n3[k] : hi[k];
-        } else if (hi[k] - lo[k] > n3[k]) {
-            hi[k] = lo[k] + n3[k];
-        }
-    }
     long long ia[7] = {0, 0, 0, 0, 0, 0, 0};         // fixed-point remainder sums
     long long ik[3] = {0, 0, 0}, it[3] = {0, 0, 0};  // exact gas-pressure sums
     bool hit = false;
@@ -1317,35 +1433,18 @@ __device__ __forceinline__ void forces_float_body(const Dev &d, const VB &vb) {
     const float rg = (float)d.rho_g, wrg1 = d.rg1_f;
     const int tid = threadIdx.x + blockDim.x * threadIdx.y;
     const int lane = tid & 31, wid = tid >> 5, nwarp = (blockDim.x * blockDim.y) >> 5;
-    const int lx = hi[0] - lo[0];
-    const unsigned ly = (unsigned)(hi[1] - lo[1]), nrows = ly * (unsigned)(hi[2] - lo[2]);
     const long long sy = d.nx, sz = (long long)d.nx * d.ny;
-    // the range's cells in x-fastest order, 32 consecutive cells per warp
-    // task (a row shorter or longer than 32 cells leaves no lanes idle); as
-    // many of the body's blocks as give each warp LBMFS_FORCE_ROWS tasks, the
-    // others contribute zeros
-    const unsigned ncell = (unsigned)lx * nrows, ntask = (ncell + 31u) / 32u;
-    const unsigned per_block = (unsigned)nwarp * LBMFS_FORCE_ROWS;
-    const unsigned used = min((unsigned)vb.nx, (ntask + per_block - 1) / per_block);
-    if ((unsigned)vb.x >= used) {
+    int lo[3], hi[3];
+    near_range(d, b, lo, hi);
+    const uint32_t ncell = (uint32_t)range_count(lo, hi);
+    const uint32_t used = min(vb.nx, (ncell + FORCE_GROUP - 1) / FORCE_GROUP);
+    if (vb.x >= used) {  // the others contribute zeros
         if (tid < 7) d.part[((long long)bi * FORCE_BLOCKS + vb.x) * 7 + tid] = 0.0;
         return;
     }
-    for (unsigned task = (unsigned)vb.x * nwarp + wid; task < ntask; task += used * nwarp) {
-        {
-            const unsigned kc = task * 32u + (unsigned)lane;
-            if (kc >= ncell) continue;
-            const unsigned row = kc / (unsigned)lx;
-            const int xo = (int)(kc - row * (unsigned)lx);
-            int y = lo[1] + (int)(row % ly), z = lo[2] + (int)(row / ly);
-            if (y < 0 || y >= d.ny) y = ((y % d.ny) + d.ny) % d.ny;  // only periodic axes leave [0, n)
-            if (z < 0 || z >= d.nz) z = ((z % d.nz) + d.nz) % d.nz;
-            int x = lo[0] + xo;
-            if (x < 0 || x >= d.nx) x = ((x % d.nx) + d.nx) % d.nx;
-            const long long i = x + sy * (y + (long long)d.ny * z);
-            const int fb = d.flags[i];
-            const int cl = fb & CL_MASK;
-            if (!(fb & NB_OBST) || cl == CL_O) continue;
+    walk_near<FORCE_GROUP>(d, lo, hi, ncell, vb, used, [](int fb) { return (fb & NB_OBST) && (fb & CL_MASK) != CL_O; },
+                           [&](int x, int y, int z, long long i) {
+            const int cl = clsv(d, i);
             // directions into body bi: all neighbour classes requested at
             // once (linear offsets away from the grid faces), then the body
             // ids of the obstacle directions
@@ -1375,9 +1474,9 @@ __device__ __forceinline__ void forces_float_body(const Dev &d, const VB &vb) {
                         if (d.bid[si] == bi) lm |= 1u << q;
                     }
             }
-            if (!lm) continue;
+            if (!lm) return;
             hit = true;
-            const float phf = cl == CL_L ? 1.0f : (cl == CL_I ? (float)d.phisrc[i] : 0.0f);
+            const float phf = cl == CL_L ? 1.0f : (cl == CL_I ? d.phifsrc[i] : 0.0f);
             // lever arm from the cell centre (minimum image on periodic
             // axes): float for the small remainder, and twice the cell
             // centre as an integer for the exact gas-pressure part
@@ -1453,8 +1552,7 @@ __device__ __forceinline__ void forces_float_body(const Dev &d, const VB &vb) {
             it[0] += c2[1] * kz - c2[2] * ky;
             it[1] += c2[2] * kx - c2[0] * kz;
             it[2] += c2[0] * ky - c2[1] * kx;
-        }
-    }
+    });
     // warp sums, then the warps' sums in the block (integers: exact); a warp
     // without any link skips the reductions (its sums are zeros)
     __shared__ long long shi[8][13];
@@ -1491,15 +1589,15 @@ __device__ __forceinline__ void forces_float_body(const Dev &d, const VB &vb) {
     }
 }
 
-template <int S>
+template <int S, bool DENSE>
 __device__ __forceinline__ void forces_body(const Dev &d, const VB &vb) {
-    if constexpr (S == 0) forces_f64_body<S>(d, vb);
-    else forces_float_body<S>(d, vb);
+    if constexpr (S == 0) forces_f64_body<S, DENSE>(d, vb);
+    else forces_float_body<S, DENSE>(d, vb);
 }
 
 template <int S>
 __global__ void __launch_bounds__(256, S == 0 ? 2 : LBMFS_FORCE_MINB) k_forces(const __grid_constant__ Dev d) {
-    forces_body<S>(d, vb_own());
+    forces_body<S, false>(d, vb_own());
 }
 
 // ---- C1 + C2 for liquid cells (Sec. 2.1 Eqs. stream, lbgk, forceterm;
@@ -1577,10 +1675,11 @@ template <int S> __device__ __forceinline__ void to_raw(typename Sto<S>::R *fp) 
 // share it, the common case; per link otherwise).  rho_x, in double for the
 // FP64 storage and in float for the float storages, sums the own populations
 // in q order.  Returns the mass the moving links add to the cell (for the
-// ledger).
+// ledger).  With owner >= 0 the cell is the caller's (mine) when its obstacle
+// neighbours' lowest body is `owner`.
 template <int S>
 __device__ __forceinline__ double gather_general(const Dev &d, int x, int y, int z, long long i,
-                                                 typename Sto<S>::R *fp) {
+                                                 typename Sto<S>::R *fp, int owner, bool &mine) {
     using P = Sto<S>;
     using R = typename P::R;
     const long long N = d.N;
@@ -1606,15 +1705,21 @@ __device__ __forceinline__ double gather_general(const Dev &d, int x, int y, int
         if (ns[q] == CL_G) atomicOr(d.status, ST_LIQUID_GAS);
     }
     fp[0] = own[0];
+    mine = true;
     if (!moving) return 0.0;
-    int b0 = -1;
+    int b0 = -1, low = MAX_BODIES;
     bool one = true;  // every obstacle link belongs to body b0
 #pragma unroll
     for (int q = 1; q < Q; ++q)
         if (obst & (1u << q)) {
             if (b0 < 0) b0 = bq[q];
             one = one && bq[q] == b0;
+            low = min(low, bq[q]);
         }
+    if (owner >= 0 && low != owner) {
+        mine = false;
+        return 0.0;
+    }
     R wall = 0;
     if constexpr (S == 0) {
         double rho_x = 0.0;
@@ -1652,68 +1757,119 @@ __device__ __forceinline__ double gather_general(const Dev &d, int x, int y, int
     return (double)wall;
 }
 
-template <int S>
-__device__ __forceinline__ double liquid_cell_general(const Dev &d, int x, int y, int z, long long i) {
-    typename Sto<S>::R fp[Q];
-    const double wall = gather_general<S>(d, x, y, z, i, fp);
-    to_raw<S>(fp);
-    collide_store<S>(d, fp, i);
-    return wall;
-}
-
-// C1 + C2 for the liquid cells the bulk kernel listed (an obstacle among the
-// neighbours, or a grid face with moving walls): the general gather, then the
-// collision.  They read the source grid and write their own cell of the
-// destination grid only, as the bulk kernel would have.
-// The mass the moving links add is summed per warp and goes to the ledger
-// with one atomic per warp (thousands of cells adding to one address would
-// queue on it).  Blocks of GEN_THREADS spread the few listed cells over many
-// SMs.
+// C1 + C2 for the liquid cells that the bulk kernel leaves out, by the general
+// gather.  They read the source grid and write their own cell of the
+// destination grid only, as the bulk kernel would have.  The mass the moving
+// links add is summed per warp and goes to the ledger with one atomic per warp
+// (thousands of cells adding to one address would queue on it).  Blocks of
+// GEN_THREADS spread the few cells over many SMs.
 constexpr int GEN_THREADS = 128;
-template <int S> __device__ __forceinline__ void general_body(const Dev &d, const VB &vb) {
-    double wacc = 0.0;
-    LIST_LOOP(WL_GEN, g) {
-        const long long i = d.list[WL_GEN][it_g];
-        int x, y, z;
-        if constexpr (S != 0) {
-            // the float storages hold N * 19 < 2^32 elements
-            const uint32_t i32 = (uint32_t)i, yz = i32 / (uint32_t)d.nx;
-            x = (int)(i32 - yz * (uint32_t)d.nx);
-            y = (int)(yz % (uint32_t)d.ny);
-            z = (int)(yz / (uint32_t)d.ny);
-        } else {
-            coords(d, i, x, y, z);
-        }
-        wacc += liquid_cell_general<S>(d, x, y, z, i);
-    }
+__device__ __forceinline__ void book_wall(const Dev &d, double wacc) {
     if (__any_sync(0xffffffffu, wacc != 0.0)) {
 #pragma unroll
         for (int off = 16; off > 0; off >>= 1) wacc += __shfl_xor_sync(0xffffffffu, wacc, off);
         if ((threadIdx.x & 31) == 0 && wacc != 0.0) atomicAdd(&d.ledger[LG_WALL], wacc);
     }
 }
+// Cells next to a body: every liquid cell with an obstacle among its
+// neighbours lies in the range around that obstacle's body, so the blocks of
+// body vb.y look through its range (a cell next to two bodies is the lower
+// one's).  Nothing here depends on the bulk kernel, beside which it runs.
+template <int S, bool DENSE> __device__ __forceinline__ void near_body(const Dev &d, const VB &vb) {
+    const int bi = vb.y, owner = d.nb > 1 ? bi : -1;
+    double wacc = 0.0;
+    uint32_t count = 0;
+    int lo[3], hi[3];
+    near_range(d, d.bodies[bi], lo, hi);
+    const uint32_t ncell = (uint32_t)range_count(lo, hi);
+    walk_near<32>(d, lo, hi, ncell, vb, near_blocks(d, vb, ncell, DENSE), [](int fb) { return (fb & ~MOVING_FACE) == (CL_L | NB_OBST); },
+                     [&](int x, int y, int z, long long i) {
+                         typename Sto<S>::R fp[Q];
+                         bool mine;
+                         const double wall = gather_general<S>(d, x, y, z, i, fp, owner, mine);
+                         if (!mine) return;
+                         to_raw<S>(fp);
+                         collide_store<S>(d, fp, i);
+                         wacc += wall;
+                         ++count;
+                     });
+    book_wall(d, wacc);
+    count = __reduce_add_sync(0xffffffffu, count);
+    if ((threadIdx.x & 31) == 0 && count) atomicAdd(&d.cnt[CN_NEAR], count);
+}
+// Liquid cells on a face of a grid with moving walls and next to no obstacle:
+// the bulk kernel leaves them out by their face bit, this walks the faces, each
+// cell once: the first and last xy-plane, then the first and last row and
+// column of the planes between.
+template <int S> __device__ __forceinline__ void faces_body(const Dev &d, const VB &vb) {
+    const uint32_t nx = d.nx, ny = d.ny, nz = d.nz, two_x = min(nx, 2u), two_y = min(ny, 2u), two_z = min(nz, 2u);
+    const uint32_t mz = nz - two_z, my = ny - two_y;  // planes, rows between
+    const uint32_t n1 = two_z * nx * ny, n2 = n1 + mz * two_y * nx, n = n2 + mz * my * two_x;
+    const int lane = threadIdx.x & 31;
+    uint32_t first, stride, count = 0;
+    list_span(vb, n, 32u, first, stride);
+    double wacc = 0.0;
+    for (uint32_t k0 = first; k0 < n; k0 += stride) {
+        uint32_t k = k0 + lane;
+        if (k < n) {
+            uint32_t x, y, z;
+            if (k < n1) {
+                x = k % nx;
+                y = k / nx % ny;
+                z = k / (nx * ny) ? nz - 1 : 0;
+            } else if (k < n2) {
+                k -= n1;
+                x = k % nx;
+                y = k / nx % two_y ? ny - 1 : 0;
+                z = 1 + k / (nx * two_y);
+            } else {
+                k -= n2;
+                x = k % two_x ? nx - 1 : 0;
+                y = 1 + k / two_x % my;
+                z = 1 + k / (two_x * my);
+            }
+            const long long i = x + (long long)nx * (y + (long long)ny * z);
+            if (d.flags[i] == (CL_L | MOVING_FACE)) {
+                typename Sto<S>::R fp[Q];
+                bool mine;
+                wacc += gather_general<S>(d, (int)x, (int)y, (int)z, i, fp, -1, mine);
+                to_raw<S>(fp);
+                collide_store<S>(d, fp, i);
+                ++count;
+            }
+        }
+        __syncwarp();
+    }
+    book_wall(d, wacc);
+    count = __reduce_add_sync(0xffffffffu, count);
+    if (lane == 0 && count) atomicAdd(&d.cnt[CN_NEAR], count);
+}
 template <int S>
-__global__ void __launch_bounds__(GEN_THREADS, 1) k_general(const __grid_constant__ Dev d) {
-    general_body<S>(d, vb_own());
+__global__ void __launch_bounds__(GEN_THREADS, 1) k_near(const __grid_constant__ Dev d) {
+    near_body<S, false>(d, vb_own());
+}
+template <int S>
+__global__ void __launch_bounds__(GEN_THREADS, 1) k_faces(const __grid_constant__ Dev d) {
+    faces_body<S>(d, vb_own());
 }
 
-// One liquid cell (class byte c, coordinates x, y, z, index i; not a
-// general_cell): gather its 18 arriving populations by the cheapest rule that
-// holds for it, collide and store.
+// One liquid cell (class byte CL_L, coordinates x, y, z, index i; not
+// next to an obstacle): gather its 18 arriving populations by the cheapest rule
+// that holds for it, collide and store.
 template <int S>
-__device__ __forceinline__ void liquid_one(const Dev &d, int c, int x, int y, int z, long long i) {
+__device__ __forceinline__ void liquid_one(const Dev &d, int x, int y, int z, long long i) {
     using P = Sto<S>;
     using R = typename P::R;
     const long long N = d.N;
     R fp[Q];
-    if (c == CL_L && x > 0 && x < d.nx - 1 && y > 0 && y < d.ny - 1 && z > 0 && z < d.nz - 1) {
+    if (x > 0 && x < d.nx - 1 && y > 0 && y < d.ny - 1 && z > 0 && z < d.nz - 1) {
         // no obstacle or wall in the neighbourhood and a liquid cell never
         // touches gas: plain pull from the 18 neighbours
         const long long sy = d.nx, sz = (long long)d.nx * d.ny;
 #pragma unroll
         for (int q = 1; q < Q; ++q) fp[q] = P::ldg_raw(d.fsrc, q, i - (cx(q) + cy(q) * sy + cz(q) * sz), N);
         fp[0] = P::ldg_raw(d.fsrc, 0, i, N);
-    } else if (c == CL_L && !d.periodic && !d.walls_move) {
+    } else if (!d.periodic) {
         // on a face of a grid without periodic axes, no obstacle
         // neighbour: a source beyond a face is a resting wall, which
         // returns the cell's own opposite population (Eq. noslip, u_w = 0)
@@ -1738,15 +1894,6 @@ __device__ __forceinline__ void liquid_one(const Dev &d, int c, int x, int y, in
     }
     collide_store<S>(d, fp, i);  // one copy of the collision in the kernel
 }
-// A liquid cell the bulk kernel leaves to k_general (class byte c): an
-// obstacle among its neighbours (the neighbour-obstacle bit), or a grid face
-// when the walls move.  Its class, body-id and body-state loads depend on one
-// another; in k_general they hold none of the bulk kernel's warps.
-__device__ __forceinline__ bool general_cell(const Dev &d, int c, int x, int y, int z) {
-    return (c & CL_MASK) == CL_L &&
-           (c != CL_L || (d.walls_move && !(x > 0 && x < d.nx - 1 && y > 0 && y < d.ny - 1 && z > 0 && z < d.nz - 1)));
-}
-
 // The cells (x, y, z0 .. z1-1) of one thread.  The flags of the whole column
 // come in one round of loads, so a thread whose column holds no fluid leaves
 // after one memory latency, and a fluid cell waits on its populations only.
@@ -1754,7 +1901,8 @@ template <int S, int ZBMAX>
 __device__ __forceinline__ void liquid_column(const Dev &d, bool in, int x, int y, int z0, int z1) {
     static_assert(ZBMAX <= 8, "flags of a column (z1 - z0 <= ZBMAX) are packed into 64 bits");
     const long long sy = d.nx, sz = (long long)d.nx * d.ny;
-    long long i = (long long)x + sy * (y + (long long)d.ny * z0);
+    // (cell indices are below 2^32)
+    long long i = (long long)((unsigned)x + (unsigned)d.nx * ((unsigned)y + (unsigned)d.ny * (unsigned)z0));
     uint64_t fl = 0;
 #pragma unroll
     for (int k = 0; k < ZBMAX; ++k)
@@ -1764,14 +1912,12 @@ __device__ __forceinline__ void liquid_column(const Dev &d, bool in, int x, int 
         atomicMax(d.ztop_wr, z1 - 1);
     if (fl == 0) return;
 #pragma unroll 1
-    for (int z = z0; z < z1; ++z, i += sz) {
+    for (int z = z0; fl != 0; ++z, i += sz) {  // up to the column's last cell with a class
         const int c = (int)(fl & 0xff);
         fl >>= 8;
         wl_append(d, (c & CL_MASK) == CL_I, WL_IFACE, (uint32_t)i);
-        const bool gen = general_cell(d, c, x, y, z);
-        wl_append(d, gen, WL_GEN, (uint32_t)i);
-        if ((c & CL_MASK) != CL_L || gen) continue;
-        liquid_one<S>(d, c, x, y, z, i);  // one copy of the collision in the kernel
+        if (c != CL_L) continue;  // (with the neighbour-obstacle bit: k_near's; with the face bit: k_faces')
+        liquid_one<S>(d, x, y, z, i);  // one copy of the collision in the kernel
     }
 }
 
@@ -1817,9 +1963,6 @@ __device__ __forceinline__ void liquid_body_pair(const Dev &d, const VB &vb, int
         const int c0 = (int)(fl[k] & 0xffu), c1 = (int)(fl[k] >> 8);
         wl_append(d, (c0 & CL_MASK) == CL_I, WL_IFACE, j);
         wl_append(d, (c1 & CL_MASK) == CL_I, WL_IFACE, j + 1);
-        const bool g0 = general_cell(d, c0, x0, y0, z), g1 = general_cell(d, c1, x0 + 1, y0, z);
-        wl_append(d, g0, WL_GEN, j);
-        wl_append(d, g1, WL_GEN, j + 1);
         if (pair_xy && c0 == CL_L && c1 == CL_L && z > 0 && z < d.nz - 1) {
             float2 fp[Q];
 #pragma unroll
@@ -1834,8 +1977,8 @@ __device__ __forceinline__ void liquid_body_pair(const Dev &d, const VB &vb, int
 #pragma unroll 1
             for (int h = 0; h < 2; ++h) {
                 const int c = h ? c1 : c0;
-                if ((c & CL_MASK) != CL_L || (h ? g1 : g0)) continue;
-                liquid_one<S>(d, c, x0 + h, y0, z, (long long)(j + h));
+                if (c != CL_L) continue;
+                liquid_one<S>(d, x0 + h, y0, z, (long long)(j + h));
             }
         }
     }
@@ -1928,9 +2071,8 @@ __global__ void __launch_bounds__(BULK_THREADS, LBMFS_BULK_MINB) k_liquid_pipe(D
                 fp[q] = Pipe<S>::get(&slots[b][0][tid], q, i - (cx(q) * sx + cy(q) * sy + cz(q) * sz), d.N);
             to_raw<S>(fp);
             collide_store<S>(d, fp, i);
-        } else if ((fl_cur & CL_MASK) == CL_L) {
-            const double w = liquid_cell_general<S>(d, x, y, z, i);
-            if (w != 0.0) atomicAdd(&d.ledger[LG_WALL], w);
+        } else if (fl_cur == CL_L) {
+            liquid_one<S>(d, x, y, z, i);
         }
         fl_cur = fl_next;
         fl_next = fl_after;
@@ -2080,9 +2222,8 @@ __global__ void __launch_bounds__(BULK_THREADS, LBMFS_BULK_MINB) k_liquid_tma(De
             for (int q = 0; q < Q; ++q) fp[q] = G::get(stage, q, tid + ((S == 2 && q > 0) ? Stage<2>::H : 4) - cx(q));
             to_raw<S>(fp);
             collide_store<S>(d, fp, i);
-        } else if ((c & CL_MASK) == CL_L) {
-            const double w = liquid_cell_general<S>(d, x, y, z, i);
-            if (w != 0.0) atomicAdd(&d.ledger[LG_WALL], w);
+        } else if (c == CL_L) {
+            liquid_one<S>(d, x, y, z, i);
         }
         fl_cur = fl_next;
         fl_next = fl_after;
@@ -2144,6 +2285,10 @@ __device__ __noinline__ double curvature_d(const Dev &d, int x, int y, int z, do
     return 0.25 * div;
 }
 // the same in float for the float storages
+__device__ __forceinline__ float fill_seen_f(const Dev &d, long long ni, float own) {
+    const int c = cls(d, ni);
+    return c == CL_L ? 1.0f : (c == CL_I ? d.phifsrc[ni] : (c == CL_G ? 0.0f : own));
+}
 __device__ __noinline__ float curvature_f(const Dev &d, int x, int y, int z, float nc0, float nc1, float nc2) {
     const float nc[3] = {nc0, nc1, nc2};
     float div = 0.0f;
@@ -2159,11 +2304,11 @@ __device__ __noinline__ float curvature_f(const Dev &d, int x, int y, int z, flo
             }
             int yx, yy, yz;
             coords(d, yi, yx, yy, yz);
-            const double own = c == CL_L ? 1.0 : (c == CL_I ? d.phisrc[yi] : 0.0);
+            const float own = c == CL_L ? 1.0f : (c == CL_I ? d.phifsrc[yi] : 0.0f);
             float n[3];
             for (int j = 0; j < 3; ++j) {
-                const float pm = (float)fill_seen(d, nbr(d, yx, yy, yz, j == 0 ? -1 : 0, j == 1 ? -1 : 0, j == 2 ? -1 : 0), own);
-                const float pp = (float)fill_seen(d, nbr(d, yx, yy, yz, j == 0 ? 1 : 0, j == 1 ? 1 : 0, j == 2 ? 1 : 0), own);
+                const float pm = fill_seen_f(d, nbr(d, yx, yy, yz, j == 0 ? -1 : 0, j == 1 ? -1 : 0, j == 2 ? -1 : 0), own);
+                const float pp = fill_seen_f(d, nbr(d, yx, yy, yz, j == 0 ? 1 : 0, j == 1 ? 1 : 0, j == 2 ? 1 : 0), own);
                 n[j] = 0.5f * (pm - pp);
             }
             const float len = sqrtf((n[0] * n[0] + n[1] * n[1]) + n[2] * n[2]);
@@ -2184,6 +2329,15 @@ __device__ __noinline__ float curvature_f(const Dev &d, int x, int y, int z, flo
 // formed per member and added as member 0 + member 1 + member 2 on all three
 // threads, so a trio agrees bit for bit.  Ten trios per warp; lanes 30 and 31
 // shadow the last trio and write nothing.
+//
+// A double operation holds a scheduler for 64 cycles (a conversion about 100,
+// a division 550), whatever the number of active lanes: they bound this kernel
+// when each trio converted the fill levels it read and did its own mass update
+// (about 1800 of those cycles per 10 cells).  The fill levels are therefore
+// also kept rounded to float, and a warp takes 30 cells as `sub` = 3 rounds of
+// ten trios before lane l does the mass update of cell l for all of them; a
+// list too short to give every scheduler a warp that way takes ten cells per
+// warp (sub = 1).
 
 // neighbour (x + dx, y + dy, z + dz) as a 32-bit cell index without
 // branches (periodic axes wrap); -1 beyond a wall
@@ -2248,7 +2402,6 @@ __device__ __forceinline__ void interface_trio(const Dev &d, const VB &vb) {
     using P = Sto<S>;
     const long long N = d.N;
     const unsigned FULL = 0xffffffffu;
-    if (vb.x == 0 && threadIdx.x == 0) *d.ztop_rd = -1;
     const int lane = threadIdx.x & 31;
     const bool lane_ok = lane < 30;
     const int g = lane_ok ? lane / 3 : 9;             // trio of the warp
@@ -2274,23 +2427,41 @@ __device__ __forceinline__ void interface_trio(const Dev &d, const VB &vb) {
 #define TRIO_EZ(k) ((int)((pk[k] >> 14) & 3u) - 1)
 #define TRIO_POS(k) ((pk[k] >> 16) & 1u)
     const float ax = d.a_f[0], ay = d.a_f[1], az = d.a_f[2];
-    const uint32_t n = wl_count(d, WL_IFACE);
+    const IfaceSeq seq = iface_seq(d);
+    const uint32_t n = seq.e[PREV_LISTS - 1];
+    // three rounds where that still gives each of the launch's warps (up to
+    // four per scheduler of the GPU) something to do
+#ifdef LBMFS_IFACE_SUB
+    const int sub = LBMFS_IFACE_SUB;
+#else
+    const int sub = 4u * (n / 30u) >= min(vb.nx * (blockDim.x >> 5), 4u * 608u) ? 3 : 1;
+#endif
     uint32_t first, stride;
-    list_span(vb, n, 10u, first, stride);
+    list_span(vb, n, 10u * sub, first, stride);
     for (uint32_t w0 = first; w0 < n; w0 += stride) {
-        const uint32_t it = w0 + (uint32_t)g;
-        const bool valid = lane_ok && it < n;
-        const long long i = d.list[WL_IFACE][valid ? it : w0];
-        const uint32_t i32 = (uint32_t)i;  // the float storages hold N * 19 < 2^32 elements
+        // lane l's cell of the 30 (10): its index, whether it is (still) an
+        // interface cell, its mass
+        const uint32_t itl = w0 + (uint32_t)min(lane, 10 * sub - 1);
+        const uint32_t il = iface_cell(d, seq, min(itl, n - 1));
+        const bool vl = lane < 10 * sub && itl < n && (d.flags[il] & CL_MASK) == CL_I;
+        const double m_old = d.m[il];  // requested with the populations
+        float dml = 0.0f, drsl = 0.0f;
+        unsigned lgl = 0;
+#pragma unroll 1
+        for (int turn = 0; turn < sub; ++turn) {
+        const uint32_t i32 = __shfl_sync(FULL, il, 10 * turn + g);  // the float storages hold N * 19 < 2^32 elements
+        const int vg = __shfl_sync(FULL, (int)vl, 10 * turn + g);  // every lane takes part
+        const bool valid = lane_ok && vg != 0;
+        if (!__any_sync(FULL, valid)) continue;
+        const long long i = i32;
         const int x = (int)(i32 % (uint32_t)d.nx);
         const uint32_t yz = i32 / (uint32_t)d.nx;
         const int y = (int)(yz % (uint32_t)d.ny), z = (int)(yz / (uint32_t)d.ny);
         // every load of the cell in one round, independent of the neighbour
         // classes: a source beyond a wall reads the cell itself (unused), so
         // no load waits on another and none sits behind a branch
-        const float phx = (float)__ldg(d.phisrc + i);
-        float foa[3], fob[3], pa[3], pb[3];
-        double ha[3], hb[3];
+        const float phx = __ldg(d.phifsrc + i);
+        float foa[3], fob[3], pa[3], pb[3], ha[3], hb[3];
         int sa[3], sb[3], ca[3], cb[3];
 #pragma unroll
         for (int k = 0; k < 3; ++k) {
@@ -2303,11 +2474,10 @@ __device__ __forceinline__ void interface_trio(const Dev &d, const VB &vb) {
             cb[k] = __ldg(d.flags + lb) & CL_MASK;
             pa[k] = trio_ld<S>(d.fsrc, TRIO_QA(k), la, N);
             pb[k] = trio_ld<S>(d.fsrc, TRIO_QB(k), lb, N);
-            ha[k] = __ldg(d.phisrc + la);
-            hb[k] = __ldg(d.phisrc + lb);
+            ha[k] = __ldg(d.phifsrc + la);
+            hb[k] = __ldg(d.phifsrc + lb);
         }
         const float fo0 = r == 0 ? P::ld(d.fsrc, 0, i, N) : 0.0f;
-        const double m_old = r == 0 ? d.m[i] : 0.0;  // requested with the populations
         // density and the velocity of the last collision (own populations)
         float drx = fo0, j0 = 0.0f, j1 = 0.0f, j2 = 0.0f;
 #pragma unroll
@@ -2338,7 +2508,7 @@ __device__ __forceinline__ void interface_trio(const Dev &d, const VB &vb) {
                 const int si = s ? sb[k] : sa[k];
                 const int ns = si < 0 ? CL_WALL : (s ? cb[k] : ca[k]);
                 const float pq = s ? pb[k] : pa[k];
-                const float phy = (float)(s ? hb[k] : ha[k]);
+                const float phy = s ? hb[k] : ha[k];
                 const float fbar = s ? foa[k] : fob[k];  // own population of the opposite direction
                 const unsigned bit = 1u << (2 * k + s);
                 const bool sol = ns == CL_WALL || ns == CL_O, gs = ns == CL_G, lq = ns == CL_L;
@@ -2451,22 +2621,34 @@ __device__ __forceinline__ void interface_trio(const Dev &d, const VB &vb) {
         drs = trio_sum(drs, b3);
         const unsigned lg = __shfl_sync(FULL, seen_lg, b3) | __shfl_sync(FULL, seen_lg, b3 + 1) |
                             __shfl_sync(FULL, seen_lg, b3 + 2);
-        const bool has_l = lg & 1u, has_g = lg & 2u;
+        if (valid && r == 0 && (!(rho > 0.0f) || !(rho < 1e30f))) atomicOr(d.status, ST_NONFINITE);
+        // to the lane that does the cell's mass update
+        const int from = 3 * min(max(lane - 10 * turn, 0), 9);
+        const float dmx = __shfl_sync(FULL, dm, from), drx2 = __shfl_sync(FULL, drs, from);
+        const unsigned lgx = __shfl_sync(FULL, lg, from);
+        if (lane >= 10 * turn && lane < 10 * turn + 10) {
+            dml = dmx;
+            drsl = drx2;
+            lgl = lgx;
+        }
+        }
+        const bool has_l = lgl & 1u, has_g = lgl & 2u;
         uint8_t mk = 0;
-        if (valid && r == 0) {
-            const double m_new = m_old + (double)dm;
-            const double phin = m_new / (1.0 + (double)drs);
-            d.m[i] = m_new;
-            d.phidst[i] = phin;
-            if (!(rho > 0.0f) || !(rho < 1e30f)) atomicOr(d.status, ST_NONFINITE);
+        if (vl) {
+            const double m_new = m_old + (double)dml;
+            const double phin = m_new / (1.0 + (double)drsl);
+            d.m[il] = m_new;
+            d.phidst[il] = phin;
+            d.phifdst[il] = (float)phin;
             mk = phin >= 1.0 + d.eps ? MK_FILLED : (phin <= -d.eps ? MK_EMPTIED : 0);
             // an interface cell without a liquid neighbour empties, one without
             // a gas neighbour fills
             if (!mk && d.nb_rule) mk = (!has_l && has_g) ? MK_EMPTIED : ((!has_g && has_l) ? MK_FILLED : 0);
-            if (mk) d.cmark[i] = mk;
+            if (mk) d.cmark[il] = mk;
         }
-        wl_append(d, mk == MK_FILLED, WL_FILLED, (uint32_t)i);
-        wl_append(d, mk == MK_EMPTIED, WL_EMPTIED, (uint32_t)i);
+        const uint32_t i32 = il;
+        wl_append(d, mk == MK_FILLED, WL_FILLED, i32);
+        wl_append(d, mk == MK_EMPTIED, WL_EMPTIED, i32);
     }
 }
 #undef TRIO_QA
@@ -2481,11 +2663,13 @@ __device__ __forceinline__ void interface_trio(const Dev &d, const VB &vb) {
 __device__ __forceinline__ void interface_d(const Dev &d, const VB &vb) {
     using P = Sto<0>;
     const long long N = d.N;
-    // the bulk kernel has read this step's fluid top: clear the slot for the
-    // next step to record into
-    if (vb.x == 0 && threadIdx.x == 0) *d.ztop_rd = -1;
-    LIST_LOOP(WL_IFACE, f) {
-        long long i = d.list[WL_IFACE][it_f];
+    const IfaceSeq seq = iface_seq(d);
+    const uint32_t n = seq.e[PREV_LISTS - 1];
+    uint32_t first, stride;
+    list_span(vb, n, 32u, first, stride);
+    for (uint32_t it = first + (threadIdx.x & 31u); it < n; it += stride) {
+        const long long i = iface_cell(d, seq, it);
+        if (clsv(d, i) != CL_I) continue;
         int x, y, z;
         coords(d, i, x, y, z);
         double own_phi = d.phisrc[i];
@@ -2627,74 +2811,100 @@ __global__ void __launch_bounds__(128, S == 0 ? 2 : LBMFS_IFACE_MINB) k_interfac
 
 // ------------------------------------------------- C3: conversions (Sec. 2.2)
 
-// filled cells: emptied neighbours are kept; gas neighbours become interface
-// set mark `bit` on the neighbours of (x, y, z) in the direction mask m (the
-// atomics issued together) and append the cells whose bit was newly set to
-// worklist `list` (one reservation for all of them)
-__device__ __forceinline__ void mark_append(const Dev &d, int x, int y, int z, unsigned m, uint8_t bit, int list) {
-    if (!m) return;
-    unsigned nw = 0;
-#pragma unroll
-    for (int q = 1; q < Q; ++q)
-        if (m & (1u << q)) {
-            const uint8_t old = mark_or(d, nbr(d, x, y, z, cx(q), cy(q), cz(q)), bit);
-            if (!(old & bit)) nw |= 1u << q;
-        }
-    if (!nw) return;
-    uint32_t pos = atomicAdd(&d.cnt[list], (uint32_t)__popc(nw));
-#pragma unroll
-    for (int q = 1; q < Q; ++q)
-        if (nw & (1u << q)) {
-            if (pos < d.cap) d.list[list][pos] = (uint32_t)nbr(d, x, y, z, cx(q), cy(q), cz(q));
-            else atomicOr(d.status, ST_OVERFLOW);
-            ++pos;
-        }
+// The conversion bodies take a warp per listed cell, lane q its neighbour in
+// direction q: the classes, marks and atomics of the 18 neighbours are in
+// flight together (one thread per cell issued its atomics one after another),
+// and the cells a warp marks are appended with one reservation.  The warps of
+// a short list go to different SMs.
+#define WARP_LOOP(L, var)                                                                                      \
+    const uint32_t n_##var = wl_count(d, L);                                                                   \
+    for (uint32_t it_##var = (threadIdx.x >> 5) * vb.nx + vb.x; it_##var < n_##var; it_##var += vb.nx * (blockDim.x >> 5))
+
+// the calling lane's neighbour of (x, y, z): direction = lane; -1 beyond a wall
+// and for the lanes without a direction
+__device__ __forceinline__ long long lane_nbr(const Dev &d, int lane, int x, int y, int z) {
+    return lane >= 1 && lane < Q ? nbr(d, x, y, z, dir_x(lane), dir_y(lane), dir_z(lane)) : -1;
+}
+// set mark `bit` on the lanes' cells (want) and append those newly marked
+__device__ __forceinline__ void mark_append(const Dev &d, bool want, long long yi, uint8_t bit, int list) {
+    const bool nw = want && !(mark_or(d, yi, bit) & bit);
+    __syncwarp();
+    wl_append(d, nw, list, (uint32_t)yi);
 }
 
+// gas neighbours of filled cells become interface
 __device__ __forceinline__ void conv_filled_body(const Dev &d, const VB &vb) {
-    LIST_LOOP(WL_FILLED, a) {
-        long long i = d.list[WL_FILLED][it_a];
+    const int lane = threadIdx.x & 31;
+    WARP_LOOP(WL_FILLED, a) {
         int x, y, z;
-        coords(d, i, x, y, z);
-        // classes and emptied marks requested at once (this kernel sets no
-        // emptied mark and changes no class)
-        unsigned em = 0, gm = 0;
-#pragma unroll
-        for (int q = 1; q < Q; ++q) {
-            long long yi = nbr(d, x, y, z, cx(q), cy(q), cz(q));
-            if (yi < 0) continue;
-            if (d.cmark[yi] & MK_EMPTIED) em |= 1u << q;
-            if (clsv(d, yi) == CL_G) gm |= 1u << q;
-        }
-#pragma unroll
-        for (int q = 1; q < Q; ++q)
-            if (em & (1u << q)) mark_and(d, nbr(d, x, y, z, cx(q), cy(q), cz(q)), MK_EMPTIED);
-        mark_append(d, x, y, z, gm, MK_NEWG, WL_NEWG);
+        coords(d, d.list[WL_FILLED][it_a], x, y, z);
+        const long long yi = lane_nbr(d, lane, x, y, z);
+        mark_append(d, cls(d, yi) == CL_G, yi, MK_NEWG, WL_NEWG);
     }
 }
 __global__ void k_conv_filled(const __grid_constant__ Dev d) { conv_filled_body(d, vb_own()); }
 
-// still-emptied cells: liquid neighbours become interface
+// an emptied cell next to a filled one is kept; liquid neighbours of the others
+// become interface
 __device__ __forceinline__ void conv_emptied_body(const Dev &d, const VB &vb) {
-    LIST_LOOP(WL_EMPTIED, a) {
-        long long i = d.list[WL_EMPTIED][it_a];
-        if (!(d.cmark[i] & MK_EMPTIED)) continue;
+    const int lane = threadIdx.x & 31;
+    WARP_LOOP(WL_EMPTIED, a) {
+        const long long i = d.list[WL_EMPTIED][it_a];
         int x, y, z;
         coords(d, i, x, y, z);
-        // classes requested at once (this kernel changes marks only)
-        unsigned lm = 0;
-#pragma unroll
-        for (int q = 1; q < Q; ++q) {
-            long long yi = nbr(d, x, y, z, cx(q), cy(q), cz(q));
-            if (yi >= 0 && clsv(d, yi) == CL_L) lm |= 1u << q;
+        const long long yi = lane_nbr(d, lane, x, y, z);
+        const int mk = yi >= 0 ? d.cmark[yi] : 0, c = cls(d, yi);
+        if (__any_sync(0xffffffffu, (mk & MK_FILLED) != 0)) {
+            if (lane == 0) mark_and(d, i, MK_EMPTIED);
+            continue;
         }
-        mark_append(d, x, y, z, lm, MK_NEWL, WL_NEWL);
+        mark_append(d, c == CL_L, yi, MK_NEWL, WL_NEWL);
     }
 }
 __global__ void k_conv_emptied(const __grid_constant__ Dev d) { conv_emptied_body(d, vb_own()); }
 
+// density of a cell by a whole warp: lane q loads population q, the sum is
+// taken in q order (as cell_density takes it) on every lane
+template <int S> __device__ __forceinline__ double warp_density(const Dev &d, const void *g, long long i) {
+    const int lane = threadIdx.x & 31;
+    typename Sto<S>::R v = 0, r = 0;
+    if (lane < Q) v = Sto<S>::ld(g, lane, i, d.N);
+#pragma unroll
+    for (int q = 0; q < Q; ++q) r += __shfl_sync(0xffffffffu, v, q);
+    if constexpr (S != 0) return 1.0 + (double)r;
+    else return r;
+}
+
 // new interface cells: from gas f = f_eq(mean rho, mean u) of the liquid and
 // interface neighbours, m = 0; from liquid m = rho
+// f_eq of the lane's direction; the products by the components are exact, so
+// this is feq_d for every q
+__device__ __forceinline__ double feq_lane(int q, double rho, const double *u) {
+    const double ex = (double)dir_x(q), ey = (double)dir_y(q), ez = (double)dir_z(q);
+    const double cu = (ex * u[0] + ey * u[1]) + ez * u[2];
+    const double usq = (u[0] * u[0] + u[1] * u[1]) + u[2] * u[2];
+    const double t = ((1.0 + 3.0 * cu) + (4.5 * cu) * cu) - 1.5 * usq;
+    return ((q == 0 ? wd(0) : (q <= 6 ? wd(1) : wd(7))) * rho) * t;
+}
+// store the cell whose population q lane q holds as f (Sto::st_cell by a warp)
+template <int S> __device__ __forceinline__ void warp_store_cell(const Dev &d, long long i, int lane, double f) {
+    if constexpr (S == 0) {
+        if (lane < Q) Sto<0>::st(d.fdst, lane, i, d.N, f);
+    } else {
+        const float dv = (float)(f - (lane == 0 ? wd(0) : (lane <= 6 ? wd(1) : wd(7))));
+        if constexpr (S == 1) {
+            if (lane < Q) Sto<1>::st(d.fdst, lane, i, d.N, dv);
+        } else {
+            // the rest population takes up what the others lose in rounding
+            float lost = 0.0f;
+            if (lane >= 1 && lane < Q) lost = dv - Sto<2>::st_one(d.fdst, lane, i, d.N, dv);
+            float rest = 0.0f;
+#pragma unroll
+            for (int q = 1; q < Q; ++q) rest += __shfl_sync(0xffffffffu, lost, q);
+            if (lane == 0) Sto<2>::st_one(d.fdst, 0, i, d.N, dv + rest);
+        }
+    }
+}
 template <int S>
 __device__ __forceinline__ void conv_init_body(const Dev &d, const VB &vb) {
     {
@@ -2719,35 +2929,27 @@ __device__ __forceinline__ void conv_init_body(const Dev &d, const VB &vb) {
                     r = cell_rho_u<S>(d, d.fdst, zi, u);
                 }
             }
-            double sr = 0.0, su[3] = {0.0, 0.0, 0.0};
-            int cnt = 0;
-#pragma unroll
-            for (int q = 1; q < Q; ++q) {
-                const int fq = __shfl_sync(0xffffffffu, fluid, q);
+            // lane c < 4 sums component c (density, velocity) in q order; lane q
+            // evaluates f_eq,q and stores population q
+            const unsigned fm = __ballot_sync(0xffffffffu, fluid != 0);
+            double sum = 0.0;
+            for (unsigned m = fm; m; m &= m - 1) {
+                const int q = __ffs(m) - 1;
                 const double rq = __shfl_sync(0xffffffffu, r, q), u0 = __shfl_sync(0xffffffffu, u[0], q),
                              u1 = __shfl_sync(0xffffffffu, u[1], q), u2 = __shfl_sync(0xffffffffu, u[2], q);
-                if (!fq) continue;
-                sr += rq;
-                su[0] += u0;
-                su[1] += u1;
-                su[2] += u2;
-                cnt++;
+                sum += lane == 0 ? rq : (lane == 1 ? u0 : (lane == 2 ? u1 : u2));
             }
-            const double rm = sr / cnt;
-            const double um[3] = {su[0] / cnt, su[1] / cnt, su[2] / cnt};
-            const double fl = feq_d(lane < Q ? lane : 0, rm, um);
-            double f[Q];
-#pragma unroll
-            for (int q = 0; q < Q; ++q) f[q] = __shfl_sync(0xffffffffu, fl, q);
-            if (lane == 0) {
-                Sto<S>::st_cell(d.fdst, i, d.N, f);
-                d.m[i] = 0.0;
-            }
+            const double mean = sum / __popc(fm);
+            const double rm = __shfl_sync(0xffffffffu, mean, 0);
+            const double um[3] = {__shfl_sync(0xffffffffu, mean, 1), __shfl_sync(0xffffffffu, mean, 2),
+                                  __shfl_sync(0xffffffffu, mean, 3)};
+            warp_store_cell<S>(d, i, lane, feq_lane(lane, rm, um));
+            if (lane == 0) d.m[i] = 0.0;
         }
     }
     {
         LIST_LOOP(WL_NEWL, b) {
-            long long i = d.list[WL_NEWL][it_b];
+            const long long i = d.list[WL_NEWL][it_b];
             d.m[i] = cell_density<S>(d, d.fdst, i);
         }
     }
@@ -2755,6 +2957,7 @@ __device__ __forceinline__ void conv_init_body(const Dev &d, const VB &vb) {
 template <int S>
 __global__ void k_conv_init(const __grid_constant__ Dev d) { conv_init_body<S>(d, vb_own()); }
 
+// the new classes
 __device__ __forceinline__ void conv_flags_body(const Dev &d, const VB &vb) {
     {
         LIST_LOOP(WL_FILLED, a) set_cls(d, d.list[WL_FILLED][it_a], CL_L);
@@ -2774,66 +2977,53 @@ __device__ __forceinline__ void conv_flags_body(const Dev &d, const VB &vb) {
 }
 __global__ void k_conv_flags(const __grid_constant__ Dev d) { conv_flags_body(d, vb_own()); }
 
-template <int S>
-__device__ __forceinline__ double excess(const Dev &d, long long i, uint8_t mk);
+// the class a cell of class c has after the conversions, by its marks
+__device__ __forceinline__ int class_after(int c, int mk) {
+    return mk & (MK_NEWG | MK_NEWL) ? CL_I : (mk & MK_FILLED ? CL_L : (mk & MK_EMPTIED ? CL_G : c));
+}
 
 // interface neighbours of converted cells receive excess mass.  The
 // converted cell's share e(x) / k(x) is computed here, once, and kept in its
 // mass entry (a converted cell is liquid or gas now, so the entry is not read
-// as a mass again before the cell next becomes interface, which sets it); a
-// cell without interface neighbours keeps its mass for the lost-mass ledger
+// as a mass again before the cell next becomes interface, which sets it); the
+// mass of a cell without interface neighbours goes to the lost-mass ledger
 template <int S>
-__device__ __forceinline__ void claim_receivers(const Dev &d, long long i, uint8_t mk) {
+__device__ __forceinline__ void claim_receivers(const Dev &d, int lane, long long i, uint8_t mk) {
     int x, y, z;
     coords(d, i, x, y, z);
-    // classes requested at once (this kernel changes marks and the converted
-    // cell's own mass entry only)
-    unsigned im = 0;
-#pragma unroll
-    for (int q = 1; q < Q; ++q) {
-        long long yi = nbr(d, x, y, z, cx(q), cy(q), cz(q));
-        if (yi >= 0 && clsv(d, yi) == CL_I) im |= 1u << q;
+    const long long yi = lane_nbr(d, lane, x, y, z);
+    // (the classes themselves change in the next phase, beside the excess)
+    const bool want = yi >= 0 && class_after(clsv(d, yi), d.cmark[yi]) == CL_I;
+    const double m = d.m[i];
+    const int k = __popc(__ballot_sync(0xffffffffu, want));
+    const double e = (mk & MK_FILLED) ? m - warp_density<S>(d, d.fdst, i) : m;
+    if (lane == 0) {
+        if (k > 0) d.m[i] = e / k;
+        else atomicAdd(&d.ledger[LG_LOST], e);
     }
-    const int k = __popc(im);
-    if (k > 0) d.m[i] = excess<S>(d, i, mk) / k;
-    mark_append(d, x, y, z, im, MK_RECV, WL_RECV);
+    __syncwarp();
+    mark_append(d, want, yi, MK_RECV, WL_RECV);
 }
 
 template <int S>
 __device__ __forceinline__ void conv_claim_body(const Dev &d, const VB &vb) {
+    const int lane = threadIdx.x & 31;
     {
-        LIST_LOOP(WL_FILLED, a) claim_receivers<S>(d, d.list[WL_FILLED][it_a], MK_FILLED);
+        WARP_LOOP(WL_FILLED, a) claim_receivers<S>(d, lane, d.list[WL_FILLED][it_a], MK_FILLED);
     }
     {
-        LIST_LOOP(WL_EMPTIED, b) {
-            long long i = d.list[WL_EMPTIED][it_b];
+        WARP_LOOP(WL_EMPTIED, b) {
+            const long long i = d.list[WL_EMPTIED][it_b];
             const uint8_t mk = d.cmark[i];
-            if (mk & MK_EMPTIED) claim_receivers<S>(d, i, mk);
+            if (mk & MK_EMPTIED) claim_receivers<S>(d, lane, i, mk);
         }
     }
 }
 template <int S>
 __global__ void k_conv_claim(const __grid_constant__ Dev d) { conv_claim_body<S>(d, vb_own()); }
 
-// k(x): interface neighbours of a converted cell (classes after conversion)
-__device__ __forceinline__ int iface_neighbours(const Dev &d, long long i) {
-    int x, y, z;
-    coords(d, i, x, y, z);
-    int k = 0;
-#pragma unroll
-    for (int q = 1; q < Q; ++q) {
-        long long yi = nbr(d, x, y, z, cx(q), cy(q), cz(q));
-        if (yi >= 0 && clsv(d, yi) == CL_I) k++;
-    }
-    return k;
-}
-
-template <int S>
-__device__ __forceinline__ double excess(const Dev &d, long long i, uint8_t mk) {
-    return (mk & MK_FILLED) ? d.m[i] - cell_density<S>(d, d.fdst, i) : d.m[i];
-}
-
 // receivers gather e(x) / k(x) over their converted neighbours in q order
+// (the receivers are many: a thread each, its loads requested at once)
 template <int S>
 __device__ __forceinline__ void conv_excess_body(const Dev &d, const VB &vb) {
     LIST_LOOP(WL_RECV, a) {
@@ -2848,106 +3038,129 @@ __device__ __forceinline__ void conv_excess_body(const Dev &d, const VB &vb) {
             long long yi = nbr(d, x, y, z, cx(q), cy(q), cz(q));
             if (yi >= 0 && (d.cmark[yi] & (MK_FILLED | MK_EMPTIED))) cm |= 1u << q;
         }
-        double sh[Q];
-#pragma unroll
-        for (int q = 1; q < Q; ++q) sh[q] = (cm & (1u << q)) ? d.m[nbr(d, x, y, z, cx(q), cy(q), cz(q))] : 0.0;
-        double acc = 0.0;
-#pragma unroll
-        for (int q = 1; q < Q; ++q)
-            if (cm & (1u << q)) acc += sh[q];
-        double m = d.m[i] + acc;
+        const double rho = cell_density<S>(d, d.fdst, i);
+        double m = d.m[i], acc = 0.0;
+        for (unsigned b = cm; b; b &= b - 1) {
+            const int q = __ffs(b) - 1;
+            acc += d.m[nbr(d, x, y, z, dir_x(q), dir_y(q), dir_z(q))];
+        }
+        m = m + acc;
         d.m[i] = m;
-        d.phidst[i] = m / cell_density<S>(d, d.fdst, i);
+        const double ph = m / rho;
+        d.phidst[i] = ph;
+        if constexpr (S != 0) d.phifdst[i] = (float)ph;
     }
 }
 template <int S>
 __global__ void k_conv_excess(const __grid_constant__ Dev d) { conv_excess_body<S>(d, vb_own()); }
 
-// mass that found no interface neighbour goes to the ledger; marks are cleared
-template <int S>
+// marks are cleared
 __device__ __forceinline__ void conv_finish_body(const Dev &d, const VB &vb) {
-    {
-        LIST_LOOP(WL_FILLED, a) {
-            long long i = d.list[WL_FILLED][it_a];
-            if (iface_neighbours(d, i) == 0) atomicAdd(&d.ledger[LG_LOST], excess<S>(d, i, MK_FILLED));
-            d.cmark[i] = 0;
-        }
-    }
-    {
-        LIST_LOOP(WL_EMPTIED, b) {
-            long long i = d.list[WL_EMPTIED][it_b];
-            uint8_t mk = d.cmark[i];
-            if ((mk & MK_EMPTIED) && iface_neighbours(d, i) == 0) atomicAdd(&d.ledger[LG_LOST], excess<S>(d, i, mk));
-            d.cmark[i] = 0;
-        }
-    }
-    {
-        LIST_LOOP(WL_NEWG, c) d.cmark[d.list[WL_NEWG][it_c]] = 0;
-    }
-    {
-        LIST_LOOP(WL_NEWL, e) d.cmark[d.list[WL_NEWL][it_e]] = 0;
-    }
-    {
-        LIST_LOOP(WL_RECV, g) d.cmark[d.list[WL_RECV][it_g]] = 0;
+    const int lists[5] = {WL_FILLED, WL_EMPTIED, WL_NEWG, WL_NEWL, WL_RECV};
+#pragma unroll
+    for (int k = 0; k < 5; ++k) {
+        LIST_LOOP(lists[k], a) d.cmark[d.list[lists[k]][it_a]] = 0;
     }
 }
-template <int S>
-__global__ void k_conv_finish(const __grid_constant__ Dev d) { conv_finish_body<S>(d, vb_own()); }
+__global__ void k_conv_finish(const __grid_constant__ Dev d) { conv_finish_body(d, vb_own()); }
 
 // ----------------------------------------------- C5: rigid-body update
 // (the role the paper gives the pe engine, Sec. 2.3: the body moves under the
 // hydrodynamic force and torque and gravity; the paper does not give the
 // integrator, this one is a virtual-mass explicit update)
 
-// one warp per body: fixed-order sum of the force partials, then the update
-__device__ __forceinline__ void body_step(const Dev &d, Body &b, const double *acc);
+// One warp per body: the fixed-order sum of the force partials, then the
+// update.  A double operation holds the scheduler for 64 cycles and a division
+// for 550 whatever the number of active lanes, so the update is written for
+// lanes: lane l works on component k = l % 3 of the vectors, lanes with
+// (l / 3) odd on the rotation where it mirrors the translation, and lanes 0..8
+// on the nine entries of a rotation matrix.  Every value is the scalar update's
+// (one thread, about 700 double operations, 22 us; now about 200), rounded the
+// same way: this unit is compiled without fused multiply-add.
+__device__ __forceinline__ double lane_of(double v, int l) { return __shfl_sync(0xffffffffu, v, l); }
+// (a_0 + a_1) + a_2 of the values that lanes base .. base + 2 hold
+__device__ __forceinline__ double sum3(double a, int base) {
+    return (lane_of(a, base) + lane_of(a, base + 1)) + lane_of(a, base + 2);
+}
+// entry lane (row-major, lanes 0..8) of the rotation matrix of the quaternion
+// whose component j lane j holds (see rotation)
+__device__ __forceinline__ double rotation_lane(double q, int lane) {
+    const int e = lane < 9 ? lane : 0, i = e / 3, j = e - 3 * i;
+    const bool diag = i == j;
+    // diagonal: 1 - 2 (a a + b b) with the two other axes; else 2 (x_i x_j +- w x_k)
+    const int o1 = i == 0 ? 1 : 0, o2 = i == 2 ? 1 : 2, k = 3 - i - j;
+    const bool neg = !diag && (j - i + 3) % 3 == 1;
+    const double p1 = lane_of(q, 1 + (diag ? o1 : i)) * lane_of(q, 1 + (diag ? o1 : j));
+    const double p2 = lane_of(q, diag ? 1 + o2 : 0) * lane_of(q, 1 + (diag ? o2 : k));
+    const double r = 2.0 * (p1 + (neg ? -p2 : p2));
+    return diag ? 1.0 - r : r;
+}
 __device__ __forceinline__ void bodies_body(const Dev &d, const VB &vb) {
-    int bi = vb.x;
-    int lane = threadIdx.x;
-    double acc[7];
+    const int bi = vb.x, lane = threadIdx.x & 31;
+    const Body &b = d.bodies[bi];
+    Body &nb = d.bodies_new[bi];
+    static_assert(sizeof(Body) % 8 == 0, "body records are copied in 8-byte words");
+    for (int w = lane; w < (int)(sizeof(Body) / 8); w += 32)
+        reinterpret_cast<unsigned long long *>(&nb)[w] = reinterpret_cast<const unsigned long long *>(&b)[w];
+    double tot;  // lane c < 7 holds sum c: force, torque, |terms|
+    const int k = lane % 3, k1 = k == 2 ? 0 : k + 1, k2 = k == 0 ? 2 : k - 1;
+    const bool rot = (lane / 3) & 1;
     if (d.part128) {
         // double storage: exact 128-bit partials (fixed96), summed exactly
         const unsigned long long *pp = reinterpret_cast<const unsigned long long *>(d.part);
-#pragma unroll 1
-        for (int c = 0; c < 7; ++c) {
-            unsigned __int128 v = 0;
-            for (int k = lane; k < FORCE_BLOCKS; k += 32) {
-                const long long j = 2 * (((long long)bi * FORCE_BLOCKS + k) * 7 + c);
-                v += ((unsigned __int128)pp[j + 1] << 64) | (unsigned __int128)pp[j];
-            }
-            for (int off = 16; off > 0; off >>= 1) v += shfl_down_128(v, off);
-            acc[c] = fixed96_value(v);
-        }
-    } else {
+        unsigned __int128 mine = 0;
 #pragma unroll
         for (int c = 0; c < 7; ++c) {
-            double v = 0.0;
-            for (int k = lane; k < FORCE_BLOCKS; k += 32) v += d.part[((long long)bi * FORCE_BLOCKS + k) * 7 + c];
-            for (int off = 16; off > 0; off >>= 1) v += __shfl_down_sync(0xffffffffu, v, off);
-            acc[c] = v;
+            unsigned __int128 v = 0;
+            for (int j = lane; j < FORCE_BLOCKS; j += 32) {
+                const long long at = 2 * (((long long)bi * FORCE_BLOCKS + j) * 7 + c);
+                v += ((unsigned __int128)pp[at + 1] << 64) | (unsigned __int128)pp[at];
+            }
+            for (int off = 16; off > 0; off >>= 1) v += shfl_xor_128(v, off);
+            if ((lane & 7) == c) mine = v;
         }
+        tot = fixed96_value(mine);
+    } else {
+        static_assert(FORCE_BLOCKS == 64, "two partials per lane");
+        // tree sums (lane l + lane l + off) of the seven components packed so
+        // that each level halves the registers: 9 additions instead of 35
+        double v[8];
+#pragma unroll
+        for (int c = 0; c < 7; ++c) {
+            const double *p = d.part + ((long long)bi * FORCE_BLOCKS + lane) * 7 + c;
+            v[c] = p[0] + p[32 * 7];
+        }
+        v[7] = 0.0;
+#pragma unroll
+        for (int h = 0; h < 3; ++h) {
+            const int off = 16 >> h;
+            const bool up = lane & off;
+#pragma unroll
+            for (int c = 0; c < (8 >> h); c += 2) {
+                const double send = up ? v[c] : v[c + 1], keep = up ? v[c + 1] : v[c];
+                v[c / 2] = keep + __shfl_xor_sync(0xffffffffu, send, off);
+            }
+        }
+        double t = v[0];
+        t += __shfl_xor_sync(0xffffffffu, t, 2);
+        t += __shfl_xor_sync(0xffffffffu, t, 1);
+        // component c sits where bit 4, 3, 2 of the lane are bit 0, 1, 2 of c
+        const int c = lane & 7;
+        tot = lane_of(t, ((c & 1) << 4) | ((c & 2) << 2) | (c & 4));
     }
-    if (lane != 0) return;
-    // the body record is read once into registers, updated, and written back
-    // (instead of a chain of dependent global-memory reads and writes)
-    Body b = d.bodies[bi];
-    body_step(d, b, acc);
-    d.bodies[bi] = b;
-}
-
-__device__ __forceinline__ void body_step(const Dev &d, Body &b, const double *acc) {
-    for (int k = 0; k < 3; ++k) {
-        b.F[k] = acc[k];
-        b.T[k] = acc[3 + k];
+    // (either way lane c holds sum c)
+    const double ft = lane_of(tot, rot ? 3 + k : k), fabs_sum = lane_of(tot, 6);
+    __syncwarp();
+    if (lane < 3) {
+        nb.F[k] = ft;
+        nb.plo[k] = b.lo[k];
+        nb.phi[k] = b.hi[k];
     }
-    b.S = acc[6];
-    for (int k = 0; k < 3; ++k) {
-        b.plo[k] = b.lo[k];
-        b.phi[k] = b.hi[k];
-    }
-    int base = b.mode & 0xff;
+    if (lane >= 3 && lane < 6) nb.T[k] = ft;
+    if (lane == 0) nb.S = fabs_sum;
+    const int base = b.mode & 0xff;
     if (base == 0) {
-        for (int k = 0; k < 3; ++k) b.v[k] = b.w[k] = b.dv[k] = b.dw[k] = 0.0;
+        if (lane < 3) nb.v[k] = nb.w[k] = nb.dv[k] = nb.dw[k] = 0.0;
         return;
     }
     // the update is driven by the mean of this step's and the previous step's
@@ -2955,137 +3168,189 @@ __device__ __forceinline__ void body_step(const Dev &d, Body &b, const double *a
     // throughout when the two-step mean is switched off): near tau = 1/2 a
     // force that flips sign every step would feed the barely damped BGK modes
     // of that period through the wall velocity
-    double Fh[3], Th[3];
-    const bool mean = d.force_mean && b.nF;
-    for (int k = 0; k < 3; ++k) {
-        Fh[k] = mean ? 0.5 * (b.F[k] + b.Fp[k]) : b.F[k];
-        Th[k] = mean ? 0.5 * (b.T[k] + b.Tp[k]) : b.T[k];
-        b.Fp[k] = b.F[k];
-        b.Tp[k] = b.T[k];
-    }
-    b.nF = 1;
-    double vol, mass, I[3];
+    const double ftp = rot ? b.Tp[k] : b.Fp[k];
+    const double fh = d.force_mean && b.nF ? 0.5 * (ft + ftp) : ft;  // force, or torque (rot)
+    const double hk = b.h[k], dens = b.dens, C = d.vmass;
+    const double h0 = b.h[0], hsq = hk * hk;
+    double vol, mass, I;
     if (b.shape == 1) {  // sphere: V = 4/3 pi r^3, I = 2/5 m r^2
-        vol = 4.1887902047863905 * ((b.h[0] * b.h[0]) * b.h[0]);
-        mass = b.dens * vol;
-        I[0] = I[1] = I[2] = (0.4 * mass) * (b.h[0] * b.h[0]);
+        vol = 4.1887902047863905 * ((h0 * h0) * h0);
+        mass = dens * vol;
+        I = (0.4 * mass) * (h0 * h0);
     } else {
-        vol = ((8.0 * b.h[0]) * b.h[1]) * b.h[2];
-        mass = b.dens * vol;
-        I[0] = (mass / 3.0) * (b.h[1] * b.h[1] + b.h[2] * b.h[2]);
-        I[1] = (mass / 3.0) * (b.h[0] * b.h[0] + b.h[2] * b.h[2]);
-        I[2] = (mass / 3.0) * (b.h[0] * b.h[0] + b.h[1] * b.h[1]);
+        vol = ((8.0 * h0) * b.h[1]) * b.h[2];
+        mass = dens * vol;
+        I = (mass / 3.0) * (lane_of(hsq, k == 0 ? 1 : 0) + lane_of(hsq, k == 2 ? 1 : 2));
     }
-    double If[3] = {I[0] / b.dens, I[1] / b.dens, I[2] / b.dens};
-    const double C = d.vmass;  // virtual-mass coefficient (Schwarz, Kempe and Froehlich 2015)
+    double q = b.q[lane & 3];
+    const double R = rotation_lane(q, lane);
+    const double c0 = lane_of(R, k), c1 = lane_of(R, 3 + k), c2 = lane_of(R, 6 + k);  // column k
+    const double T0 = lane_of(fh, 3), T1 = lane_of(fh, 4), T2 = lane_of(fh, 5);
+    const double w0 = b.w[0], w1 = b.w[1], w2 = b.w[2];
+    double num = (fh + mass * d.grav[k]) + C * (vol * b.dv[k]);  // translation (virtual mass: Schwarz, Kempe and Froehlich 2015)
     double den = mass + C * vol;
-    for (int k = 0; k < 3; ++k) {
-        double num = (Fh[k] + mass * d.grav[k]) + C * (vol * b.dv[k]);
-        b.dv[k] = num / den;
-        b.v[k] = b.v[k] + b.dv[k];
-    }
-    if (b.mode & 0x100)
-        for (int k = 0; k < 3; ++k) b.v[k] = b.v[k] * (1.0 - b.damp);
-    double R[9];
-    rotation(b.q, R);
+    double wb = 0.0, rnum, rden;
     if (base == 2) {
-        const double *ax = b.axis;
-        double ta = (Th[0] * ax[0] + Th[1] * ax[1]) + Th[2] * ax[2];
-        double ab[3];
-        for (int k = 0; k < 3; ++k) ab[k] = (R[0 * 3 + k] * ax[0] + R[1 * 3 + k] * ax[1]) + R[2 * 3 + k] * ax[2];
-        double Ia = (ab[0] * ab[0] * I[0] + ab[1] * ab[1] * I[1]) + ab[2] * ab[2] * I[2];
-        double Ifa = Ia / b.dens;
-        double ws = (b.w[0] * ax[0] + b.w[1] * ax[1]) + b.w[2] * ax[2];
-        b.dw[0] = (ta + C * (Ifa * b.dw[0])) / (Ia + C * Ifa);
-        ws = ws + b.dw[0];
-        for (int k = 0; k < 3; ++k) b.w[k] = ws * ax[k];
+        const double a0 = b.axis[0], a1 = b.axis[1], a2 = b.axis[2];
+        const double ta = (T0 * a0 + T1 * a1) + T2 * a2;
+        const double ab = (c0 * a0 + c1 * a1) + c2 * a2;
+        const double Ia = sum3((ab * ab) * I, 0);
+        const double Ifa = Ia / dens;
+        wb = (w0 * a0 + w1 * a1) + w2 * a2;
+        rnum = ta + C * (Ifa * b.dw[0]);
+        rden = Ia + C * Ifa;
     } else {
-        double wb[3], tb[3], L[3], gy[3];
-        for (int k = 0; k < 3; ++k) {
-            wb[k] = (R[0 * 3 + k] * b.w[0] + R[1 * 3 + k] * b.w[1]) + R[2 * 3 + k] * b.w[2];
-            tb[k] = (R[0 * 3 + k] * Th[0] + R[1 * 3 + k] * Th[1]) + R[2 * 3 + k] * Th[2];
-            L[k] = I[k] * wb[k];
-        }
-        gy[0] = wb[1] * L[2] - wb[2] * L[1];
-        gy[1] = wb[2] * L[0] - wb[0] * L[2];
-        gy[2] = wb[0] * L[1] - wb[1] * L[0];
-        for (int k = 0; k < 3; ++k) {
-            b.dw[k] = ((tb[k] - gy[k]) + C * (If[k] * b.dw[k])) / (I[k] + C * If[k]);
-            wb[k] = wb[k] + b.dw[k];
-        }
-        for (int k = 0; k < 3; ++k) b.w[k] = (R[k * 3 + 0] * wb[0] + R[k * 3 + 1] * wb[1]) + R[k * 3 + 2] * wb[2];
+        const double If = I / dens;
+        wb = (c0 * w0 + c1 * w1) + c2 * w2;
+        const double tb = (c0 * T0 + c1 * T1) + c2 * T2;
+        const double L = I * wb;
+        const double gy = lane_of(wb, k1) * lane_of(L, k2) - lane_of(wb, k2) * lane_of(L, k1);
+        rnum = (tb - gy) + C * (If * b.dw[k]);
+        rden = I + C * If;
     }
-    double nn[3] = {(double)d.nx, (double)d.ny, (double)d.nz};
-    for (int k = 0; k < 3; ++k) {
-        b.o[k] = b.o[k] + b.v[k];
-        if (d.periodic & (1u << k)) {
-            if (b.o[k] >= nn[k]) b.o[k] = b.o[k] - nn[k];
-            else if (b.o[k] < 0.0) b.o[k] = b.o[k] + nn[k];
-        }
+    const double acc = (rot ? rnum : num) / (rot ? rden : den);  // dv (lanes 0..2), dw (lanes 3..5)
+    const double dv = lane_of(acc, k), dw = lane_of(acc, 3 + k);
+    double v = b.v[k] + dv;
+    if (b.mode & 0x100) v = v * (1.0 - b.damp);
+    double w;
+    if (base == 2) {
+        w = (wb + lane_of(dw, 0)) * b.axis[k];
+    } else {
+        wb = wb + dw;
+        w = (lane_of(R, 3 * k) * lane_of(wb, 0) + lane_of(R, 3 * k + 1) * lane_of(wb, 1)) +
+            lane_of(R, 3 * k + 2) * lane_of(wb, 2);
     }
-    double qw = b.q[0], qx = b.q[1], qy = b.q[2], qz = b.q[3];
-    const double *w = b.w;
-    double dw = -((w[0] * qx + w[1] * qy) + w[2] * qz);
-    double dx = qw * w[0] + (w[1] * qz - w[2] * qy);
-    double dy = qw * w[1] + (w[2] * qx - w[0] * qz);
-    double dz = qw * w[2] + (w[0] * qy - w[1] * qx);
-    double nq[4] = {qw + 0.5 * dw, qx + 0.5 * dx, qy + 0.5 * dy, qz + 0.5 * dz};
-    double norm = sqrt(((nq[0] * nq[0] + nq[1] * nq[1]) + nq[2] * nq[2]) + nq[3] * nq[3]);
-    for (int k = 0; k < 4; ++k) b.q[k] = nq[k] / norm;
-    body_bounds(d, b);
-    // a moving box that reaches a wall plane would need a contact model
-    // (the paper's rigid-body engine); report it instead of running on
-    for (int k = 0; k < 3; ++k) {
-        if (d.periodic & (1u << k)) continue;
-        const double e = b.shape == 1 ? b.h[0]
-                                      : (fabs(b.R[k * 3 + 0]) * b.h[0] + fabs(b.R[k * 3 + 1]) * b.h[1]) +
-                                            fabs(b.R[k * 3 + 2]) * b.h[2];
-        const double n = k == 0 ? d.nx : (k == 1 ? d.ny : d.nz);
-        if (b.o[k] - e < 0.0 || b.o[k] + e > n) atomicOr(d.status, ST_CONTACT);
+    const int nk = k == 0 ? d.nx : (k == 1 ? d.ny : d.nz);
+    const double nn = (double)nk;
+    double o = b.o[k] + v;
+    if (d.periodic & (1u << k)) {
+        if (o >= nn) o = o - nn;
+        else if (o < 0.0) o = o + nn;
+    }
+    {
+        // lane j < 4: component j of the quaternion's rate of change,
+        //   -((w0 qx + w1 qy) + w2 qz), qw w0 + (w1 qz - w2 qy), ...
+        const int j = lane & 3;
+        const double v0 = lane_of(w, 0), v1 = lane_of(w, 1), v2 = lane_of(w, 2);
+        const double qw = lane_of(q, 0), qx = lane_of(q, 1), qy = lane_of(q, 2), qz = lane_of(q, 3);
+        const double m1 = (j == 0 ? v0 : qw) * (j == 0 ? qx : (j == 1 ? v0 : (j == 2 ? v1 : v2)));
+        const double m2 = (j == 0 ? v1 : (j == 1 ? v1 : (j == 2 ? v2 : v0))) * (j == 0 ? qy : (j == 1 ? qz : (j == 2 ? qx : qy)));
+        const double m3 = (j == 0 ? v2 : (j == 1 ? v2 : (j == 2 ? v0 : v1))) * (j == 0 ? qz : (j == 1 ? qy : (j == 2 ? qz : qx)));
+        const double s = (j == 0 ? m1 : m2) + (j == 0 ? m2 : -m3);
+        const double t = s + (j == 0 ? m3 : m1);
+        const double nq = q + 0.5 * (j == 0 ? -t : t);
+        const double sq = nq * nq;
+        const double norm = sqrt(((lane_of(sq, 0) + lane_of(sq, 1)) + lane_of(sq, 2)) + lane_of(sq, 3));
+        q = nq / norm;
+    }
+    // the new pose's rotation, its float copies and the cells it may cover
+    const double Rn = rotation_lane(q, lane);
+    const double fl = floor(o);
+    const double e = b.shape == 1 ? h0
+                                  : (fabs(lane_of(Rn, 3 * k)) * h0 + fabs(lane_of(Rn, 3 * k + 1)) * b.h[1]) +
+                                        fabs(lane_of(Rn, 3 * k + 2)) * b.h[2];
+    const double olo = o - e, ohi = o + e;
+    int lo = (int)floor(olo) - 1, hi = (int)floor(ohi) + 2;
+    if (!(d.periodic & (1u << k))) {
+        lo = lo < 0 ? 0 : lo;
+        hi = hi > nk ? nk : hi;
+    } else if (hi - lo > nk) {
+        hi = lo + nk;
+    }
+    if (hi < lo) hi = lo;
+    if (lane < 9) {
+        nb.R[lane] = Rn;
+        nb.Rf[lane] = (float)Rn;
+    }
+    if (lane < 4) nb.q[lane] = q;
+    if (lane == 0) nb.nF = 1;
+    if (lane < 3) {
+        nb.Fp[k] = ft;
+        nb.dv[k] = dv;
+        nb.v[k] = v;
+        nb.o[k] = o;
+        nb.oi[k] = (int)fl;
+        nb.of[k] = (float)(o - fl);
+        nb.hf[k] = (float)(b.shape == 1 && k == 0 ? h0 * h0 : hk);
+        nb.lo[k] = lo;
+        nb.hi[k] = hi;
+        // a moving box that reaches a wall plane would need a contact model
+        // (the paper's rigid-body engine); report it instead of running on
+        if (!(d.periodic & (1u << k)) && (olo < 0.0 || ohi > nn)) atomicOr(d.status, ST_CONTACT);
+    }
+    if (lane >= 3 && lane < 6) {
+        nb.Tp[k] = ft;
+        if (base != 2 || k == 0) nb.dw[k] = dw;
+        nb.w[k] = w;
     }
 }
 __global__ void k_bodies(const __grid_constant__ Dev d) { bodies_body(d, vb_own()); }
 
 // ----------------------------------------------- C6: remap (Sec. 2.3, 2.4)
 
-// cells inside body vb.y at its new pose become obstacle
-template <int S>
-__device__ __forceinline__ void remap_cover_body(const Dev &d, const VB &vb) {
-    int bi = vb.y;
-    const Body &b = d.bodies[bi];
-    long long n = range_count(b.lo, b.hi);
-    for (long long k = vb.x * (long long)blockDim.x + threadIdx.x; k < n; k += (long long)vb.nx * blockDim.x) {
-        int x, y, z;
-        range_cell(d, b.lo, b.hi, k, x, y, z);
-        long long i = x + (long long)d.nx * (y + (long long)d.ny * z);
-        int c = clsv(d, i);
-        bool cover = c != CL_O && inside(d, b, x, y, z);
-        wl_append(d, cover, WL_COVER, (uint32_t)i);
-        if (!cover) continue;
-        double mass = c == CL_L ? cell_density<S>(d, d.fdst, i) : (c == CL_I ? d.m[i] : 0.0);
-        if (mass != 0.0) atomicAdd(&d.ledger[LG_COVERED], mass);
-        set_cls(d, i, CL_O);
-        d.bid[i] = (uint8_t)bi;
+// Which cells body vb.y covers and which it leaves with its new pose: the
+// obstacle set is not touched by the conversions, so the lists are made from
+// it and the two poses alone, beside the bulk kernel; remap_apply_body acts on
+// them once the conversions are done.
+__device__ __forceinline__ void remap_scan_body(const Dev &d, const VB &vb) {
+    const int bi = vb.y;
+    const Body &b = d.bodies_new[bi];
+    const uint32_t lane = threadIdx.x & 31u;
+    uint32_t first, stride;
+    const uint32_t n = (uint32_t)range_count(b.lo, b.hi);
+    list_span(vb, n, 32u, first, stride);
+    for (uint32_t k0 = first; k0 < n; k0 += stride) {
+        const uint32_t kk = k0 + lane;
+        long long i = 0;
+        bool cover = false;
+        if (kk < n) {
+            int x, y, z;
+            range_cell(d, b.lo, b.hi, kk, x, y, z);
+            i = x + (long long)d.nx * (y + (long long)d.ny * z);
+            cover = clsv(d, i) != CL_O && inside(d, b, x, y, z);
+        }
+        if (__any_sync(0xffffffffu, cover)) wl_append(d, cover, WL_COVER, (uint32_t)i);
+        // the covering body, for remap_apply_body (an obstacle's id is set
+        // there; until then nothing reads a fluid cell's id)
+        if (cover) d.bid[i] = (uint8_t)bi;
+    }
+    const uint32_t m = (uint32_t)range_count(b.plo, b.phi);
+    list_span(vb, m, 32u, first, stride);
+    for (uint32_t k0 = first; k0 < m; k0 += stride) {
+        const uint32_t kk = k0 + lane;
+        long long i = 0;
+        bool pend = false;
+        if (kk < m) {
+            int x, y, z;
+            range_cell(d, b.plo, b.phi, kk, x, y, z);
+            i = x + (long long)d.nx * (y + (long long)d.ny * z);
+            pend = clsv(d, i) == CL_O && d.bid[i] == bi && !inside(d, b, x, y, z);
+        }
+        if (__any_sync(0xffffffffu, pend)) wl_append(d, pend, WL_PEND, (uint32_t)i);
     }
 }
-template <int S>
-__global__ void k_remap_cover(const __grid_constant__ Dev d) { remap_cover_body<S>(d, vb_own()); }
+__global__ void k_remap_scan(const __grid_constant__ Dev d) { remap_scan_body(d, vb_own()); }
 
-// obstacle cells of body vb.y outside its new pose are pending
-__device__ __forceinline__ void remap_pending_body(const Dev &d, const VB &vb) {
-    int bi = vb.y;
-    const Body &b = d.bodies[bi];
-    long long n = range_count(b.plo, b.phi);
-    for (long long k = vb.x * (long long)blockDim.x + threadIdx.x; k < n; k += (long long)vb.nx * blockDim.x) {
-        int x, y, z;
-        range_cell(d, b.plo, b.phi, k, x, y, z);
-        long long i = x + (long long)d.nx * (y + (long long)d.ny * z);
-        bool pend = clsv(d, i) == CL_O && d.bid[i] == bi && !inside(d, b, x, y, z);
-        if (pend) d.cmark[i] = MK_PEND;
-        wl_append(d, pend, WL_PEND, (uint32_t)i);
+// listed cells inside a body's new pose become obstacle, their mass is booked;
+// listed obstacle cells outside it are pending
+template <int S>
+__device__ __forceinline__ void remap_apply_body(const Dev &d, const VB &vb) {
+    {
+        LIST_LOOP(WL_COVER, a) {
+            const long long i = d.list[WL_COVER][it_a];
+            const int c = clsv(d, i);
+            if (c == CL_O) continue;  // two bodies cover it
+            const double mass = c == CL_L ? cell_density<S>(d, d.fdst, i) : (c == CL_I ? d.m[i] : 0.0);
+            if (mass != 0.0) atomicAdd(&d.ledger[LG_COVERED], mass);
+            set_cls(d, i, CL_O);
+        }
+    }
+    {
+        LIST_LOOP(WL_PEND, b) d.cmark[d.list[WL_PEND][it_b]] = MK_PEND;
     }
 }
-__global__ void k_remap_pending(const __grid_constant__ Dev d) { remap_pending_body(d, vb_own()); }
+template <int S>
+__global__ void k_remap_apply(const __grid_constant__ Dev d) { remap_apply_body<S>(d, vb_own()); }
 
 // Jacobi passes of the obstacle-to-fluid rule over the pending cells, closure,
 // uncovered-mass ledger (one block)
@@ -3095,79 +3360,81 @@ __device__ __forceinline__ void remap_resolve_body(const Dev &d, const VB &vb) {
     if (n == 0) return;
     __shared__ int s_any;
     for (int pass = 0; pass < 4; ++pass) {
-        for (uint32_t it = threadIdx.x; it < n; it += blockDim.x) {
-            long long i = d.list[WL_PEND][it];
-            d.rdec[it] = 0;
-            if (!(d.cmark[i] & MK_PEND)) continue;
+        // a warp per pending cell, lane q its neighbour in direction q
+        for (uint32_t it = threadIdx.x >> 5; it < n; it += blockDim.x >> 5) {
+            const int lane = threadIdx.x & 31;
+            const long long i = d.list[WL_PEND][it];
+            if (!(d.cmark[i] & MK_PEND)) {
+                if (lane == 0) d.rdec[it] = 0;
+                continue;
+            }
             int x, y, z;
             coords(d, i, x, y, z);
-            int nL = 0, nI = 0, nG = 0;
+            const long long yi = lane_nbr(d, lane, x, y, z);
+            const int c = (yi < 0 || (d.cmark[yi] & MK_PEND)) ? 0 : clsv(d, yi);
+            const unsigned full = 0xffffffffu;
+            const unsigned mL = __ballot_sync(full, c == CL_L), mI = __ballot_sync(full, c == CL_I),
+                           mG = __ballot_sync(full, c == CL_G);
+            const int nL = __popc(mL), nI = __popc(mI), nG = __popc(mG);
+            double r = 0.0, ph = 0.0;
+            if (c == CL_L || c == CL_I) r = cell_density<S>(d, d.fdst, yi);
+            if (c == CL_I) ph = d.phidst[yi];
+            // sums in q order
             double sr = 0.0, sp = 0.0;
-            // marks and classes requested at once, then the neighbours in q order
-            uint8_t cs[Q];
-#pragma unroll
-            for (int q = 1; q < Q; ++q) {
-                long long yi = nbr(d, x, y, z, cx(q), cy(q), cz(q));
-                cs[q] = (yi < 0 || (d.cmark[yi] & MK_PEND)) ? (uint8_t)0 : (uint8_t)clsv(d, yi);
-            }
-#pragma unroll 1
-            for (int q = 1; q < Q; ++q) {
-                const int c = cs[q];
-                if (c == 0 || c == CL_O) continue;
-                long long yi = nbr(d, x, y, z, cx(q), cy(q), cz(q));
-                if (c == CL_L) {
-                    nL++;
-                    sr += cell_density<S>(d, d.fdst, yi);
-                } else if (c == CL_I) {
-                    nI++;
-                    sr += cell_density<S>(d, d.fdst, yi);
-                    sp += d.phidst[yi];
-                } else if (c == CL_G) {
-                    nG++;
+            for (unsigned m = mL | mI; m; m &= m - 1) sr += __shfl_sync(full, r, __ffs(m) - 1);
+            for (unsigned m = mI; m; m &= m - 1) sp += __shfl_sync(full, ph, __ffs(m) - 1);
+            if (lane == 0) {
+                uint8_t dec = 0;
+                if (nL > 0 && nG > 0) {
+                    dec = CL_I;
+                    d.rrho[it] = sr / (nL + nI);
+                    d.rphi[it] = nI > 0 ? sp / nI : 0.5;
+                } else if (nG == 0 && nL + nI > 0) {
+                    dec = CL_L;
+                    d.rrho[it] = sr / (nL + nI);
+                } else if (nL == 0 && nG > 0) {
+                    dec = CL_G;
                 }
+                d.rdec[it] = dec;
             }
-            uint8_t dec = 0;
-            if (nL > 0 && nG > 0) {
-                dec = CL_I;
-                d.rrho[it] = sr / (nL + nI);
-                d.rphi[it] = nI > 0 ? sp / nI : 0.5;
-            } else if (nG == 0 && nL + nI > 0) {
-                dec = CL_L;
-                d.rrho[it] = sr / (nL + nI);
-            } else if (nL == 0 && nG > 0) {
-                dec = CL_G;
-            }
-            d.rdec[it] = dec;
         }
         if (threadIdx.x == 0) s_any = 0;
         __syncthreads();
-        for (uint32_t it = threadIdx.x; it < n; it += blockDim.x) {
-            long long i = d.list[WL_PEND][it];
-            if (!(d.cmark[i] & MK_PEND)) continue;
+        for (uint32_t it = threadIdx.x >> 5; it < n; it += blockDim.x >> 5) {
+            const int lane = threadIdx.x & 31;
+            const long long i = d.list[WL_PEND][it];
+            const bool open = d.cmark[i] & MK_PEND;
+            __syncwarp();
+            if (!open) continue;
             int dec = d.rdec[it];
             if (dec == 0 && pass == 3) dec = CL_G;
             if (dec == 0) {
-                s_any = 1;
+                if (lane == 0) s_any = 1;
                 continue;
             }
-            const Body &b = d.bodies[d.bid[i]];
-            d.cmark[i] = MK_FRESH;
-            set_cls(d, i, dec);
+            const Body &b = d.bodies_new[d.bid[i]];
+            if (lane == 0) {
+                d.cmark[i] = MK_FRESH;
+                set_cls(d, i, dec);
+            }
             if (dec == CL_G) continue;
             int x, y, z;
             coords(d, i, x, y, z);
-            if (z > *d.ztop_wr + ZTOP_MARGIN) atomicOr(d.status, ST_TOP);
+            if (lane == 0 && z > *d.ztop_wr + ZTOP_MARGIN) atomicOr(d.status, ST_TOP);
             double p[3] = {x + 0.5, y + 0.5, z + 0.5}, uw[3];
             body_velocity_at(d, b, p, uw);
-            double f[Q];
-            double rho = d.rrho[it];
-#pragma unroll
-            for (int q = 0; q < Q; ++q) f[q] = feq_d(q, rho, uw);
-            Sto<S>::st_cell(d.fdst, i, d.N, f);
+            const double rho = d.rrho[it];
+            warp_store_cell<S>(d, i, lane, feq_lane(lane, rho, uw));
+            __syncwarp();
             if (dec == CL_I) {
-                double m = d.rphi[it] * rho;
-                d.m[i] = m;
-                d.phidst[i] = m / cell_density<S>(d, d.fdst, i);
+                const double dens = warp_density<S>(d, d.fdst, i);
+                if (lane == 0) {
+                    const double m = d.rphi[it] * rho;
+                    d.m[i] = m;
+                    const double ph = m / dens;
+                    d.phidst[i] = ph;
+                    if constexpr (S != 0) d.phifdst[i] = (float)ph;
+                }
             }
         }
         __syncthreads();
@@ -3175,31 +3442,33 @@ __device__ __forceinline__ void remap_resolve_body(const Dev &d, const VB &vb) {
         __syncthreads();
     }
     // closure: a new liquid cell next to gas becomes interface with phi = 1
-    for (uint32_t it = threadIdx.x; it < n; it += blockDim.x) {
-        long long i = d.list[WL_PEND][it];
+    for (uint32_t it = threadIdx.x >> 5; it < n; it += blockDim.x >> 5) {
+        const int lane = threadIdx.x & 31;
+        const long long i = d.list[WL_PEND][it];
         if (!(d.cmark[i] & MK_FRESH) || clsv(d, i) != CL_L) continue;
         int x, y, z;
         coords(d, i, x, y, z);
-        bool gas = false;
-        for (int q = 1; q < Q; ++q) {
-            long long yi = nbr(d, x, y, z, cx(q), cy(q), cz(q));
-            if (yi >= 0 && clsv(d, yi) == CL_G) gas = true;
-        }
-        d.rdec[it] = gas ? 1 : 0;
+        const bool gas = __any_sync(0xffffffffu, cls(d, lane_nbr(d, lane, x, y, z)) == CL_G);
+        if (lane == 0) d.rdec[it] = gas ? 1 : 0;
     }
     __syncthreads();
     double acc = 0.0;
     for (uint32_t it = threadIdx.x; it < n; it += blockDim.x) {
         long long i = d.list[WL_PEND][it];
         if (!(d.cmark[i] & MK_FRESH)) continue;
-        if (clsv(d, i) == CL_L && d.rdec[it]) {
-            set_cls(d, i, CL_I);
-            double r = cell_density<S>(d, d.fdst, i);
-            d.m[i] = r;
-            d.phidst[i] = d.m[i] / cell_density<S>(d, d.fdst, i);
+        const int c = clsv(d, i);
+        if (c == CL_L) {
+            const double r = cell_density<S>(d, d.fdst, i);
+            acc += r;
+            if (d.rdec[it]) {
+                set_cls(d, i, CL_I);
+                d.m[i] = r;
+                d.phidst[i] = 1.0;  // r / r
+                if constexpr (S != 0) d.phifdst[i] = 1.0f;
+            }
+        } else if (c == CL_I) {
+            acc += d.m[i];
         }
-        if (clsv(d, i) == CL_L) acc += cell_density<S>(d, d.fdst, i);
-        else if (clsv(d, i) == CL_I) acc += d.m[i];
         d.cmark[i] = 0;
     }
     __shared__ double sh[REMAP_THREADS / 32];
@@ -3214,6 +3483,94 @@ __device__ __forceinline__ void remap_resolve_body(const Dev &d, const VB &vb) {
 }
 template <int S>
 __global__ void __launch_bounds__(REMAP_THREADS) k_remap_resolve(const __grid_constant__ Dev d) { remap_resolve_body<S>(d, vb_own()); }
+
+// ------------------------------------------- conversions and remap in one launch
+//
+// What follows the collision in a step -- the conversions, then the obstacle
+// remapping -- is eleven short phases, each of which needs the one before it
+// complete everywhere.  As kernels of their own they cost 3 to 6 us each even
+// with empty lists, more than the work of a small tank's step, so one launch
+// runs them with a barrier in between, and leaves out the conversions' (the
+// remap's) barriers when nothing converts (no cell is covered or left).
+//  - CLUSTER: one cluster of TAIL_CLUSTER blocks with the hardware's cluster
+//    barrier, for tanks whose lists are short;
+//  - else a cooperative grid with a barrier in global memory, for large tanks
+//    (hundreds to thousands of conversions a step want all SMs).
+constexpr int TAIL_THREADS = REMAP_THREADS, TAIL_CLUSTER = 8, TAIL_BLOCKS = 152;
+
+// one warp-wide poll limit for the grid barrier: far beyond the time that the
+// resident blocks of a cooperative launch can be apart
+constexpr unsigned BARRIER_POLLS = 1u << 24;
+template <bool CLUSTER> __device__ __forceinline__ bool tail_barrier(const Dev &d) {
+    if constexpr (CLUSTER) {
+        // (the form without .aligned: the warps may arrive diverged)
+        asm volatile("barrier.cluster.arrive.release;" ::: "memory");
+        asm volatile("barrier.cluster.wait.acquire;" ::: "memory");
+        return true;
+    } else {
+        __shared__ int s_ok;
+        __syncthreads();
+        if (threadIdx.x == 0) {
+            unsigned *count = d.status + 1, *turn = d.status + 2;
+            unsigned now;
+            asm volatile("ld.relaxed.gpu.global.u32 %0, [%1];" : "=r"(now) : "l"(turn) : "memory");
+            __threadfence();
+            bool ok = true;
+            if (atomicAdd(count, 1u) == gridDim.x - 1) {
+                *count = 0;
+                __threadfence();
+                atomicAdd(turn, 1u);
+            } else {
+                unsigned seen = now, polls = 0;
+                while (seen == now && polls < BARRIER_POLLS) {
+                    asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(seen) : "l"(turn) : "memory");
+                    ++polls;
+                }
+                ok = seen != now;
+                if (!ok) atomicOr(d.status, ST_TIMEOUT);
+            }
+            __threadfence();
+            s_ok = ok;
+        }
+        __syncthreads();
+        return s_ok != 0;
+    }
+}
+
+template <int S, bool CLUSTER>
+__global__ void __launch_bounds__(TAIL_THREADS) k_tail(const __grid_constant__ Dev d) {
+    const VB vb = vb_own();
+    if (vb.x == 0) {
+        // for the next step: its counters (this step's previous ones), and the
+        // slot its bulk pass records the fluid top in
+        if (threadIdx.x < CN_COUNT) d.pcnt[threadIdx.x] = 0;
+        if (threadIdx.x == 0) *d.ztop_rd = -1;
+    }
+    const bool conv = wl_count(d, WL_FILLED) + wl_count(d, WL_EMPTIED) > 0;
+    const bool remap = d.nb > 0 && wl_count(d, WL_COVER) + wl_count(d, WL_PEND) > 0;
+    if (conv) {
+        // new interface cells are marked (the two lists mark disjoint cells)
+        conv_filled_body(d, vb);
+        conv_emptied_body(d, vb);
+        if (!tail_barrier<CLUSTER>(d)) return;
+        // their states; the converted cells' shares and who receives them
+        // (from the classes before and the marks)
+        conv_init_body<S>(d, vb);
+        conv_claim_body<S>(d, vb);
+        if (!tail_barrier<CLUSTER>(d)) return;
+        conv_flags_body(d, vb);
+        conv_excess_body<S>(d, vb);
+        if (!tail_barrier<CLUSTER>(d)) return;
+        conv_finish_body(d, vb);
+    }
+    if (remap) {
+        remap_apply_body<S>(d, vb);
+        if (!tail_barrier<CLUSTER>(d)) return;
+        if (vb.x == 0) remap_resolve_body<S>(d, vb);
+        if (!tail_barrier<CLUSTER>(d)) return;
+        nb_update_body(d, vb);
+    }
+}
 
 // ------------------------------------------------------ reductions, output
 
@@ -3288,7 +3645,7 @@ __global__ void __launch_bounds__(K::THREADS, K::MINB)
     k_batch(const __grid_constant__ TankSet ts, const Tile *__restrict__ table, unsigned n, int zb) {
     for (unsigned t = blockIdx.x; t < n; t += gridDim.x) {
         const Tile e = table[t];
-        const VB vb{e.x, e.y, e.z, e.nx, e.ny, e.nz};
+        const VB vb{e.x, e.y, e.z, e.nx, e.ny, e.nz, e.kind};
         K::run(ts.d[e.tank], vb, zb);
         // the next entry's body reuses this one's shared memory; bodies
         // without shared memory let a block's warps move on independently
@@ -3296,39 +3653,42 @@ __global__ void __launch_bounds__(K::THREADS, K::MINB)
     }
 }
 
-#define LBMFS_BATCH_BODY_SM(NAME, THR, MB, SM, CALL)                                          \
+#define LBMFS_BATCH_BODY_SM(NAME, THR, MB, SM, ...)                                           \
     struct NAME {                                                                              \
         static constexpr int THREADS = THR, MINB = MB;                                         \
         static constexpr bool SMEM = SM;                                                       \
-        static __device__ __forceinline__ void run(const Dev &d, const VB &vb, int zb) { CALL; } \
+        static __device__ __forceinline__ void run(const Dev &d, const VB &vb, int zb) { __VA_ARGS__; } \
     };
-#define LBMFS_BATCH_BODY(NAME, THR, MB, CALL) LBMFS_BATCH_BODY_SM(NAME, THR, MB, false, CALL)
+#define LBMFS_BATCH_BODY(NAME, THR, MB, ...) LBMFS_BATCH_BODY_SM(NAME, THR, MB, false, __VA_ARGS__)
 struct BkReset {
     static constexpr int THREADS = 32, MINB = 1;
     static constexpr bool SMEM = false;
     static __device__ __forceinline__ void run(const Dev &d, const VB &, int) {
-        if (threadIdx.x < WL_COUNT) d.cnt[threadIdx.x] = 0;
+        if (threadIdx.x < CN_COUNT) d.cnt[threadIdx.x] = 0;
     }
 };
-template <int S> LBMFS_BATCH_BODY_SM(BkForces, 256, S == 0 ? 2 : LBMFS_FORCE_MINB, true, forces_body<S>(d, vb))
+template <int S> LBMFS_BATCH_BODY_SM(BkForces, 256, S == 0 ? 2 : LBMFS_FORCE_MINB, true, forces_body<S, true>(d, vb))
 // one instantiation per z-planes-per-tile choice (the column loop unrolled to it)
 template <int S, int ZB>
 LBMFS_BATCH_BODY(BkLiquid, BULK_THREADS, S == 0 ? 1 : (LBMFS_BULK_PAIR ? LBMFS_PAIR_MINB : LBMFS_BULK_MINB),
                  (bulk_body<S, ZB>(d, vb, zb)))
 // the batch's listed cells are spread over many more blocks: 4 resident per SM
 // (128 registers) beat 1 there, not on the single tank
-template <int S> LBMFS_BATCH_BODY(BkGeneral, GEN_THREADS, 4, general_body<S>(d, vb))
+template <int S>
+LBMFS_BATCH_BODY_SM(BkGeneral, GEN_THREADS, 4, true, if (vb.kind == 0) near_body<S, true>(d, vb); else faces_body<S>(d, vb))
 template <int S> LBMFS_BATCH_BODY(BkInterface, 128, S == 0 ? 2 : LBMFS_IFACE_MINB, interface_body<S>(d, vb))
-LBMFS_BATCH_BODY(BkConvFilled, LIST_THREADS, 1, conv_filled_body(d, vb))
+// (runs after the bulk kernel, which has read this step's fluid top: clears the
+// slot that the next step records its own in)
+LBMFS_BATCH_BODY(BkConvFilled, LIST_THREADS, 1, if (vb.x == 0 && threadIdx.x == 0) *d.ztop_rd = -1; conv_filled_body(d, vb))
 LBMFS_BATCH_BODY(BkConvEmptied, LIST_THREADS, 1, conv_emptied_body(d, vb))
 template <int S> LBMFS_BATCH_BODY(BkConvInit, LIST_THREADS, 1, conv_init_body<S>(d, vb))
 LBMFS_BATCH_BODY(BkConvFlags, LIST_THREADS, 1, conv_flags_body(d, vb))
 template <int S> LBMFS_BATCH_BODY(BkConvClaim, LIST_THREADS, 1, conv_claim_body<S>(d, vb))
 template <int S> LBMFS_BATCH_BODY(BkConvExcess, LIST_THREADS, 1, conv_excess_body<S>(d, vb))
-template <int S> LBMFS_BATCH_BODY(BkConvFinish, LIST_THREADS, 1, conv_finish_body<S>(d, vb))
+LBMFS_BATCH_BODY(BkConvFinish, LIST_THREADS, 1, conv_finish_body(d, vb))
 LBMFS_BATCH_BODY(BkBodies, 32, 1, bodies_body(d, vb))
-template <int S> LBMFS_BATCH_BODY(BkRemapCover, 256, 1, remap_cover_body<S>(d, vb))
-LBMFS_BATCH_BODY(BkRemapPending, 256, 1, remap_pending_body(d, vb))
+LBMFS_BATCH_BODY(BkRemapScan, 256, 1, remap_scan_body(d, vb))
+template <int S> LBMFS_BATCH_BODY(BkRemapApply, LIST_THREADS, 1, remap_apply_body<S>(d, vb))
 template <int S> LBMFS_BATCH_BODY_SM(BkRemapResolve, REMAP_THREADS, 1, true, remap_resolve_body<S>(d, vb))
 LBMFS_BATCH_BODY(BkNbUpdate, LIST_THREADS, 1, nb_update_body(d, vb))
 #undef LBMFS_BATCH_BODY
@@ -3362,11 +3722,23 @@ inline int bulk_planes(int storage, unsigned gx, int nz) {
     return blocks(2) >= 2000 ? 2 : 1;
 }
 
+// largest xy-plane whose tail runs as one cluster
+#ifndef LBMFS_TAIL_CLUSTER_CELLS
+#define LBMFS_TAIL_CLUSTER_CELLS 131072
+#endif
+constexpr long long TAIL_CLUSTER_CELLS = LBMFS_TAIL_CLUSTER_CELLS;
+
+constexpr int STEP_SLOTS = 7, BATCH_SLOTS = 17;  // kernel slots of a step (names below)
+
 template <int S> struct Launch {
     static void init_cells(const Dev &d, const uint8_t *flags, const double *fill, const double *rho, const double *vel,
                            cudaStream_t st) {
         unsigned blocks = (unsigned)((d.N + 255) / 256);
         k_init<S><<<blocks, 256, 0, st>>>(d, flags, fill, rho, vel);
+        Dev prev = d;  // the lists of the step before the first
+        prev.list[WL_IFACE] = const_cast<uint32_t *>(d.plist[0]);
+        prev.cnt = d.pcnt;
+        k_list_interface<<<blocks, 256, 0, st>>>(prev);
         k_nb_all<<<dim3((d.nx + 127) / 128, d.ny, d.nz), 128, 0, st>>>(d);
     }
     static void body_prepare(const Dev &d, int b, cudaStream_t st) { k_body_prepare<<<1, 32, 0, st>>>(d, b); }
@@ -3400,67 +3772,106 @@ template <int S> struct Launch {
             if (zb == 8) bulk_zb<8>(d, gx, st);
         }
     }
-    // one time step; with ev != nullptr, event k is recorded before kernel k
-    // and ev[count] after the last one
-    static int step(const Dev &d, cudaStream_t st, float *, cudaEvent_t *ev) {
+    static void faces(const Dev &d, cudaStream_t st) { k_faces<S><<<LIST_BLOCKS, GEN_THREADS, 0, st>>>(d); }
+    static void near(const Dev &d, cudaStream_t st) {
+        k_near<S><<<dim3(FORCE_BLOCKS, d.nb), GEN_THREADS, 0, st>>>(d);
+    }
+    static void forces(const Dev &d, cudaStream_t st) {
+        k_forces<S><<<dim3(FORCE_BLOCKS, d.nb), dim3(32, 8), 0, st>>>(d);
+    }
+    static void scan(const Dev &d, cudaStream_t st) { k_remap_scan<<<dim3(FORCE_BLOCKS, d.nb), 256, 0, st>>>(d); }
+    static void interface(const Dev &d, cudaStream_t st) { k_interface<S><<<LBMFS_IFACE_GRID, 128, 0, st>>>(d); }
+    static void bulk_any(const Dev &d, cudaStream_t st) {
+        if constexpr (S != 0) {
+            // the staged variants tile rows: (ceil(nx / BULK_THREADS), ny, z-blocks)
+            dim3 rgrid((d.nx + BULK_THREADS - 1) / BULK_THREADS, d.ny, (d.nz + LBMFS_BULK_ZB - 1) / LBMFS_BULK_ZB);
+            dim3 pgrid(rgrid.x, rgrid.y, (d.nz + LBMFS_BULK_PIPE_ZB - 1) / LBMFS_BULK_PIPE_ZB);
+            if (d.bulk == BULK_TMA) k_liquid_tma<S><<<rgrid, BULK_THREADS, 128 + 2 * Stage<S>::BYTES, st>>>(d);
+            else if (d.bulk == BULK_PIPE) k_liquid_pipe<S><<<pgrid, BULK_THREADS, 0, st>>>(d);
+            else bulk(d, st);
+        } else {
+            bulk(d, st);
+        }
+    }
+    static void tail(const Dev &d, cudaStream_t st) {
+        cudaLaunchConfig_t c = {};
+        cudaLaunchAttribute a = {};
+        c.blockDim = dim3(TAIL_THREADS);
+        c.stream = st;
+        c.attrs = &a;
+        c.numAttrs = 1;
+        if ((long long)d.nx * d.ny <= TAIL_CLUSTER_CELLS) {
+            c.gridDim = dim3(TAIL_CLUSTER);
+            a.id = cudaLaunchAttributeClusterDimension;
+            a.val.clusterDim.x = TAIL_CLUSTER;
+            a.val.clusterDim.y = a.val.clusterDim.z = 1;
+            cudaLaunchKernelEx(&c, k_tail<S, true>, d);
+        } else {
+            c.gridDim = dim3(TAIL_BLOCKS);
+            a.id = cudaLaunchAttributeCooperative;
+            a.val.cooperative = 1;
+            cudaLaunchKernelEx(&c, k_tail<S, false>, d);
+        }
+    }
+    // One time step.  The force kernel, the rigid-body update and the remap's
+    // scan (a chain), the cells next to bodies or on moving walls, and the
+    // interface cells need only the state at t: with `sides` (while a graph is
+    // captured) these chains run beside the bulk kernel, on streams of a higher
+    // priority, and join before the tail.  Without, all run in one chain.  With
+    // ev != nullptr event k is recorded before kernel slot k (step_names).
+    static int step(const Dev &d, cudaStream_t st, const Sides *sides, cudaEvent_t *ev) {
+        const bool bodies = d.nb > 0, walls = d.walls_move != 0;
+        const int launches = 3 + (bodies ? 4 : 0) + (walls ? 1 : 0);
+        if (sides) {
+            const bool used[SIDE_STREAMS] = {true, bodies, bodies || walls};
+            cudaEventRecord(sides->fork, st);
+            for (int k = 0; k < SIDE_STREAMS; ++k)
+                if (used[k]) cudaStreamWaitEvent(sides->st[k], sides->fork, 0);
+            if (bodies) forces(d, sides->st[1]);
+            if (bodies) near(d, sides->st[2]);
+            if (walls) faces(d, sides->st[2]);
+            interface(d, sides->st[0]);
+            if (bodies) launch_bodies(d, sides->st[1]);
+            if (bodies) scan(d, sides->st[1]);
+            bulk_any(d, st);
+            for (int k = 0; k < SIDE_STREAMS; ++k)
+                if (used[k]) {
+                    cudaEventRecord(sides->join[k], sides->st[k]);
+                    cudaStreamWaitEvent(st, sides->join[k], 0);
+                }
+            tail(d, st);
+            return launches;
+        }
         int k = 0;
         auto mark = [&]() {
             if (ev) cudaEventRecord(ev[k], st);
             ++k;
         };
         mark();
-        cudaMemsetAsync(d.cnt, 0, WL_COUNT * sizeof(uint32_t), st);
+        if (bodies) forces(d, st);
         mark();
-        if (d.nb > 0) k_forces<S><<<dim3(FORCE_BLOCKS, d.nb), dim3(32, 8), 0, st>>>(d);
+        bulk_any(d, st);
         mark();
-        {
-            if constexpr (S != 0) {
-                // the staged variants tile rows: (ceil(nx / BULK_THREADS), ny, z-blocks)
-                dim3 rgrid((d.nx + BULK_THREADS - 1) / BULK_THREADS, d.ny, (d.nz + LBMFS_BULK_ZB - 1) / LBMFS_BULK_ZB);
-                dim3 pgrid(rgrid.x, rgrid.y, (d.nz + LBMFS_BULK_PIPE_ZB - 1) / LBMFS_BULK_PIPE_ZB);
-                if (d.bulk == BULK_TMA) k_liquid_tma<S><<<rgrid, BULK_THREADS, 128 + 2 * Stage<S>::BYTES, st>>>(d);
-                else if (d.bulk == BULK_PIPE) k_liquid_pipe<S><<<pgrid, BULK_THREADS, 0, st>>>(d);
-                else bulk(d, st);
-            } else {
-                bulk(d, st);
-            }
-        }
+        if (bodies) near(d, st);
+        if (walls) faces(d, st);
         mark();
-        k_general<S><<<LIST_BLOCKS, GEN_THREADS, 0, st>>>(d);
+        interface(d, st);
         mark();
-        k_interface<S><<<LBMFS_IFACE_GRID, 128, 0, st>>>(d);
+        if (bodies) launch_bodies(d, st);
         mark();
-        k_conv_filled<<<LIST_BLOCKS, LIST_THREADS, 0, st>>>(d);
+        if (bodies) scan(d, st);
         mark();
-        k_conv_emptied<<<LIST_BLOCKS, LIST_THREADS, 0, st>>>(d);
+        tail(d, st);
         mark();
-        k_conv_init<S><<<LIST_BLOCKS, LIST_THREADS, 0, st>>>(d);
-        mark();
-        k_conv_flags<<<LIST_BLOCKS, LIST_THREADS, 0, st>>>(d);
-        mark();
-        k_conv_claim<S><<<LIST_BLOCKS, LIST_THREADS, 0, st>>>(d);
-        mark();
-        k_conv_excess<S><<<LIST_BLOCKS, LIST_THREADS, 0, st>>>(d);
-        mark();
-        k_conv_finish<S><<<LIST_BLOCKS, LIST_THREADS, 0, st>>>(d);
-        mark();
-        if (d.nb > 0) launch_bodies(d, st);
-        mark();
-        if (d.nb > 0) k_remap_cover<S><<<dim3(FORCE_BLOCKS, d.nb), 256, 0, st>>>(d);
-        mark();
-        if (d.nb > 0) k_remap_pending<<<dim3(FORCE_BLOCKS, d.nb), 256, 0, st>>>(d);
-        mark();
-        if (d.nb > 0) k_remap_resolve<S><<<1, REMAP_THREADS, 0, st>>>(d);
-        mark();
-        if (d.nb > 0) k_nb_update<<<LIST_BLOCKS, LIST_THREADS, 0, st>>>(d);
-        mark();
-        return d.nb > 0 ? 16 : 10;  // kernels (the counter reset is a memset node)
+        return launches;
     }
 };
 
 // The batched counterpart of Launch<S>::step (same kernel slots).
 template <int S> struct BatchStep {
-    static int step(const BatchLaunch &b, cudaStream_t st, cudaEvent_t *ev) {
+    // (with sides: the chains that need only the state at t beside the bulk
+    // kernel, as in Launch<S>::step)
+    static int step(const BatchLaunch &b, cudaStream_t st, const Sides *sides, cudaEvent_t *ev) {
         int k = 0;
         auto mark = [&]() {
             if (ev) cudaEventRecord(ev[k], st);
@@ -3468,42 +3879,62 @@ template <int S> struct BatchStep {
         };
         mark();
         batch_launch<BkReset>(b, SH_TANK, 32, st);
+        cudaStream_t s0 = st, s1 = st, s2 = st;
+        if (sides) {
+            cudaEventRecord(sides->fork, st);
+            for (int j = 0; j < SIDE_STREAMS; ++j) cudaStreamWaitEvent(sides->st[j], sides->fork, 0);
+            s0 = sides->st[0];
+            s1 = sides->st[1];
+            s2 = sides->st[2];
+        }
         mark();
-        batch_launch<BkForces<S>>(b, SH_FORCE, dim3(32, 8), st);
+        batch_launch<BkForces<S>>(b, SH_FORCE, dim3(32, 8), s1);
+        if (sides) {
+            // in the order in which they should get the SMs
+            batch_launch<BkGeneral<S>>(b, SH_GEN, GEN_THREADS, s2);
+            batch_launch<BkInterface<S>>(b, SH_IFACE, 128, s0);
+            launch_bodies_batch(b, s1);
+            batch_launch<BkRemapScan>(b, SH_FORCE, 256, s1);
+        }
         mark();
         batch_bulk_launch<S>(b, st);
         mark();
-        batch_launch<BkGeneral<S>>(b, SH_IFACE, GEN_THREADS, st);
+        if (!sides) batch_launch<BkGeneral<S>>(b, SH_GEN, GEN_THREADS, s2);
         mark();
-        batch_launch<BkInterface<S>>(b, SH_IFACE, 128, st);
+        if (!sides) batch_launch<BkInterface<S>>(b, SH_IFACE, 128, st);
         mark();
+        if (sides)
+            for (int j = 0; j < SIDE_STREAMS; ++j) {
+                cudaEventRecord(sides->join[j], sides->st[j]);
+                cudaStreamWaitEvent(st, sides->join[j], 0);
+            }
         batch_launch<BkConvFilled>(b, SH_LIST, LIST_THREADS, st);
         mark();
         batch_launch<BkConvEmptied>(b, SH_LIST, LIST_THREADS, st);
         mark();
         batch_launch<BkConvInit<S>>(b, SH_LIST, LIST_THREADS, st);
         mark();
-        batch_launch<BkConvFlags>(b, SH_LIST, LIST_THREADS, st);
-        mark();
         batch_launch<BkConvClaim<S>>(b, SH_LIST, LIST_THREADS, st);
+        mark();
+        batch_launch<BkConvFlags>(b, SH_LIST, LIST_THREADS, st);
         mark();
         batch_launch<BkConvExcess<S>>(b, SH_LIST, LIST_THREADS, st);
         mark();
-        batch_launch<BkConvFinish<S>>(b, SH_LIST, LIST_THREADS, st);
+        batch_launch<BkConvFinish>(b, SH_LIST, LIST_THREADS, st);
         mark();
-        launch_bodies_batch(b, st);
+        if (!sides) launch_bodies_batch(b, st);
         mark();
-        batch_launch<BkRemapCover<S>>(b, SH_FORCE, 256, st);
+        if (!sides) batch_launch<BkRemapScan>(b, SH_FORCE, 256, st);
         mark();
-        batch_launch<BkRemapPending>(b, SH_FORCE, 256, st);
+        batch_launch<BkRemapApply<S>>(b, SH_LIST, LIST_THREADS, st);
         mark();
         batch_launch<BkRemapResolve<S>>(b, SH_ONE, REMAP_THREADS, st);
         mark();
         batch_launch<BkNbUpdate>(b, SH_LIST, LIST_THREADS, st);
         mark();
         int n = 0;
-        const int shapes[] = {SH_TANK, SH_FORCE, SH_BULK, SH_IFACE, SH_IFACE, SH_LIST, SH_LIST, SH_LIST, SH_LIST,
-                              SH_LIST, SH_LIST, SH_LIST, SH_BODY, SH_FORCE, SH_FORCE, SH_ONE, SH_LIST};
+        const int shapes[] = {SH_TANK, SH_FORCE, SH_BULK, SH_GEN, SH_IFACE, SH_LIST, SH_LIST, SH_LIST, SH_LIST,
+                              SH_LIST, SH_LIST, SH_LIST, SH_BODY, SH_FORCE, SH_LIST, SH_ONE, SH_LIST};
         for (int sh : shapes) n += b.sh[sh].n ? 1 : 0;
         return n;
     }
@@ -3516,10 +3947,16 @@ template <int S> struct BatchStep {
     }
 };
 
-inline const char *const *kernel_names() {
-    static const char *const n[] = {"reset_counters", "forces", "liquid", "general", "interface", "conv_filled",
-                                    "conv_emptied",    "conv_init", "conv_flags", "conv_claim", "conv_excess",
-                                    "conv_finish",     "bodies",  "remap_cover", "remap_pending", "remap_resolve", "nb_update"};
+inline const char *const *step_names() {
+    static const char *const n[] = {"forces", "liquid", "general", "interface", "bodies", "remap_scan", "convert_remap"};
+    static_assert(sizeof n / sizeof n[0] == STEP_SLOTS, "one name per slot");
+    return n;
+}
+inline const char *const *batch_names() {
+    static const char *const n[] = {"reset_counters", "forces",     "liquid",     "general",     "interface",   "conv_filled",
+                                    "conv_emptied",   "conv_init",  "conv_claim", "conv_flags",  "conv_excess", "conv_finish",
+                                    "bodies",         "remap_scan", "remap_apply", "remap_resolve", "nb_update"};
+    static_assert(sizeof n / sizeof n[0] == BATCH_SLOTS, "one name per slot");
     return n;
 }
 
@@ -3534,8 +3971,10 @@ template <int S> KernelSet make_kernel_set() {
     k.batch_step = &BatchStep<S>::step;
     k.batch_bulk = &BatchStep<S>::bulk;
     k.bulk_blocks_per_sm = &BatchStep<S>::bulk_blocks_per_sm;
-    k.nkernels = 17;
-    k.names = kernel_names();
+    k.nkernels = STEP_SLOTS;
+    k.names = step_names();
+    k.batch_kernels = BATCH_SLOTS;
+    k.batch_names = batch_names();
     return k;
 }
 
