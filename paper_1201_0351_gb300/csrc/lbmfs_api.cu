@@ -219,7 +219,7 @@ lbm_fs_status lbm_fs_create(const lbm_fs_params *p, lbm_fs **out) {
     d.vmass = rd_vm ? p->virtual_mass : 1.0;
     d.force_mean = (p->readings & LBM_FS_READING_FORCE_MEAN) ? (p->force_mean != 0) : 1;
     d.nb_rule = (p->readings & LBM_FS_READING_NEIGHBOUR_RULE) ? (p->neighbour_rule != 0) : 1;
-    d.pair_ok = p->storage != LBM_FS_F64 && p->nx % 2 == 0 && N % 2 == 0;
+    d.pair_ok = p->nx % 2 == 0 && N % 2 == 0;
     // row segments are 16-byte aligned when nx is a multiple of 16 / element size
     // bulk-kernel variant (float storages): direct loads by default;
     // LBMFS_BULK=pipe|tma selects the shared-memory staged variants (both
@@ -234,15 +234,21 @@ lbm_fs_status lbm_fs_create(const lbm_fs_params *p, lbm_fs **out) {
         d.bulk = BULK_PLAIN;
     size_t fb = storage_bytes(p->storage, N);
     size_t nb4 = ((size_t)N + 3) & ~(size_t)3;
-    d.flags = (uint8_t *)h->alloc(nb4);
+    // (the ring kernel reads the class bytes of whole tiles: zeros after the grid)
+    const size_t nflags = ((size_t)N + RING_TILE - 1) / RING_TILE * RING_TILE;
+    d.flags = (uint8_t *)h->alloc(nflags);
     d.bid = (uint8_t *)h->alloc(nb4);
     d.cmark = (uint8_t *)h->alloc(nb4);
     // population grids with guard bands: the staged bulk kernel reads a
-    // 16-byte halo around each row segment, which at the grid's first and
-    // last rows reaches past the population array
-    void *fA = h->alloc(fb + 2 * GRID_GUARD), *fB = h->alloc(fb + 2 * GRID_GUARD);
-    if (fA) fA = (char *)fA + GRID_GUARD;
-    if (fB) fB = (char *)fB + GRID_GUARD;
+    // 16-byte halo around each row segment, which at the grid's
+    // first and last rows reaches past the population array; the ring kernel's
+    // tiles reach a z-plane, a row and a tile further (multiples of 16 bytes)
+    size_t guard = GRID_GUARD;
+    if (p->storage != LBM_FS_F64)
+        guard += (((size_t)p->nx * p->ny + p->nx + 1024) * (p->storage == LBM_FS_F32 ? 4 : 2) + 255) & ~(size_t)255;
+    void *fA = h->alloc(fb + 2 * guard), *fB = h->alloc(fb + 2 * guard);
+    if (fA) fA = (char *)fA + guard;
+    if (fB) fB = (char *)fB + guard;
     double *pA = (double *)h->alloc(N * 8), *pB = (double *)h->alloc(N * 8);
     d.m = (double *)h->alloc(N * 8);
     for (int k = 0; k < WL_COUNT; ++k) d.list[k] = (uint32_t *)h->alloc(N * 4);
@@ -280,8 +286,9 @@ lbm_fs_status lbm_fs_create(const lbm_fs_params *p, lbm_fs **out) {
         if (e_ != cudaSuccess) return bail(cuda_fail(e_, #call));   \
     } while (0)
     CKB(cudaMemsetAsync(d.cmark, 0, nb4, st));
-    CKB(cudaMemsetAsync((char *)fA - GRID_GUARD, 0, fb + 2 * GRID_GUARD, st));
-    CKB(cudaMemsetAsync((char *)fB - GRID_GUARD, 0, fb + 2 * GRID_GUARD, st));
+    CKB(cudaMemsetAsync(d.flags, 0, nflags, st));
+    CKB(cudaMemsetAsync((char *)fA - guard, 0, fb + 2 * guard, st));
+    CKB(cudaMemsetAsync((char *)fB - guard, 0, fb + 2 * guard, st));
     CKB(cudaMemsetAsync(pA, 0, N * 8, st));
     CKB(cudaMemsetAsync(pB, 0, N * 8, st));
     CKB(cudaMemsetAsync(d.m, 0, N * 8, st));

@@ -33,6 +33,7 @@ struct Chunk {
     int lane = 0;          // concurrent chain the chunk's launches belong to
     TankSet ts[2];         // descriptors for even / odd steps
     Shape sh[SH_COUNT];
+    bool zg = true;        // as in BatchLaunch
 };
 
 }  // namespace
@@ -126,6 +127,7 @@ lbm_fs_status build(lbm_fs_batch *b) {
             for (int j = 0; j < (int)c.idx.size(); ++j) c.ts[k].d[j] = b->tanks[c.idx[j]]->d[k];
         }
         std::vector<Tile> tb[SH_COUNT];
+        c.zg = true;
         for (int j = 0; j < (int)c.idx.size(); ++j) {
             const lbm_fs *t = b->tanks[c.idx[j]];
             const Dev &d = t->d[0];
@@ -134,11 +136,16 @@ lbm_fs_status build(lbm_fs_batch *b) {
             tb[SH_TANK].push_back(tile(j, 0, 0, 0, 1, 1, 1));
             for (int y = 0; y < nb; ++y)
                 for (int x = 0; x < FORCE_BLOCKS; ++x) tb[SH_FORCE].push_back(tile(j, x, y, 0, FORCE_BLOCKS, nb, 1));
-            const int bc = bulk_cells(t->p.storage, d);
-            const int gx = (int)(((long long)d.nx * d.ny + bc - 1) / bc);
-            const int gz = (d.nz + b->zb - 1) / b->zb;
-            for (int z = 0; z < gz; ++z)
-                for (int x = 0; x < gx; ++x) tb[SH_BULK].push_back(tile(j, x, 0, z, gx, 1, gz));
+            if (t->p.storage == LBM_FS_F16S) {
+                const long long tiles = (d.N + RING_TILE - 1) / RING_TILE;
+                for (long long k = 0; k < tiles; ++k) tb[SH_BULK].push_back(tile(j, (int)(k & 0xffff), (int)(k >> 16), 0, 1, 1, 1));
+            } else {
+                const int gx = (int)(((long long)d.nx * d.ny + BULK_THREADS - 1) / BULK_THREADS);
+                const int gz = (d.nz + b->zb - 1) / b->zb;
+                for (int z = 0; z < gz; ++z)
+                    for (int x = 0; x < gx; ++x) tb[SH_BULK].push_back(tile(j, x, 0, z, gx, 1, gz));
+            }
+            c.zg = c.zg && d.a_f[0] == 0.0f && d.a_f[1] == 0.0f;
             const int lb = list_blocks(t, b->list_cells);
             for (int x = 0; x < 2 * lb; ++x) tb[SH_IFACE].push_back(tile(j, x, 0, 0, 2 * lb, 1, 1));
             for (int x = 0; x < lb; ++x) tb[SH_LIST].push_back(tile(j, x, 0, 0, lb, 1, 1));
@@ -159,7 +166,10 @@ lbm_fs_status build(lbm_fs_batch *b) {
             all.insert(all.end(), tb[s].begin(), tb[s].end());
             c.sh[s].n = (unsigned)tb[s].size();
             unsigned grid = c.sh[s].n;
-            if (s == SH_BULK && b->bulk_blocks > 0) grid = std::min<unsigned>(grid, (unsigned)b->bulk_blocks);
+            // the FP16 storage's bulk kernel is a persistent grid
+            if (s == SH_BULK && b->tanks[0]->p.storage == LBM_FS_F16S)
+                grid = std::min<unsigned>(grid, (unsigned)(b->bulk_blocks > 0 ? b->bulk_blocks : RING_CTAS * b->sms));
+            else if (s == SH_BULK && b->bulk_blocks > 0) grid = std::min<unsigned>(grid, (unsigned)b->bulk_blocks);
             c.sh[s].grid = grid;
             c.sh[s].table = nullptr;
         }
@@ -194,6 +204,7 @@ BatchLaunch launch_of(lbm_fs_batch *b, Chunk &c, int parity) {
     L.ts = &c.ts[parity];
     for (int s = 0; s < SH_COUNT; ++s) L.sh[s] = c.sh[s];
     L.zb = b->zb;
+    L.zg = c.zg;
     return L;
 }
 

@@ -20,16 +20,11 @@ constexpr int GRID_GUARD = 1024;
 #define LBMFS_BULK_THREADS 128
 #endif
 constexpr int BULK_THREADS = LBMFS_BULK_THREADS;  // x extent of a bulk-kernel block
-// cells of an xy-plane per bulk-kernel block, by storage: one per thread for
-// double, two per thread for the float storages
-#ifndef LBMFS_BULK_PAIR
-#define LBMFS_BULK_PAIR 0  // tuning knob: float storages on even grids take two cells per bulk-kernel thread
-#endif
 
 // cell classes (as in the C ABI) in the low nibble of the flag byte; bit 4
-// marks a cell with an obstacle among its 18 neighbours, bit 5 a cell on a face
-// of a grid with moving walls
-enum : uint8_t { CL_L = 1, CL_I = 2, CL_G = 4, CL_O = 8, CL_MASK = 15, NB_OBST = 16, MOVING_FACE = 32 };
+// marks a cell with an obstacle among its 18 neighbours, bits 7 and 6 a
+// cell on an x face, on a y or z face of the grid, bit 5 either where walls move
+enum : uint8_t { CL_L = 1, CL_I = 2, CL_G = 4, CL_O = 8, CL_MASK = 15, NB_OBST = 16, MOVING_FACE = 32, FACE_YZ = 64, FACE_X = 128 };
 // per-cell conversion marks (separate byte array, zero between steps)
 enum : uint8_t {
     MK_FILLED = 1, MK_EMPTIED = 2, MK_NEWG = 4, MK_NEWL = 8, MK_RECV = 16, MK_PEND = 32, MK_FRESH = 64
@@ -112,7 +107,7 @@ struct Dev {
     double vmass;      // virtual-mass coefficient of the rigid-body update
     int force_mean;    // rigid-body update driven by (F_n + F_{n-1}) / 2
     int nb_rule;       // interface cells without liquid (gas) neighbours empty (fill)
-    int pair_ok;       // nx and N even: the float bulk kernel takes two cells per thread
+    int pair_ok;       // nx and N even: pairs of cells start on even elements of every plane
 };
 
 // bulk-kernel variants: direct loads, per-thread cp.async pipeline over z,
@@ -138,7 +133,8 @@ struct Tile {
 // block tables by launch shape
 enum {
     SH_FORCE = 0,  // (FORCE_BLOCKS, bodies): forces, remap cover / pending
-    SH_BULK,       // (ceil(nx / BULK_THREADS), ny, ceil(nz / zb)): bulk stream + collide
+    SH_BULK,       // bulk stream + collide: (ceil(nx ny / BULK_THREADS), 1, ceil(nz / zb));
+                   // FP16 storage: tile x + 2^16 y of RING_TILE cells
     SH_IFACE,      // (2 lb): interface cells
     SH_LIST,       // (lb): conversion worklists, neighbour-bit refresh
     SH_BODY,       // (bodies): rigid-body step
@@ -156,7 +152,10 @@ struct BatchLaunch {
     const TankSet *ts;  // host copy, passed by value to every launch
     Shape sh[SH_COUNT];
     int zb;             // z-planes per bulk tile
+    bool zg;            // every tank's acceleration is along z
 };
+// FP16 storage: cells per tile of the ring kernel, and its blocks per SM
+constexpr int RING_TILE = 512, RING_CTAS = 2;
 // Streams (and events to fork to and join from them) on which a step's kernels
 // that do not depend on the bulk kernel run beside it.  They are created with
 // the highest priority: the bulk kernel fills every SM, and its thousands of
@@ -190,12 +189,6 @@ struct KernelSet {
     int batch_kernels;         // slots of batch_step
     const char *const *batch_names;
 };
-
-// cells of an xy-plane per bulk-kernel block: two per thread for the float
-// storages on grids with nx and the cell count even, one otherwise
-inline int bulk_cells(int storage, const Dev &d) {
-    return (storage != 0 && LBMFS_BULK_PAIR && d.pair_ok) ? 2 * BULK_THREADS : BULK_THREADS;
-}
 
 // The rigid-body update (double precision, independent of the storage) is
 // compiled once, in the unit built without fused multiply-add, and launched

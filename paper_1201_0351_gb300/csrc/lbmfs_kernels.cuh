@@ -14,6 +14,8 @@
 #include <math.h>
 #include <stdint.h>
 
+#include <algorithm>
+
 #include "lbmfs_internal.h"
 
 namespace lbmfs {
@@ -62,12 +64,6 @@ __host__ __device__ __forceinline__ constexpr float wf(int q) {
 #ifndef LBMFS_BULK_MINB
 #define LBMFS_BULK_MINB 8  // resident blocks per SM asked of ptxas for the bulk kernel (64 registers)
 #endif
-#ifndef LBMFS_BULK_PAIR
-#define LBMFS_BULK_PAIR 0  // tuning knob: float storages on even grids take two cells per bulk-kernel thread
-#endif
-#ifndef LBMFS_PAIR_MINB
-#define LBMFS_PAIR_MINB 5  // resident blocks per SM of the two-cell bulk kernel (float storages, 96 registers)
-#endif
 #ifndef LBMFS_BULK_ZB
 #define LBMFS_BULK_ZB 8    // z-planes per bulk-kernel block (measured: 8 beat 4 by 2 % for FP32, 2 was far slower)
 #endif
@@ -75,10 +71,7 @@ __host__ __device__ __forceinline__ constexpr float wf(int q) {
 #define LBMFS_BULK_PIPE_ZB 16  // z-planes per block of the software-pipelined bulk kernel
 #endif
 #ifndef LBMFS_FORCE_MINB
-#define LBMFS_FORCE_MINB 3  // resident 256-thread blocks per SM of the float-storage force kernel
-#endif
-#ifndef LBMFS_FORCE_ROWS
-#define LBMFS_FORCE_ROWS 1  // 32-cell tasks of a body's range per warp in the float-storage force kernel
+#define LBMFS_FORCE_MINB 6  // resident blocks per SM of the float-storage force kernel (80 registers)
 #endif
 #ifndef LBMFS_IFACE_MINB
 #define LBMFS_IFACE_MINB 6  // resident blocks per SM asked of ptxas for the interface kernel (80 registers)
@@ -182,26 +175,6 @@ template <> struct Sto<1> {
     static __device__ __forceinline__ float st_raw(void *g, int q, long long i, long long N, float v) {
         return st_one(g, q, i, N, v);
     }
-    // the populations q of the cells j, j + 1 (one 8-byte load when the pair
-    // starts on an even element, two loads otherwise), through the read-only path
-    static __device__ __forceinline__ float2 ldg_pair_raw(const void *g, int q, long long j, long long N) {
-        const long long k = (long long)q * N + j;
-        const float *b = reinterpret_cast<const float *>(g) + k;
-        if (k & 1) return make_float2(pop_ldg(b), pop_ldg(b + 1));
-        return pop_ldg(reinterpret_cast<const float2 *>(b));
-    }
-    // store population q of the cells i, i + 1; returns the values as stored
-    static __device__ __forceinline__ float2 st_pair_raw(void *g, int q, long long i, long long N, float2 v) {
-        const long long k = (long long)q * N + i;
-        float *b = reinterpret_cast<float *>(g) + k;
-        if (k & 1) {
-            pop_st(b, v.x);
-            pop_st(b + 1, v.y);
-        } else {
-            pop_st(reinterpret_cast<float2 *>(b), v);
-        }
-        return v;
-    }
 };
 
 template <> struct Sto<2> {
@@ -271,123 +244,6 @@ template <> struct Sto<2> {
         __half hq = __float2half_rn(v);
         pop_st(const_cast<__half *>(hp(g, N)) + ((long long)(q - 1) * N + i), hq);
         return __half2float(hq);
-    }
-    // the populations q of the cells j, j + 1 in raw units: one 4-byte load
-    // (8 bytes for the rest population) when the pair starts on an even
-    // element, otherwise the two aligned words around it
-    static __device__ __forceinline__ float2 ldg_pair_raw(const void *g, int q, long long j, long long N) {
-        if (q == 0) {
-            const float *b = reinterpret_cast<const float *>(g) + j;
-            if (j & 1) return make_float2(pop_ldg(b), pop_ldg(b + 1));
-            return pop_ldg(reinterpret_cast<const float2 *>(b));
-        }
-        const long long k = (long long)(q - 1) * N + j;
-        const __half *h = hp(g, N) + k;
-        if (k & 1) {
-            const __half2 a = pop_ldg(reinterpret_cast<const __half2 *>(h - 1));
-            const __half2 b = pop_ldg(reinterpret_cast<const __half2 *>(h + 1));
-            return make_float2(__high2float(a), __low2float(b));
-        }
-        return __half22float2(pop_ldg(reinterpret_cast<const __half2 *>(h)));
-    }
-    // store population q of the cells i, i + 1 (raw units); returns the
-    // values as stored
-    static __device__ __forceinline__ float2 st_pair_raw(void *g, int q, long long i, long long N, float2 v) {
-        if (q == 0) {
-            float *b = reinterpret_cast<float *>(g) + i;
-            if (i & 1) {
-                pop_st(b, v.x);
-                pop_st(b + 1, v.y);
-            } else {
-                pop_st(reinterpret_cast<float2 *>(b), v);
-            }
-            return v;
-        }
-        const long long k = (long long)(q - 1) * N + i;
-        __half *h = const_cast<__half *>(hp(g, N)) + k;
-        const __half2 hv = __floats2half2_rn(v.x, v.y);
-        if (k & 1) {
-            pop_st(h, __low2half(hv));
-            pop_st(h + 1, __high2half(hv));
-        } else {
-            pop_st(reinterpret_cast<__half2 *>(h), hv);
-        }
-        return __half22float2(hv);
-    }
-};
-
-// The bulk kernel's view of one population grid: 32-bit element indices
-// (q N + j < 2^32 for the float storages, checked at create) from one base
-// pointer per kind of plane, so an access costs one index multiply-add and
-// one widening address computation instead of 64-bit index arithmetic.
-template <int S> struct Planes;
-template <> struct Planes<1> {
-    const float *r;
-    float *w;
-    uint32_t N;
-    __device__ __forceinline__ Planes(const void *src, void *dst, long long n)
-        : r(reinterpret_cast<const float *>(src)), w(reinterpret_cast<float *>(dst)), N((uint32_t)n) {}
-    __device__ __forceinline__ float ld(int q, uint32_t j) const { return pop_ldg(r + ((uint32_t)q * N + j)); }
-    __device__ __forceinline__ float st(int q, uint32_t j, float v) const {
-        pop_st(w + ((uint32_t)q * N + j), v);
-        return v;
-    }
-    // the pair j, j + 1 when j + q N is even (one 8-byte load / store)
-    __device__ __forceinline__ float2 ld2(int q, uint32_t j) const {
-        return pop_ldg(reinterpret_cast<const float2 *>(r + ((uint32_t)q * N + j)));
-    }
-    // the pair j, j + 1 when j + q N is odd (two loads)
-    __device__ __forceinline__ float2 ld2_odd(int q, uint32_t j) const {
-        const float *b = r + ((uint32_t)q * N + j);
-        return make_float2(pop_ldg(b), pop_ldg(b + 1));
-    }
-    __device__ __forceinline__ float2 st2(int q, uint32_t j, float2 v) const {
-        pop_st(reinterpret_cast<float2 *>(w + ((uint32_t)q * N + j)), v);
-        return v;
-    }
-};
-template <> struct Planes<2> {
-    const float *r0;
-    const __half *rh;
-    float *w0;
-    __half *wh;
-    uint32_t N;
-    __device__ __forceinline__ Planes(const void *src, void *dst, long long n)
-        : r0(reinterpret_cast<const float *>(src)), rh(reinterpret_cast<const __half *>(r0 + n)),
-          w0(reinterpret_cast<float *>(dst)), wh(reinterpret_cast<__half *>(w0 + n)), N((uint32_t)n) {}
-    // raw units: q >= 1 times the storage's scale, the rest population unscaled
-    __device__ __forceinline__ float ld(int q, uint32_t j) const {
-        if (q == 0) return pop_ldg(r0 + j);
-        return __half2float(pop_ldg(rh + ((uint32_t)(q - 1) * N + j)));
-    }
-    __device__ __forceinline__ float st(int q, uint32_t j, float v) const {
-        if (q == 0) {
-            pop_st(w0 + j, v);
-            return v;
-        }
-        const __half h = __float2half_rn(v);
-        pop_st(wh + ((uint32_t)(q - 1) * N + j), h);
-        return __half2float(h);
-    }
-    __device__ __forceinline__ float2 ld2(int q, uint32_t j) const {
-        if (q == 0) return pop_ldg(reinterpret_cast<const float2 *>(r0 + j));
-        return __half22float2(pop_ldg(reinterpret_cast<const __half2 *>(rh + ((uint32_t)(q - 1) * N + j))));
-    }
-    __device__ __forceinline__ float2 ld2_odd(int q, uint32_t j) const {
-        if (q == 0) return make_float2(pop_ldg(r0 + j), pop_ldg(r0 + j + 1));
-        const __half *h = rh + ((uint32_t)(q - 1) * N + j);
-        const __half2 a = pop_ldg(reinterpret_cast<const __half2 *>(h - 1));
-        const __half2 b = pop_ldg(reinterpret_cast<const __half2 *>(h + 1));
-        return make_float2(__high2float(a), __low2float(b));
-    }
-    __device__ __forceinline__ float2 st2(int q, uint32_t j, float2 v) const {
-        if (q == 0) {
-            pop_st(reinterpret_cast<float2 *>(w0 + j), v);
-            return v;
-        }
-        const __half2 h = __floats2half2_rn(v.x, v.y);
-        pop_st(reinterpret_cast<__half2 *>(wh + ((uint32_t)(q - 1) * N + j)), h);
-        return __half22float2(h);
     }
 };
 
@@ -489,6 +345,16 @@ __device__ __forceinline__ uint32_t iface_cell(const Dev &d, const IfaceSeq &r, 
     for (int k = 1; k < PREV_LISTS; ++k)
         if (it >= r.e[k - 1]) p = d.plist[k] + (it - r.e[k - 1]);
     return *p;
+}
+
+// opposite of a direction known at run time only
+__host__ __device__ constexpr unsigned long long opp_bits(int half) {
+    unsigned long long b = 0;
+    for (int q = 10 * half; q < (half ? Q : 10); ++q) b |= (unsigned long long)opp(q) << (5 * (q - 10 * half));
+    return b;
+}
+__device__ __forceinline__ int opp_lane(int q) {
+    return (int)((q < 10 ? opp_bits(0) >> (5 * q) : opp_bits(1) >> (5 * (q - 10))) & 31u);
 }
 
 // atomic OR / AND on one byte of the mark array; returns the old byte
@@ -860,7 +726,10 @@ __device__ __forceinline__ bool vpos_finite(float2 r) { return vpos_finite(r.x) 
 // (c of the pair's member with the positive leading component) so that
 //   dn = (1 - omega) dp + (E +- G),  E = omega A + C,  G = omega B + D.
 // Returns the collision density.
-template <int SC, class V, class Store>
+// ZG (ax = ay = 0: gravity along z alone) leaves out the products by the zero
+// accelerations (x + 0 y = x, so every value is the same): 212 instead of 228
+// operations.
+template <int SC, bool ZG, class V, class Store>
 __device__ __forceinline__ V collide_store_v(const Dev &d, const V *dp, Store store) {
     constexpr float sc = (float)SC, isc = 1.0f / (float)SC;
     V dr = dp[0];
@@ -882,11 +751,14 @@ __device__ __forceinline__ V collide_store_v(const Dev &d, const V *dp, Store st
     const V nusq15 = vmul(vfma(uz, uz, vfma(uy, uy, vmul(ux, ux))), vbc<V>(-1.5f));  // -1.5 u.u
     const float om = d.omega_f, om1 = 1.0f - om;
     const float ax = d.a_f[0], ay = d.a_f[1], az = d.a_f[2];
-    const V nua3 = vmul(vfma(uz, vbc<V>(az), vfma(uy, vbc<V>(ay), vmul(ux, vbc<V>(ax)))), vbc<V>(-3.0f));
+    const V nua3 = vmul(ZG ? vmul(uz, vbc<V>(az)) : vfma(uz, vbc<V>(az), vfma(uy, vbc<V>(ay), vmul(ux, vbc<V>(ax)))),
+                        vbc<V>(-3.0f));
     // per weight class: w dr, w rho, 3 w rho (times SC)
     const V wdr1 = vmul(dr, vbc<V>(wf(1) * sc)), wr1 = vmul(rho, vbc<V>(wf(1) * sc));
     const V wdr2 = vmul(dr, vbc<V>(wf(7) * sc)), wr2 = vmul(rho, vbc<V>(wf(7) * sc));
     const V wr13 = vmul(wr1, vbc<V>(3.0f)), wr23 = vmul(wr2, vbc<V>(3.0f));
+    // ZG: C of the directions with c_z = 0, and 3 w rho az of those with c_z = 1
+    const V c1 = vmul(wr1, nua3), c2 = vmul(wr2, nua3), d1 = vmul(wr13, vbc<V>(az)), d2 = vmul(wr23, vbc<V>(az));
     V rest = vbc<V>(0.0f);
 #pragma unroll
     for (int q = 1; q < Q; ++q) {
@@ -903,9 +775,14 @@ __device__ __forceinline__ V collide_store_v(const Dev &d, const V *dp, Store st
         if ((cx(p) || cy(p)) && cz(p) < 0) cu = vsub(cu, uz);
         const float ca = (float)cx(p) * ax + (float)cy(p) * ay + (float)cz(p) * az;
         const V A = vfma(wr, vfma(vmul(cu, cu), vbc<V>(4.5f), nusq15), wdr);
-        const V C = vmul(wr, vfma(cu, vbc<V>(9.0f * ca), nua3));
+        const V C = ZG && cz(p) == 0 ? (axis ? c1 : c2) : vmul(wr, vfma(cu, vbc<V>(9.0f * (ZG ? (float)cz(p) * az : ca)), nua3));
         const V E = vfma(A, vbc<V>(om), C);
-        const V G = vfma(vmul(wr3, cu), vbc<V>(om), vmul(wr3, vbc<V>(ca)));
+        const V wcu = vmul(wr3, cu);
+        V G;
+        if (!ZG) G = vfma(wcu, vbc<V>(om), vmul(wr3, vbc<V>(ca)));
+        else if (cz(p) == 0) G = vmul(wcu, vbc<V>(om));
+        else if (cz(p) > 0) G = vfma(wcu, vbc<V>(om), axis ? d1 : d2);
+        else G = vfma(wcu, vbc<V>(om), vmul(axis ? d1 : d2, vbc<V>(-1.0f)));
         const V dnp = vfma(dp[p], vbc<V>(om1), vadd(E, G));
         const int m = p == q ? qb : q;
         const V dnm = vfma(dp[m], vbc<V>(om1), vsub(E, G));
@@ -935,8 +812,8 @@ __global__ void k_init(Dev d, const uint8_t *flags, const double *fill, const do
     const int c = flags[i] & CL_MASK;
     int x, y, z;
     coords(d, i, x, y, z);
-    const bool face = x == 0 || x == d.nx - 1 || y == 0 || y == d.ny - 1 || z == 0 || z == d.nz - 1;
-    d.flags[i] = (uint8_t)(c | (face && d.walls_move ? MOVING_FACE : 0));
+    const int fx = x == 0 || x == d.nx - 1 ? FACE_X : 0, fyz = y == 0 || y == d.ny - 1 || z == 0 || z == d.nz - 1 ? FACE_YZ : 0;
+    d.flags[i] = (uint8_t)(c | fx | fyz | (d.walls_move && (fx | fyz) ? MOVING_FACE : 0));
     d.bid[i] = 0;
     d.cmark[i] = 0;
     if (c != CL_L && c != CL_I) return;
@@ -1095,13 +972,14 @@ __device__ __forceinline__ void list_span(const VB &vb, uint32_t n, uint32_t per
 // it wants into shared memory, then works on them with full warps
 // (`work(x, y, z, i)`).
 constexpr uint32_t CHUNK = 1024;
+constexpr int FORCE_THREADS = 128;
 template <uint32_t G, class Want, class Work>
 __device__ __forceinline__ void walk_near(const Dev &d, const int *lo, const int *hi, uint32_t ncell, const VB &vb,
                                           uint32_t blocks, Want want, Work work) {
     __shared__ uint32_t s_cell[CHUNK];
     __shared__ uint32_t s_n;
     if (vb.x >= blocks) return;
-    const uint32_t nthr = blockDim.x * blockDim.y, tid = threadIdx.x + blockDim.x * threadIdx.y, lane = tid & 31u;
+    const uint32_t nthr = blockDim.x, tid = threadIdx.x, lane = tid & 31u;
     const uint32_t groups = (ncell + G - 1) / G;
     const uint32_t mine = groups > vb.x ? (groups - vb.x + blocks - 1) / blocks * G : 0;  // cells of this block
     constexpr int U = 4;  // flag loads in flight per thread
@@ -1374,8 +1252,8 @@ __device__ __forceinline__ void forces_f64_body(const Dev &d, const VB &vb) {
     // block reduction of the exact integer sums (any order gives the same
     // bits); a warp without any link skips the tree (its sums are zeros).
     // The block's partials go out as 128-bit integers (low, high word).
-    __shared__ unsigned __int128 sh[8][7];
-    const int tid = threadIdx.x + blockDim.x * threadIdx.y;
+    __shared__ unsigned __int128 sh[FORCE_THREADS / 32][7];
+    const int tid = threadIdx.x;
     int lane = tid & 31, wid = tid >> 5;
     const bool any = __any_sync(0xffffffffu, (acc[6] | acc[0] | acc[1] | acc[2]) != 0);
 #pragma unroll
@@ -1388,7 +1266,7 @@ __device__ __forceinline__ void forces_f64_body(const Dev &d, const VB &vb) {
     __syncthreads();
     if (tid < 7) {
         unsigned __int128 v = 0;
-        for (int w = 0; w < 8; ++w) v += sh[w][tid];
+        for (int w = 0; w < FORCE_THREADS / 32; ++w) v += sh[w][tid];
         unsigned long long *p = reinterpret_cast<unsigned long long *>(d.part) +
                                 2 * (((long long)bi * FORCE_BLOCKS + vb.x) * 7 + tid);
         p[0] = (unsigned long long)v;
@@ -1431,8 +1309,7 @@ __device__ __forceinline__ void forces_float_body(const Dev &d, const VB &vb) {
     const float vf[3] = {(float)b.v[0], (float)b.v[1], (float)b.v[2]};
     const float wfv[3] = {(float)b.w[0], (float)b.w[1], (float)b.w[2]};
     const float rg = (float)d.rho_g, wrg1 = d.rg1_f;
-    const int tid = threadIdx.x + blockDim.x * threadIdx.y;
-    const int lane = tid & 31, wid = tid >> 5, nwarp = (blockDim.x * blockDim.y) >> 5;
+    const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5, nwarp = blockDim.x >> 5;
     const long long sy = d.nx, sz = (long long)d.nx * d.ny;
     int lo[3], hi[3];
     near_range(d, b, lo, hi);
@@ -1555,7 +1432,7 @@ __device__ __forceinline__ void forces_float_body(const Dev &d, const VB &vb) {
     });
     // warp sums, then the warps' sums in the block (integers: exact); a warp
     // without any link skips the reductions (its sums are zeros)
-    __shared__ long long shi[8][13];
+    __shared__ long long shi[FORCE_THREADS / 32][13];
     const bool any = __any_sync(0xffffffffu, hit);
 #pragma unroll
     for (int c = 0; c < 13; ++c) {
@@ -1596,7 +1473,7 @@ __device__ __forceinline__ void forces_body(const Dev &d, const VB &vb) {
 }
 
 template <int S>
-__global__ void __launch_bounds__(256, S == 0 ? 2 : LBMFS_FORCE_MINB) k_forces(const __grid_constant__ Dev d) {
+__global__ void __launch_bounds__(FORCE_THREADS, S == 0 ? 4 : LBMFS_FORCE_MINB) k_forces(const __grid_constant__ Dev d) {
     forces_body<S, false>(d, vb_own());
 }
 
@@ -1604,8 +1481,6 @@ __global__ void __launch_bounds__(256, S == 0 ? 2 : LBMFS_FORCE_MINB) k_forces(c
 // Sec. 2.3 Eq. noslip); interface cells are listed for k_interface
 template <int S, int ZBMAX>
 __device__ __forceinline__ void liquid_column(const Dev &d, bool in, int x, int y, int z0, int z1);
-template <int S, int ZBMAX>
-__device__ __forceinline__ void liquid_body_pair(const Dev &d, const VB &vb, int zb);
 
 // A block covers BULK_THREADS consecutive cells of an xy-plane (row ends
 // wrap to the next row, so narrow grids keep every lane busy) for zb
@@ -1622,17 +1497,10 @@ __device__ __forceinline__ void liquid_body(const Dev &d, const VB &vb, int zb) 
     const int z1 = min(z0 + zb, d.nz);
     liquid_column<S, ZBMAX>(d, in, x, y, z0, z1);
 }
-// the bulk body of a storage: one cell per thread (double), two (float)
-template <int S, int ZBMAX>
-__device__ __forceinline__ void bulk_body(const Dev &d, const VB &vb, int zb) {
-    if constexpr (S == 0 || !LBMFS_BULK_PAIR) liquid_body<S, ZBMAX>(d, vb, zb);
-    else if (d.pair_ok) liquid_body_pair<S, ZBMAX>(d, vb, zb);
-    else liquid_body<S, ZBMAX>(d, vb, zb);
-}
 template <int S, int ZB>
-__global__ void __launch_bounds__(BULK_THREADS, S == 0 ? 1 : (LBMFS_BULK_PAIR ? LBMFS_PAIR_MINB : LBMFS_BULK_MINB))
+__global__ void __launch_bounds__(BULK_THREADS, S == 0 ? 1 : LBMFS_BULK_MINB)
     k_liquid(const __grid_constant__ Dev d) {
-    bulk_body<S, ZB>(d, vb_own(), ZB);
+    liquid_body<S, ZB>(d, vb_own(), ZB);
 }
 
 template <int S>
@@ -1652,7 +1520,7 @@ __device__ __forceinline__ void collide_store(const Dev &d, typename Sto<S>::R *
         // fp in the storage's raw units (to_raw)
         void *g = d.fdst;
         const long long N = d.N;
-        float rho = collide_store_v<P::SCALE, float>(d, fp, [&](int q, float v) { return P::st_raw(g, q, i, N, v); });
+        float rho = collide_store_v<P::SCALE, false, float>(d, fp, [&](int q, float v) { return P::st_raw(g, q, i, N, v); });
         if (!vpos_finite(rho)) atomicOr(d.status, ST_NONFINITE);
     }
 }
@@ -1782,7 +1650,7 @@ template <int S, bool DENSE> __device__ __forceinline__ void near_body(const Dev
     int lo[3], hi[3];
     near_range(d, d.bodies[bi], lo, hi);
     const uint32_t ncell = (uint32_t)range_count(lo, hi);
-    walk_near<32>(d, lo, hi, ncell, vb, near_blocks(d, vb, ncell, DENSE), [](int fb) { return (fb & ~MOVING_FACE) == (CL_L | NB_OBST); },
+    walk_near<32>(d, lo, hi, ncell, vb, near_blocks(d, vb, ncell, DENSE), [](int fb) { return (fb & (CL_MASK | NB_OBST)) == (CL_L | NB_OBST); },
                      [&](int x, int y, int z, long long i) {
                          typename Sto<S>::R fp[Q];
                          bool mine;
@@ -1829,7 +1697,7 @@ template <int S> __device__ __forceinline__ void faces_body(const Dev &d, const 
                 z = 1 + k / (two_x * my);
             }
             const long long i = x + (long long)nx * (y + (long long)ny * z);
-            if (d.flags[i] == (CL_L | MOVING_FACE)) {
+            if ((d.flags[i] & (CL_MASK | NB_OBST)) == CL_L) {
                 typename Sto<S>::R fp[Q];
                 bool mine;
                 wacc += gather_general<S>(d, (int)x, (int)y, (int)z, i, fp, -1, mine);
@@ -1853,16 +1721,21 @@ __global__ void __launch_bounds__(GEN_THREADS, 1) k_faces(const __grid_constant_
     faces_body<S>(d, vb_own());
 }
 
-// One liquid cell (class byte CL_L, coordinates x, y, z, index i; not
+// The liquid cells that the bulk kernel steps: not those with the
+// neighbour-obstacle bit (k_near) or on a face of a grid with moving walls
+// (k_faces).  With the byte CL_L the cell is also on no
+// face.
+__device__ __forceinline__ bool bulk_cell(int c) { return (c & (CL_MASK | NB_OBST | MOVING_FACE)) == CL_L; }
+// One such cell (class byte c, coordinates x, y, z, index i; not
 // next to an obstacle): gather its 18 arriving populations by the cheapest rule
 // that holds for it, collide and store.
 template <int S>
-__device__ __forceinline__ void liquid_one(const Dev &d, int x, int y, int z, long long i) {
+__device__ __forceinline__ void liquid_one(const Dev &d, int c, int x, int y, int z, long long i) {
     using P = Sto<S>;
     using R = typename P::R;
     const long long N = d.N;
     R fp[Q];
-    if (x > 0 && x < d.nx - 1 && y > 0 && y < d.ny - 1 && z > 0 && z < d.nz - 1) {
+    if (c == CL_L) {
         // no obstacle or wall in the neighbourhood and a liquid cell never
         // touches gas: plain pull from the 18 neighbours
         const long long sy = d.nx, sz = (long long)d.nx * d.ny;
@@ -1900,7 +1773,7 @@ __device__ __forceinline__ void liquid_one(const Dev &d, int x, int y, int z, lo
 template <int S, int ZBMAX>
 __device__ __forceinline__ void liquid_column(const Dev &d, bool in, int x, int y, int z0, int z1) {
     static_assert(ZBMAX <= 8, "flags of a column (z1 - z0 <= ZBMAX) are packed into 64 bits");
-    const long long sy = d.nx, sz = (long long)d.nx * d.ny;
+    const long long sz = (long long)d.nx * d.ny;
     // (cell indices are below 2^32)
     long long i = (long long)((unsigned)x + (unsigned)d.nx * ((unsigned)y + (unsigned)d.ny * (unsigned)z0));
     uint64_t fl = 0;
@@ -1916,71 +1789,8 @@ __device__ __forceinline__ void liquid_column(const Dev &d, bool in, int x, int 
         const int c = (int)(fl & 0xff);
         fl >>= 8;
         wl_append(d, (c & CL_MASK) == CL_I, WL_IFACE, (uint32_t)i);
-        if (c != CL_L) continue;  // (with the neighbour-obstacle bit: k_near's; with the face bit: k_faces')
-        liquid_one<S>(d, x, y, z, i);  // one copy of the collision in the kernel
-    }
-}
-
-// Float storages on grids with nx and the cell count even (Dev::pair_ok):
-// two cells per thread, the cells p = 2t and 2t + 1 of the xy-plane (a block
-// covers 2 BULK_THREADS of them), zb z-planes.  Every pair then starts on an
-// even element of each plane, so where both cells are interior liquid cells
-// -- almost every liquid cell -- each direction's two arriving populations come
-// in one load (two for the +-x directions, whose sources start one element
-// off), the two cells collide together in packed FP32 arithmetic (float2
-// operations with the same roundings per cell as the single-cell path), and
-// each direction's pair is stored at once.  Every other cell takes the
-// single-cell path.
-template <int S, int ZBMAX>
-__device__ __forceinline__ void liquid_body_pair(const Dev &d, const VB &vb, int zb) {
-    using P = Sto<S>;
-    static_assert(S != 0, "pairs serve the float storages");
-    if ((int)(vb.z * zb) > __ldg(d.ztop_rd) + ZTOP_MARGIN) return;
-    const unsigned nxy = (unsigned)d.nx * (unsigned)d.ny;
-    const unsigned p0 = 2u * (vb.x * BULK_THREADS + threadIdx.x);
-    const bool in = p0 < nxy;  // nx even: the pair lies in one row
-    const int y0 = in ? (int)(p0 / (unsigned)d.nx) : 0;
-    const int x0 = in ? (int)p0 - y0 * d.nx : 0;
-    const int z0 = vb.z * zb, z1 = min(z0 + zb, d.nz);
-    const uint32_t sy = (uint32_t)d.nx, sz = (uint32_t)nxy;
-    uint32_t j = p0 + sz * (uint32_t)z0;  // cell 0 at z (even); cell 1 is j + 1
-    // classes of both columns in one round of loads: cell 0 in the low byte
-    unsigned fl[ZBMAX];
-    unsigned any = 0;
-#pragma unroll
-    for (int k = 0; k < ZBMAX; ++k) {
-        fl[k] = (in && z0 + k < z1) ? (unsigned)*reinterpret_cast<const uint16_t *>(d.flags + j + k * sz) : 0u;
-        any |= fl[k];
-    }
-    if (__any_sync(0xffffffffu, (any & 0x0303u) != 0) && (threadIdx.x & 31) == 0) atomicMax(d.ztop_wr, z1 - 1);
-    if (any == 0) return;
-    const bool pair_xy = x0 > 0 && x0 + 1 < d.nx - 1 && y0 > 0 && y0 < d.ny - 1;
-    const Planes<S> pl(d.fsrc, d.fdst, d.N);
-#pragma unroll 1
-    for (int k = 0; k < ZBMAX; ++k, j += sz) {
-        const int z = z0 + k;
-        if (z >= z1) break;
-        const int c0 = (int)(fl[k] & 0xffu), c1 = (int)(fl[k] >> 8);
-        wl_append(d, (c0 & CL_MASK) == CL_I, WL_IFACE, j);
-        wl_append(d, (c1 & CL_MASK) == CL_I, WL_IFACE, j + 1);
-        if (pair_xy && c0 == CL_L && c1 == CL_L && z > 0 && z < d.nz - 1) {
-            float2 fp[Q];
-#pragma unroll
-            for (int q = 1; q < Q; ++q) {
-                const uint32_t src = j - (uint32_t)cx(q) - (uint32_t)cy(q) * sy - (uint32_t)cz(q) * sz;
-                fp[q] = cx(q) == 0 ? pl.ld2(q, src) : pl.ld2_odd(q, src);
-            }
-            fp[0] = pl.ld2(0, j);
-            const float2 rho = collide_store_v<P::SCALE, float2>(d, fp, [&](int q, float2 v) { return pl.st2(q, j, v); });
-            if (!vpos_finite(rho)) atomicOr(d.status, ST_NONFINITE);
-        } else {
-#pragma unroll 1
-            for (int h = 0; h < 2; ++h) {
-                const int c = h ? c1 : c0;
-                if (c != CL_L) continue;
-                liquid_one<S>(d, x0 + h, y0, z, (long long)(j + h));
-            }
-        }
+        if (!bulk_cell(c)) continue;
+        liquid_one<S>(d, c, x, y, z, i);  // one copy of the collision in the kernel
     }
 }
 
@@ -2071,8 +1881,8 @@ __global__ void __launch_bounds__(BULK_THREADS, LBMFS_BULK_MINB) k_liquid_pipe(D
                 fp[q] = Pipe<S>::get(&slots[b][0][tid], q, i - (cx(q) * sx + cy(q) * sy + cz(q) * sz), d.N);
             to_raw<S>(fp);
             collide_store<S>(d, fp, i);
-        } else if (fl_cur == CL_L) {
-            liquid_one<S>(d, x, y, z, i);
+        } else if (bulk_cell(fl_cur)) {
+            liquid_one<S>(d, fl_cur, x, y, z, i);
         }
         fl_cur = fl_next;
         fl_next = fl_after;
@@ -2136,6 +1946,9 @@ __device__ __forceinline__ void bulk_g2s(void *dst, const void *src, unsigned by
                      smem_addr(dst)),
                  "l"(src), "r"(bytes), "r"(smem_addr(bar))
                  : "memory");
+}
+__device__ __forceinline__ void mbar_arrive(uint64_t *bar) {
+    asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_addr(bar)) : "memory");
 }
 __device__ __forceinline__ bool mbar_try_wait(uint64_t *bar, unsigned parity) {
     unsigned ok;
@@ -2222,8 +2035,8 @@ __global__ void __launch_bounds__(BULK_THREADS, LBMFS_BULK_MINB) k_liquid_tma(De
             for (int q = 0; q < Q; ++q) fp[q] = G::get(stage, q, tid + ((S == 2 && q > 0) ? Stage<2>::H : 4) - cx(q));
             to_raw<S>(fp);
             collide_store<S>(d, fp, i);
-        } else if (c == CL_L) {
-            liquid_one<S>(d, x, y, z, i);
+        } else if (bulk_cell(c)) {
+            liquid_one<S>(d, c, x, y, z, i);
         }
         fl_cur = fl_next;
         fl_next = fl_after;
@@ -2234,6 +2047,437 @@ __global__ void __launch_bounds__(BULK_THREADS, LBMFS_BULK_MINB) k_liquid_tma(De
         // has had its (bounded) wait above, so no copy is left unawaited
         if (tid == 0) atomicOr(d.status, ST_TIMEOUT);
     }
+}
+
+// --------------------------------------------------- ring bulk kernel
+//
+// The bulk kernel of the FP16 storage.  Pull streaming reads population q of
+// cell i at i - (c_x + c_y nx + c_z nx ny): a shift of the linear cell index, so
+// the sources of TILE consecutive cells are TILE consecutive elements of each
+// plane whatever the grid's sizes, and 19 linear bulk copies (1 KB each) bring a
+// tile's arriving populations into shared memory.  A producer warp keeps a ring
+// of STAGES tiles in flight per block with no registers held for them, which
+// was what bound the one-cell-per-thread kernel (64 registers, 24 warps with one
+// cell's loads each; FP16S: 73 % of the issue slots, 52 % of the copy
+// bandwidth); the consumer warps take two cells per thread, in packed FP32
+// arithmetic with half the instructions per cell.  Copies start at the 16-byte
+// boundary below the source; the remainder m_q depends on q only (tiles start
+// at multiples of TILE).  Reads past a plane's ends meet the next plane or the
+// guard bands and belong to cells on grid faces, whose populations from beyond
+// the face are their own (resting walls) or a periodic image's.  On the x faces
+// -- two cells of every row, so some in nearly every warp -- a second warp
+// fetches them as soon as a tile is announced and patches them into the staged
+// tile; the consumers fetch those of the y and z faces (whole warps) themselves.
+// Fetching the x faces in the consumers too cost a global load's latency per
+// warp: FP16S bulk kernel, 768x384x256 763 us against 581 without any face work.
+constexpr int RING_STAGES = 4;
+struct RingShape {
+    static constexpr int TILE = RING_TILE, ESZ = 2;         // cells, bytes per moving population
+    static constexpr int WORKERS = TILE / 2, THREADS = WORKERS + 64;  // and the producer and the patching warp
+    static constexpr int ALIGN = 16 / ESZ;                  // elements per 16 bytes
+    static constexpr int ROW = (TILE + ALIGN) * ESZ;        // bytes of one staged plane, q >= 1
+    static constexpr int COPY = TILE * 4 + (Q - 1) * ROW;   // bytes of a tile's copies
+    static constexpr int STAGE = (COPY + TILE + 127) / 128 * 128;  // populations, then the flags
+    static constexpr int HEAD = 256;                        // barriers, tile descriptors
+    static constexpr int SMEM = HEAD + RING_STAGES * STAGE;
+};
+// offset of direction q's source in the linear cell index
+__device__ __forceinline__ int src_offset(const Dev &d, int q) { return cx(q) + d.nx * (cy(q) + d.ny * cz(q)); }
+// element index, from the grid's (16-byte aligned) start, of the first staged
+// element of plane q >= 1 for the tile at i0, before the rounding to 16 bytes
+// (the FP16 planes start after plane 0, whose N floats are 2 N of their
+// elements)
+__device__ __forceinline__ long long ring_plane(const Dev &d, int q) { return (long long)(q + 1) * d.N; }
+
+// what a tile is: its tank (batch) and first cell; tank < 0 ends the ring
+struct RingTile {
+    int tank;
+    uint32_t i0;
+};
+
+// The populations of the cells 2p, 2p + 1 of the staged tile in raw units.
+// EVEN (nx and the cell count even): a pair starts on an even element exactly
+// when c_x = 0; else that is decided per direction at run time.
+template <bool EVEN>
+__device__ __forceinline__ float2 ring_pair(const char *stage, const Dev &d, int q, int p) {
+    using G = RingShape;
+    if (q == 0) return *reinterpret_cast<const float2 *>(stage + 8 * p);
+    const int m = (int)(ring_plane(d, q) - src_offset(d, q)) & (G::ALIGN - 1);  // (tiles start at multiples of ALIGN)
+    const uint32_t *w = reinterpret_cast<const uint32_t *>(stage + G::TILE * 4 + (q - 1) * G::ROW) + p + (m >> 1);
+    uint32_t v;
+    if (EVEN && cx(q) == 0) v = w[0];
+    else v = __funnelshift_r(w[0], w[1], EVEN ? 16 : (m & 1) * 16);
+    return __half22float2(*reinterpret_cast<const __half2 *>(&v));
+}
+// the five directions with component `sign` along an axis, 5 bits each
+__host__ __device__ constexpr unsigned face_dirs(int axis, int sign) {
+    unsigned b = 0;
+    int n = 0;
+    for (int q = 1; q < Q; ++q)
+        if ((axis == 0 ? cx(q) : (axis == 1 ? cy(q) : cz(q))) == sign) b |= (unsigned)q << (5 * n++);
+    return b;
+}
+// Where the population that arrives at face cell i from beyond the grid in
+// direction q is read: the cell's own opposite one (resting wall) or the
+// periodic image's, as an element index.
+__device__ __forceinline__ long long face_source(const Dev &d, uint32_t i, int q) {
+    if (d.periodic) {
+        int x, y, z;
+        coords(d, i, x, y, z);
+        const long long si = nbr(d, x, y, z, -dir_x(q), -dir_y(q), -dir_z(q));
+        if (si >= 0) return ring_plane(d, q) + si;
+    }
+    return ring_plane(d, opp_lane(q)) + i;
+}
+// byte offset in a stage of population q of the tile's cell `local`
+__device__ __forceinline__ int stage_slot(const Dev &d, int q, int local) {
+    using G = RingShape;
+    const int off = dir_x(q) + d.nx * (dir_y(q) + d.ny * dir_z(q));
+    const int m = (int)(ring_plane(d, q) - off) & (G::ALIGN - 1);
+    return G::TILE * 4 + (q - 1) * G::ROW + (local + m) * G::ESZ;
+}
+// A cell on a y or z face, by the consumer that owns it: its populations from
+// beyond the face into its own slots of the staged tile.  (A loop over the two
+// axes and five directions each: the code stays small.)
+__device__ __forceinline__ void ring_face(const Dev &d, char *stage, uint32_t i, int local) {
+    const uint16_t *src = reinterpret_cast<const uint16_t *>(d.fsrc);
+    int x, y, z;
+    coords(d, i, x, y, z);
+#pragma unroll 1
+    for (int s = 0; s < 4; ++s) {  // y low, y high, z low, z high
+        const int p = s < 2 ? y : z, end = (s < 2 ? d.ny : d.nz) - 1;
+        if (p != (s & 1 ? end : 0)) continue;
+        const unsigned dirs = s < 2 ? (s & 1 ? face_dirs(1, -1) : face_dirs(1, 1)) : (s & 1 ? face_dirs(2, -1) : face_dirs(2, 1));
+        uint16_t v[5];
+#pragma unroll
+        for (int j = 0; j < 5; ++j) v[j] = __ldg(src + face_source(d, i, (int)(dirs >> (5 * j) & 31u)));
+#pragma unroll
+        for (int j = 0; j < 5; ++j)
+            *reinterpret_cast<uint16_t *>(stage + stage_slot(d, (int)(dirs >> (5 * j) & 31u), local)) = v[j];
+    }
+}
+// The patching warp's work on one tile: per row boundary b inside it, the five
+// directions with c_x > 0 of cell b (x = 0) and the five with c_x < 0 of cell
+// b - 1 (x = nx - 1).  A lane keeps one of the ten (three rows at a time), so
+// that an item is an addition, a load and a 2-byte store.  The loads of a tile
+// are issued before the previous tile's are stored.
+struct RingPatch {
+    static constexpr int U = 4;  // items per lane held at a time: 12 rows, enough for one round from nx = 47 up
+    uint16_t v[U];
+    int at[U];  // byte offset of the slot in the stage, -1: none
+    uint32_t rows, row0, i0;
+    // boundaries b = row nx with i0 <= b <= i0 + TILE
+    __device__ __forceinline__ void begin(const Dev &d, uint32_t first) {
+        const uint32_t nx = (uint32_t)d.nx;
+        i0 = first;
+        row0 = (i0 + nx - 1) / nx;
+        rows = (i0 + RingShape::TILE) / nx + 1 - row0;
+    }
+    __device__ __forceinline__ void load(const Dev &d, uint32_t r0) {
+        const uint32_t lane = threadIdx.x & 31u, j = lane % 10u;
+        const bool high = j >= 5;
+        const int q = (int)((high ? face_dirs(0, -1) >> (5 * (j - 5u)) : face_dirs(0, 1) >> (5 * j)) & 31u);
+        const uint16_t *own = reinterpret_cast<const uint16_t *>(d.fsrc) + ring_plane(d, opp_lane(q));
+        const int slot = stage_slot(d, q, 0);
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+            const uint32_t r = r0 + 3u * u + lane / 10u;
+            const uint32_t i = (row0 + r) * (uint32_t)d.nx - (high ? 1u : 0u);  // (of b = i0: before the tile)
+            at[u] = -1;
+            if (lane < 30 && r < rows && i >= i0 && i < i0 + RingShape::TILE && i < (uint32_t)d.N) {
+                v[u] = __ldg(d.periodic ? reinterpret_cast<const uint16_t *>(d.fsrc) + face_source(d, i, q) : own + i);
+                at[u] = slot + (int)(i - i0) * RingShape::ESZ;
+            }
+        }
+    }
+    __device__ __forceinline__ void store(char *stage) const {
+#pragma unroll
+        for (int u = 0; u < U; ++u)
+            if (at[u] >= 0) *reinterpret_cast<uint16_t *>(stage + at[u]) = v[u];
+    }
+};
+
+// One staged tile by the consumer warps.  The kernel holds one copy of the
+// collision (with one per parity and per kind of store its instructions did not
+// fit the caches: 4.7 of 14 stall cycles per instruction in a batch): the
+// gather and the stores branch on the tank's parity, and the collided pairs are
+// kept packed, a register per direction, until the stores.
+template <bool ZG>
+__device__ __forceinline__ void ring_tile(const Dev &d, char *stage, uint64_t *empty, uint32_t i0, int p) {
+    using G = RingShape;
+    const unsigned cc = *reinterpret_cast<const uint16_t *>(stage + G::COPY + 2 * p);
+    const int c0 = (int)(cc & 0xffu), c1 = (int)(cc >> 8);
+    const int lane = threadIdx.x & 31;
+    const uint32_t i = i0 + 2u * (uint32_t)p;
+    // interface cells are listed, in cell order
+    const bool f0 = (c0 & CL_MASK) == CL_I, f1 = (c1 & CL_MASK) == CL_I;
+    const unsigned m0 = __ballot_sync(0xffffffffu, f0), m1 = __ballot_sync(0xffffffffu, f1);
+    if (m0 | m1) {
+        uint32_t at = 0;
+        if (lane == 0) at = atomicAdd(&d.cnt[WL_IFACE], (uint32_t)(__popc(m0) + __popc(m1)));
+        at = __shfl_sync(0xffffffffu, at, 0) + __popc(m0 & ((1u << lane) - 1u)) + __popc(m1 & ((1u << lane) - 1u));
+        // (repeated launches on one state, as the batch's autotuner does them,
+        // append again)
+        if (at + 2 <= d.cap || at + (f0 ? 1 : 0) + (f1 ? 1 : 0) <= d.cap) {
+            if (f0) d.list[WL_IFACE][at++] = i;
+            if (f1) d.list[WL_IFACE][at] = i + 1;
+        } else {
+            atomicOr(d.status, ST_OVERFLOW);
+        }
+    }
+    const bool s0 = bulk_cell(c0), s1 = bulk_cell(c1);
+    if (!__any_sync(0xffffffffu, s0 || s1)) {
+        if (lane == 0) mbar_arrive(empty);
+        return;
+    }
+    if ((s0 && (c0 & FACE_YZ)) || (s1 && (c1 & FACE_YZ))) {
+#pragma unroll 1
+        for (int h = 0; h < 2; ++h)
+            if (h ? s1 && (c1 & FACE_YZ) : s0 && (c0 & FACE_YZ)) ring_face(d, stage, i + h, 2 * p + h);
+    }
+    float2 fp[Q];
+    if (d.pair_ok) {
+#pragma unroll
+        for (int q = 0; q < Q; ++q) fp[q] = ring_pair<true>(stage, d, q, p);
+    } else {
+#pragma unroll
+        for (int q = 0; q < Q; ++q) fp[q] = ring_pair<false>(stage, d, q, p);
+    }
+    __syncwarp();
+    if (lane == 0) mbar_arrive(empty);  // the stage is in registers
+    if (!(s0 || s1)) return;
+    float2 rest;
+    uint32_t hp[Q];  // the collided pairs as stored
+    const float2 rho = collide_store_v<Sto<2>::SCALE, ZG, float2>(d, fp, [&](int q, float2 v) {
+        if (q == 0) {
+            rest = v;
+            return v;
+        }
+        const __half2 h = __floats2half2_rn(v.x, v.y);
+        hp[q] = *reinterpret_cast<const uint32_t *>(&h);
+        return __half22float2(h);
+    });
+    float *w0 = reinterpret_cast<float *>(d.fdst) + i;
+    const bool both = s0 && s1;
+    if (__all_sync(__activemask(), both) && d.pair_ok) {
+        *reinterpret_cast<float2 *>(w0) = rest;
+#pragma unroll
+        for (int q = 1; q < Q; ++q)
+            *reinterpret_cast<uint32_t *>(reinterpret_cast<uint16_t *>(d.fdst) + ring_plane(d, q) + i) = hp[q];
+    } else {
+        // some pair has a cell that is not stepped here, or an odd cell count
+        // puts every other plane on an odd element
+        const bool skew = d.N & 1;
+        if (s0) w0[0] = rest.x;
+        if (s1) w0[1] = rest.y;
+#pragma unroll
+        for (int q = 1; q < Q; ++q) {
+            uint16_t *w = reinterpret_cast<uint16_t *>(d.fdst) + ring_plane(d, q) + i;
+            const bool word = both && !(q % 2 == 0 && skew);
+            if (word) *reinterpret_cast<uint32_t *>(w) = hp[q];
+            if (s0 && !word) w[0] = (uint16_t)hp[q];
+            if (s1 && !word) w[1] = (uint16_t)(hp[q] >> 16);
+        }
+    }
+    if ((s0 && !vpos_finite(rho.x)) || (s1 && !vpos_finite(rho.y))) atomicOr(d.status, ST_NONFINITE);
+}
+
+// The ring over a launch's n entries: tile_of(entry) gives an entry's tank and
+// first cell (single tank: tank 0), dev_of(tank) its descriptor.  Warps 0 .. are
+// the consumers, then the producer, then the patching warp.  A stage goes
+// through four barriers: announced (its tile and class bytes are written),
+// landed (its copies are complete), full (patched), empty (in registers).
+// Every wait is bounded (mbar_wait); one that gives up ends its role with a
+// sticky status.
+template <bool ZG, class TileOf, class DevOf>
+__device__ __forceinline__ void ring_run(uint32_t n, TileOf tile_of, DevOf dev_of) {
+    using G = RingShape;
+    extern __shared__ __align__(128) char smem[];
+    uint64_t *said = reinterpret_cast<uint64_t *>(smem), *landed = said + RING_STAGES, *full = landed + RING_STAGES,
+             *empty = full + RING_STAGES;
+    RingTile *desc = reinterpret_cast<RingTile *>(empty + RING_STAGES);
+    static_assert(RING_STAGES * (4 * 8 + sizeof(RingTile)) <= G::HEAD, "barriers and descriptors fit the head");
+    char *stages = smem + G::HEAD;
+    const int tid = threadIdx.x, lane = tid & 31;
+    if (tid == 0) {
+        for (int k = 0; k < RING_STAGES; ++k) {
+            mbar_init(&said[k], 1);
+            mbar_init(&landed[k], 1);
+            mbar_init(&full[k], 1);
+            mbar_init(&empty[k], G::WORKERS / 32);
+        }
+        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    }
+    __syncthreads();
+    bool ok = true;
+    if (tid < G::WORKERS) {
+        for (uint32_t k = 0;; ++k) {
+            const int st = (int)(k % RING_STAGES);
+            const unsigned ph = (k / RING_STAGES) & 1u;
+            if (!(mbar_wait(&full[st], ph) && mbar_wait(&landed[st], ph))) {
+                ok = false;
+                break;
+            }
+            const RingTile t = desc[st];
+            if (t.tank < 0) break;
+            ring_tile<ZG>(dev_of(t.tank), stages + st * G::STAGE, &empty[st], t.i0, tid);
+        }
+    } else if (tid < G::WORKERS + 32) {
+        uint32_t k = 0;  // tiles produced
+        int top_tank = -1, top = -1;  // highest plane with fluid of the current tank's tiles
+        auto flush_top = [&]() {
+            if (lane == 0 && top >= 0) atomicMax(dev_of(top_tank).ztop_wr, top);
+        };
+        for (uint32_t base = blockIdx.x; base < n && ok; base += 32u * gridDim.x) {
+            // a lane per entry: tiles above the previous step's fluid (plus a
+            // margin) hold only gas
+            const uint32_t e = base + (uint32_t)lane * gridDim.x;
+            RingTile t{-1, 0};
+            if (e < n) {
+                t = tile_of(e);
+                const Dev &d = dev_of(t.tank);
+                if ((int)(t.i0 / ((uint32_t)d.nx * (uint32_t)d.ny)) > __ldg(d.ztop_rd) + ZTOP_MARGIN) t.tank = -1;
+            }
+            // the class bytes of the next tile are requested before the current
+            // one waits for a free stage (the flags are padded to whole tiles)
+            unsigned todo = __ballot_sync(0xffffffffu, t.tank >= 0);
+            auto fetch = [&](unsigned rest, int &tank, uint32_t &i0) {
+                const int l = rest ? __ffs(rest) - 1 : 0;
+                tank = __shfl_sync(0xffffffffu, t.tank, l);
+                i0 = __shfl_sync(0xffffffffu, t.i0, l);
+                uint4 f = make_uint4(0, 0, 0, 0);
+                if (rest) {
+                    const char *src = reinterpret_cast<const char *>(dev_of(tank).flags) + i0;
+                    static_assert(G::TILE == 512, "16 class bytes per lane");
+                    f = reinterpret_cast<const uint4 *>(src)[lane];
+                }
+                return f;
+            };
+            int tank;
+            uint32_t i0;
+            uint4 fl = fetch(todo, tank, i0);
+            while (todo && ok) {
+                todo &= todo - 1;
+                int tank1;
+                uint32_t i1;
+                const uint4 fl1 = fetch(todo, tank1, i1);
+                const Dev &d = dev_of(tank);
+                const unsigned any = fl.x | fl.y | fl.z | fl.w;
+                const bool any_wet = __any_sync(0xffffffffu, (any & 0x03030303u) != 0),
+                           any_liq = __any_sync(0xffffffffu, (any & 0x01010101u) != 0);
+                if (any_wet) {
+                    const int st = (int)(k % RING_STAGES);
+                    char *stage = stages + st * G::STAGE;
+                    if (tank != top_tank) {
+                        flush_top();
+                        top_tank = tank;
+                        top = -1;
+                    }
+                    top = max(top, min(d.nz - 1, (int)((i0 + G::TILE - 1) / ((uint32_t)d.nx * (uint32_t)d.ny))));
+                    if (k >= RING_STAGES) ok = __all_sync(0xffffffffu, mbar_wait(&empty[st], (k / RING_STAGES - 1) & 1u));
+                    if (!ok) break;
+                    reinterpret_cast<uint4 *>(stage + G::COPY)[lane] = fl;
+                    if (lane == 0) desc[st] = RingTile{tank, i0};
+                    fence_async_shared();
+                    __syncwarp();
+                    if (lane == 0) {
+                        mbar_arrive(&said[st]);
+                        mbar_expect_tx(&landed[st], any_liq ? (unsigned)G::COPY : 0u);
+                    }
+                    __syncwarp();
+                    if (any_liq && lane < Q) {
+                        if (lane == 0) {
+                            bulk_g2s(stage, reinterpret_cast<const float *>(d.fsrc) + i0, G::TILE * 4, &landed[st]);
+                        } else {
+                            const int off = dir_x(lane) + d.nx * (dir_y(lane) + d.ny * dir_z(lane));
+                            const long long first = ring_plane(d, lane) + i0 - off;
+                            bulk_g2s(stage + G::TILE * 4 + (lane - 1) * G::ROW,
+                                     reinterpret_cast<const char *>(d.fsrc) + (first & ~(long long)(G::ALIGN - 1)) * G::ESZ,
+                                     G::ROW, &landed[st]);
+                        }
+                    }
+                    ++k;
+                }
+                tank = tank1;
+                i0 = i1;
+                fl = fl1;
+            }
+        }
+        flush_top();
+        const int st = (int)(k % RING_STAGES);
+        if (ok && k >= RING_STAGES) ok = __all_sync(0xffffffffu, mbar_wait(&empty[st], (k / RING_STAGES - 1) & 1u));
+        if (lane == 0) {
+            desc[st] = RingTile{-1, 0};
+            mbar_arrive(&said[st]);
+            mbar_expect_tx(&landed[st], 0u);
+        }
+    } else {
+        // tile k is patched while tile k + 1's loads, where it is announced
+        // already, are under way
+        RingPatch cur, next;
+        auto stage_of = [&](uint32_t k) { return (int)(k % RING_STAGES); };
+        auto phase_of = [&](uint32_t k) { return (k / RING_STAGES) & 1u; };
+        auto begin = [&](RingPatch &r, uint32_t k) {  // after tile k's announcement; its tank
+            const RingTile t = desc[stage_of(k)];
+            if (t.tank >= 0) {
+                r.begin(dev_of(t.tank), t.i0);
+                if (r.rows) r.load(dev_of(t.tank), 0);
+            }
+            return t.tank;
+        };
+        ok = __all_sync(0xffffffffu, mbar_wait(&said[0], 0));
+        int tank = ok ? begin(cur, 0) : -1;
+        for (uint32_t k = 0; ok; ++k) {
+            const int st = stage_of(k);
+            int tank1 = -1;
+            const bool more = tank >= 0;
+            const bool ready = more && __all_sync(0xffffffffu, mbar_try_wait(&said[stage_of(k + 1)], phase_of(k + 1)));
+            if (ready) tank1 = begin(next, k + 1);
+            if (more && cur.rows) {
+                ok = __all_sync(0xffffffffu, mbar_wait(&landed[st], phase_of(k)));
+                char *stage = stages + st * G::STAGE;
+                cur.store(stage);
+                for (uint32_t r0 = 3u * RingPatch::U; r0 < cur.rows; r0 += 3u * RingPatch::U) {
+                    cur.load(dev_of(tank), r0);
+                    cur.store(stage);
+                }
+                __syncwarp();
+            }
+            if (lane == 0) mbar_arrive(&full[st]);
+            if (!more || !ok) break;
+            if (!ready) {
+                ok = __all_sync(0xffffffffu, mbar_wait(&said[stage_of(k + 1)], phase_of(k + 1)));
+                tank1 = ok ? begin(next, k + 1) : -1;
+            }
+            cur = next;
+            tank = tank1;
+        }
+    }
+    if (!ok) atomicOr(dev_of(0).status, ST_TIMEOUT);
+}
+struct OneTank {
+    const Dev &d;
+    __device__ __forceinline__ const Dev &operator()(int) const { return d; }
+};
+struct ManyTanks {
+    const TankSet &ts;
+    __device__ __forceinline__ const Dev &operator()(int tank) const { return ts.d[tank]; }
+};
+template <bool ZG>
+__global__ void __launch_bounds__(RingShape::THREADS, RING_CTAS) k_ring(const __grid_constant__ Dev d, uint32_t n) {
+    ring_run<ZG>(n, [](uint32_t e) { return RingTile{0, e * (uint32_t)RingShape::TILE}; }, OneTank{d});
+}
+
+// the ring over all tanks of a batch's launch (entries: tank, tile in x + 2^16 y)
+template <bool ZG>
+__global__ void __launch_bounds__(RingShape::THREADS, RING_CTAS)
+    k_batch_ring(const __grid_constant__ TankSet ts, const Tile *__restrict__ table, unsigned n) {
+    ring_run<ZG>(n,
+                         [&](uint32_t e) {
+                             const Tile t = table[e];
+                             return RingTile{t.tank, (t.x + ((uint32_t)t.y << 16)) * (uint32_t)RingShape::TILE};
+                         },
+                         ManyTanks{ts});
 }
 
 // fill level of a neighbour as seen by the normal estimate
@@ -3667,11 +3911,10 @@ struct BkReset {
         if (threadIdx.x < CN_COUNT) d.cnt[threadIdx.x] = 0;
     }
 };
-template <int S> LBMFS_BATCH_BODY_SM(BkForces, 256, S == 0 ? 2 : LBMFS_FORCE_MINB, true, forces_body<S, true>(d, vb))
+template <int S> LBMFS_BATCH_BODY_SM(BkForces, FORCE_THREADS, S == 0 ? 4 : LBMFS_FORCE_MINB, true, forces_body<S, true>(d, vb))
 // one instantiation per z-planes-per-tile choice (the column loop unrolled to it)
 template <int S, int ZB>
-LBMFS_BATCH_BODY(BkLiquid, BULK_THREADS, S == 0 ? 1 : (LBMFS_BULK_PAIR ? LBMFS_PAIR_MINB : LBMFS_BULK_MINB),
-                 (bulk_body<S, ZB>(d, vb, zb)))
+LBMFS_BATCH_BODY(BkLiquid, BULK_THREADS, S == 0 ? 1 : LBMFS_BULK_MINB, (liquid_body<S, ZB>(d, vb, zb)))
 // the batch's listed cells are spread over many more blocks: 4 resident per SM
 // (128 registers) beat 1 there, not on the single tank
 template <int S>
@@ -3699,6 +3942,16 @@ template <class K> void batch_launch(const BatchLaunch &b, int sh, dim3 block, c
     if (x.n) k_batch<K><<<x.grid, block, 0, st>>>(*b.ts, x.table, x.n, b.zb);
 }
 template <int S> void batch_bulk_launch(const BatchLaunch &b, cudaStream_t st) {
+    if constexpr (S == 2) {
+        const Shape &x = b.sh[SH_BULK];
+        if (!x.n) return;
+        auto go = [&](void (*k)(TankSet, const Tile *, unsigned)) {
+            cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, RingShape::SMEM);
+            k<<<x.grid, RingShape::THREADS, RingShape::SMEM, st>>>(*b.ts, x.table, x.n);
+        };
+        go(b.zg ? k_batch_ring<true> : k_batch_ring<false>);
+        return;
+    }
     switch (b.zb) {
     case 1: batch_launch<BkLiquid<S, 1>>(b, SH_BULK, BULK_THREADS, st); break;
     case 2: batch_launch<BkLiquid<S, 2>>(b, SH_BULK, BULK_THREADS, st); break;
@@ -3762,8 +4015,7 @@ template <int S> struct Launch {
     }
     // the bulk kernel with the z-planes per block of bulk_planes
     static void bulk(const Dev &d, cudaStream_t st) {
-        const int bc = bulk_cells(S, d);
-        const unsigned gx = (unsigned)(((long long)d.nx * d.ny + bc - 1) / bc);
+        const unsigned gx = (unsigned)(((long long)d.nx * d.ny + BULK_THREADS - 1) / BULK_THREADS);
         const int zb = bulk_planes(S, gx, d.nz);
         if (zb == 1) bulk_zb<1>(d, gx, st);
         if constexpr (S != 0) {
@@ -3777,7 +4029,7 @@ template <int S> struct Launch {
         k_near<S><<<dim3(FORCE_BLOCKS, d.nb), GEN_THREADS, 0, st>>>(d);
     }
     static void forces(const Dev &d, cudaStream_t st) {
-        k_forces<S><<<dim3(FORCE_BLOCKS, d.nb), dim3(32, 8), 0, st>>>(d);
+        k_forces<S><<<dim3(FORCE_BLOCKS, d.nb), FORCE_THREADS, 0, st>>>(d);
     }
     static void scan(const Dev &d, cudaStream_t st) { k_remap_scan<<<dim3(FORCE_BLOCKS, d.nb), 256, 0, st>>>(d); }
     static void interface(const Dev &d, cudaStream_t st) { k_interface<S><<<LBMFS_IFACE_GRID, 128, 0, st>>>(d); }
@@ -3788,9 +4040,22 @@ template <int S> struct Launch {
             dim3 pgrid(rgrid.x, rgrid.y, (d.nz + LBMFS_BULK_PIPE_ZB - 1) / LBMFS_BULK_PIPE_ZB);
             if (d.bulk == BULK_TMA) k_liquid_tma<S><<<rgrid, BULK_THREADS, 128 + 2 * Stage<S>::BYTES, st>>>(d);
             else if (d.bulk == BULK_PIPE) k_liquid_pipe<S><<<pgrid, BULK_THREADS, 0, st>>>(d);
+            else if (S == 2) ring(d, st);
             else bulk(d, st);
         } else {
             bulk(d, st);
+        }
+    }
+    static void ring(const Dev &d, cudaStream_t st) {
+        if constexpr (S == 2) {
+            using G = RingShape;
+            const uint32_t n = (uint32_t)((d.N + G::TILE - 1) / G::TILE);
+            const bool zg = d.a_f[0] == 0.0f && d.a_f[1] == 0.0f;
+            auto go = [&](void (*k)(Dev, uint32_t)) {
+                cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, G::SMEM);
+                k<<<std::min(n, 152u * RING_CTAS), G::THREADS, G::SMEM, st>>>(d, n);
+            };
+            go(zg ? k_ring<true> : k_ring<false>);
         }
     }
     static void tail(const Dev &d, cudaStream_t st) {
@@ -3888,7 +4153,7 @@ template <int S> struct BatchStep {
             s2 = sides->st[2];
         }
         mark();
-        batch_launch<BkForces<S>>(b, SH_FORCE, dim3(32, 8), s1);
+        batch_launch<BkForces<S>>(b, SH_FORCE, FORCE_THREADS, s1);
         if (sides) {
             // in the order in which they should get the SMs
             batch_launch<BkGeneral<S>>(b, SH_GEN, GEN_THREADS, s2);
@@ -3941,6 +4206,7 @@ template <int S> struct BatchStep {
     static void bulk(const BatchLaunch &b, cudaStream_t st) { batch_bulk_launch<S>(b, st); }
     static int bulk_blocks_per_sm() {
         int nb = 0;
+        if (S == 2) return RING_CTAS;
         if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k_batch<BkLiquid<S, 4>>, BULK_THREADS, 0) != cudaSuccess)
             return 1;
         return nb > 0 ? nb : 1;
