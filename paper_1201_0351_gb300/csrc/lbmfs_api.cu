@@ -68,6 +68,7 @@ cudaError_t Sides::create() {
         if (e == cudaSuccess) e = cudaEventCreateWithFlags(&join[k], cudaEventDisableTiming);
     }
     if (e == cudaSuccess) e = cudaEventCreateWithFlags(&fork, cudaEventDisableTiming);
+    if (e == cudaSuccess) e = cudaEventCreateWithFlags(&fork2, cudaEventDisableTiming);
     return e;
 }
 void Sides::destroy() {
@@ -78,7 +79,8 @@ void Sides::destroy() {
         join[k] = nullptr;
     }
     if (fork) cudaEventDestroy(fork);
-    fork = nullptr;
+    if (fork2) cudaEventDestroy(fork2);
+    fork = fork2 = nullptr;
 }
 
 void begin_mass(lbm_fs *h) {

@@ -163,7 +163,7 @@ constexpr int RING_TILE = 512, RING_CTAS = 2;
 constexpr int SIDE_STREAMS = 3;
 struct Sides {
     cudaStream_t st[SIDE_STREAMS] = {};
-    cudaEvent_t fork = nullptr, join[SIDE_STREAMS] = {};
+    cudaEvent_t fork = nullptr, fork2 = nullptr, join[SIDE_STREAMS] = {};
     cudaError_t create();
     void destroy();
 };

@@ -71,7 +71,7 @@ __host__ __device__ __forceinline__ constexpr float wf(int q) {
 #define LBMFS_BULK_PIPE_ZB 16  // z-planes per block of the software-pipelined bulk kernel
 #endif
 #ifndef LBMFS_FORCE_MINB
-#define LBMFS_FORCE_MINB 6  // resident blocks per SM of the float-storage force kernel (80 registers)
+#define LBMFS_FORCE_MINB 6  // resident 128-thread blocks per SM of the float-storage force kernel (80 registers)
 #endif
 #ifndef LBMFS_IFACE_MINB
 #define LBMFS_IFACE_MINB 6  // resident blocks per SM asked of ptxas for the interface kernel (80 registers)
@@ -248,6 +248,13 @@ template <> struct Sto<2> {
 };
 
 // ---------------------------------------------------------------- helpers
+
+// Programmatic launch: lets a kernel that was launched as this one's dependent
+// begin once all of this launch's blocks have got here.  The bulk kernel is
+// launched so behind the force kernel, which it does not depend on: the force
+// kernel's few blocks, the first of a chain of short kernels, then get their
+// SMs before the bulk kernel's blocks fill the GPU.
+__device__ __forceinline__ void launch_dependents() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 
 __device__ __forceinline__ unsigned smem_addr(const void *p) { return (unsigned)__cvta_generic_to_shared(p); }
 // order earlier generic-proxy accesses to shared memory before the async-proxy
@@ -972,7 +979,11 @@ __device__ __forceinline__ void list_span(const VB &vb, uint32_t n, uint32_t per
 // it wants into shared memory, then works on them with full warps
 // (`work(x, y, z, i)`).
 constexpr uint32_t CHUNK = 1024;
-constexpr int FORCE_THREADS = 128;
+// The force kernel's blocks: on a single tank one thread per cell of a group (a
+// block's group may lie wholly in a face of the body: 128^3 heeled box 34 us
+// with 128 threads, 24 with 256); in a batch, where most of a group's cells are
+// passed over, smaller ones so that more groups are resident.
+constexpr int FORCE_THREADS = 256, FORCE_THREADS_BATCH = 128;
 template <uint32_t G, class Want, class Work>
 __device__ __forceinline__ void walk_near(const Dev &d, const int *lo, const int *hi, uint32_t ncell, const VB &vb,
                                           uint32_t blocks, Want want, Work work) {
@@ -1085,37 +1096,33 @@ __global__ void k_nb_body(Dev d, int bi) {
     }
 }
 
-// cells whose obstacle status changed this step (covered, uncovered): refresh
-// the bit of each and of its 18 neighbours
-__device__ __forceinline__ void nb_refresh_around(const Dev &d, long long i) {
-    int x, y, z;
-    coords(d, i, x, y, z);
-    nb_refresh(d, i);
-#pragma unroll 1
-    for (int q = 1; q < Q; ++q) {
-        long long yi = nbr(d, x, y, z, cx(q), cy(q), cz(q));
-        if (yi >= 0) nb_refresh(d, yi);
-    }
+// the calling lane's neighbour of (x, y, z): direction = lane; -1 beyond a wall
+// and for the lanes without a direction
+__device__ __forceinline__ long long lane_nbr(const Dev &d, int lane, int x, int y, int z) {
+    return lane >= 1 && lane < Q ? nbr(d, x, y, z, dir_x(lane), dir_y(lane), dir_z(lane)) : -1;
 }
-
-// one thread per (listed cell, direction): the cell itself (q = 0) or its
-// neighbour in direction q; cells refreshed twice get the same value (the
-// classes do not change in this kernel)
+// Cells whose obstacle status changed this step (covered, uncovered): the bit
+// of each and of its 18 neighbours is refreshed.
+// A warp per (listed cell, direction): the target is the cell itself (q = 0) or
+// its neighbour in direction q, lane p looks at the target's neighbour p.
+// Targets refreshed twice get the same value (the classes do not change in this
+// kernel).
 __device__ __forceinline__ void nb_update_body(const Dev &d, const VB &vb) {
-    const uint32_t nc = wl_count(d, WL_COVER), np = wl_count(d, WL_PEND);
-    const unsigned long long n = (unsigned long long)(nc + np) * Q;
-    for (unsigned long long it = (unsigned long long)vb.x * blockDim.x + threadIdx.x; it < n;
-         it += (unsigned long long)vb.nx * blockDim.x) {
-        const uint32_t e = (uint32_t)(it / Q);
-        const int q = (int)(it % Q);
+    const uint32_t nc = wl_count(d, WL_COVER), n = (nc + wl_count(d, WL_PEND)) * Q;
+    const int lane = threadIdx.x & 31;
+    for (uint32_t it = (threadIdx.x >> 5) * vb.nx + vb.x; it < n; it += vb.nx * (blockDim.x >> 5)) {
+        const uint32_t e = it / Q;
+        const int q = (int)(it - e * Q);
         const long long c = e < nc ? (long long)d.list[WL_COVER][e] : (long long)d.list[WL_PEND][e - nc];
-        long long t = c;
-        if (q > 0) {
-            int x, y, z;
-            coords(d, c, x, y, z);
-            t = nbr(d, x, y, z, cx(q), cy(q), cz(q));
-        }
-        if (t >= 0) nb_refresh(d, t);
+        int x, y, z;
+        coords(d, c, x, y, z);
+        const long long t = q > 0 ? nbr(d, x, y, z, dir_x(q), dir_y(q), dir_z(q)) : c;
+        if (t < 0) continue;
+        coords(d, t, x, y, z);
+        const bool obst = cls(d, lane_nbr(d, lane, x, y, z)) == CL_O;
+        const bool nb = __any_sync(0xffffffffu, obst);
+        if (lane == 0) d.flags[t] = (uint8_t)((d.flags[t] & ~NB_OBST) | (nb ? NB_OBST : 0));
+        __syncwarp();
     }
 }
 __global__ void k_nb_update(const __grid_constant__ Dev d) { nb_update_body(d, vb_own()); }
@@ -1266,7 +1273,7 @@ __device__ __forceinline__ void forces_f64_body(const Dev &d, const VB &vb) {
     __syncthreads();
     if (tid < 7) {
         unsigned __int128 v = 0;
-        for (int w = 0; w < FORCE_THREADS / 32; ++w) v += sh[w][tid];
+        for (int w = 0; w < (int)(blockDim.x >> 5); ++w) v += sh[w][tid];
         unsigned long long *p = reinterpret_cast<unsigned long long *>(d.part) +
                                 2 * (((long long)bi * FORCE_BLOCKS + vb.x) * 7 + tid);
         p[0] = (unsigned long long)v;
@@ -1473,7 +1480,8 @@ __device__ __forceinline__ void forces_body(const Dev &d, const VB &vb) {
 }
 
 template <int S>
-__global__ void __launch_bounds__(FORCE_THREADS, S == 0 ? 4 : LBMFS_FORCE_MINB) k_forces(const __grid_constant__ Dev d) {
+__global__ void __launch_bounds__(FORCE_THREADS, S == 0 ? 2 : LBMFS_FORCE_MINB / 2) k_forces(const __grid_constant__ Dev d) {
+    launch_dependents();
     forces_body<S, false>(d, vb_own());
 }
 
@@ -3060,15 +3068,13 @@ __global__ void __launch_bounds__(128, S == 0 ? 2 : LBMFS_IFACE_MINB) k_interfac
 // flight together (one thread per cell issued its atomics one after another),
 // and the cells a warp marks are appended with one reservation.  The warps of
 // a short list go to different SMs.
-#define WARP_LOOP(L, var)                                                                                      \
-    const uint32_t n_##var = wl_count(d, L);                                                                   \
-    for (uint32_t it_##var = (threadIdx.x >> 5) * vb.nx + vb.x; it_##var < n_##var; it_##var += vb.nx * (blockDim.x >> 5))
+// (`skip` items of other lists that the same phase works on come first: the
+// lists share the warps instead of all starting at the first one)
+#define WARP_LOOP(L, var, skip)                                                                                \
+    const uint32_t n_##var = wl_count(d, L), w_##var = vb.nx * (blockDim.x >> 5), s_##var = (skip) % w_##var;   \
+    for (uint32_t it_##var = ((threadIdx.x >> 5) * vb.nx + vb.x + w_##var - s_##var) % w_##var; it_##var < n_##var; \
+         it_##var += w_##var)
 
-// the calling lane's neighbour of (x, y, z): direction = lane; -1 beyond a wall
-// and for the lanes without a direction
-__device__ __forceinline__ long long lane_nbr(const Dev &d, int lane, int x, int y, int z) {
-    return lane >= 1 && lane < Q ? nbr(d, x, y, z, dir_x(lane), dir_y(lane), dir_z(lane)) : -1;
-}
 // set mark `bit` on the lanes' cells (want) and append those newly marked
 __device__ __forceinline__ void mark_append(const Dev &d, bool want, long long yi, uint8_t bit, int list) {
     const bool nw = want && !(mark_or(d, yi, bit) & bit);
@@ -3079,7 +3085,7 @@ __device__ __forceinline__ void mark_append(const Dev &d, bool want, long long y
 // gas neighbours of filled cells become interface
 __device__ __forceinline__ void conv_filled_body(const Dev &d, const VB &vb) {
     const int lane = threadIdx.x & 31;
-    WARP_LOOP(WL_FILLED, a) {
+    WARP_LOOP(WL_FILLED, a, 0u) {
         int x, y, z;
         coords(d, d.list[WL_FILLED][it_a], x, y, z);
         const long long yi = lane_nbr(d, lane, x, y, z);
@@ -3092,7 +3098,7 @@ __global__ void k_conv_filled(const __grid_constant__ Dev d) { conv_filled_body(
 // become interface
 __device__ __forceinline__ void conv_emptied_body(const Dev &d, const VB &vb) {
     const int lane = threadIdx.x & 31;
-    WARP_LOOP(WL_EMPTIED, a) {
+    WARP_LOOP(WL_EMPTIED, a, wl_count(d, WL_FILLED)) {
         const long long i = d.list[WL_EMPTIED][it_a];
         int x, y, z;
         coords(d, i, x, y, z);
@@ -3156,10 +3162,8 @@ __device__ __forceinline__ void conv_init_body(const Dev &d, const VB &vb) {
         // populations in flight together), the sums are taken in q order
         // from the gathered values, lane q evaluates f_eq,q
         const int lane = threadIdx.x & 31;
-        const unsigned wpb = blockDim.x >> 5;
-        const uint32_t n = wl_count(d, WL_NEWG);
-        for (uint32_t w = vb.x * wpb + (threadIdx.x >> 5); w < n; w += vb.nx * wpb) {
-            const long long i = d.list[WL_NEWG][w];
+        WARP_LOOP(WL_NEWG, w, 0u) {
+            const long long i = d.list[WL_NEWG][it_w];
             int x, y, z;
             coords(d, i, x, y, z);
             if (lane == 0 && z > *d.ztop_wr + ZTOP_MARGIN) atomicOr(d.status, ST_TOP);
@@ -3253,10 +3257,10 @@ template <int S>
 __device__ __forceinline__ void conv_claim_body(const Dev &d, const VB &vb) {
     const int lane = threadIdx.x & 31;
     {
-        WARP_LOOP(WL_FILLED, a) claim_receivers<S>(d, lane, d.list[WL_FILLED][it_a], MK_FILLED);
+        WARP_LOOP(WL_FILLED, a, wl_count(d, WL_NEWG)) claim_receivers<S>(d, lane, d.list[WL_FILLED][it_a], MK_FILLED);
     }
     {
-        WARP_LOOP(WL_EMPTIED, b) {
+        WARP_LOOP(WL_EMPTIED, b, wl_count(d, WL_NEWG) + wl_count(d, WL_FILLED)) {
             const long long i = d.list[WL_EMPTIED][it_b];
             const uint8_t mk = d.cmark[i];
             if (mk & MK_EMPTIED) claim_receivers<S>(d, lane, i, mk);
@@ -3266,16 +3270,41 @@ __device__ __forceinline__ void conv_claim_body(const Dev &d, const VB &vb) {
 template <int S>
 __global__ void k_conv_claim(const __grid_constant__ Dev d) { conv_claim_body<S>(d, vb_own()); }
 
-// receivers gather e(x) / k(x) over their converted neighbours in q order
-// (the receivers are many: a thread each, its loads requested at once)
+// Receivers gather e(x) / k(x) over their converted neighbours in q order: the
+// neighbours' marks, then the converted ones' shares (computed when the
+// receivers were claimed).  A warp per receiver with a lane per neighbour while
+// there are warps for it (a thread's thousand instructions for its 18
+// neighbours, at the rate of a lone warp, took 10 us for a single receiver); a
+// thread each for the long lists of large tanks.
+template <int S> __device__ __forceinline__ void set_mass(const Dev &d, long long i, double m, double rho) {
+    d.m[i] = m;
+    const double ph = m / rho;
+    d.phidst[i] = ph;
+    if constexpr (S != 0) d.phifdst[i] = (float)ph;
+}
 template <int S>
 __device__ __forceinline__ void conv_excess_body(const Dev &d, const VB &vb) {
+    if (wl_count(d, WL_RECV) <= 2u * vb.nx * (blockDim.x >> 5)) {
+        const int lane = threadIdx.x & 31;
+        WARP_LOOP(WL_RECV, w, 0u) {
+            const long long i = d.list[WL_RECV][it_w];
+            int x, y, z;
+            coords(d, i, x, y, z);
+            const long long yi = lane_nbr(d, lane, x, y, z);
+            const bool conv = yi >= 0 && (d.cmark[yi] & (MK_FILLED | MK_EMPTIED));
+            const double share = conv ? d.m[yi] : 0.0, m = d.m[i], rho = warp_density<S>(d, d.fdst, i);
+            double acc = 0.0;
+            for (unsigned b = __ballot_sync(0xffffffffu, conv); b; b &= b - 1)
+                acc += __shfl_sync(0xffffffffu, share, __ffs(b) - 1);
+            if (lane == 0) set_mass<S>(d, i, m + acc, rho);
+            __syncwarp();
+        }
+        return;
+    }
     LIST_LOOP(WL_RECV, a) {
         long long i = d.list[WL_RECV][it_a];
         int x, y, z;
         coords(d, i, x, y, z);
-        // the neighbours' marks, then the converted ones' shares e(y) / k(y)
-        // (computed when the receivers were claimed), summed in q order
         unsigned cm = 0;
 #pragma unroll
         for (int q = 1; q < Q; ++q) {
@@ -3283,16 +3312,12 @@ __device__ __forceinline__ void conv_excess_body(const Dev &d, const VB &vb) {
             if (yi >= 0 && (d.cmark[yi] & (MK_FILLED | MK_EMPTIED))) cm |= 1u << q;
         }
         const double rho = cell_density<S>(d, d.fdst, i);
-        double m = d.m[i], acc = 0.0;
+        double acc = 0.0;
         for (unsigned b = cm; b; b &= b - 1) {
             const int q = __ffs(b) - 1;
             acc += d.m[nbr(d, x, y, z, dir_x(q), dir_y(q), dir_z(q))];
         }
-        m = m + acc;
-        d.m[i] = m;
-        const double ph = m / rho;
-        d.phidst[i] = ph;
-        if constexpr (S != 0) d.phifdst[i] = (float)ph;
+        set_mass<S>(d, i, d.m[i] + acc, rho);
     }
 }
 template <int S>
@@ -3540,40 +3565,48 @@ __device__ __forceinline__ void remap_scan_body(const Dev &d, const VB &vb) {
     const int bi = vb.y;
     const Body &b = d.bodies_new[bi];
     const uint32_t lane = threadIdx.x & 31u;
+    // one pass over the cells of both poses' ranges (they differ by a cell or
+    // two; across a periodic seam the old one is shifted to the new)
+    const int n3[3] = {d.nx, d.ny, d.nz};
+    int lo[3], hi[3];
+#pragma unroll
+    for (int k = 0; k < 3; ++k) {
+        int shift = 0;
+        if (d.periodic & (1u << k)) shift = b.plo[k] - b.lo[k] > n3[k] / 2 ? -n3[k] : (b.lo[k] - b.plo[k] > n3[k] / 2 ? n3[k] : 0);
+        // (an empty range, of a body that has left the grid, adds nothing)
+        const bool now = b.hi[k] > b.lo[k], was = b.phi[k] > b.plo[k];
+        lo[k] = now && was ? min(b.lo[k], b.plo[k] + shift) : (now ? b.lo[k] : b.plo[k]);
+        hi[k] = now && was ? max(b.hi[k], b.phi[k] + shift) : (now ? b.hi[k] : b.phi[k]);
+        if ((d.periodic & (1u << k)) && hi[k] - lo[k] > n3[k]) hi[k] = lo[k] + n3[k];
+        if (hi[k] < lo[k]) hi[k] = lo[k];
+    }
+    const uint32_t n = (uint32_t)range_count(lo, hi);
     uint32_t first, stride;
-    const uint32_t n = (uint32_t)range_count(b.lo, b.hi);
     list_span(vb, n, 32u, first, stride);
     for (uint32_t k0 = first; k0 < n; k0 += stride) {
         const uint32_t kk = k0 + lane;
         long long i = 0;
-        bool cover = false;
+        bool cover = false, pend = false;
         if (kk < n) {
             int x, y, z;
-            range_cell(d, b.lo, b.hi, kk, x, y, z);
+            range_cell(d, lo, hi, kk, x, y, z);
             i = x + (long long)d.nx * (y + (long long)d.ny * z);
-            cover = clsv(d, i) != CL_O && inside(d, b, x, y, z);
+            const bool solid = clsv(d, i) == CL_O, own = solid && d.bid[i] == bi;
+            if (!solid || own) {
+                const bool in = inside(d, b, x, y, z);
+                cover = !solid && in;
+                pend = own && !in;
+            }
         }
         if (__any_sync(0xffffffffu, cover)) wl_append(d, cover, WL_COVER, (uint32_t)i);
         // the covering body, for remap_apply_body (an obstacle's id is set
         // there; until then nothing reads a fluid cell's id)
         if (cover) d.bid[i] = (uint8_t)bi;
-    }
-    const uint32_t m = (uint32_t)range_count(b.plo, b.phi);
-    list_span(vb, m, 32u, first, stride);
-    for (uint32_t k0 = first; k0 < m; k0 += stride) {
-        const uint32_t kk = k0 + lane;
-        long long i = 0;
-        bool pend = false;
-        if (kk < m) {
-            int x, y, z;
-            range_cell(d, b.plo, b.phi, kk, x, y, z);
-            i = x + (long long)d.nx * (y + (long long)d.ny * z);
-            pend = clsv(d, i) == CL_O && d.bid[i] == bi && !inside(d, b, x, y, z);
-        }
         if (__any_sync(0xffffffffu, pend)) wl_append(d, pend, WL_PEND, (uint32_t)i);
     }
 }
-__global__ void k_remap_scan(const __grid_constant__ Dev d) { remap_scan_body(d, vb_own()); }
+constexpr int SCAN_THREADS = 64;
+__global__ void __launch_bounds__(SCAN_THREADS) k_remap_scan(const __grid_constant__ Dev d) { remap_scan_body(d, vb_own()); }
 
 // listed cells inside a body's new pose become obstacle, their mass is booked;
 // listed obstacle cells outside it are pending
@@ -3615,14 +3648,16 @@ __device__ __forceinline__ void remap_resolve_body(const Dev &d, const VB &vb) {
             int x, y, z;
             coords(d, i, x, y, z);
             const long long yi = lane_nbr(d, lane, x, y, z);
-            const int c = (yi < 0 || (d.cmark[yi] & MK_PEND)) ? 0 : clsv(d, yi);
+            // mark, class, density and fill level of the neighbour requested
+            // together (those of a cell without populations are not used)
+            const int mk = yi < 0 ? MK_PEND : d.cmark[yi], cl = cls(d, yi), c = (mk & MK_PEND) ? 0 : cl;
+            double r = 0.0, ph = 0.0;
+            if (cl == CL_L || cl == CL_I) r = cell_density<S>(d, d.fdst, yi);
+            if (cl == CL_I) ph = d.phidst[yi];
             const unsigned full = 0xffffffffu;
             const unsigned mL = __ballot_sync(full, c == CL_L), mI = __ballot_sync(full, c == CL_I),
                            mG = __ballot_sync(full, c == CL_G);
             const int nL = __popc(mL), nI = __popc(mI), nG = __popc(mG);
-            double r = 0.0, ph = 0.0;
-            if (c == CL_L || c == CL_I) r = cell_density<S>(d, d.fdst, yi);
-            if (c == CL_I) ph = d.phidst[yi];
             // sums in q order
             double sr = 0.0, sp = 0.0;
             for (unsigned m = mL | mI; m; m &= m - 1) sr += __shfl_sync(full, r, __ffs(m) - 1);
@@ -3670,15 +3705,10 @@ __device__ __forceinline__ void remap_resolve_body(const Dev &d, const VB &vb) {
             const double rho = d.rrho[it];
             warp_store_cell<S>(d, i, lane, feq_lane(lane, rho, uw));
             __syncwarp();
-            if (dec == CL_I) {
-                const double dens = warp_density<S>(d, d.fdst, i);
-                if (lane == 0) {
-                    const double m = d.rphi[it] * rho;
-                    d.m[i] = m;
-                    const double ph = m / dens;
-                    d.phidst[i] = ph;
-                    if constexpr (S != 0) d.phifdst[i] = (float)ph;
-                }
+            const double dens = warp_density<S>(d, d.fdst, i);
+            if (lane == 0) {
+                if (dec == CL_I) set_mass<S>(d, i, d.rphi[it] * rho, dens);
+                d.rrho[it] = dens;  // as stored, for what follows
             }
         }
         __syncthreads();
@@ -3702,7 +3732,7 @@ __device__ __forceinline__ void remap_resolve_body(const Dev &d, const VB &vb) {
         if (!(d.cmark[i] & MK_FRESH)) continue;
         const int c = clsv(d, i);
         if (c == CL_L) {
-            const double r = cell_density<S>(d, d.fdst, i);
+            const double r = d.rrho[it];
             acc += r;
             if (d.rdec[it]) {
                 set_cls(d, i, CL_I);
@@ -3715,7 +3745,7 @@ __device__ __forceinline__ void remap_resolve_body(const Dev &d, const VB &vb) {
         }
         d.cmark[i] = 0;
     }
-    __shared__ double sh[REMAP_THREADS / 32];
+    __shared__ double sh[32];
     for (int off = 16; off > 0; off >>= 1) acc += __shfl_down_sync(0xffffffffu, acc, off);
     if ((threadIdx.x & 31) == 0) sh[threadIdx.x >> 5] = acc;
     __syncthreads();
@@ -3740,7 +3770,10 @@ __global__ void __launch_bounds__(REMAP_THREADS) k_remap_resolve(const __grid_co
 //    barrier, for tanks whose lists are short;
 //  - else a cooperative grid with a barrier in global memory, for large tanks
 //    (hundreds to thousands of conversions a step want all SMs).
-constexpr int TAIL_THREADS = REMAP_THREADS, TAIL_CLUSTER = 8, TAIL_BLOCKS = 152;
+constexpr int TAIL_CLUSTER = 8, TAIL_BLOCKS = 152;
+// (1024 threads of the cluster's blocks give its short lists a warp each; on the
+// grid they only make the block barriers longer: 768x384x256 103 us against 89)
+constexpr int tail_threads(bool cluster) { return cluster ? 1024 : 512; }
 
 // one warp-wide poll limit for the grid barrier: far beyond the time that the
 // resident blocks of a cooperative launch can be apart
@@ -3782,7 +3815,7 @@ template <bool CLUSTER> __device__ __forceinline__ bool tail_barrier(const Dev &
 }
 
 template <int S, bool CLUSTER>
-__global__ void __launch_bounds__(TAIL_THREADS) k_tail(const __grid_constant__ Dev d) {
+__global__ void __launch_bounds__(tail_threads(CLUSTER)) k_tail(const __grid_constant__ Dev d) {
     const VB vb = vb_own();
     if (vb.x == 0) {
         // for the next step: its counters (this step's previous ones), and the
@@ -3823,14 +3856,26 @@ template <int S>
 __global__ void __launch_bounds__(256) k_mass_partial(Dev d) {
     double acc = 0.0;
     for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < d.N; i += (long long)gridDim.x * blockDim.x) {
-        int c = clsv(d, i);
+        const int fb = d.flags[i], c = fb & CL_MASK;
         if (c == CL_L) {
+            // closed interface layer (Sec. 2.2): no liquid cell touches gas; the
+            // neighbours' classes are requested with the populations, off the
+            // grid faces by constant index offsets
+            bool gas = false;
+            if (fb & (FACE_X | FACE_YZ)) {
+                int x, y, z;
+                coords(d, i, x, y, z);
+#pragma unroll 1
+                for (int q = 1; q < Q; ++q) gas = gas || cls(d, nbr(d, x, y, z, dir_x(q), dir_y(q), dir_z(q))) == CL_G;
+            } else {
+                const long long sy = d.nx, sz = (long long)d.nx * d.ny;
+                unsigned any = 0;
+#pragma unroll
+                for (int q = 1; q < Q; ++q) any |= d.flags[i + (cx(q) + cy(q) * sy + cz(q) * sz)];
+                gas = any & CL_G;
+            }
             acc += cell_density<S>(d, d.fsrc, i);
-            // closed interface layer (Sec. 2.2): no liquid cell touches gas
-            int x, y, z;
-            coords(d, i, x, y, z);
-            for (int q = 1; q < Q; ++q)
-                if (cls(d, nbr(d, x, y, z, cx(q), cy(q), cz(q))) == CL_G) atomicOr(d.status, ST_LIQUID_GAS);
+            if (gas) atomicOr(d.status, ST_LIQUID_GAS);
         } else if (c == CL_I) {
             acc += d.m[i];
         }
@@ -3847,10 +3892,12 @@ __global__ void __launch_bounds__(256) k_mass_partial(Dev d) {
 }
 
 __global__ void k_mass_final(Dev d, int nblk) {
-    if (threadIdx.x != 0) return;
+    // one warp, in a fixed order (a double addition takes 65 cycles: one thread's
+    // chain over all blocks took 10 us)
     double t = 0.0;
-    for (int k = 0; k < nblk; ++k) t += d.red[k];
-    d.ledger[LG_MASS] = t;
+    for (int k = threadIdx.x; k < nblk; k += 32) t += d.red[k];
+    for (int off = 16; off > 0; off >>= 1) t += __shfl_down_sync(0xffffffffu, t, off);
+    if (threadIdx.x == 0) d.ledger[LG_MASS] = t;
 }
 
 template <int S>
@@ -3887,6 +3934,7 @@ __global__ void k_read_fields(Dev d, unsigned mask, uint8_t *flags, double *fill
 template <class K>
 __global__ void __launch_bounds__(K::THREADS, K::MINB)
     k_batch(const __grid_constant__ TankSet ts, const Tile *__restrict__ table, unsigned n, int zb) {
+    launch_dependents();  // (only the bulk kernel is launched so, behind the force kernel)
     for (unsigned t = blockIdx.x; t < n; t += gridDim.x) {
         const Tile e = table[t];
         const VB vb{e.x, e.y, e.z, e.nx, e.ny, e.nz, e.kind};
@@ -3911,7 +3959,7 @@ struct BkReset {
         if (threadIdx.x < CN_COUNT) d.cnt[threadIdx.x] = 0;
     }
 };
-template <int S> LBMFS_BATCH_BODY_SM(BkForces, FORCE_THREADS, S == 0 ? 4 : LBMFS_FORCE_MINB, true, forces_body<S, true>(d, vb))
+template <int S> LBMFS_BATCH_BODY_SM(BkForces, FORCE_THREADS_BATCH, S == 0 ? 4 : LBMFS_FORCE_MINB, true, forces_body<S, true>(d, vb))
 // one instantiation per z-planes-per-tile choice (the column loop unrolled to it)
 template <int S, int ZB>
 LBMFS_BATCH_BODY(BkLiquid, BULK_THREADS, S == 0 ? 1 : LBMFS_BULK_MINB, (liquid_body<S, ZB>(d, vb, zb)))
@@ -3930,7 +3978,7 @@ template <int S> LBMFS_BATCH_BODY(BkConvClaim, LIST_THREADS, 1, conv_claim_body<
 template <int S> LBMFS_BATCH_BODY(BkConvExcess, LIST_THREADS, 1, conv_excess_body<S>(d, vb))
 LBMFS_BATCH_BODY(BkConvFinish, LIST_THREADS, 1, conv_finish_body(d, vb))
 LBMFS_BATCH_BODY(BkBodies, 32, 1, bodies_body(d, vb))
-LBMFS_BATCH_BODY(BkRemapScan, 256, 1, remap_scan_body(d, vb))
+LBMFS_BATCH_BODY(BkRemapScan, SCAN_THREADS, 1, remap_scan_body(d, vb))
 template <int S> LBMFS_BATCH_BODY(BkRemapApply, LIST_THREADS, 1, remap_apply_body<S>(d, vb))
 template <int S> LBMFS_BATCH_BODY_SM(BkRemapResolve, REMAP_THREADS, 1, true, remap_resolve_body<S>(d, vb))
 LBMFS_BATCH_BODY(BkNbUpdate, LIST_THREADS, 1, nb_update_body(d, vb))
@@ -3941,25 +3989,6 @@ template <class K> void batch_launch(const BatchLaunch &b, int sh, dim3 block, c
     const Shape &x = b.sh[sh];
     if (x.n) k_batch<K><<<x.grid, block, 0, st>>>(*b.ts, x.table, x.n, b.zb);
 }
-template <int S> void batch_bulk_launch(const BatchLaunch &b, cudaStream_t st) {
-    if constexpr (S == 2) {
-        const Shape &x = b.sh[SH_BULK];
-        if (!x.n) return;
-        auto go = [&](void (*k)(TankSet, const Tile *, unsigned)) {
-            cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, RingShape::SMEM);
-            k<<<x.grid, RingShape::THREADS, RingShape::SMEM, st>>>(*b.ts, x.table, x.n);
-        };
-        go(b.zg ? k_batch_ring<true> : k_batch_ring<false>);
-        return;
-    }
-    switch (b.zb) {
-    case 1: batch_launch<BkLiquid<S, 1>>(b, SH_BULK, BULK_THREADS, st); break;
-    case 2: batch_launch<BkLiquid<S, 2>>(b, SH_BULK, BULK_THREADS, st); break;
-    case 4: batch_launch<BkLiquid<S, 4>>(b, SH_BULK, BULK_THREADS, st); break;
-    default: batch_launch<BkLiquid<S, 8>>(b, SH_BULK, BULK_THREADS, st); break;
-    }
-}
-
 // z-planes per block of the single-tank bulk kernel.  A thread steps its planes
 // one after another, so blocks of 8 planes suit only grids whose blocks still
 // fill the GPU several times over; on smaller ones a few threads would walk 8
@@ -4010,20 +4039,6 @@ template <int S> struct Launch {
             (mask & 4u) ? (double *)dst[2] : nullptr, (mask & 8u) ? (double *)dst[3] : nullptr,
             (mask & 16u) ? (double *)dst[4] : nullptr, (mask & 32u) ? (double *)dst[5] : nullptr);
     }
-    template <int ZB> static void bulk_zb(const Dev &d, unsigned gx, cudaStream_t st) {
-        k_liquid<S, ZB><<<dim3(gx, 1, (d.nz + ZB - 1) / ZB), BULK_THREADS, 0, st>>>(d);
-    }
-    // the bulk kernel with the z-planes per block of bulk_planes
-    static void bulk(const Dev &d, cudaStream_t st) {
-        const unsigned gx = (unsigned)(((long long)d.nx * d.ny + BULK_THREADS - 1) / BULK_THREADS);
-        const int zb = bulk_planes(S, gx, d.nz);
-        if (zb == 1) bulk_zb<1>(d, gx, st);
-        if constexpr (S != 0) {
-            if (zb == 2) bulk_zb<2>(d, gx, st);
-            if (zb == 4) bulk_zb<4>(d, gx, st);
-            if (zb == 8) bulk_zb<8>(d, gx, st);
-        }
-    }
     static void faces(const Dev &d, cudaStream_t st) { k_faces<S><<<LIST_BLOCKS, GEN_THREADS, 0, st>>>(d); }
     static void near(const Dev &d, cudaStream_t st) {
         k_near<S><<<dim3(FORCE_BLOCKS, d.nb), GEN_THREADS, 0, st>>>(d);
@@ -4031,48 +4046,78 @@ template <int S> struct Launch {
     static void forces(const Dev &d, cudaStream_t st) {
         k_forces<S><<<dim3(FORCE_BLOCKS, d.nb), FORCE_THREADS, 0, st>>>(d);
     }
-    static void scan(const Dev &d, cudaStream_t st) { k_remap_scan<<<dim3(FORCE_BLOCKS, d.nb), 256, 0, st>>>(d); }
+    static void scan(const Dev &d, cudaStream_t st) { 
+        // a cell or two per thread; blocks small enough to run beside the ring
+        // kernel's, which leave 4096 registers of an SM
+        k_remap_scan<<<dim3(std::max(FORCE_BLOCKS, 1216 / d.nb), d.nb), SCAN_THREADS, 0, st>>>(d);
+    }
     static void interface(const Dev &d, cudaStream_t st) { k_interface<S><<<LBMFS_IFACE_GRID, 128, 0, st>>>(d); }
-    static void bulk_any(const Dev &d, cudaStream_t st) {
+    // launch k, with `early` as a programmatic dependent of the stream's last
+    // kernel (see launch_dependents)
+    template <class... P, class... A>
+    static void launch(void (*k)(P...), dim3 grid, int block, size_t smem, cudaStream_t st, bool early, A... args) {
+        cudaLaunchConfig_t c = {};
+        cudaLaunchAttribute a = {};
+        c.gridDim = grid;
+        c.blockDim = dim3(block);
+        c.dynamicSmemBytes = smem;
+        c.stream = st;
+        a.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+        a.val.programmaticStreamSerializationAllowed = 1;
+        c.attrs = &a;
+        c.numAttrs = early ? 1 : 0;
+        cudaLaunchKernelEx(&c, k, P(args)...);
+    }
+    // the bulk kernel: FP64 and FP32 one cell per thread, with the z-planes per
+    // block of bulk_planes; FP16 the ring; LBMFS_BULK selects the staged forms
+    static void bulk_any(const Dev &d, cudaStream_t st, bool early) {
         if constexpr (S != 0) {
             // the staged variants tile rows: (ceil(nx / BULK_THREADS), ny, z-blocks)
             dim3 rgrid((d.nx + BULK_THREADS - 1) / BULK_THREADS, d.ny, (d.nz + LBMFS_BULK_ZB - 1) / LBMFS_BULK_ZB);
             dim3 pgrid(rgrid.x, rgrid.y, (d.nz + LBMFS_BULK_PIPE_ZB - 1) / LBMFS_BULK_PIPE_ZB);
-            if (d.bulk == BULK_TMA) k_liquid_tma<S><<<rgrid, BULK_THREADS, 128 + 2 * Stage<S>::BYTES, st>>>(d);
-            else if (d.bulk == BULK_PIPE) k_liquid_pipe<S><<<pgrid, BULK_THREADS, 0, st>>>(d);
-            else if (S == 2) ring(d, st);
-            else bulk(d, st);
-        } else {
-            bulk(d, st);
+            if (d.bulk == BULK_TMA) {
+                k_liquid_tma<S><<<rgrid, BULK_THREADS, 128 + 2 * Stage<S>::BYTES, st>>>(d);
+                return;
+            }
+            if (d.bulk == BULK_PIPE) {
+                k_liquid_pipe<S><<<pgrid, BULK_THREADS, 0, st>>>(d);
+                return;
+            }
         }
-    }
-    static void ring(const Dev &d, cudaStream_t st) {
         if constexpr (S == 2) {
             using G = RingShape;
             const uint32_t n = (uint32_t)((d.N + G::TILE - 1) / G::TILE);
-            const bool zg = d.a_f[0] == 0.0f && d.a_f[1] == 0.0f;
-            auto go = [&](void (*k)(Dev, uint32_t)) {
-                cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, G::SMEM);
-                k<<<std::min(n, 152u * RING_CTAS), G::THREADS, G::SMEM, st>>>(d, n);
-            };
-            go(zg ? k_ring<true> : k_ring<false>);
+            const auto k = d.a_f[0] == 0.0f && d.a_f[1] == 0.0f ? k_ring<true> : k_ring<false>;
+            cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, G::SMEM);
+            launch(k, dim3(std::min(n, 152u * RING_CTAS)), G::THREADS, G::SMEM, st, early, d, n);
+        } else {
+            const unsigned gx = (unsigned)(((long long)d.nx * d.ny + BULK_THREADS - 1) / BULK_THREADS);
+            const int zb = bulk_planes(S, gx, d.nz);
+            auto go = [&](void (*k)(Dev)) { launch(k, dim3(gx, 1, (d.nz + zb - 1) / zb), BULK_THREADS, 0, st, early, d); };
+            if (zb == 1) go(k_liquid<S, 1>);
+            if constexpr (S == 1) {
+                if (zb == 2) go(k_liquid<S, 2>);
+                if (zb == 4) go(k_liquid<S, 4>);
+                if (zb == 8) go(k_liquid<S, 8>);
+            }
         }
     }
     static void tail(const Dev &d, cudaStream_t st) {
         cudaLaunchConfig_t c = {};
         cudaLaunchAttribute a = {};
-        c.blockDim = dim3(TAIL_THREADS);
         c.stream = st;
         c.attrs = &a;
         c.numAttrs = 1;
         if ((long long)d.nx * d.ny <= TAIL_CLUSTER_CELLS) {
             c.gridDim = dim3(TAIL_CLUSTER);
+            c.blockDim = dim3(tail_threads(true));
             a.id = cudaLaunchAttributeClusterDimension;
             a.val.clusterDim.x = TAIL_CLUSTER;
             a.val.clusterDim.y = a.val.clusterDim.z = 1;
             cudaLaunchKernelEx(&c, k_tail<S, true>, d);
         } else {
             c.gridDim = dim3(TAIL_BLOCKS);
+            c.blockDim = dim3(tail_threads(false));
             a.id = cudaLaunchAttributeCooperative;
             a.val.cooperative = 1;
             cudaLaunchKernelEx(&c, k_tail<S, false>, d);
@@ -4082,7 +4127,9 @@ template <int S> struct Launch {
     // scan (a chain), the cells next to bodies or on moving walls, and the
     // interface cells need only the state at t: with `sides` (while a graph is
     // captured) these chains run beside the bulk kernel, on streams of a higher
-    // priority, and join before the tail.  Without, all run in one chain.  With
+    // priority, and join before the tail; the bulk kernel is launched behind the
+    // start of the force kernel, the first of the longest chain
+    // (launch_dependents).  Without, all run in one chain.  With
     // ev != nullptr event k is recorded before kernel slot k (step_names).
     static int step(const Dev &d, cudaStream_t st, const Sides *sides, cudaEvent_t *ev) {
         const bool bodies = d.nb > 0, walls = d.walls_move != 0;
@@ -4090,15 +4137,19 @@ template <int S> struct Launch {
         if (sides) {
             const bool used[SIDE_STREAMS] = {true, bodies, bodies || walls};
             cudaEventRecord(sides->fork, st);
-            for (int k = 0; k < SIDE_STREAMS; ++k)
+            for (int k = 0; k < SIDE_STREAMS; k += 2)
                 if (used[k]) cudaStreamWaitEvent(sides->st[k], sides->fork, 0);
-            if (bodies) forces(d, sides->st[1]);
+            if (bodies) {
+                forces(d, st);
+                cudaEventRecord(sides->fork2, st);
+                cudaStreamWaitEvent(sides->st[1], sides->fork2, 0);
+            }
             if (bodies) near(d, sides->st[2]);
             if (walls) faces(d, sides->st[2]);
             interface(d, sides->st[0]);
             if (bodies) launch_bodies(d, sides->st[1]);
             if (bodies) scan(d, sides->st[1]);
-            bulk_any(d, st);
+            bulk_any(d, st, bodies);  // (behind the force kernel's start)
             for (int k = 0; k < SIDE_STREAMS; ++k)
                 if (used[k]) {
                     cudaEventRecord(sides->join[k], sides->st[k]);
@@ -4115,7 +4166,7 @@ template <int S> struct Launch {
         mark();
         if (bodies) forces(d, st);
         mark();
-        bulk_any(d, st);
+        bulk_any(d, st, false);
         mark();
         if (bodies) near(d, st);
         if (walls) faces(d, st);
@@ -4132,6 +4183,25 @@ template <int S> struct Launch {
     }
 };
 
+// (early: behind the start of the stream's last kernel, see launch_dependents)
+template <int S> void batch_bulk_launch(const BatchLaunch &b, cudaStream_t st, bool early) {
+    const Shape &x = b.sh[SH_BULK];
+    if (!x.n) return;
+    if constexpr (S == 2) {
+        const auto k = b.zg ? k_batch_ring<true> : k_batch_ring<false>;
+        cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, RingShape::SMEM);
+        Launch<S>::launch(k, dim3(x.grid), RingShape::THREADS, RingShape::SMEM, st, early, *b.ts, x.table, x.n);
+    } else {
+        auto go = [&](void (*k)(TankSet, const Tile *, unsigned, int)) {
+            Launch<S>::launch(k, dim3(x.grid), BULK_THREADS, 0, st, early, *b.ts, x.table, x.n, b.zb);
+        };
+        if (b.zb == 1) go(k_batch<BkLiquid<S, 1>>);
+        else if (b.zb == 2) go(k_batch<BkLiquid<S, 2>>);
+        else if (b.zb == 4) go(k_batch<BkLiquid<S, 4>>);
+        else go(k_batch<BkLiquid<S, 8>>);
+    }
+}
+
 // The batched counterpart of Launch<S>::step (same kernel slots).
 template <int S> struct BatchStep {
     // (with sides: the chains that need only the state at t beside the bulk
@@ -4147,22 +4217,23 @@ template <int S> struct BatchStep {
         cudaStream_t s0 = st, s1 = st, s2 = st;
         if (sides) {
             cudaEventRecord(sides->fork, st);
-            for (int j = 0; j < SIDE_STREAMS; ++j) cudaStreamWaitEvent(sides->st[j], sides->fork, 0);
+            for (int j = 0; j < SIDE_STREAMS; j += 2) cudaStreamWaitEvent(sides->st[j], sides->fork, 0);
             s0 = sides->st[0];
             s1 = sides->st[1];
             s2 = sides->st[2];
         }
         mark();
-        batch_launch<BkForces<S>>(b, SH_FORCE, FORCE_THREADS, s1);
+        batch_launch<BkForces<S>>(b, SH_FORCE, FORCE_THREADS_BATCH, st);
         if (sides) {
-            // in the order in which they should get the SMs
+            cudaEventRecord(sides->fork2, st);
+            cudaStreamWaitEvent(s1, sides->fork2, 0);
             batch_launch<BkGeneral<S>>(b, SH_GEN, GEN_THREADS, s2);
             batch_launch<BkInterface<S>>(b, SH_IFACE, 128, s0);
             launch_bodies_batch(b, s1);
-            batch_launch<BkRemapScan>(b, SH_FORCE, 256, s1);
+            batch_launch<BkRemapScan>(b, SH_FORCE, SCAN_THREADS, s1);
         }
         mark();
-        batch_bulk_launch<S>(b, st);
+        batch_bulk_launch<S>(b, st, sides != nullptr && b.sh[SH_FORCE].n > 0);
         mark();
         if (!sides) batch_launch<BkGeneral<S>>(b, SH_GEN, GEN_THREADS, s2);
         mark();
@@ -4189,7 +4260,7 @@ template <int S> struct BatchStep {
         mark();
         if (!sides) launch_bodies_batch(b, st);
         mark();
-        if (!sides) batch_launch<BkRemapScan>(b, SH_FORCE, 256, st);
+        if (!sides) batch_launch<BkRemapScan>(b, SH_FORCE, SCAN_THREADS, st);
         mark();
         batch_launch<BkRemapApply<S>>(b, SH_LIST, LIST_THREADS, st);
         mark();
@@ -4203,7 +4274,7 @@ template <int S> struct BatchStep {
         for (int sh : shapes) n += b.sh[sh].n ? 1 : 0;
         return n;
     }
-    static void bulk(const BatchLaunch &b, cudaStream_t st) { batch_bulk_launch<S>(b, st); }
+    static void bulk(const BatchLaunch &b, cudaStream_t st) { batch_bulk_launch<S>(b, st, false); }
     static int bulk_blocks_per_sm() {
         int nb = 0;
         if (S == 2) return RING_CTAS;
