@@ -44,9 +44,10 @@ lbm_fs_status check_handle(lbm_fs *h) {
 #define CK LBMFS_CK
 
 lbm_fs_status read_status(lbm_fs *h) {
-    uint32_t st = 0;
-    CK(cudaMemcpyAsync(&st, h->d[0].status, sizeof st, cudaMemcpyDeviceToHost, h->st));
+    CK(cudaMemcpyAsync(h->pin + lbm_fs::PIN_STATUS, h->d[0].status, sizeof(uint32_t), cudaMemcpyDeviceToHost, h->st));
     CK(cudaStreamSynchronize(h->st));
+    uint32_t st;
+    memcpy(&st, h->pin + lbm_fs::PIN_STATUS, sizeof st);
     return status_bits(st);
 }
 
@@ -194,6 +195,7 @@ lbm_fs_status lbm_fs_create(const lbm_fs_params *p, lbm_fs **out) {
     };
     cudaError_t e = cudaStreamCreateWithFlags(&h->cap_st, cudaStreamNonBlocking);
     if (e == cudaSuccess && p->use_graphs) e = h->sides.create();
+    if (e == cudaSuccess) e = cudaHostAlloc((void **)&h->pin, lbm_fs::PIN_BYTES, cudaHostAllocDefault);
     if (e != cudaSuccess) return bail(cuda_fail(e, "cudaStreamCreate"));
 
     Dev d{};
@@ -443,19 +445,7 @@ lbm_fs_status lbm_fs_body_state(lbm_fs *h, int32_t id, lbm_fs_body_state_t *out)
     lbm_fs_status s = check_handle(h);
     if (s) return s;
     if (id < 0 || id >= h->nb || !out) return fail(LBM_FS_EINVAL, "bad body id%s");
-    CK(cudaStreamSynchronize(h->st));
-    Body hb;
-    CK(cudaMemcpy(&hb, h->d[h->cur].bodies + id, sizeof hb, cudaMemcpyDeviceToHost));
-    for (int k = 0; k < 3; ++k) {
-        out->F[k] = hb.F[k];
-        out->T[k] = hb.T[k];
-        out->center[k] = hb.o[k];
-        out->vel[k] = hb.v[k];
-        out->omega[k] = hb.w[k];
-    }
-    for (int k = 0; k < 4; ++k) out->quat[k] = hb.q[k];
-    out->S = hb.S;
-    return read_status(h);
+    return lbm_fs_body_states(h, id, 1, out);
 }
 
 lbm_fs_status lbm_fs_body_states(lbm_fs *h, int32_t first, int32_t count, lbm_fs_body_state_t *out) {
@@ -464,11 +454,17 @@ lbm_fs_status lbm_fs_body_states(lbm_fs *h, int32_t first, int32_t count, lbm_fs
     if (first < 0 || count < 0 || first + count > h->nb || (count > 0 && !out))
         return fail(LBM_FS_EINVAL, "bad body range%s");
     if (count == 0) return read_status(h);
-    std::vector<Body> hb(count);
-    uint32_t st = 0;  // the status word comes with the bodies: one synchronisation
-    CK(cudaMemcpyAsync(hb.data(), h->d[h->cur].bodies + first, sizeof(Body) * count, cudaMemcpyDeviceToHost, h->st));
-    CK(cudaMemcpyAsync(&st, h->d[0].status, sizeof st, cudaMemcpyDeviceToHost, h->st));
-    CK(cudaStreamSynchronize(h->st));
+    // the status word comes with the bodies: one synchronisation
+    const size_t bytes = sizeof(Body) * (size_t)count;
+    std::vector<Body> many;
+    Body *hb = reinterpret_cast<Body *>(h->pin + lbm_fs::PIN_DATA);
+    if (bytes > lbm_fs::PIN_BYTES - lbm_fs::PIN_DATA) {
+        many.resize(count);
+        hb = many.data();
+    }
+    CK(cudaMemcpyAsync(hb, h->d[h->cur].bodies + first, bytes, cudaMemcpyDeviceToHost, h->st));
+    const lbm_fs_status s1 = read_status(h);
+    if (s1 == LBM_FS_ECUDA || s1 == LBM_FS_ENOMEM) return s1;
     for (int32_t b = 0; b < count; ++b) {
         for (int k = 0; k < 3; ++k) {
             out[b].F[k] = hb[b].F[k];
@@ -480,7 +476,7 @@ lbm_fs_status lbm_fs_body_states(lbm_fs *h, int32_t first, int32_t count, lbm_fs
         for (int k = 0; k < 4; ++k) out[b].quat[k] = hb[b].q[k];
         out[b].S = hb[b].S;
     }
-    return status_bits(st);
+    return s1;
 }
 
 lbm_fs_status lbm_fs_forces(lbm_fs *h, int32_t id, double F[3], double T[3], double center[3], double quat[4]) {
@@ -527,6 +523,7 @@ lbm_fs_status lbm_fs_read_fields(lbm_fs *h, uint32_t mask, void *const *dst, int
     cudaError_t e = cudaGetLastError();
     for (int k = 0; k < 6 && e == cudaSuccess; ++k)
         if (!dst_on_device && (mask & (1u << k))) e = cudaMemcpyAsync(dst[k], ddst[k], sz[k], cudaMemcpyDeviceToHost, st);
+    if (e == cudaSuccess && tmp.empty()) return read_status(h);  // (waits for the fields too)
     if (e == cudaSuccess) e = cudaStreamSynchronize(st);
     for (void *t : tmp) cudaFree(t);
     if (e != cudaSuccess) return cuda_fail(e, "read_fields");
@@ -540,13 +537,18 @@ lbm_fs_status lbm_fs_stats(lbm_fs *h, lbm_fs_stats_t *out) {
     cudaStream_t st = h->st;
     h->ks.liquid_mass(h->d[h->cur], st);
     CK(cudaGetLastError());
-    CK(cudaStreamSynchronize(st));
     double lg[LG_COUNT];
     uint32_t cnt[CN_COUNT], status;
-    CK(cudaMemcpy(lg, h->d[0].ledger, sizeof lg, cudaMemcpyDeviceToHost));
-    memset(cnt, 0, sizeof cnt);
-    if (h->step > 0) CK(cudaMemcpy(cnt, h->d[h->cur ^ 1].cnt, sizeof cnt, cudaMemcpyDeviceToHost));  // of the last step
-    CK(cudaMemcpy(&status, h->d[0].status, sizeof status, cudaMemcpyDeviceToHost));
+    static_assert(lbm_fs::PIN_DATA + sizeof lg + sizeof cnt <= lbm_fs::PIN_BYTES, "the statistics fit the pinned buffer");
+    char *plg = h->pin + lbm_fs::PIN_DATA, *pcnt = plg + sizeof lg;
+    CK(cudaMemcpyAsync(plg, h->d[0].ledger, sizeof lg, cudaMemcpyDeviceToHost, st));
+    CK(cudaMemcpyAsync(pcnt, h->d[h->cur ^ 1].cnt, sizeof cnt, cudaMemcpyDeviceToHost, st));  // of the last step
+    const lbm_fs_status s1 = read_status(h);
+    if (s1 == LBM_FS_ECUDA || s1 == LBM_FS_ENOMEM) return s1;
+    memcpy(lg, plg, sizeof lg);
+    memcpy(cnt, pcnt, sizeof cnt);
+    if (h->step == 0) memset(cnt, 0, sizeof cnt);
+    memcpy(&status, h->pin + lbm_fs::PIN_STATUS, sizeof status);
     memset(out, 0, sizeof *out);
     out->step = h->step;
     out->liquid_mass = lg[LG_MASS];
@@ -564,7 +566,7 @@ lbm_fs_status lbm_fs_stats(lbm_fs *h, lbm_fs_stats_t *out) {
     out->kernel_launches = h->launches;
     out->wall_source = lg[LG_WALL];
     out->n_general = cnt[CN_NEAR];
-    return read_status(h);
+    return s1;
 }
 
 lbm_fs_status lbm_fs_kernel_times(lbm_fs *h, int32_t nsteps, double *ms, const char **names, int32_t cap, int32_t *nk) {

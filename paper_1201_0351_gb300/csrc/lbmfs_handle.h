@@ -16,6 +16,10 @@ struct lbm_fs {
     cudaStream_t st = nullptr;
     cudaStream_t cap_st = nullptr;
     lbmfs::Sides sides;
+    // pinned host memory for what the synchronising calls read back: copies into
+    // it queue behind one another, with one wait for all of a call's
+    static constexpr size_t PIN_BYTES = 8192, PIN_STATUS = 0, PIN_DATA = 64;
+    char *pin = nullptr;
     std::vector<void *> allocs;
     int nb = 0;
     bool started = false;
@@ -51,6 +55,7 @@ struct lbm_fs {
         allocs.clear();
         if (cap_st) cudaStreamDestroy(cap_st);
         sides.destroy();
+        if (pin) cudaFreeHost(pin);
     }
 };
 
@@ -59,7 +64,8 @@ namespace lbmfs {
 lbm_fs_status fail(lbm_fs_status s, const char *fmt, const char *detail = nullptr);
 lbm_fs_status cuda_fail(cudaError_t e, const char *where);
 lbm_fs_status check_handle(lbm_fs *h);
-// synchronise the handle's stream and map its sticky device bits to a status
+// copy the sticky device bits after the stream's work, synchronise it and map
+// them to a status
 lbm_fs_status read_status(lbm_fs *h);
 // map a copy of the device status word to a status (first sticky bit wins)
 lbm_fs_status status_bits(uint32_t st);
