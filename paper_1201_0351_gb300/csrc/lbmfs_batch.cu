@@ -32,6 +32,7 @@ struct Chunk {
     std::vector<int> idx;  // the batch's tank indices, in descriptor order
     int lane = 0;          // concurrent chain the chunk's launches belong to
     TankSet ts[2];         // descriptors for even / odd steps
+    const TankSet *dts = nullptr;  // their copies on the device
     Shape sh[SH_COUNT];
     bool zg = true;        // as in BatchLaunch
 };
@@ -56,6 +57,8 @@ struct lbm_fs_batch {
     bool built = false;
     void *tables = nullptr;
     size_t table_cap = 0;
+    TankSet *dsets = nullptr;  // device copies of the descriptors, two per chunk
+    size_t dsets_cap = 0;
     cudaGraphExec_t gexec[2] = {nullptr, nullptr};
     int per_step = 0;
     int cur = 0;
@@ -182,9 +185,20 @@ lbm_fs_status build(lbm_fs_batch *b) {
         b->table_cap = b->tables ? bytes : 0;
         if (!b->tables) return fail(LBM_FS_ENOMEM, "batch table allocation failed%s");
     }
+    const size_t sets = 2 * b->chunks.size();
+    if (sets > b->dsets_cap) {
+        CK(cudaStreamSynchronize(b->st));
+        b->free_(b->dsets);
+        b->dsets = (TankSet *)b->alloc(sets * sizeof(TankSet));
+        b->dsets_cap = b->dsets ? sets : 0;
+        if (!b->dsets) return fail(LBM_FS_ENOMEM, "batch descriptor allocation failed%s");
+    }
+    for (size_t k = 0; k < b->chunks.size(); ++k)
+        CK(cudaMemcpyAsync(b->dsets + 2 * k, b->chunks[k]->ts, 2 * sizeof(TankSet), cudaMemcpyHostToDevice, b->st));
     CK(cudaMemcpyAsync(b->tables, all.data(), all.size() * sizeof(Tile), cudaMemcpyHostToDevice, b->st));
     CK(cudaStreamSynchronize(b->st));
     size_t q = 0;
+    for (size_t k = 0; k < b->chunks.size(); ++k) b->chunks[k]->dts = b->dsets + 2 * k;
     for (auto &cp : b->chunks)
         for (int s = 0; s < SH_COUNT; ++s) cp->sh[s].table = (const Tile *)b->tables + offs[q++];
     b->built = true;
@@ -202,6 +216,7 @@ bool stale(lbm_fs_batch *b) {
 BatchLaunch launch_of(lbm_fs_batch *b, Chunk &c, int parity) {
     BatchLaunch L;
     L.ts = &c.ts[parity];
+    L.dts = c.dts + parity;
     for (int s = 0; s < SH_COUNT; ++s) L.sh[s] = c.sh[s];
     L.zb = b->zb;
     L.zg = c.zg;
@@ -299,6 +314,7 @@ void destroy_all(lbm_fs_batch *b) {
     if (b->st) cudaStreamSynchronize(b->st);
     b->drop_graphs();
     b->free_(b->tables);
+    b->free_(b->dsets);
     for (lbm_fs *t : b->tanks) {
         t->owner = nullptr;
         lbm_fs_destroy(t);

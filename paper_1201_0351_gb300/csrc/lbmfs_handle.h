@@ -18,7 +18,7 @@ struct lbm_fs {
     lbmfs::Sides sides;
     // pinned host memory for what the synchronising calls read back: copies into
     // it queue behind one another, with one wait for all of a call's
-    static constexpr size_t PIN_BYTES = 8192, PIN_STATUS = 0, PIN_DATA = 64;
+    static constexpr size_t PIN_BYTES = 16384, PIN_STATUS = 0, PIN_DATA = 64;
     char *pin = nullptr;
     std::vector<void *> allocs;
     int nb = 0;

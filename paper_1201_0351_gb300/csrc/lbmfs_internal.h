@@ -56,6 +56,7 @@ struct Body {
     double F[3], T[3], S;
     double Fp[3], Tp[3];  // the previous step's force and torque (rigid-body update)
     int nF, pad2;         // 1 once Fp, Tp hold a step
+    double vol, mass, I[3];  // of the body (set when it is added)
     double R[9];        // rotation of q (row-major), recomputed with the pose
     int mode, shape;  // shape 0: box of half extents h; 1: sphere of radius h[0]
     int lo[3], hi[3];   // cells that may be inside at the current pose, [lo, hi)
@@ -149,7 +150,8 @@ struct Shape {
     unsigned grid;      // blocks of the launch (each walks entries grid apart)
 };
 struct BatchLaunch {
-    const TankSet *ts;  // host copy, passed by value to every launch
+    const TankSet *ts;  // host copy, passed by value to the launches with much work per tank
+    const TankSet *dts; // device copy, for the short kernels
     Shape sh[SH_COUNT];
     int zb;             // z-planes per bulk tile
     bool zg;            // every tank's acceleration is along z
@@ -195,7 +197,7 @@ struct KernelSet {
 // from there for every storage: its rounding is then the same in every
 // kernel set and in single-tank and batched launches.
 void launch_bodies(const Dev &d, cudaStream_t st);
-void launch_bodies_batch(const BatchLaunch &b, cudaStream_t st);
+void launch_bodies_batch(const BatchLaunch &b, cudaStream_t st, bool early);
 
 KernelSet kernels_f64();
 KernelSet kernels_f32();

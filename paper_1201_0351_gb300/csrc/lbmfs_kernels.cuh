@@ -255,6 +255,10 @@ template <> struct Sto<2> {
 // kernel's few blocks, the first of a chain of short kernels, then get their
 // SMs before the bulk kernel's blocks fill the GPU.
 __device__ __forceinline__ void launch_dependents() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+// In a kernel so launched that does depend on the one before it: waits for that
+// one's end (nothing to wait for otherwise).  The launch itself is then already
+// behind it, about 1.5 us of each short kernel in a chain.
+__device__ __forceinline__ void wait_for_launch() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 
 __device__ __forceinline__ unsigned smem_addr(const void *p) { return (unsigned)__cvta_generic_to_shared(p); }
 // order earlier generic-proxy accesses to shared memory before the async-proxy
@@ -882,6 +886,22 @@ __global__ void k_body_prepare(Dev d, int bi) {
     if (threadIdx.x != 0) return;
     Body &b = d.bodies[bi];
     body_bounds(d, b);
+    // volume, mass and principal moments, every operation rounded by itself as
+    // in the rigid-body update's unit
+    const double *h = b.h;
+    if (b.shape == 1) {  // sphere: V = 4/3 pi r^3, I = 2/5 m r^2
+        b.vol = __dmul_rn(4.1887902047863905, __dmul_rn(__dmul_rn(h[0], h[0]), h[0]));
+        b.mass = __dmul_rn(b.dens, b.vol);
+        b.I[0] = b.I[1] = b.I[2] = __dmul_rn(__dmul_rn(0.4, b.mass), __dmul_rn(h[0], h[0]));
+    } else {
+        b.vol = __dmul_rn(__dmul_rn(__dmul_rn(8.0, h[0]), h[1]), h[2]);
+        b.mass = __dmul_rn(b.dens, b.vol);
+        const double m3 = __ddiv_rn(b.mass, 3.0);
+        const double s0 = __dmul_rn(h[0], h[0]), s1 = __dmul_rn(h[1], h[1]), s2 = __dmul_rn(h[2], h[2]);
+        b.I[0] = __dmul_rn(m3, __dadd_rn(s1, s2));
+        b.I[1] = __dmul_rn(m3, __dadd_rn(s0, s2));
+        b.I[2] = __dmul_rn(m3, __dadd_rn(s0, s1));
+    }
     for (int k = 0; k < 3; ++k) {
         b.plo[k] = b.lo[k];
         b.phi[k] = b.hi[k];
@@ -2536,39 +2556,47 @@ __device__ __noinline__ double curvature_d(const Dev &d, int x, int y, int z, do
     }
     return 0.25 * div;
 }
-// the same in float for the float storages
-__device__ __forceinline__ float fill_seen_f(const Dev &d, long long ni, float own) {
-    const int c = cls(d, ni);
-    return c == CL_L ? 1.0f : (c == CL_I ? d.phifsrc[ni] : (c == CL_G ? 0.0f : own));
-}
-__device__ __noinline__ float curvature_f(const Dev &d, int x, int y, int z, float nc0, float nc1, float nc2) {
-    const float nc[3] = {nc0, nc1, nc2};
-    float div = 0.0f;
-    for (int k = 0; k < 3; ++k) {
-        float comp[2];
-        for (int sgn = 0; sgn < 2; ++sgn) {
-            const int s = sgn ? -1 : 1;
-            const long long yi = nbr(d, x, y, z, k == 0 ? s : 0, k == 1 ? s : 0, k == 2 ? s : 0);
-            const int c = cls(d, yi);
-            if (c == CL_WALL || c == CL_O) {
-                comp[sgn] = nc[k];
-                continue;
-            }
-            int yx, yy, yz;
-            coords(d, yi, yx, yy, yz);
-            const float own = c == CL_L ? 1.0f : (c == CL_I ? d.phifsrc[yi] : 0.0f);
-            float n[3];
-            for (int j = 0; j < 3; ++j) {
-                const float pm = fill_seen_f(d, nbr(d, yx, yy, yz, j == 0 ? -1 : 0, j == 1 ? -1 : 0, j == 2 ? -1 : 0), own);
-                const float pp = fill_seen_f(d, nbr(d, yx, yy, yz, j == 0 ? 1 : 0, j == 1 ? 1 : 0, j == 2 ? 1 : 0), own);
-                n[j] = 0.5f * (pm - pp);
-            }
-            const float len = sqrtf((n[0] * n[0] + n[1] * n[1]) + n[2] * n[2]);
-            comp[sgn] = len > 0.0f ? n[k] / len : 0.0f;
+// The same in float for the float storages, one axis: member r of a cell's trio
+// takes the two neighbours on axis r, own the cell's unit normal's component r;
+// the caller adds the three in axis order.  All classes and fill levels around
+// the two neighbours are requested at once (one thread walking the six
+// neighbours' six neighbours class by class was most of the interface kernel:
+// 64^3 bubble 20 us).
+__device__ __noinline__ float curvature_axis_f(const Dev &d, int x, int y, int z, int r, float own) {
+    const int ex = r == 0, ey = r == 1, ez = r == 2;
+    float comp[2], f[2][6];
+    int cy0[2];
+#pragma unroll
+    for (int s = 0; s < 2; ++s) {
+        const int sg = s ? -1 : 1;
+        const long long yi = nbr(d, x, y, z, sg * ex, sg * ey, sg * ez);
+        cy0[s] = cls(d, yi);
+        int yx = x, yy = y, yz = z;
+        if (yi >= 0) coords(d, yi, yx, yy, yz);
+        const long long at = yi >= 0 ? yi : x + (long long)d.nx * (y + (long long)d.ny * z);
+        const float ph = d.phifsrc[at];
+        const float self = cy0[s] == CL_L ? 1.0f : (cy0[s] == CL_I ? ph : 0.0f);
+        int c[6];
+        float p[6];
+#pragma unroll
+        for (int j = 0; j < 6; ++j) {
+            const int sj = j & 1 ? 1 : -1;
+            const long long ni = nbr(d, yx, yy, yz, j < 2 ? sj : 0, j >= 2 && j < 4 ? sj : 0, j >= 4 ? sj : 0);
+            c[j] = cls(d, ni);
+            p[j] = d.phifsrc[ni < 0 ? at : ni];
         }
-        div += comp[0] - comp[1];
+#pragma unroll
+        for (int j = 0; j < 6; ++j)
+            f[s][j] = c[j] == CL_L ? 1.0f : (c[j] == CL_I ? p[j] : (c[j] == CL_G ? 0.0f : self));
     }
-    return 0.25f * div;
+#pragma unroll
+    for (int s = 0; s < 2; ++s) {
+        const float n0 = 0.5f * (f[s][0] - f[s][1]), n1 = 0.5f * (f[s][2] - f[s][3]), n2 = 0.5f * (f[s][4] - f[s][5]);
+        const float len = sqrtf((n0 * n0 + n1 * n1) + n2 * n2);
+        const float nr = r == 0 ? n0 : (r == 1 ? n1 : n2);
+        comp[s] = (cy0[s] == CL_WALL || cy0[s] == CL_O) ? own : (len > 0.0f ? nr / len : 0.0f);
+    }
+    return comp[0] - comp[1];
 }
 
 // ---- C1 + C2 for interface cells of the float storages: three threads per
@@ -2793,13 +2821,10 @@ __device__ __forceinline__ void interface_trio(const Dev &d, const VB &vb) {
                     nv2 = __shfl_sync(FULL, nvr, b3 + 2);
         float drg = d.drg_f;
         if (d.sigma != 0.0) {
-            // gas density raised by the Laplace pressure (curvature by member 0)
+            // gas density raised by the Laplace pressure
             const float len = sqrtf((nv0 * nv0 + nv1 * nv1) + nv2 * nv2);
-            const float nu0 = len > 0.0f ? nv0 / len : 0.0f, nu1 = len > 0.0f ? nv1 / len : 0.0f,
-                        nu2 = len > 0.0f ? nv2 / len : 0.0f;
-            float kap = 0.0f;
-            if (r == 0) kap = curvature_f(d, x, y, z, nu0, nu1, nu2);
-            kap = __shfl_sync(FULL, kap, b3);
+            const float nur = len > 0.0f ? (r == 0 ? nv0 : (r == 1 ? nv1 : nv2)) / len : 0.0f;
+            const float kap = 0.25f * trio_sum(curvature_axis_f(d, x, y, z, r, nur), b3);
             drg = d.drg_f + (6.0f * d.sigma_f) * kap;
         }
         // Eq. reconstruct for gas-sourced directions and every non-solid
@@ -3344,8 +3369,9 @@ __global__ void k_conv_finish(const __grid_constant__ Dev d) { conv_finish_body(
 // lanes: lane l works on component k = l % 3 of the vectors, lanes with
 // (l / 3) odd on the rotation where it mirrors the translation, and lanes 0..8
 // on the nine entries of a rotation matrix.  Every value is the scalar update's
-// (one thread, about 700 double operations, 22 us; now about 200), rounded the
-// same way: this unit is compiled without fused multiply-add.
+// (one thread, about 700 double operations, 22 us; now about 80 and four
+// divisions), rounded the same way: this unit is compiled without fused
+// multiply-add.
 __device__ __forceinline__ double lane_of(double v, int l) { return __shfl_sync(0xffffffffu, v, l); }
 // (a_0 + a_1) + a_2 of the values that lanes base .. base + 2 hold
 __device__ __forceinline__ double sum3(double a, int base) {
@@ -3439,45 +3465,48 @@ __device__ __forceinline__ void bodies_body(const Dev &d, const VB &vb) {
     // of that period through the wall velocity
     const double ftp = rot ? b.Tp[k] : b.Fp[k];
     const double fh = d.force_mean && b.nF ? 0.5 * (ft + ftp) : ft;  // force, or torque (rot)
-    const double hk = b.h[k], dens = b.dens, C = d.vmass;
-    const double h0 = b.h[0], hsq = hk * hk;
-    double vol, mass, I;
-    if (b.shape == 1) {  // sphere: V = 4/3 pi r^3, I = 2/5 m r^2
-        vol = 4.1887902047863905 * ((h0 * h0) * h0);
-        mass = dens * vol;
-        I = (0.4 * mass) * (h0 * h0);
-    } else {
-        vol = ((8.0 * h0) * b.h[1]) * b.h[2];
-        mass = dens * vol;
-        I = (mass / 3.0) * (lane_of(hsq, k == 0 ? 1 : 0) + lane_of(hsq, k == 2 ? 1 : 2));
-    }
+    const double hk = b.h[k], h0 = b.h[0], dens = b.dens, C = d.vmass;
+    const double vol = b.vol, mass = b.mass, I = b.I[k];  // (set with the body)
     double q = b.q[lane & 3];
     const double R = rotation_lane(q, lane);
     const double c0 = lane_of(R, k), c1 = lane_of(R, 3 + k), c2 = lane_of(R, 6 + k);  // column k
     const double T0 = lane_of(fh, 3), T1 = lane_of(fh, 4), T2 = lane_of(fh, 5);
     const double w0 = b.w[0], w1 = b.w[1], w2 = b.w[2];
-    double num = (fh + mass * d.grav[k]) + C * (vol * b.dv[k]);  // translation (virtual mass: Schwarz, Kempe and Froehlich 2015)
-    double den = mass + C * vol;
-    double wb = 0.0, rnum, rden;
+    // translation (virtual mass: Schwarz, Kempe and Froehlich 2015) and rotation
+    // have the form (A + C (B D)) / (E + C B), D the last acceleration
+    double A = fh + mass * d.grav[k], B = vol, E = mass, wb;
+    const double Dl = rot ? (base == 2 ? b.dw[0] : b.dw[k]) : b.dv[k];
     if (base == 2) {
-        const double a0 = b.axis[0], a1 = b.axis[1], a2 = b.axis[2];
-        const double ta = (T0 * a0 + T1 * a1) + T2 * a2;
-        const double ab = (c0 * a0 + c1 * a1) + c2 * a2;
-        const double Ia = sum3((ab * ab) * I, 0);
+        // the dot products with the axis: of column k (lanes 0..2: the axis in the
+        // body's frame), of the torque (lane 3) and of the angular velocity (lane 4)
+        const double v0 = lane < 3 ? c0 : (lane == 3 ? T0 : w0), v1 = lane < 3 ? c1 : (lane == 3 ? T1 : w1),
+                     v2 = lane < 3 ? c2 : (lane == 3 ? T2 : w2);
+        const double dot = (v0 * b.axis[0] + v1 * b.axis[1]) + v2 * b.axis[2];
+        const double Ia = sum3((dot * dot) * I, 0);
         const double Ifa = Ia / dens;
-        wb = (w0 * a0 + w1 * a1) + w2 * a2;
-        rnum = ta + C * (Ifa * b.dw[0]);
-        rden = Ia + C * Ifa;
+        wb = lane_of(dot, 4);
+        const double ta = lane_of(dot, 3);
+        if (rot) {
+            A = ta;
+            B = Ifa;
+            E = Ia;
+        }
     } else {
+        // column k times the angular velocity (lanes 0..2) and the torque (3..5)
+        const double dot = (c0 * (rot ? T0 : w0) + c1 * (rot ? T1 : w1)) + c2 * (rot ? T2 : w2);
         const double If = I / dens;
-        wb = (c0 * w0 + c1 * w1) + c2 * w2;
-        const double tb = (c0 * T0 + c1 * T1) + c2 * T2;
+        wb = lane_of(dot, k);
+        const double tb = lane_of(dot, 3 + k);
         const double L = I * wb;
         const double gy = lane_of(wb, k1) * lane_of(L, k2) - lane_of(wb, k2) * lane_of(L, k1);
-        rnum = (tb - gy) + C * (If * b.dw[k]);
-        rden = I + C * If;
+        const double Ar = tb - gy;
+        if (rot) {
+            A = Ar;
+            B = If;
+            E = I;
+        }
     }
-    const double acc = (rot ? rnum : num) / (rot ? rden : den);  // dv (lanes 0..2), dw (lanes 3..5)
+    const double acc = (A + C * (B * Dl)) / (E + C * B);  // dv (lanes 0..2), dw (lanes 3..5)
     const double dv = lane_of(acc, k), dw = lane_of(acc, 3 + k);
     double v = b.v[k] + dv;
     if (b.mode & 0x100) v = v * (1.0 - b.damp);
@@ -3553,7 +3582,10 @@ __device__ __forceinline__ void bodies_body(const Dev &d, const VB &vb) {
         nb.w[k] = w;
     }
 }
-__global__ void k_bodies(const __grid_constant__ Dev d) { bodies_body(d, vb_own()); }
+__global__ void k_bodies(const __grid_constant__ Dev d) {
+    launch_dependents();  // the remap's scan, which waits for this launch's end
+    bodies_body(d, vb_own());
+}
 
 // ----------------------------------------------- C6: remap (Sec. 2.3, 2.4)
 
@@ -3606,7 +3638,10 @@ __device__ __forceinline__ void remap_scan_body(const Dev &d, const VB &vb) {
     }
 }
 constexpr int SCAN_THREADS = 64;
-__global__ void __launch_bounds__(SCAN_THREADS) k_remap_scan(const __grid_constant__ Dev d) { remap_scan_body(d, vb_own()); }
+__global__ void __launch_bounds__(SCAN_THREADS) k_remap_scan(const __grid_constant__ Dev d) {
+    wait_for_launch();
+    remap_scan_body(d, vb_own());
+}
 
 // listed cells inside a body's new pose become obstacle, their mass is booked;
 // listed obstacle cells outside it are pending
@@ -3934,13 +3969,31 @@ __global__ void k_read_fields(Dev d, unsigned mask, uint8_t *flags, double *fill
 template <class K>
 __global__ void __launch_bounds__(K::THREADS, K::MINB)
     k_batch(const __grid_constant__ TankSet ts, const Tile *__restrict__ table, unsigned n, int zb) {
-    launch_dependents();  // (only the bulk kernel is launched so, behind the force kernel)
+    launch_dependents();  // (of these only the bulk kernel is launched so, behind the force kernel)
     for (unsigned t = blockIdx.x; t < n; t += gridDim.x) {
         const Tile e = table[t];
         const VB vb{e.x, e.y, e.z, e.nx, e.ny, e.nz, e.kind};
         K::run(ts.d[e.tank], vb, zb);
         // the next entry's body reuses this one's shared memory; bodies
         // without shared memory let a block's warps move on independently
+        if constexpr (K::SMEM) __syncthreads();
+    }
+}
+
+// The short kernels of a batch's step (counters, conversions, rigid bodies,
+// remap): the descriptors come from memory instead of the parameter space, 25 KB
+// of which cost every launch a few us, and each launch is a programmatic
+// dependent of the one before it in the chain.
+template <class K>
+__global__ void __launch_bounds__(K::THREADS, K::MINB)
+    k_batch_short(const TankSet *__restrict__ ts, const Tile *__restrict__ table, unsigned n) {
+    launch_dependents();
+    wait_for_launch();
+    for (unsigned t = blockIdx.x; t < n; t += gridDim.x) {
+        const Tile e = table[t];
+        const VB vb{e.x, e.y, e.z, e.nx, e.ny, e.nz, e.kind};
+        const Dev d = ts->d[e.tank];  // (the fields that the body uses)
+        K::run(d, vb, 0);
         if constexpr (K::SMEM) __syncthreads();
     }
 }
@@ -3985,6 +4038,26 @@ LBMFS_BATCH_BODY(BkNbUpdate, LIST_THREADS, 1, nb_update_body(d, vb))
 #undef LBMFS_BATCH_BODY
 #undef LBMFS_BATCH_BODY_SM
 
+// launch k, with `early` as a programmatic dependent of the stream's last kernel
+// (see launch_dependents)
+template <class... P, class... A>
+void launch(void (*k)(P...), dim3 grid, int block, size_t smem, cudaStream_t st, bool early, A... args) {
+    cudaLaunchConfig_t c = {};
+    cudaLaunchAttribute a = {};
+    c.gridDim = grid;
+    c.blockDim = dim3(block);
+    c.dynamicSmemBytes = smem;
+    c.stream = st;
+    a.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    a.val.programmaticStreamSerializationAllowed = 1;
+    c.attrs = &a;
+    c.numAttrs = early ? 1 : 0;
+    cudaLaunchKernelEx(&c, k, P(args)...);
+}
+template <class K> void batch_short(const BatchLaunch &b, int sh, int block, cudaStream_t st, bool early) {
+    const Shape &x = b.sh[sh];
+    if (x.n) launch(k_batch_short<K>, dim3(x.grid), block, 0, st, early, b.dts, x.table, x.n);
+}
 template <class K> void batch_launch(const BatchLaunch &b, int sh, dim3 block, cudaStream_t st) {
     const Shape &x = b.sh[sh];
     if (x.n) k_batch<K><<<x.grid, block, 0, st>>>(*b.ts, x.table, x.n, b.zb);
@@ -4046,28 +4119,12 @@ template <int S> struct Launch {
     static void forces(const Dev &d, cudaStream_t st) {
         k_forces<S><<<dim3(FORCE_BLOCKS, d.nb), FORCE_THREADS, 0, st>>>(d);
     }
-    static void scan(const Dev &d, cudaStream_t st) { 
+    static void scan(const Dev &d, cudaStream_t st, bool early) {
         // a cell or two per thread; blocks small enough to run beside the ring
         // kernel's, which leave 4096 registers of an SM
-        k_remap_scan<<<dim3(std::max(FORCE_BLOCKS, 1216 / d.nb), d.nb), SCAN_THREADS, 0, st>>>(d);
+        launch(k_remap_scan, dim3(std::max(FORCE_BLOCKS, 1216 / d.nb), d.nb), SCAN_THREADS, 0, st, early, d);
     }
     static void interface(const Dev &d, cudaStream_t st) { k_interface<S><<<LBMFS_IFACE_GRID, 128, 0, st>>>(d); }
-    // launch k, with `early` as a programmatic dependent of the stream's last
-    // kernel (see launch_dependents)
-    template <class... P, class... A>
-    static void launch(void (*k)(P...), dim3 grid, int block, size_t smem, cudaStream_t st, bool early, A... args) {
-        cudaLaunchConfig_t c = {};
-        cudaLaunchAttribute a = {};
-        c.gridDim = grid;
-        c.blockDim = dim3(block);
-        c.dynamicSmemBytes = smem;
-        c.stream = st;
-        a.id = cudaLaunchAttributeProgrammaticStreamSerialization;
-        a.val.programmaticStreamSerializationAllowed = 1;
-        c.attrs = &a;
-        c.numAttrs = early ? 1 : 0;
-        cudaLaunchKernelEx(&c, k, P(args)...);
-    }
     // the bulk kernel: FP64 and FP32 one cell per thread, with the z-planes per
     // block of bulk_planes; FP16 the ring; LBMFS_BULK selects the staged forms
     static void bulk_any(const Dev &d, cudaStream_t st, bool early) {
@@ -4148,7 +4205,7 @@ template <int S> struct Launch {
             if (walls) faces(d, sides->st[2]);
             interface(d, sides->st[0]);
             if (bodies) launch_bodies(d, sides->st[1]);
-            if (bodies) scan(d, sides->st[1]);
+            if (bodies) scan(d, sides->st[1], true);
             bulk_any(d, st, bodies);  // (behind the force kernel's start)
             for (int k = 0; k < SIDE_STREAMS; ++k)
                 if (used[k]) {
@@ -4175,7 +4232,7 @@ template <int S> struct Launch {
         mark();
         if (bodies) launch_bodies(d, st);
         mark();
-        if (bodies) scan(d, st);
+        if (bodies) scan(d, st, false);
         mark();
         tail(d, st);
         mark();
@@ -4190,10 +4247,10 @@ template <int S> void batch_bulk_launch(const BatchLaunch &b, cudaStream_t st, b
     if constexpr (S == 2) {
         const auto k = b.zg ? k_batch_ring<true> : k_batch_ring<false>;
         cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, RingShape::SMEM);
-        Launch<S>::launch(k, dim3(x.grid), RingShape::THREADS, RingShape::SMEM, st, early, *b.ts, x.table, x.n);
+        launch(k, dim3(x.grid), RingShape::THREADS, RingShape::SMEM, st, early, *b.ts, x.table, x.n);
     } else {
         auto go = [&](void (*k)(TankSet, const Tile *, unsigned, int)) {
-            Launch<S>::launch(k, dim3(x.grid), BULK_THREADS, 0, st, early, *b.ts, x.table, x.n, b.zb);
+            launch(k, dim3(x.grid), BULK_THREADS, 0, st, early, *b.ts, x.table, x.n, b.zb);
         };
         if (b.zb == 1) go(k_batch<BkLiquid<S, 1>>);
         else if (b.zb == 2) go(k_batch<BkLiquid<S, 2>>);
@@ -4213,7 +4270,8 @@ template <int S> struct BatchStep {
             ++k;
         };
         mark();
-        batch_launch<BkReset>(b, SH_TANK, 32, st);
+        const bool chain = ev == nullptr;  // (an event between two launches breaks the chain)
+        batch_short<BkReset>(b, SH_TANK, 32, st, false);
         cudaStream_t s0 = st, s1 = st, s2 = st;
         if (sides) {
             cudaEventRecord(sides->fork, st);
@@ -4229,8 +4287,8 @@ template <int S> struct BatchStep {
             cudaStreamWaitEvent(s1, sides->fork2, 0);
             batch_launch<BkGeneral<S>>(b, SH_GEN, GEN_THREADS, s2);
             batch_launch<BkInterface<S>>(b, SH_IFACE, 128, s0);
-            launch_bodies_batch(b, s1);
-            batch_launch<BkRemapScan>(b, SH_FORCE, SCAN_THREADS, s1);
+            launch_bodies_batch(b, s1, false);
+            batch_short<BkRemapScan>(b, SH_FORCE, SCAN_THREADS, s1, true);
         }
         mark();
         batch_bulk_launch<S>(b, st, sides != nullptr && b.sh[SH_FORCE].n > 0);
@@ -4244,29 +4302,29 @@ template <int S> struct BatchStep {
                 cudaEventRecord(sides->join[j], sides->st[j]);
                 cudaStreamWaitEvent(st, sides->join[j], 0);
             }
-        batch_launch<BkConvFilled>(b, SH_LIST, LIST_THREADS, st);
+        batch_short<BkConvFilled>(b, SH_LIST, LIST_THREADS, st, false);
         mark();
-        batch_launch<BkConvEmptied>(b, SH_LIST, LIST_THREADS, st);
+        batch_short<BkConvEmptied>(b, SH_LIST, LIST_THREADS, st, chain);
         mark();
-        batch_launch<BkConvInit<S>>(b, SH_LIST, LIST_THREADS, st);
+        batch_short<BkConvInit<S>>(b, SH_LIST, LIST_THREADS, st, chain);
         mark();
-        batch_launch<BkConvClaim<S>>(b, SH_LIST, LIST_THREADS, st);
+        batch_short<BkConvClaim<S>>(b, SH_LIST, LIST_THREADS, st, chain);
         mark();
-        batch_launch<BkConvFlags>(b, SH_LIST, LIST_THREADS, st);
+        batch_short<BkConvFlags>(b, SH_LIST, LIST_THREADS, st, chain);
         mark();
-        batch_launch<BkConvExcess<S>>(b, SH_LIST, LIST_THREADS, st);
+        batch_short<BkConvExcess<S>>(b, SH_LIST, LIST_THREADS, st, chain);
         mark();
-        batch_launch<BkConvFinish>(b, SH_LIST, LIST_THREADS, st);
+        batch_short<BkConvFinish>(b, SH_LIST, LIST_THREADS, st, chain);
         mark();
-        if (!sides) launch_bodies_batch(b, st);
+        if (!sides) launch_bodies_batch(b, st, false);
         mark();
-        if (!sides) batch_launch<BkRemapScan>(b, SH_FORCE, SCAN_THREADS, st);
+        if (!sides) batch_short<BkRemapScan>(b, SH_FORCE, SCAN_THREADS, st, false);
         mark();
-        batch_launch<BkRemapApply<S>>(b, SH_LIST, LIST_THREADS, st);
+        batch_short<BkRemapApply<S>>(b, SH_LIST, LIST_THREADS, st, chain);
         mark();
-        batch_launch<BkRemapResolve<S>>(b, SH_ONE, REMAP_THREADS, st);
+        batch_short<BkRemapResolve<S>>(b, SH_ONE, REMAP_THREADS, st, chain);
         mark();
-        batch_launch<BkNbUpdate>(b, SH_LIST, LIST_THREADS, st);
+        batch_short<BkNbUpdate>(b, SH_LIST, LIST_THREADS, st, chain);
         mark();
         int n = 0;
         const int shapes[] = {SH_TANK, SH_FORCE, SH_BULK, SH_GEN, SH_IFACE, SH_LIST, SH_LIST, SH_LIST, SH_LIST,
