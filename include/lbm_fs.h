@@ -268,8 +268,9 @@ lbm_fs_status lbm_fs_stats(lbm_fs *h, lbm_fs_stats_t *out);
 /* Synchronises the handle's stream and reports sticky device errors. */
 lbm_fs_status lbm_fs_sync(lbm_fs *h);
 
-/* Runs nsteps steps without graphs, timing every kernel with CUDA events on the
- * handle's stream; ms[k] receives the summed milliseconds of kernel k over the
+/* Runs nsteps steps without graphs, all kernels in one chain (a captured step
+ * runs several of them beside the bulk kernel, so a step takes less than the
+ * sum), timing every kernel with CUDA events on the handle's stream; ms[k] receives the summed milliseconds of kernel k over the
  * steps and names (may be NULL) a static name per kernel.  Returns the number
  * of kernels in *nk (at most cap entries are written). */
 lbm_fs_status lbm_fs_kernel_times(lbm_fs *h, int32_t nsteps, double *ms,
@@ -310,8 +311,10 @@ lbm_fs_status lbm_fs_batch_step(lbm_fs_batch *b, int32_t nsteps);
 lbm_fs_status lbm_fs_batch_sync(lbm_fs_batch *b);
 
 /* Launch configuration of a batch:
- *   zb          z-planes per bulk tile (1..8);
- *   bulk_blocks persistent grid of the bulk kernel (0: one block per tile);
+ *   zb          z-planes per bulk tile (1..8; FP64 and FP32 storage: the FP16
+ *               storage's bulk kernel walks tiles of consecutive cells);
+ *   bulk_blocks persistent grid of the bulk kernel (0: one block per tile, FP16
+ *               storage: as many as are resident);
  *   list_cells  nx*ny cells of a tank per block of the worklist kernels
  *               (a tank gets ceil(nx*ny / list_cells) blocks, at most 304);
  *   lanes       groups of tanks (of about equal cell count) whose step

@@ -1063,8 +1063,8 @@ __device__ __forceinline__ uint32_t near_blocks(const Dev &d, const VB &vb, uint
 }
 
 // neighbour-obstacle bit: set when any of the 18 neighbours is an obstacle
-// (the bulk kernel then lists the cell for k_general; walls and periodic
-// seams are recognised from the cell's coordinates)
+// (the bulk kernel then leaves a liquid cell to k_near; walls and periodic
+// seams have their own bits, set at creation)
 __device__ __forceinline__ void nb_refresh(const Dev &d, long long i) {
     int x, y, z;
     coords(d, i, x, y, z);
@@ -1506,7 +1506,7 @@ __global__ void __launch_bounds__(FORCE_THREADS, S == 0 ? 2 : LBMFS_FORCE_MINB /
 }
 
 // ---- C1 + C2 for liquid cells (Sec. 2.1 Eqs. stream, lbgk, forceterm;
-// Sec. 2.3 Eq. noslip); interface cells are listed for k_interface
+// Sec. 2.3 Eq. noslip); interface cells are listed for the next step's k_interface
 template <int S, int ZBMAX>
 __device__ __forceinline__ void liquid_column(const Dev &d, bool in, int x, int y, int z0, int z1);
 
@@ -2711,11 +2711,7 @@ __device__ __forceinline__ void interface_trio(const Dev &d, const VB &vb) {
     const uint32_t n = seq.e[PREV_LISTS - 1];
     // three rounds where that still gives each of the launch's warps (up to
     // four per scheduler of the GPU) something to do
-#ifdef LBMFS_IFACE_SUB
-    const int sub = LBMFS_IFACE_SUB;
-#else
     const int sub = 4u * (n / 30u) >= min(vb.nx * (blockDim.x >> 5), 4u * 608u) ? 3 : 1;
-#endif
     uint32_t first, stride;
     list_span(vb, n, 10u * sub, first, stride);
     for (uint32_t w0 = first; w0 < n; w0 += stride) {
@@ -3810,7 +3806,7 @@ constexpr int TAIL_CLUSTER = 8, TAIL_BLOCKS = 152;
 // grid they only make the block barriers longer: 768x384x256 103 us against 89)
 constexpr int tail_threads(bool cluster) { return cluster ? 1024 : 512; }
 
-// one warp-wide poll limit for the grid barrier: far beyond the time that the
+// poll limit of the grid barrier: far beyond the time that the
 // resident blocks of a cooperative launch can be apart
 constexpr unsigned BARRIER_POLLS = 1u << 24;
 template <bool CLUSTER> __device__ __forceinline__ bool tail_barrier(const Dev &d) {
@@ -4078,10 +4074,9 @@ inline int bulk_planes(int storage, unsigned gx, int nz) {
 }
 
 // largest xy-plane whose tail runs as one cluster
-#ifndef LBMFS_TAIL_CLUSTER_CELLS
-#define LBMFS_TAIL_CLUSTER_CELLS 131072
-#endif
-constexpr long long TAIL_CLUSTER_CELLS = LBMFS_TAIL_CLUSTER_CELLS;
+// (measured with both forms, us: 385x190 plane 55 as a cluster, 65 as a grid;
+// 768x384 109 and 82; a tank whose lists are empty 5 and 8)
+constexpr long long TAIL_CLUSTER_CELLS = 131072;
 
 constexpr int STEP_SLOTS = 7, BATCH_SLOTS = 17;  // kernel slots of a step (names below)
 
@@ -4173,7 +4168,11 @@ template <int S> struct Launch {
             a.val.clusterDim.y = a.val.clusterDim.z = 1;
             cudaLaunchKernelEx(&c, k_tail<S, true>, d);
         } else {
-            c.gridDim = dim3(TAIL_BLOCKS);
+            // a block per SM, of the SMs that there are (all blocks are resident)
+            int dev = 0, sms = TAIL_BLOCKS;
+            cudaGetDevice(&dev);
+            cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+            c.gridDim = dim3(std::min(TAIL_BLOCKS, sms));
             c.blockDim = dim3(tail_threads(false));
             a.id = cudaLaunchAttributeCooperative;
             a.val.cooperative = 1;
