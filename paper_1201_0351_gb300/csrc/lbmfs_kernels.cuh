@@ -2110,7 +2110,13 @@ __global__ void __launch_bounds__(BULK_THREADS, LBMFS_BULK_MINB) k_liquid_tma(De
 // fetches them as soon as a tile is announced and patches them into the staged
 // tile; the consumers fetch those of the y and z faces (whole warps) themselves.
 // Fetching the x faces in the consumers too cost a global load's latency per
-// warp: FP16S bulk kernel, 768x384x256 763 us against 581 without any face work.
+// warp: 768x384x256 bulk kernel 763 us against 581 without any face work.
+// Measured, us, before (one cell per thread) and now: 768x384x256 856 and 593
+// (5.1 TB/s, 76 % of the copy bandwidth; on 384x192x128 issue is 58 % and the FMA
+// pipe 46 % active, so no unit alone is the bound),
+// 385x190x127 127 and 91, 64 tanks of edge 48..112 626 and 408.  On grids too
+// small to fill the GPU it is even (130x40x40 11 and 12).  The FP32 storage
+// keeps the other kernel: 944 us against 1021 in a ring, HBM-bound either way.
 constexpr int RING_STAGES = 4;
 struct RingShape {
     static constexpr int TILE = RING_TILE, ESZ = 2;         // cells, bytes per moving population
@@ -2630,7 +2636,8 @@ __device__ __noinline__ float curvature_axis_f(const Dev &d, int x, int y, int z
 // also kept rounded to float, and a warp takes 30 cells as `sub` = 3 rounds of
 // ten trios before lane l does the mass update of cell l for all of them; a
 // list too short to give every scheduler a warp that way takes ten cells per
-// warp (sub = 1).
+// warp (sub = 1).  64-tank FP16S batch 154 us with sub = 1, 137 with 3; alone on
+// 768x384x256 102 and 116, beside the bulk kernel the step is the same.
 
 // neighbour (x + dx, y + dy, z + dz) as a 32-bit cell index without
 // branches (periodic axes wrap); -1 beyond a wall
@@ -3601,7 +3608,8 @@ __global__ void k_bodies(const __grid_constant__ Dev d) {
 // Which cells body vb.y covers and which it leaves with its new pose: the
 // obstacle set is not touched by the conversions, so the lists are made from
 // it and the two poses alone, beside the bulk kernel; remap_apply_body acts on
-// them once the conversions are done.
+// them once the conversions are done.  (Two scans behind the
+// conversions before, 6 to 8 us each on a small tank; now one of 6 to 10 us.)
 __device__ __forceinline__ void remap_scan_body(const Dev &d, const VB &vb) {
     const int bi = vb.y;
     const Body &b = d.bodies_new[bi];
@@ -3810,6 +3818,9 @@ __global__ void __launch_bounds__(REMAP_THREADS) k_remap_resolve(const __grid_co
 // with empty lists, more than the work of a small tank's step, so one launch
 // runs them with a barrier in between, and leaves out the conversions' (the
 // remap's) barriers when nothing converts (no cell is covered or left).
+// Measured, us, sum of the ten kernels timed one by one and this launch: 64^3
+// without bodies 53 and 5; 130x40x40 117 and 40; 385x190x127 143 and 55;
+// 768x384x256 172 and 72.
 //  - CLUSTER: one cluster of TAIL_CLUSTER blocks with the hardware's cluster
 //    barrier, for tanks whose lists are short;
 //  - else a cooperative grid with a barrier in global memory, for large tanks
