@@ -616,9 +616,10 @@ __device__ __forceinline__ double cell_rho_u(const Dev &d, const void *g, long l
 // pair shares 3 cu, 9 cu and (4.5 cu) cu, and a component with c = 0
 // contributes (-3 u) a to every such direction.  ZG (ax = ay = 0, gravity
 // along z alone, chosen per launch from the uniform parameters) also drops the
-// products by those zero accelerations.  612 double operations per liquid cell
-// before, 311 with ZG and about 400 without (96^3 bulk kernel 565 -> 287 us; at
-// 529 G double operations per second it is within 7 % of that rate).
+// products by those zero accelerations.  Double operations per
+// liquid cell of the bulk kernel (wave tank): 612 before, 329 with this, 310 with
+// the stored sum checked by exponents; 96^3 bulk kernel 565, 287 and 270 us, now
+// within 4 % of 529 G double operations per second.
 // Returns rho.
 template <bool ZG> __device__ __forceinline__ double collide_d_t(const Dev &d, const double *fp, double *fnew) {
     double rho = fp[0], j0 = 0.0, j1 = 0.0, j2 = 0.0;
