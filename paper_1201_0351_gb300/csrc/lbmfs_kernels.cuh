@@ -3646,6 +3646,9 @@ __device__ __forceinline__ void remap_scan_body(const Dev &d, const VB &vb) {
                 const bool in = inside(d, b, x, y, z);
                 cover = !solid && in;
                 pend = own && !in;
+                // of the bodies that cover a cell at once the first has it
+#pragma unroll 1
+                for (int j = 0; cover && j < bi; ++j) cover = !inside(d, d.bodies_new[j], x, y, z);
             }
         }
         if (__any_sync(0xffffffffu, cover)) wl_append(d, cover, WL_COVER, (uint32_t)i);
@@ -3669,7 +3672,6 @@ __device__ __forceinline__ void remap_apply_body(const Dev &d, const VB &vb) {
         LIST_LOOP(WL_COVER, a) {
             const long long i = d.list[WL_COVER][it_a];
             const int c = clsv(d, i);
-            if (c == CL_O) continue;  // two bodies cover it
             const double mass = c == CL_L ? cell_density<S>(d, d.fdst, i) : (c == CL_I ? d.m[i] : 0.0);
             if (mass != 0.0) atomicAdd(&d.ledger[LG_COVERED], mass);
             set_cls(d, i, CL_O);
