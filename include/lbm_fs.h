@@ -91,8 +91,11 @@ typedef struct {
     double eps;            /* conversion threshold: fill at phi >= 1+eps, empty at phi <= -eps */
     int32_t storage;       /* LBM_FS_F64 / LBM_FS_F32 / LBM_FS_F16S */
     /* initial state, nx*ny*nz entries each (3 per cell for init_vel, xyz):
-     * classes 1/2/4, fill level, density, velocity (NULL = at rest).  Fluid cells
-     * start at f = f_eq(rho, u).  The arrays are copied; the caller keeps them.
+     * classes 1/2/4/8, fill level, density, velocity (NULL = at rest).  Fluid cells
+     * start at f = f_eq(rho, u).  Obstacle cells (8) given here are a fixed solid;
+     * in a tank with bodies they count as cells of body 0 (its force, its velocity
+     * at their links, and they turn into fluid where its bounding range passes).
+     * The arrays are copied; the caller keeps them.
      * init_flags, init_fill and init_rho are required. */
     const uint8_t *init_flags;
     const double *init_fill;

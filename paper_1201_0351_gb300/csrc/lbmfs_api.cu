@@ -351,9 +351,12 @@ lbm_fs_status lbm_fs_create(const lbm_fs_params *p, lbm_fs **out) {
     }
     h->ks.init_cells(h->d[0], dfl, dfi, drh, dvl, st);
     e = cudaGetLastError();
+    uint32_t loose = 0;  // obstacles among the initial classes
+    if (e == cudaSuccess) e = cudaMemcpyAsync(&loose, d.status + 3, sizeof loose, cudaMemcpyDeviceToHost, st);
     if (e == cudaSuccess) e = cudaStreamSynchronize(st);
     if (tmp) cudaFree(tmp);
     if (e != cudaSuccess) return bail(cuda_fail(e, "initial upload"));
+    h->d[0].loose = h->d[1].loose = loose != 0;
 #undef CKB
     *out = h;
     return LBM_FS_OK;

@@ -154,8 +154,11 @@ lbm_fs_status build(lbm_fs_batch *b) {
             for (int x = 0; x < lb; ++x) tb[SH_LIST].push_back(tile(j, x, 0, 0, lb, 1, 1));
             for (int x = 0; x < nb; ++x) tb[SH_BODY].push_back(tile(j, x, 0, 0, nb, 1, 1));
             if (nb > 0) tb[SH_ONE].push_back(tile(j, 0, 0, 0, 1, 1, 1));
-            for (int y = 0; y < nb; ++y)
-                for (int x = 0; x < FORCE_BLOCKS; ++x) tb[SH_GEN].push_back(tile(j, x, y, 0, FORCE_BLOCKS, nb, 1));
+            if (d.loose)
+                for (int x = 0; x < 2 * lb; ++x) tb[SH_GEN].push_back(tile(j, x, 0, 0, 2 * lb, 1, 1));
+            else
+                for (int y = 0; y < nb; ++y)
+                    for (int x = 0; x < FORCE_BLOCKS; ++x) tb[SH_GEN].push_back(tile(j, x, y, 0, FORCE_BLOCKS, nb, 1));
             if (d.walls_move) {
                 for (int x = 0; x < 2 * lb; ++x) {
                     Tile t2 = tile(j, x, 0, 0, 2 * lb, 1, 1);

@@ -87,7 +87,7 @@ struct Dev {
     double *part;   // force partials: MAX_BODIES * FORCE_BLOCKS * 7 slots of 16 bytes
     int part128;    // partials are exact 128-bit fixed-point sums (double storage)
     double *ledger; // LG_COUNT
-    uint32_t *status;  // [0] sticky bits, [1], [2] the tail kernel's grid barrier
+    uint32_t *status;  // [0] sticky bits, [1], [2] the tail kernel's grid barrier, [3] obstacles among the initial classes
     uint8_t *rdec;  // remap scratch: decision per pending item
     double *rrho, *rphi;
     double *red;    // reduction scratch
@@ -109,6 +109,7 @@ struct Dev {
     int force_mean;    // rigid-body update driven by (F_n + F_{n-1}) / 2
     int nb_rule;       // interface cells without liquid (gas) neighbours empty (fill)
     int pair_ok;       // nx and N even: pairs of cells start on even elements of every plane
+    int loose;         // obstacle cells came with the initial classes: they may lie away from every body
 };
 
 // bulk-kernel variants: direct loads, per-thread cp.async pipeline over z,
@@ -141,7 +142,8 @@ enum {
     SH_BODY,       // (bodies): rigid-body step
     SH_ONE,        // (1) per tank with bodies: remap resolution
     SH_TANK,       // (1) per tank: counter reset
-    SH_GEN,        // liquid cells next to bodies: (FORCE_BLOCKS, bodies), kind 0; on moving walls: (2 lb), kind 1
+    SH_GEN,        // liquid cells next to bodies: (FORCE_BLOCKS, bodies), or next to any obstacle (Dev::loose):
+                   // (2 lb), kind 0; on moving walls: (2 lb), kind 1
     SH_COUNT
 };
 struct Shape {

@@ -831,6 +831,7 @@ __global__ void k_init(Dev d, const uint8_t *flags, const double *fill, const do
     d.flags[i] = (uint8_t)(c | fx | fyz | (d.walls_move && (fx | fyz) ? MOVING_FACE : 0));
     d.bid[i] = 0;
     d.cmark[i] = 0;
+    if (c == CL_O) d.status[3] = 1;
     if (c != CL_L && c != CL_I) return;
     double u[3] = {0.0, 0.0, 0.0};
     if (vel) {
@@ -1684,15 +1685,17 @@ __device__ __forceinline__ void book_wall(const Dev &d, double wacc) {
 // Cells next to a body: every liquid cell with an obstacle among its
 // neighbours lies in the range around that obstacle's body, so the blocks of
 // body vb.y look through its range (a cell next to two bodies is the lower
-// one's).  Nothing here depends on the bulk kernel, beside which it runs.
+// one's).  Obstacles of the initial classes may lie anywhere: in a tank with
+// such (Dev::loose) the blocks look through the whole grid.  Nothing here
+// depends on the bulk kernel, beside which it runs.
 template <int S, bool DENSE> __device__ __forceinline__ void near_body(const Dev &d, const VB &vb) {
-    const int bi = vb.y, owner = d.nb > 1 ? bi : -1;
+    const int bi = vb.y, owner = d.nb > 1 && !d.loose ? bi : -1;
     double wacc = 0.0;
     uint32_t count = 0;
-    int lo[3], hi[3];
-    near_range(d, d.bodies[bi], lo, hi);
-    const uint32_t ncell = (uint32_t)range_count(lo, hi);
-    walk_near<32>(d, lo, hi, ncell, vb, near_blocks(d, vb, ncell, DENSE), [](int fb) { return (fb & (CL_MASK | NB_OBST)) == (CL_L | NB_OBST); },
+    int lo[3] = {0, 0, 0}, hi[3] = {d.nx, d.ny, d.nz};
+    if (!d.loose) near_range(d, d.bodies[bi], lo, hi);
+    const uint32_t ncell = (uint32_t)range_count(lo, hi), blocks = d.loose ? vb.nx : near_blocks(d, vb, ncell, DENSE);
+    walk_near<32>(d, lo, hi, ncell, vb, blocks, [](int fb) { return (fb & (CL_MASK | NB_OBST)) == (CL_L | NB_OBST); },
                      [&](int x, int y, int z, long long i) {
                          typename Sto<S>::R fp[Q];
                          bool mine;
@@ -3606,6 +3609,18 @@ __global__ void k_bodies(const __grid_constant__ Dev d) {
 
 // ----------------------------------------------- C6: remap (Sec. 2.3, 2.4)
 
+// whether a cell lies in the body's range at its previous pose
+__device__ __forceinline__ bool in_prev_range(const Dev &d, const Body &b, int x, int y, int z) {
+    const int c[3] = {x, y, z}, n3[3] = {d.nx, d.ny, d.nz};
+    bool in = true;
+#pragma unroll
+    for (int k = 0; k < 3; ++k) {
+        int t = c[k] - b.plo[k];
+        if (d.periodic & (1u << k)) t = ((t % n3[k]) + n3[k]) % n3[k];
+        in = in && t >= 0 && t < b.phi[k] - b.plo[k];
+    }
+    return in;
+}
 // Which cells body vb.y covers and which it leaves with its new pose: the
 // obstacle set is not touched by the conversions, so the lists are made from
 // it and the two poses alone, beside the bulk kernel; remap_apply_body acts on
@@ -3645,7 +3660,7 @@ __device__ __forceinline__ void remap_scan_body(const Dev &d, const VB &vb) {
             if (!solid || own) {
                 const bool in = inside(d, b, x, y, z);
                 cover = !solid && in;
-                pend = own && !in;
+                pend = own && !in && (!d.loose || in_prev_range(d, b, x, y, z));
                 // of the bodies that cover a cell at once the first has it
 #pragma unroll 1
                 for (int j = 0; cover && j < bi; ++j) cover = !inside(d, d.bodies_new[j], x, y, z);
@@ -4136,7 +4151,7 @@ template <int S> struct Launch {
     }
     static void faces(const Dev &d, cudaStream_t st) { k_faces<S><<<LIST_BLOCKS, GEN_THREADS, 0, st>>>(d); }
     static void near(const Dev &d, cudaStream_t st) {
-        k_near<S><<<dim3(FORCE_BLOCKS, d.nb), GEN_THREADS, 0, st>>>(d);
+        k_near<S><<<d.loose ? dim3(4 * LIST_BLOCKS) : dim3(FORCE_BLOCKS, d.nb), GEN_THREADS, 0, st>>>(d);
     }
     static void forces(const Dev &d, cudaStream_t st) {
         k_forces<S><<<dim3(FORCE_BLOCKS, d.nb), FORCE_THREADS, 0, st>>>(d);
@@ -4215,10 +4230,10 @@ template <int S> struct Launch {
     // (launch_dependents).  Without, all run in one chain.  With
     // ev != nullptr event k is recorded before kernel slot k (step_names).
     static int step(const Dev &d, cudaStream_t st, const Sides *sides, cudaEvent_t *ev) {
-        const bool bodies = d.nb > 0, walls = d.walls_move != 0;
-        const int launches = 3 + (bodies ? 4 : 0) + (walls ? 1 : 0);
+        const bool bodies = d.nb > 0, obstacles = bodies || d.loose, walls = d.walls_move != 0;
+        const int launches = 3 + (bodies ? 3 : 0) + (obstacles ? 1 : 0) + (walls ? 1 : 0);
         if (sides) {
-            const bool used[SIDE_STREAMS] = {true, bodies, bodies || walls};
+            const bool used[SIDE_STREAMS] = {true, bodies, obstacles || walls};
             cudaEventRecord(sides->fork, st);
             for (int k = 0; k < SIDE_STREAMS; k += 2)
                 if (used[k]) cudaStreamWaitEvent(sides->st[k], sides->fork, 0);
@@ -4227,7 +4242,7 @@ template <int S> struct Launch {
                 cudaEventRecord(sides->fork2, st);
                 cudaStreamWaitEvent(sides->st[1], sides->fork2, 0);
             }
-            if (bodies) near(d, sides->st[2]);
+            if (obstacles) near(d, sides->st[2]);
             if (walls) faces(d, sides->st[2]);
             interface(d, sides->st[0]);
             if (bodies) launch_bodies(d, sides->st[1]);
@@ -4251,7 +4266,7 @@ template <int S> struct Launch {
         mark();
         bulk_any(d, st, false);
         mark();
-        if (bodies) near(d, st);
+        if (obstacles) near(d, st);
         if (walls) faces(d, st);
         mark();
         interface(d, st);
