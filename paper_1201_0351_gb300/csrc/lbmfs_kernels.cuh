@@ -2006,8 +2006,9 @@ __device__ __forceinline__ bool mbar_try_wait(uint64_t *bar, unsigned parity) {
 }
 // bounded wait: gives up after ~2^22 polls (each try_wait also suspends for a
 // hardware-chosen interval), far beyond any copy latency
-__device__ __forceinline__ bool mbar_wait(uint64_t *bar, unsigned parity) {
-    for (int it = 0; it < (1 << 22); ++it)
+constexpr int WAIT_POLLS = 1 << 22;
+template <int POLLS = WAIT_POLLS> __device__ __forceinline__ bool mbar_wait(uint64_t *bar, unsigned parity) {
+    for (int it = 0; it < POLLS; ++it)
         if (mbar_try_wait(bar, parity)) return true;
     return false;
 }
@@ -2338,8 +2339,16 @@ __device__ __forceinline__ void ring_tile(const Dev &d, char *stage, uint64_t *e
 // the consumers, then the producer, then the patching warp.  A stage goes
 // through four barriers: announced (its tile and class bytes are written),
 // landed (its copies are complete), full (patched), empty (in registers).
-// Every wait is bounded (mbar_wait); one that gives up ends its role with a
-// sticky status.
+// Every wait is bounded (ring_wait); one that gives up ends its warp's role, and
+// the others' by their own waits.  The block then waits for its copies in
+// flight and sets the sticky status of every tank that it had tiles of: any of
+// them may hold cells that were not stepped.
+#ifndef LBMFS_RING_POLLS
+#define LBMFS_RING_POLLS WAIT_POLLS  // polls of a role's wait (0: a test's waits that all give up)
+#endif
+__device__ __forceinline__ bool ring_wait(uint64_t *bar, unsigned parity) {
+    return __all_sync(0xffffffffu, mbar_wait<LBMFS_RING_POLLS>(bar, parity));
+}
 template <bool ZG, class TileOf, class DevOf>
 __device__ __forceinline__ void ring_run(uint32_t n, TileOf tile_of, DevOf dev_of) {
     using G = RingShape;
@@ -2361,20 +2370,19 @@ __device__ __forceinline__ void ring_run(uint32_t n, TileOf tile_of, DevOf dev_o
     }
     __syncthreads();
     bool ok = true;
+    uint32_t made = 0;  // tiles produced
     if (tid < G::WORKERS) {
         for (uint32_t k = 0;; ++k) {
             const int st = (int)(k % RING_STAGES);
             const unsigned ph = (k / RING_STAGES) & 1u;
-            if (!(mbar_wait(&full[st], ph) && mbar_wait(&landed[st], ph))) {
-                ok = false;
-                break;
-            }
+            ok = ring_wait(&full[st], ph) && ring_wait(&landed[st], ph);
+            if (!ok) break;
             const RingTile t = desc[st];
             if (t.tank < 0) break;
             ring_tile<ZG>(dev_of(t.tank), stages + st * G::STAGE, &empty[st], t.i0, tid);
         }
     } else if (tid < G::WORKERS + 32) {
-        uint32_t k = 0;  // tiles produced
+        uint32_t &k = made;
         int top_tank = -1, top = -1;  // highest plane with fluid of the current tank's tiles
         auto flush_top = [&]() {
             if (lane == 0 && top >= 0) atomicMax(dev_of(top_tank).ztop_wr, top);
@@ -2425,7 +2433,7 @@ __device__ __forceinline__ void ring_run(uint32_t n, TileOf tile_of, DevOf dev_o
                         top = -1;
                     }
                     top = max(top, min(d.nz - 1, (int)((i0 + G::TILE - 1) / ((uint32_t)d.nx * (uint32_t)d.ny))));
-                    if (k >= RING_STAGES) ok = __all_sync(0xffffffffu, mbar_wait(&empty[st], (k / RING_STAGES - 1) & 1u));
+                    if (k >= RING_STAGES) ok = ring_wait(&empty[st], (k / RING_STAGES - 1) & 1u);
                     if (!ok) break;
                     reinterpret_cast<uint4 *>(stage + G::COPY)[lane] = fl;
                     if (lane == 0) desc[st] = RingTile{tank, i0};
@@ -2456,8 +2464,8 @@ __device__ __forceinline__ void ring_run(uint32_t n, TileOf tile_of, DevOf dev_o
         }
         flush_top();
         const int st = (int)(k % RING_STAGES);
-        if (ok && k >= RING_STAGES) ok = __all_sync(0xffffffffu, mbar_wait(&empty[st], (k / RING_STAGES - 1) & 1u));
-        if (lane == 0) {
+        if (ok && k >= RING_STAGES) ok = ring_wait(&empty[st], (k / RING_STAGES - 1) & 1u);
+        if (ok && lane == 0) {
             desc[st] = RingTile{-1, 0};
             mbar_arrive(&said[st]);
             mbar_expect_tx(&landed[st], 0u);
@@ -2476,7 +2484,7 @@ __device__ __forceinline__ void ring_run(uint32_t n, TileOf tile_of, DevOf dev_o
             }
             return t.tank;
         };
-        ok = __all_sync(0xffffffffu, mbar_wait(&said[0], 0));
+        ok = ring_wait(&said[0], 0);
         int tank = ok ? begin(cur, 0) : -1;
         for (uint32_t k = 0; ok; ++k) {
             const int st = stage_of(k);
@@ -2485,7 +2493,7 @@ __device__ __forceinline__ void ring_run(uint32_t n, TileOf tile_of, DevOf dev_o
             const bool ready = more && __all_sync(0xffffffffu, mbar_try_wait(&said[stage_of(k + 1)], phase_of(k + 1)));
             if (ready) tank1 = begin(next, k + 1);
             if (more && cur.rows) {
-                ok = __all_sync(0xffffffffu, mbar_wait(&landed[st], phase_of(k)));
+                ok = ring_wait(&landed[st], phase_of(k));
                 char *stage = stages + st * G::STAGE;
                 cur.store(stage);
                 for (uint32_t r0 = 3u * RingPatch::U; r0 < cur.rows; r0 += 3u * RingPatch::U) {
@@ -2497,14 +2505,20 @@ __device__ __forceinline__ void ring_run(uint32_t n, TileOf tile_of, DevOf dev_o
             if (lane == 0) mbar_arrive(&full[st]);
             if (!more || !ok) break;
             if (!ready) {
-                ok = __all_sync(0xffffffffu, mbar_wait(&said[stage_of(k + 1)], phase_of(k + 1)));
+                ok = ring_wait(&said[stage_of(k + 1)], phase_of(k + 1));
                 tank1 = ok ? begin(next, k + 1) : -1;
             }
             cur = next;
             tank = tank1;
         }
     }
-    if (!ok) atomicOr(dev_of(0).status, ST_TIMEOUT);
+    if (__syncthreads_or(!ok)) {
+        if (tid >= G::WORKERS && tid < G::WORKERS + 32)
+            for (uint32_t k = made > RING_STAGES ? made - RING_STAGES : 0; k < made; ++k)
+                mbar_wait(&landed[k % RING_STAGES], (k / RING_STAGES) & 1u);
+        for (uint32_t e = blockIdx.x + (uint32_t)tid * gridDim.x; e < n; e += G::THREADS * gridDim.x)
+            atomicOr(dev_of(tile_of(e).tank).status, ST_TIMEOUT);
+    }
 }
 struct OneTank {
     const Dev &d;
