@@ -248,18 +248,17 @@ lbm_fs_status lbm_fs_create(const lbm_fs_params *p, lbm_fs **out) {
     // first and last rows reaches past the population array; the ring kernel's
     // tiles reach a z-plane, a row and a tile further (multiples of 16 bytes)
     size_t guard = GRID_GUARD;
-    if (p->storage != LBM_FS_F64)
-        guard += (((size_t)p->nx * p->ny + p->nx + 1024) * (p->storage == LBM_FS_F32 ? 4 : 2) + 255) & ~(size_t)255;
+    if (p->storage == LBM_FS_F16S) guard += (((size_t)p->nx * p->ny + p->nx + 1024) * 2 + 255) & ~(size_t)255;
     void *fA = h->alloc(fb + 2 * guard), *fB = h->alloc(fb + 2 * guard);
     if (fA) fA = (char *)fA + guard;
     if (fB) fB = (char *)fB + guard;
     double *pA = (double *)h->alloc(N * 8), *pB = (double *)h->alloc(N * 8);
     d.m = (double *)h->alloc(N * 8);
-    for (int k = 0; k < WL_COUNT; ++k) d.list[k] = (uint32_t *)h->alloc(N * 4);
-    // what a step reads of the one before it: second copies of some lists, of
-    // the counters and of the body records
-    uint32_t *list2[PREV_LISTS];
-    for (int k = 0; k < PREV_LISTS; ++k) list2[k] = (uint32_t *)h->alloc(N * 4);
+    for (int k : {WL_FILLED, WL_EMPTIED, WL_COVER}) d.list[k] = (uint32_t *)h->alloc(N * 4);
+    // what a step reads of the one before it, in turn: the lists prev_wl(k), the
+    // counters and the body records
+    uint32_t *lists[2];
+    for (auto &l : lists) l = (uint32_t *)h->alloc((size_t)N * 4 * PREV_LISTS);
     d.cnt = (uint32_t *)h->alloc(2 * CN_COUNT * 4);
     d.bodies = (Body *)h->alloc(2 * sizeof(Body) * MAX_BODIES);
     const size_t pfb = p->storage == LBM_FS_F64 ? 0 : (size_t)N * 4;
@@ -268,16 +267,13 @@ lbm_fs_status lbm_fs_create(const lbm_fs_params *p, lbm_fs **out) {
     d.part128 = p->storage == LBM_FS_F64;
     d.ledger = (double *)h->alloc(sizeof(double) * LG_COUNT);
     d.status = (uint32_t *)h->alloc(16);
-    d.rdec = (uint8_t *)h->alloc(nb4);
-    d.rrho = (double *)h->alloc(N * 8);
-    d.rphi = (double *)h->alloc(N * 8);
     d.red = (double *)h->alloc(sizeof(double) * LIST_BLOCKS);
     double *wallv = (double *)h->alloc(sizeof(double) * 18);
     d.wallv = wallv;
     int *ztop = (int *)h->alloc(sizeof(int) * 2);
     for (void *ptr : h->allocs)
         if (!ptr) return bail(fail(LBM_FS_ENOMEM, "device allocation failed%s"));
-    if (h->allocs.size() != 21 + WL_COUNT + PREV_LISTS) return bail(fail(LBM_FS_ENOMEM, "device allocation failed%s"));
+    if (h->allocs.size() != 23) return bail(fail(LBM_FS_ENOMEM, "device allocation failed%s"));
     if (h->misaligned) return bail(fail(LBM_FS_EINVAL, "dev_alloc must return 16-byte aligned memory%s"));
     d.walls_move = 0;
     for (int f = 0; f < 6; ++f)
@@ -319,9 +315,20 @@ lbm_fs_status lbm_fs_create(const lbm_fs_params *p, lbm_fs **out) {
         e.cnt = d.cnt + k * CN_COUNT;
         e.pcnt = d.cnt + (k ^ 1) * CN_COUNT;
         for (int j = 0; j < PREV_LISTS; ++j) {
-            if (k) e.list[prev_wl(j)] = list2[j];
-            e.plist[j] = k ? d.list[prev_wl(j)] : list2[j];
+            e.list[prev_wl(j)] = lists[k] + (size_t)N * j;
+            e.plist[j] = lists[k ^ 1] + (size_t)N * j;
         }
+        // What the conversions and the remap need for themselves lies in arrays
+        // that the step has read by then: its previous step's lists (by the
+        // interface kernel; next written by the next step) and its source fill
+        // levels (by the force and interface kernels).  With them on their own
+        // a cell took 21 bytes more.
+        static_assert(PREV_LISTS == 4, "an entry's 16 bytes: rphi 8, receivers 4, rdec 1");
+        uint32_t *spent = lists[k ^ 1];
+        e.rphi = (double *)spent;
+        e.list[WL_RECV] = spent + (size_t)N * 2;
+        e.rdec = (uint8_t *)(spent + (size_t)N * 3);
+        e.rrho = e.phisrc;
     }
     h->d[0].ztop_rd = ztop;
     h->d[0].ztop_wr = ztop + 1;
