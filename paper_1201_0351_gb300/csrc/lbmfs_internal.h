@@ -38,8 +38,8 @@ constexpr int ZTOP_MARGIN = 4;
 // worklists
 enum { WL_IFACE = 0, WL_FILLED, WL_EMPTIED, WL_NEWG, WL_NEWL, WL_RECV, WL_PEND, WL_COVER, WL_COUNT };
 // counters of a step: one per worklist, then the liquid cells next to a body or
-// on a moving wall
-enum { CN_NEAR = WL_COUNT, CN_COUNT = 16 };
+// on a moving wall, and the blocks of the tail that work on long lists
+enum { CN_NEAR = WL_COUNT, CN_TEAM_NAMES, CN_TEAM_SIZE, CN_COUNT = 16 };
 // lists of the previous step that hold every cell that may be interface now:
 // the interface cells its bulk pass met and those its conversions and its
 // remap may have added

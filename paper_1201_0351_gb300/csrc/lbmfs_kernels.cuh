@@ -3853,85 +3853,150 @@ __global__ void __launch_bounds__(REMAP_THREADS) k_remap_resolve(const __grid_co
 // Measured, us, sum of the ten kernels timed one by one and this launch: 64^3
 // without bodies 53 and 5; 130x40x40 117 and 40; 385x190x127 143 and 55;
 // 768x384x256 172 and 72.
-//  - CLUSTER: one cluster of TAIL_CLUSTER blocks with the hardware's cluster
-//    barrier, for tanks whose lists are short;
+//  - CLUSTER, for tanks up to TAIL_CLUSTER_CELLS per plane: short lists by the
+//    first cluster of TAIL_CLUSTER blocks with the hardware's cluster barrier,
+//    the launch's other blocks leave at once (which costs nothing measurable);
+//    long ones, of a splashing tank, by all blocks that have started by then
+//    (tail_team);
 //  - else a cooperative grid with a barrier in global memory, for large tanks
 //    (hundreds to thousands of conversions a step want all SMs).
 constexpr int TAIL_CLUSTER = 8, TAIL_BLOCKS = 152;
+// Clusters launched: one per 65536 cells, at most the 15 that are resident at
+// once (a tank of 32^3 cells has no list worth more than one).
+constexpr int TAIL_CLUSTERS = 15;
+constexpr long long TAIL_CLUSTER_PER = 65536;
 // (1024 threads of the cluster's blocks give its short lists a warp each; on the
 // grid they only make the block barriers longer: 768x384x256 103 us against 89)
 constexpr int tail_threads(bool cluster) { return cluster ? 1024 : 512; }
+// Entries (conversions, cells covered and left) up to which the first cluster
+// works alone.  Measured, us of this launch, alone and with all blocks: 170
+// entries 39 and 49, 210 41 and 48, 440 (FP32) 48 and 52, 450 (FP64) 84 and 60,
+// 460 61 and 55, 840 64 and 49, 2900 199 and 67, 10900 677 and 132 (as ten
+// kernels, timed one by one: 204 and 287 for the last two).
+#ifndef LBMFS_TAIL_SHORT
+#define LBMFS_TAIL_SHORT 512
+#endif
+constexpr uint32_t TAIL_SHORT = LBMFS_TAIL_SHORT;
 
-// poll limit of the grid barrier: far beyond the time that the
-// resident blocks of a cooperative launch can be apart
+// poll limit of the waits in global memory: far beyond the time that blocks
+// which are all running can be apart
 constexpr unsigned BARRIER_POLLS = 1u << 24;
-template <bool CLUSTER> __device__ __forceinline__ bool tail_barrier(const Dev &d) {
-    if constexpr (CLUSTER) {
+__device__ __forceinline__ unsigned ld_acquire(const unsigned *p) {
+    unsigned v;
+    asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
+    return v;
+}
+// Barrier of the phases: of the cluster, or through global memory of the vb.nx
+// blocks that work on them.
+__device__ __forceinline__ bool tail_barrier(const Dev &d, const VB &vb, bool cluster) {
+    if (cluster) {
         // (the form without .aligned: the warps may arrive diverged)
         asm volatile("barrier.cluster.arrive.release;" ::: "memory");
         asm volatile("barrier.cluster.wait.acquire;" ::: "memory");
         return true;
-    } else {
-        __shared__ int s_ok;
-        __syncthreads();
-        if (threadIdx.x == 0) {
-            unsigned *count = d.status + 1, *turn = d.status + 2;
-            unsigned now;
-            asm volatile("ld.relaxed.gpu.global.u32 %0, [%1];" : "=r"(now) : "l"(turn) : "memory");
-            __threadfence();
-            bool ok = true;
-            if (atomicAdd(count, 1u) == gridDim.x - 1) {
-                *count = 0;
-                __threadfence();
-                atomicAdd(turn, 1u);
-            } else {
-                unsigned seen = now, polls = 0;
-                while (seen == now && polls < BARRIER_POLLS) {
-                    asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(seen) : "l"(turn) : "memory");
-                    ++polls;
-                }
-                ok = seen != now;
-                if (!ok) atomicOr(d.status, ST_TIMEOUT);
-            }
-            __threadfence();
-            s_ok = ok;
-        }
-        __syncthreads();
-        return s_ok != 0;
     }
+    __shared__ int s_ok;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        unsigned *count = d.status + 1, *turn = d.status + 2;
+        unsigned now;
+        asm volatile("ld.relaxed.gpu.global.u32 %0, [%1];" : "=r"(now) : "l"(turn) : "memory");
+        __threadfence();
+        bool ok = true;
+        if (atomicAdd(count, 1u) == vb.nx - 1) {
+            *count = 0;
+            __threadfence();
+            atomicAdd(turn, 1u);
+        } else {
+            unsigned seen = now, polls = 0;
+            for (; seen == now && polls < BARRIER_POLLS; ++polls) seen = ld_acquire(turn);
+            ok = seen != now;
+            if (!ok) atomicOr(d.status, ST_TIMEOUT);
+        }
+        __threadfence();
+        s_ok = ok;
+    }
+    __syncthreads();
+    return s_ok != 0;
 }
+// The blocks of an ordinary launch that work on long lists together: those that
+// have come by the time the first of them closes the list of names, a few us
+// after it started.  They are all running, so they can wait for one another
+// whatever else the GPU is doing; blocks that come later leave.  The names are
+// in the step's own counters, which are zero when it starts.  Sets the block's
+// number and the number of blocks; false: not one of them.
+constexpr unsigned TEAM_CLOSED = 1u << 31, TEAM_JOIN_POLLS = 16;
+__device__ __forceinline__ bool tail_team(const Dev &d, VB &vb) {
+    __shared__ unsigned s_rank, s_team;
+    if (threadIdx.x == 0) {
+        unsigned *names = d.cnt + CN_TEAM_NAMES, *size = d.cnt + CN_TEAM_SIZE;
+        const unsigned rank = atomicAdd(names, 1u);
+        unsigned team = 0;
+        if (rank == 0) {
+            for (unsigned polls = 0; polls < TEAM_JOIN_POLLS && ld_acquire(names) < gridDim.x; ++polls) {}
+            team = atomicOr(names, TEAM_CLOSED);
+            atomicExch(size, team);
+        } else if (!(rank & TEAM_CLOSED)) {
+            for (unsigned polls = 0; team == 0 && polls < BARRIER_POLLS; ++polls) team = ld_acquire(size);
+            if (team == 0) atomicOr(d.status, ST_TIMEOUT);
+        }
+        s_rank = rank;
+        s_team = team;
+    }
+    __syncthreads();
+    vb.x = s_rank;
+    vb.nx = s_team;
+    return s_team != 0;
+}
+
+__device__ __forceinline__ uint32_t tail_conversions(const Dev &d) { return wl_count(d, WL_FILLED) + wl_count(d, WL_EMPTIED); }
+__device__ __forceinline__ uint32_t tail_moved(const Dev &d) {
+    return d.nb > 0 ? wl_count(d, WL_COVER) + wl_count(d, WL_PEND) : 0u;
+}
+__device__ __forceinline__ uint32_t tail_items(const Dev &d) { return tail_conversions(d) + tail_moved(d); }
 
 template <int S, bool CLUSTER>
 __global__ void __launch_bounds__(tail_threads(CLUSTER)) k_tail(const __grid_constant__ Dev d) {
-    const VB vb = vb_own();
+    VB vb = vb_own();
+    if (CLUSTER && vb.x >= TAIL_CLUSTER) {
+        // (one thread looks: the counters of all 120 blocks' threads queueing at
+        // one address cost 3 us)
+        if (!__syncthreads_or(threadIdx.x == 0 && tail_items(d) > TAIL_SHORT)) return;
+    }
     if (vb.x == 0) {
         // for the next step: its counters (this step's previous ones), and the
         // slot its bulk pass records the fluid top in
         if (threadIdx.x < CN_COUNT) d.pcnt[threadIdx.x] = 0;
         if (threadIdx.x == 0) *d.ztop_rd = -1;
     }
-    const bool conv = wl_count(d, WL_FILLED) + wl_count(d, WL_EMPTIED) > 0;
-    const bool remap = d.nb > 0 && wl_count(d, WL_COVER) + wl_count(d, WL_PEND) > 0;
-    if (conv) {
+    const uint32_t nconv = tail_conversions(d), nmoved = tail_moved(d);
+    bool cluster = false;
+    if (CLUSTER && nconv + nmoved <= TAIL_SHORT) {
+        vb.nx = TAIL_CLUSTER;
+        cluster = true;
+    } else if (CLUSTER && !tail_team(d, vb)) {
+        return;
+    }
+    if (nconv) {
         // new interface cells are marked (the two lists mark disjoint cells)
         conv_filled_body(d, vb);
         conv_emptied_body(d, vb);
-        if (!tail_barrier<CLUSTER>(d)) return;
+        if (!tail_barrier(d, vb, cluster)) return;
         // their states; the converted cells' shares and who receives them
         // (from the classes before and the marks)
         conv_init_body<S>(d, vb);
         conv_claim_body<S>(d, vb);
-        if (!tail_barrier<CLUSTER>(d)) return;
+        if (!tail_barrier(d, vb, cluster)) return;
         conv_flags_body(d, vb);
         conv_excess_body<S>(d, vb);
-        if (!tail_barrier<CLUSTER>(d)) return;
+        if (!tail_barrier(d, vb, cluster)) return;
         conv_finish_body(d, vb);
     }
-    if (remap) {
+    if (nmoved) {
         remap_apply_body<S>(d, vb);
-        if (!tail_barrier<CLUSTER>(d)) return;
+        if (!tail_barrier(d, vb, cluster)) return;
         if (vb.x == 0) remap_resolve_body<S>(d, vb);
-        if (!tail_barrier<CLUSTER>(d)) return;
+        if (!tail_barrier(d, vb, cluster)) return;
         nb_update_body(d, vb);
     }
 }
@@ -4129,9 +4194,10 @@ inline int bulk_planes(int storage, unsigned gx, int nz) {
     return blocks(2) >= 2000 ? 2 : 1;
 }
 
-// largest xy-plane whose tail runs as one cluster
-// (measured with both forms, us: 385x190 plane 55 as a cluster, 65 as a grid;
-// 768x384 109 and 82; a tank whose lists are empty 5 and 8)
+// largest xy-plane whose tail starts as clusters; with a larger one hundreds of
+// conversions a step are the rule (calm wave tanks measured with both forms, us:
+// 385x190 plane 55 as a cluster, 65 as a grid; 768x384 109 and 82; a tank whose
+// lists are empty 5 and 8)
 constexpr long long TAIL_CLUSTER_CELLS = 131072;
 
 constexpr int STEP_SLOTS = 7, BATCH_SLOTS = 17;  // kernel slots of a step (names below)
@@ -4217,7 +4283,7 @@ template <int S> struct Launch {
         c.attrs = &a;
         c.numAttrs = 1;
         if ((long long)d.nx * d.ny <= TAIL_CLUSTER_CELLS) {
-            c.gridDim = dim3(TAIL_CLUSTER);
+            c.gridDim = dim3(TAIL_CLUSTER * std::max(1, (int)std::min<long long>(TAIL_CLUSTERS, d.N / TAIL_CLUSTER_PER)));
             c.blockDim = dim3(tail_threads(true));
             a.id = cudaLaunchAttributeClusterDimension;
             a.val.clusterDim.x = TAIL_CLUSTER;
