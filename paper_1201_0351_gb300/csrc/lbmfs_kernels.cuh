@@ -1129,20 +1129,39 @@ __device__ __forceinline__ long long lane_nbr(const Dev &d, int lane, int x, int
 // Cells whose obstacle status changed this step (covered, uncovered): the bit
 // of each and of its 18 neighbours is refreshed.
 // A warp per (listed cell, direction): the target is the cell itself (q = 0) or
-// its neighbour in direction q, lane p looks at the target's neighbour p.
-// Targets refreshed twice get the same value (the classes do not change in this
-// kernel).
+// its neighbour in direction q, lane p looks at the target's neighbour p; for
+// long lists, of which each warp would take more than NB_WARP in turn, a thread
+// per target.  Targets refreshed twice get the same value (the classes do not
+// change in this kernel).  Measured, us, four 96^3 tanks of a batch with about
+// 18000 targets each (on 18 blocks): 99 and 26.
+#ifndef LBMFS_NB_WARP
+#define LBMFS_NB_WARP 8
+#endif
+constexpr uint32_t NB_WARP = LBMFS_NB_WARP;
+__device__ __forceinline__ long long nb_target(const Dev &d, uint32_t it, uint32_t nc) {
+    const uint32_t e = it / Q;
+    const int q = (int)(it - e * Q);
+    const long long c = e < nc ? (long long)d.list[WL_COVER][e] : (long long)d.list[WL_PEND][e - nc];
+    if (q == 0) return c;
+    int x, y, z;
+    coords(d, c, x, y, z);
+    return nbr(d, x, y, z, dir_x(q), dir_y(q), dir_z(q));
+}
 __device__ __forceinline__ void nb_update_body(const Dev &d, const VB &vb) {
     const uint32_t nc = wl_count(d, WL_COVER), n = (nc + wl_count(d, WL_PEND)) * Q;
+    const uint32_t warps = vb.nx * (blockDim.x >> 5);
     const int lane = threadIdx.x & 31;
-    for (uint32_t it = (threadIdx.x >> 5) * vb.nx + vb.x; it < n; it += vb.nx * (blockDim.x >> 5)) {
-        const uint32_t e = it / Q;
-        const int q = (int)(it - e * Q);
-        const long long c = e < nc ? (long long)d.list[WL_COVER][e] : (long long)d.list[WL_PEND][e - nc];
-        int x, y, z;
-        coords(d, c, x, y, z);
-        const long long t = q > 0 ? nbr(d, x, y, z, dir_x(q), dir_y(q), dir_z(q)) : c;
+    if (n > NB_WARP * warps) {
+        for (uint32_t it = vb.x * blockDim.x + threadIdx.x; it < n; it += vb.nx * blockDim.x) {
+            const long long t = nb_target(d, it, nc);
+            if (t >= 0) nb_refresh(d, t);
+        }
+        return;
+    }
+    for (uint32_t it = (threadIdx.x >> 5) * vb.nx + vb.x; it < n; it += warps) {
+        const long long t = nb_target(d, it, nc);
         if (t < 0) continue;
+        int x, y, z;
         coords(d, t, x, y, z);
         const bool obst = cls(d, lane_nbr(d, lane, x, y, z)) == CL_O;
         const bool nb = __any_sync(0xffffffffu, obst);
@@ -3713,16 +3732,107 @@ __device__ __forceinline__ void remap_apply_body(const Dev &d, const VB &vb) {
 template <int S>
 __global__ void k_remap_apply(const __grid_constant__ Dev d) { remap_apply_body<S>(d, vb_own()); }
 
+// What a pending cell becomes (Sec. 2.4), from its numbers of liquid, interface
+// and gas neighbours and their sums of density and fill level.
+__device__ __forceinline__ void resolve_decide(const Dev &d, uint32_t it, int nL, int nI, int nG, double sr, double sp) {
+    uint8_t dec = 0;
+    if (nL > 0 && nG > 0) {
+        dec = CL_I;
+        d.rrho[it] = sr / (nL + nI);
+        d.rphi[it] = nI > 0 ? sp / nI : 0.5;
+    } else if (nG == 0 && nL + nI > 0) {
+        dec = CL_L;
+        d.rrho[it] = sr / (nL + nI);
+    } else if (nL == 0 && nG > 0) {
+        dec = CL_G;
+    }
+    d.rdec[it] = dec;
+}
+// The two halves of a pass for a long list, a thread per pending cell: the
+// decision, and the cells that have one (false: undecided yet).
+template <int S> __device__ __forceinline__ void resolve_look(const Dev &d, uint32_t it) {
+    const long long i = d.list[WL_PEND][it];
+    if (!(d.cmark[i] & MK_PEND)) {
+        d.rdec[it] = 0;
+        return;
+    }
+    int x, y, z;
+    coords(d, i, x, y, z);
+    // marks and classes, then the neighbours in q order
+    unsigned mL = 0, mI = 0, mG = 0;
+#pragma unroll 6
+    for (int q = 1; q < Q; ++q) {
+        const long long yi = nbr(d, x, y, z, dir_x(q), dir_y(q), dir_z(q));
+        const int c = yi < 0 || (d.cmark[yi] & MK_PEND) ? 0 : clsv(d, yi);
+        mL |= (c == CL_L ? 1u : 0u) << q;
+        mI |= (c == CL_I ? 1u : 0u) << q;
+        mG |= (c == CL_G ? 1u : 0u) << q;
+    }
+    double sr = 0.0, sp = 0.0;
+    for (unsigned m = mL | mI; m; m &= m - 1) {
+        const int q = __ffs(m) - 1;
+        const long long yi = nbr(d, x, y, z, dir_x(q), dir_y(q), dir_z(q));
+        sr += cell_density<S>(d, d.fdst, yi);
+        if (mI & (1u << q)) sp += d.phidst[yi];
+    }
+    resolve_decide(d, it, __popc(mL), __popc(mI), __popc(mG), sr, sp);
+}
+template <int S> __device__ __forceinline__ bool resolve_set(const Dev &d, uint32_t it, bool last) {
+    const long long i = d.list[WL_PEND][it];
+    if (!(d.cmark[i] & MK_PEND)) return true;
+    int dec = d.rdec[it];
+    if (dec == 0 && last) dec = CL_G;
+    if (dec == 0) return false;
+    d.cmark[i] = MK_FRESH;
+    set_cls(d, i, dec);
+    if (dec == CL_G) return true;
+    int x, y, z;
+    coords(d, i, x, y, z);
+    if (z > *d.ztop_wr + ZTOP_MARGIN) atomicOr(d.status, ST_TOP);
+    double p[3] = {x + 0.5, y + 0.5, z + 0.5}, uw[3];
+    body_velocity_at(d, d.bodies_new[d.bid[i]], p, uw);
+    const double rho = d.rrho[it];
+    float dv0 = 0.0f, rest = 0.0f;  // (as warp_store_cell rounds them)
+#pragma unroll 1
+    for (int q = 0; q < Q; ++q) {
+        const double f = feq_lane(q, rho, uw);
+        if constexpr (S == 0) {
+            Sto<0>::st(d.fdst, q, i, d.N, f);
+        } else {
+            const float dv = (float)(f - (q == 0 ? wd(0) : (q <= 6 ? wd(1) : wd(7))));
+            if constexpr (S == 1) Sto<1>::st(d.fdst, q, i, d.N, dv);
+            else if (q == 0) dv0 = dv;
+            else rest += dv - Sto<2>::st_one(d.fdst, q, i, d.N, dv);
+        }
+    }
+    if constexpr (S == 2) Sto<2>::st_one(d.fdst, 0, i, d.N, dv0 + rest);
+    const double dens = cell_density<S>(d, d.fdst, i);
+    if (dec == CL_I) set_mass<S>(d, i, d.rphi[it] * rho, dens);
+    d.rrho[it] = dens;  // as stored, for what follows
+    return true;
+}
+
 // Jacobi passes of the obstacle-to-fluid rule over the pending cells, closure,
-// uncovered-mass ledger (one block)
+// uncovered-mass ledger (one block).  Up to RESOLVE_WARP pending cells a warp
+// each, whose latency is short; more by a thread each: a warp's double
+// operations hold their scheduler as long for one cell as for 32.  Measured, us
+// of the tail with 36, 72, 150, 366 and 1145 pending cells: a warp each 75, 98,
+// 169, 350 and 1032, a thread each 69, 77, 94, 127 and 307.
+#ifndef LBMFS_RESOLVE_WARP
+#define LBMFS_RESOLVE_WARP 36
+#endif
+constexpr uint32_t RESOLVE_WARP = LBMFS_RESOLVE_WARP;
 template <int S>
 __device__ __forceinline__ void remap_resolve_body(const Dev &d, const VB &vb) {
     uint32_t n = wl_count(d, WL_PEND);
     if (n == 0) return;
     __shared__ int s_any;
+    const bool wide = n > RESOLVE_WARP;
     for (int pass = 0; pass < 4; ++pass) {
+        if (wide)
+            for (uint32_t it = threadIdx.x; it < n; it += blockDim.x) resolve_look<S>(d, it);
         // a warp per pending cell, lane q its neighbour in direction q
-        for (uint32_t it = threadIdx.x >> 5; it < n; it += blockDim.x >> 5) {
+        for (uint32_t it = threadIdx.x >> 5; !wide && it < n; it += blockDim.x >> 5) {
             const int lane = threadIdx.x & 31;
             const long long i = d.list[WL_PEND][it];
             if (!(d.cmark[i] & MK_PEND)) {
@@ -3746,24 +3856,14 @@ __device__ __forceinline__ void remap_resolve_body(const Dev &d, const VB &vb) {
             double sr = 0.0, sp = 0.0;
             for (unsigned m = mL | mI; m; m &= m - 1) sr += __shfl_sync(full, r, __ffs(m) - 1);
             for (unsigned m = mI; m; m &= m - 1) sp += __shfl_sync(full, ph, __ffs(m) - 1);
-            if (lane == 0) {
-                uint8_t dec = 0;
-                if (nL > 0 && nG > 0) {
-                    dec = CL_I;
-                    d.rrho[it] = sr / (nL + nI);
-                    d.rphi[it] = nI > 0 ? sp / nI : 0.5;
-                } else if (nG == 0 && nL + nI > 0) {
-                    dec = CL_L;
-                    d.rrho[it] = sr / (nL + nI);
-                } else if (nL == 0 && nG > 0) {
-                    dec = CL_G;
-                }
-                d.rdec[it] = dec;
-            }
+            if (lane == 0) resolve_decide(d, it, nL, nI, nG, sr, sp);
         }
         if (threadIdx.x == 0) s_any = 0;
         __syncthreads();
-        for (uint32_t it = threadIdx.x >> 5; it < n; it += blockDim.x >> 5) {
+        if (wide)
+            for (uint32_t it = threadIdx.x; it < n; it += blockDim.x)
+                if (!resolve_set<S>(d, it, pass == 3)) s_any = 1;
+        for (uint32_t it = threadIdx.x >> 5; !wide && it < n; it += blockDim.x >> 5) {
             const int lane = threadIdx.x & 31;
             const long long i = d.list[WL_PEND][it];
             const bool open = d.cmark[i] & MK_PEND;

@@ -9,7 +9,7 @@ import pytest
 
 from paper_1201_0351_gb300 import inputs as I
 
-from parity import assert_f64_parity, run_both
+from parity import assert_f64_parity, macro_errors, run_both
 
 pytestmark = pytest.mark.gpu
 
@@ -48,6 +48,16 @@ def large_moving_box(n):
     box = I.Box(center=(n / 2 + 0.1, n / 2 + 0.2, n / 2), half=(0.31 * n, 0.27 * n, 0.23 * n), density_ratio=50.0,
                 quat=I.heel_quat(17.0, (0.0, 0.6, 0.8)), vel=(0.12, 0.06, 0.0), mode=I.MODE_FREE)
     return I.Scenario("moving_box", n, n, n, 7, 0.8, (0.0, 0.0, 0.0), (0.0, 0.0, 0.0), 1.0, 1e-2, flags, fill, rho,
+                      [box], 0)
+
+
+def half_immersed_box(n):
+    """a fast box through the surface of a half-full tank: cells that it leaves
+    become liquid, interface and gas, about a hundred a step"""
+    flags, fill, rho = I.hydrostatic_tank(n, n, n, lambda X, Y: 0.5 * n + 0.3, 1e-5, 1.0, 3)
+    box = I.Box(center=(n / 2 + 0.1, n / 2 + 0.2, n / 2), half=(0.31 * n, 0.27 * n, 0.23 * n), density_ratio=50.0,
+                quat=I.heel_quat(17.0, (0.0, 0.6, 0.8)), vel=(0.12, 0.06, 0.0), mode=I.MODE_FREE)
+    return I.Scenario("half_immersed", n, n, n, 3, 0.8, (0.0, 0.0, -1e-5), (0.0, 0.0, 0.0), 1.0, 1e-2, flags, fill, rho,
                       [box], 0)
 
 
@@ -90,6 +100,39 @@ def test_long_lists_equal_the_batch(scene, storage):
             assert np.array_equal(a[key], other[key]), key
         for key in ("n_interface", "n_filled", "n_emptied", "n_new_from_gas", "n_new_from_liquid", "n_pending"):
             assert s[key] == st[key], key
+
+
+PENDING_BY_WARPS = 36  # pending cells up to which each has a warp
+
+
+@pytest.mark.parametrize("scene", ["half_immersed", "inside"])
+def test_many_uncovered_cells_against_the_oracle(scene):
+    """the remap's rule for long pending lists, a thread per cell"""
+    sc = half_immersed_box(44) if scene == "half_immersed" else large_moving_box(40)
+    g, o, gb, ob, gs, ref = run_both(sc, 6)
+    assert gs["n_pending"] > PENDING_BY_WARPS
+    assert_f64_parity(g, o, gb, ob)
+    led = ref.ledger()
+    for key in ("covered", "uncovered"):
+        assert abs(gs[key] - led[key]) <= 1e-11 * led[key], key
+
+
+@pytest.mark.parametrize("storage", ["f32", "f16s"])
+def test_many_uncovered_cells_in_the_float_storages(storage):
+    """alone and in a batch bit for bit; density within 2e-3 and classes of the
+    oracle, the bounds of the parity tests"""
+    import oracle
+
+    sc = half_immersed_box(44)
+    a, s, _ = _alone(sc, storage, 6)
+    b, t = _batched(sc, storage, 6)
+    assert s["n_pending"] > PENDING_BY_WARPS and s["status"] == 0
+    for key in ("flags", "f", "fill", "mass"):
+        assert np.array_equal(a[key], b[key]), key
+    ref = oracle.OracleSim(sc)
+    ref.step(6)
+    e = macro_errors(a, ref.fields(want_f=True))
+    assert e["flag_diff"] == 0 and e["rho"] <= 2e-3, e
 
 
 def test_long_lists_against_the_oracle():
