@@ -4,6 +4,7 @@
 #include <stdio.h>
 #include <string.h>
 
+#include <algorithm>
 #include <cmath>
 #include <cstdlib>
 #include <string>
@@ -265,6 +266,7 @@ lbm_fs_status lbm_fs_create(const lbm_fs_params *p, lbm_fs **out) {
     float *pfA = (float *)h->alloc(pfb), *pfB = (float *)h->alloc(pfb);
     d.part = (double *)h->alloc(2 * sizeof(double) * MAX_BODIES * FORCE_BLOCKS * 7);
     d.part128 = p->storage == LBM_FS_F64;
+    d.range_blocks = FORCE_BLOCKS;
     d.ledger = (double *)h->alloc(sizeof(double) * LG_COUNT);
     d.status = (uint32_t *)h->alloc(16);
     d.red = (double *)h->alloc(sizeof(double) * LIST_BLOCKS);
@@ -406,11 +408,26 @@ lbm_fs_status lbm_fs_add_box(lbm_fs *h, const lbm_fs_box *b, int32_t *out_id) {
     hb.mode = b->mode;
     hb.shape = b->shape;
     int id = h->nb;
+    // the cells of its range, for the launches that look through it
+    double range = 1.0;
+    const double *q = b->quat, R[9] = {1 - 2 * (q[2] * q[2] + q[3] * q[3]), 2 * (q[1] * q[2] - q[0] * q[3]), 2 * (q[1] * q[3] + q[0] * q[2]),
+                                       2 * (q[1] * q[2] + q[0] * q[3]), 1 - 2 * (q[1] * q[1] + q[3] * q[3]), 2 * (q[2] * q[3] - q[0] * q[1]),
+                                       2 * (q[1] * q[3] - q[0] * q[2]), 2 * (q[2] * q[3] + q[0] * q[1]), 1 - 2 * (q[1] * q[1] + q[2] * q[2])};
+    const int n3[3] = {h->p.nx, h->p.ny, h->p.nz};
+    for (int k = 0; k < 3; ++k) {
+        double e = b->half[0];
+        if (b->shape == 0) e = fabs(R[3 * k]) * b->half[0] + fabs(R[3 * k + 1]) * b->half[1] + fabs(R[3 * k + 2]) * b->half[2];
+        range *= std::min(2.0 * e + 5.0, (double)n3[k]);
+    }
+    const int blocks = (int)std::min<double>(range / RANGE_CELLS, RANGE_BLOCKS_MAX);
     cudaStream_t st = h->st;
     CK(cudaMemcpyAsync(h->d[h->cur].bodies + id, &hb, sizeof hb, cudaMemcpyHostToDevice, st));
     CK(cudaStreamSynchronize(st));
     h->nb++;
-    for (int k = 0; k < 2; ++k) h->d[k].nb = h->nb;
+    for (int k = 0; k < 2; ++k) {
+        h->d[k].nb = h->nb;
+        h->d[k].range_blocks = std::max(h->d[k].range_blocks, blocks);
+    }
     h->ks.body_prepare(h->d[h->cur], id, st);
     h->ks.map_body(h->d[h->cur], id, h->started ? 1 : 0, st);
     CK(cudaGetLastError());

@@ -139,6 +139,9 @@ lbm_fs_status build(lbm_fs_batch *b) {
             tb[SH_TANK].push_back(tile(j, 0, 0, 0, 1, 1, 1));
             for (int y = 0; y < nb; ++y)
                 for (int x = 0; x < FORCE_BLOCKS; ++x) tb[SH_FORCE].push_back(tile(j, x, y, 0, FORCE_BLOCKS, nb, 1));
+            const int rb = d.range_blocks;
+            for (int y = 0; y < nb; ++y)
+                for (int x = 0; x < rb; ++x) tb[SH_SCAN].push_back(tile(j, x, y, 0, rb, nb, 1));
             if (t->p.storage == LBM_FS_F16S) {
                 const long long tiles = (d.N + RING_TILE - 1) / RING_TILE;
                 for (long long k = 0; k < tiles; ++k) tb[SH_BULK].push_back(tile(j, (int)(k & 0xffff), (int)(k >> 16), 0, 1, 1, 1));
@@ -158,7 +161,7 @@ lbm_fs_status build(lbm_fs_batch *b) {
                 for (int x = 0; x < 2 * lb; ++x) tb[SH_GEN].push_back(tile(j, x, 0, 0, 2 * lb, 1, 1));
             else
                 for (int y = 0; y < nb; ++y)
-                    for (int x = 0; x < FORCE_BLOCKS; ++x) tb[SH_GEN].push_back(tile(j, x, y, 0, FORCE_BLOCKS, nb, 1));
+                    for (int x = 0; x < rb; ++x) tb[SH_GEN].push_back(tile(j, x, y, 0, rb, nb, 1));
             if (d.walls_move) {
                 for (int x = 0; x < 2 * lb; ++x) {
                     Tile t2 = tile(j, x, 0, 0, 2 * lb, 1, 1);

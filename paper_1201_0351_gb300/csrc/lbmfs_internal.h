@@ -8,7 +8,14 @@ namespace lbmfs {
 
 constexpr int Q = 19;
 constexpr int MAX_BODIES = 255;
-constexpr int FORCE_BLOCKS = 64;   // blocks per body in the force / remap kernels
+constexpr int FORCE_BLOCKS = 64;   // blocks per body in the force kernel
+// Blocks per body where nothing depends on their number (the cells next to it,
+// the remap's scan): one per 1024 cells of its range, from the force kernel's up
+// to RANGE_BLOCKS_MAX.  With 64 whatever the body, boxes of half extents 55 in
+// four 160^3 tanks of a batch (FP32) took 425 us (scan) and 360 us (cells next to
+// it) per step, 100 and 216 now; one of 90 in a 256^3 tank 1290 us (cells next to
+// it), 384 now.
+constexpr int RANGE_CELLS = 1024, RANGE_BLOCKS_MAX = 1024;
 constexpr int LIST_BLOCKS = 304;   // 2 x 152 SMs: grid of the worklist kernels
 constexpr int LIST_THREADS = 256;
 constexpr int REMAP_THREADS = 512;
@@ -109,6 +116,7 @@ struct Dev {
     int force_mean;    // rigid-body update driven by (F_n + F_{n-1}) / 2
     int nb_rule;       // interface cells without liquid (gas) neighbours empty (fill)
     int pair_ok;       // nx and N even: pairs of cells start on even elements of every plane
+    int range_blocks;  // blocks per body of the kernels that look through its range (host)
     int loose;         // obstacle cells came with the initial classes: they may lie away from every body
 };
 
@@ -134,7 +142,8 @@ struct Tile {
 
 // block tables by launch shape
 enum {
-    SH_FORCE = 0,  // (FORCE_BLOCKS, bodies): forces, remap cover / pending
+    SH_FORCE = 0,  // (FORCE_BLOCKS, bodies): forces
+    SH_SCAN,       // (range_blocks, bodies): remap cover / pending
     SH_BULK,       // bulk stream + collide: (ceil(nx ny / BULK_THREADS), 1, ceil(nz / zb));
                    // FP16 storage: tile x + 2^16 y of RING_TILE cells
     SH_IFACE,      // (2 lb): interface cells
@@ -142,7 +151,7 @@ enum {
     SH_BODY,       // (bodies): rigid-body step
     SH_ONE,        // (1) per tank with bodies: remap resolution
     SH_TANK,       // (1) per tank: counter reset
-    SH_GEN,        // liquid cells next to bodies: (FORCE_BLOCKS, bodies), or next to any obstacle (Dev::loose):
+    SH_GEN,        // liquid cells next to bodies: (range_blocks, bodies), or next to any obstacle (Dev::loose):
                    // (2 lb), kind 0; on moving walls: (2 lb), kind 1
     SH_COUNT
 };

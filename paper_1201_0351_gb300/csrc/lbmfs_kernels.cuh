@@ -4331,7 +4331,7 @@ template <int S> struct Launch {
     }
     static void faces(const Dev &d, cudaStream_t st) { k_faces<S><<<LIST_BLOCKS, GEN_THREADS, 0, st>>>(d); }
     static void near(const Dev &d, cudaStream_t st) {
-        k_near<S><<<d.loose ? dim3(4 * LIST_BLOCKS) : dim3(FORCE_BLOCKS, d.nb), GEN_THREADS, 0, st>>>(d);
+        k_near<S><<<d.loose ? dim3(4 * LIST_BLOCKS) : dim3(d.range_blocks, d.nb), GEN_THREADS, 0, st>>>(d);
     }
     static void forces(const Dev &d, cudaStream_t st) {
         k_forces<S><<<dim3(FORCE_BLOCKS, d.nb), FORCE_THREADS, 0, st>>>(d);
@@ -4339,7 +4339,7 @@ template <int S> struct Launch {
     static void scan(const Dev &d, cudaStream_t st, bool early) {
         // a cell or two per thread; blocks small enough to run beside the ring
         // kernel's, which leave 4096 registers of an SM
-        launch(k_remap_scan, dim3(std::max(FORCE_BLOCKS, 1216 / d.nb), d.nb), SCAN_THREADS, 0, st, early, d);
+        launch(k_remap_scan, dim3(std::max(d.range_blocks, 1216 / d.nb), d.nb), SCAN_THREADS, 0, st, early, d);
     }
     static void interface(const Dev &d, cudaStream_t st) { k_interface<S><<<LBMFS_IFACE_GRID, 128, 0, st>>>(d); }
     // the bulk kernel: FP64 and FP32 one cell per thread, with the z-planes per
@@ -4509,7 +4509,7 @@ template <int S> struct BatchStep {
             batch_launch<BkGeneral<S>>(b, SH_GEN, GEN_THREADS, s2);
             batch_launch<BkInterface<S>>(b, SH_IFACE, 128, s0);
             launch_bodies_batch(b, s1, false);
-            batch_short<BkRemapScan>(b, SH_FORCE, SCAN_THREADS, s1, true);
+            batch_short<BkRemapScan>(b, SH_SCAN, SCAN_THREADS, s1, true);
         }
         mark();
         batch_bulk_launch<S>(b, st, sides != nullptr && b.sh[SH_FORCE].n > 0);
@@ -4539,7 +4539,7 @@ template <int S> struct BatchStep {
         mark();
         if (!sides) launch_bodies_batch(b, st, false);
         mark();
-        if (!sides) batch_short<BkRemapScan>(b, SH_FORCE, SCAN_THREADS, st, false);
+        if (!sides) batch_short<BkRemapScan>(b, SH_SCAN, SCAN_THREADS, st, false);
         mark();
         batch_short<BkRemapApply<S>>(b, SH_LIST, LIST_THREADS, st, chain);
         mark();
@@ -4549,7 +4549,7 @@ template <int S> struct BatchStep {
         mark();
         int n = 0;
         const int shapes[] = {SH_TANK, SH_FORCE, SH_BULK, SH_GEN, SH_IFACE, SH_LIST, SH_LIST, SH_LIST, SH_LIST,
-                              SH_LIST, SH_LIST, SH_LIST, SH_BODY, SH_FORCE, SH_LIST, SH_ONE, SH_LIST};
+                              SH_LIST, SH_LIST, SH_LIST, SH_BODY, SH_SCAN, SH_LIST, SH_ONE, SH_LIST};
         for (int sh : shapes) n += b.sh[sh].n ? 1 : 0;
         return n;
     }

@@ -135,6 +135,27 @@ def test_many_uncovered_cells_in_the_float_storages(storage):
     assert e["flag_diff"] == 0 and e["rho"] <= 2e-3, e
 
 
+@pytest.mark.parametrize("storage", ["f64", "f32", "f16s"])
+def test_large_body_range(storage):
+    """a body whose range takes more blocks than the force kernel's 64: the
+    cells next to it and the remap's lists in a batch beside a small tank equal
+    those alone, and (FP64) the oracle's"""
+    from paper_1201_0351_gb300 import lbm_fs
+
+    sc, small = half_immersed_box(72), half_immersed_box(30)
+    a, s, _ = _alone(sc, storage, 4)
+    bt = lbm_fs.Batch([small, sc], storage=storage)
+    bt.step(4)
+    b, t = bt.tanks[1].fields(want_f=True), bt.tanks[1].stats()
+    bt.close()
+    for key in ("flags", "f", "fill", "mass"):
+        assert np.array_equal(a[key], b[key]), key
+    assert s["n_general"] == t["n_general"] > 1000 and s["n_pending"] == t["n_pending"] > 0
+    if storage == "f64":
+        g, o, gb, ob, gs, ref = run_both(sc, 4)
+        assert_f64_parity(g, o, gb, ob)
+
+
 def test_long_lists_against_the_oracle():
     sc = splash(64, 60, 56, 90)
     g, o, gb, ob, gs, ref = run_both(sc, 4)
