@@ -34,7 +34,7 @@ constexpr int BULK_THREADS = LBMFS_BULK_THREADS;  // x extent of a bulk-kernel b
 enum : uint8_t { CL_L = 1, CL_I = 2, CL_G = 4, CL_O = 8, CL_MASK = 15, NB_OBST = 16, MOVING_FACE = 32, FACE_YZ = 64, FACE_X = 128 };
 // per-cell conversion marks (separate byte array, zero between steps)
 enum : uint8_t {
-    MK_FILLED = 1, MK_EMPTIED = 2, MK_NEWG = 4, MK_NEWL = 8, MK_RECV = 16, MK_PEND = 32, MK_FRESH = 64
+    MK_FILLED = 1, MK_EMPTIED = 2, MK_NEWG = 4, MK_NEWL = 8, MK_RECV = 16, MK_PEND = 32, MK_FRESH = 64, MK_COVER = 128
 };
 // sticky device status bits
 enum : uint32_t { ST_LIQUID_GAS = 1, ST_NONFINITE = 2, ST_OVERFLOW = 4, ST_TIMEOUT = 8, ST_CONTACT = 16, ST_TOP = 32 };

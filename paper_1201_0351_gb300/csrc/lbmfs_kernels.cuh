@@ -1148,6 +1148,9 @@ __device__ __forceinline__ long long nb_target(const Dev &d, uint32_t it, uint32
     return nbr(d, x, y, z, dir_x(q), dir_y(q), dir_z(q));
 }
 __device__ __forceinline__ void nb_update_body(const Dev &d, const VB &vb) {
+    if (d.nb > 1) {
+        LIST_LOOP(WL_COVER, a) d.cmark[d.list[WL_COVER][it_a]] = 0;
+    }
     const uint32_t nc = wl_count(d, WL_COVER), n = (nc + wl_count(d, WL_PEND)) * Q;
     const uint32_t warps = vb.nx * (blockDim.x >> 5);
     const int lane = threadIdx.x & 31;
@@ -3401,12 +3404,12 @@ __device__ __forceinline__ void conv_excess_body(const Dev &d, const VB &vb) {
 template <int S>
 __global__ void k_conv_excess(const __grid_constant__ Dev d) { conv_excess_body<S>(d, vb_own()); }
 
-// marks are cleared
+// marks are cleared (bit by bit: the remap may be marking covered cells by then)
 __device__ __forceinline__ void conv_finish_body(const Dev &d, const VB &vb) {
     const int lists[5] = {WL_FILLED, WL_EMPTIED, WL_NEWG, WL_NEWL, WL_RECV};
 #pragma unroll
     for (int k = 0; k < 5; ++k) {
-        LIST_LOOP(lists[k], a) d.cmark[d.list[lists[k]][it_a]] = 0;
+        LIST_LOOP(lists[k], a) mark_and(d, d.list[lists[k]][it_a], MK_FILLED | MK_EMPTIED | MK_NEWG | MK_NEWL | MK_RECV);
     }
 }
 __global__ void k_conv_finish(const __grid_constant__ Dev d) { conv_finish_body(d, vb_own()); }
@@ -3694,14 +3697,11 @@ __device__ __forceinline__ void remap_scan_body(const Dev &d, const VB &vb) {
                 const bool in = inside(d, b, x, y, z);
                 cover = !solid && in;
                 pend = own && !in && (!d.loose || in_prev_range(d, b, x, y, z));
-                // of the bodies that cover a cell at once the first has it
-#pragma unroll 1
-                for (int j = 0; cover && j < bi; ++j) cover = !inside(d, d.bodies_new[j], x, y, z);
             }
         }
         if (__any_sync(0xffffffffu, cover)) wl_append(d, cover, WL_COVER, (uint32_t)i);
-        // the covering body, for remap_apply_body (an obstacle's id is set
-        // there; until then nothing reads a fluid cell's id)
+        // the covering body (until remap_apply_body makes the cell an obstacle
+        // nothing reads its id)
         if (cover) d.bid[i] = (uint8_t)bi;
         if (__any_sync(0xffffffffu, pend)) wl_append(d, pend, WL_PEND, (uint32_t)i);
     }
@@ -3713,12 +3713,23 @@ __global__ void __launch_bounds__(SCAN_THREADS) k_remap_scan(const __grid_consta
 }
 
 // listed cells inside a body's new pose become obstacle, their mass is booked;
-// listed obstacle cells outside it are pending
+// listed obstacle cells outside it are pending.  A cell that several bodies
+// cover in one step is listed once for each: it is booked once, and the first of
+// those bodies has it.  (Looking for lower bodies at each covered cell in the
+// scan instead: 200 spheres 257 -> 319 us per step.)
 template <int S>
 __device__ __forceinline__ void remap_apply_body(const Dev &d, const VB &vb) {
     {
         LIST_LOOP(WL_COVER, a) {
             const long long i = d.list[WL_COVER][it_a];
+            if (d.nb > 1 && (mark_or(d, i, MK_COVER) & MK_COVER)) {
+                int x, y, z, j = 0;
+                coords(d, i, x, y, z);
+#pragma unroll 1
+                while (j < d.nb - 1 && !inside(d, d.bodies_new[j], x, y, z)) ++j;
+                d.bid[i] = (uint8_t)j;
+                continue;
+            }
             const int c = clsv(d, i);
             const double mass = c == CL_L ? cell_density<S>(d, d.fdst, i) : (c == CL_I ? d.m[i] : 0.0);
             if (mass != 0.0) atomicAdd(&d.ledger[LG_COVERED], mass);
@@ -3726,7 +3737,7 @@ __device__ __forceinline__ void remap_apply_body(const Dev &d, const VB &vb) {
         }
     }
     {
-        LIST_LOOP(WL_PEND, b) d.cmark[d.list[WL_PEND][it_b]] = MK_PEND;
+        LIST_LOOP(WL_PEND, b) mark_or(d, d.list[WL_PEND][it_b], MK_PEND);
     }
 }
 template <int S>
