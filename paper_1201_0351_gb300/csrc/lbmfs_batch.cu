@@ -142,7 +142,11 @@ lbm_fs_status build(lbm_fs_batch *b) {
             const int rb = d.range_blocks;
             for (int y = 0; y < nb; ++y)
                 for (int x = 0; x < rb; ++x) tb[SH_SCAN].push_back(tile(j, x, y, 0, rb, nb, 1));
-            if (t->p.storage == LBM_FS_F16S) {
+            if (t->p.storage == LBM_FS_F16S && d.nx < RING_MIN_NX) {
+                const int gx = (int)(((long long)d.nx * d.ny + BULK_THREADS - 1) / BULK_THREADS);
+                for (int z = 0; z < d.nz; ++z)
+                    for (int x = 0; x < gx; ++x) tb[SH_NARROW].push_back(tile(j, x, 0, z, gx, 1, d.nz));
+            } else if (t->p.storage == LBM_FS_F16S) {
                 const long long tiles = (d.N + RING_TILE - 1) / RING_TILE;
                 for (long long k = 0; k < tiles; ++k) tb[SH_BULK].push_back(tile(j, (int)(k & 0xffff), (int)(k >> 16), 0, 1, 1, 1));
             } else {

@@ -146,6 +146,7 @@ enum {
     SH_SCAN,       // (range_blocks, bodies): remap cover / pending
     SH_BULK,       // bulk stream + collide: (ceil(nx ny / BULK_THREADS), 1, ceil(nz / zb));
                    // FP16 storage: tile x + 2^16 y of RING_TILE cells
+    SH_NARROW,     // FP16 storage, tanks too narrow for the ring: (ceil(nx ny / BULK_THREADS), 1, nz)
     SH_IFACE,      // (2 lb): interface cells
     SH_LIST,       // (lb): conversion worklists, neighbour-bit refresh
     SH_BODY,       // (bodies): rigid-body step
@@ -169,6 +170,13 @@ struct BatchLaunch {
 };
 // FP16 storage: cells per tile of the ring kernel, and its blocks per SM
 constexpr int RING_TILE = 512, RING_CTAS = 2;
+// Grids narrower than this take the one-cell kernel instead, a z-plane per
+// block: two of a row's cells lie on the x faces, whose populations the ring's
+// one patching warp fetches, 12 rows of a tile at a time.  Measured, us per
+// step, ring and one-cell: nx = 1 (1x2048x2048) 869 and 211, 2 (2x1024x1024) 263
+// and 111, 4 (4x700x700) 133 and 80, 5 (5x700x700) 145 and 101, 6 (6x600x600) 65
+// and 64, 8 (8x512x512) 56 and 63.
+constexpr int RING_MIN_NX = 6;
 // Streams (and events to fork to and join from them) on which a step's kernels
 // that do not depend on the bulk kernel run beside it.  They are created with
 // the highest priority: the bulk kernel fills every SM, and its thousands of

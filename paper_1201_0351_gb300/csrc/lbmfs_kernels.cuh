@@ -4354,7 +4354,8 @@ template <int S> struct Launch {
     }
     static void interface(const Dev &d, cudaStream_t st) { k_interface<S><<<LBMFS_IFACE_GRID, 128, 0, st>>>(d); }
     // the bulk kernel: FP64 and FP32 one cell per thread, with the z-planes per
-    // block of bulk_planes; FP16 the ring; LBMFS_BULK selects the staged forms
+    // block of bulk_planes; FP16 the ring, or on narrow grids one cell per thread
+    // and a plane per block; LBMFS_BULK selects the staged forms
     static void bulk_any(const Dev &d, cudaStream_t st, bool early) {
         if constexpr (S != 0) {
             // the staged variants tile rows: (ceil(nx / BULK_THREADS), ny, z-blocks)
@@ -4369,7 +4370,7 @@ template <int S> struct Launch {
                 return;
             }
         }
-        if constexpr (S == 2) {
+        if (S == 2 && d.nx >= RING_MIN_NX) {
             using G = RingShape;
             const uint32_t n = (uint32_t)((d.N + G::TILE - 1) / G::TILE);
             const auto k = d.a_f[0] == 0.0f && d.a_f[1] == 0.0f ? k_ring<true> : k_ring<false>;
@@ -4377,7 +4378,7 @@ template <int S> struct Launch {
             launch(k, dim3(std::min(n, 152u * RING_CTAS)), G::THREADS, G::SMEM, st, early, d, n);
         } else {
             const unsigned gx = (unsigned)(((long long)d.nx * d.ny + BULK_THREADS - 1) / BULK_THREADS);
-            const int zb = bulk_planes(S, gx, d.nz);
+            const int zb = S == 2 ? 1 : bulk_planes(S, gx, d.nz);
             auto go = [&](void (*k)(Dev)) { launch(k, dim3(gx, 1, (d.nz + zb - 1) / zb), BULK_THREADS, 0, st, early, d); };
             if (zb == 1) go(k_liquid<S, 1>);
             if constexpr (S == 1) {
@@ -4475,11 +4476,14 @@ template <int S> struct Launch {
 // (early: behind the start of the stream's last kernel, see launch_dependents)
 template <int S> void batch_bulk_launch(const BatchLaunch &b, cudaStream_t st, bool early) {
     const Shape &x = b.sh[SH_BULK];
-    if (!x.n) return;
     if constexpr (S == 2) {
+        const Shape &narrow = b.sh[SH_NARROW];
+        if (narrow.n)
+            launch(k_batch<BkLiquid<S, 1>>, dim3(narrow.grid), BULK_THREADS, 0, st, early, *b.ts, narrow.table, narrow.n, 1);
+        if (!x.n) return;
         const auto k = b.zg ? k_batch_ring<true> : k_batch_ring<false>;
         cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, RingShape::SMEM);
-        launch(k, dim3(x.grid), RingShape::THREADS, RingShape::SMEM, st, early, *b.ts, x.table, x.n);
+        launch(k, dim3(x.grid), RingShape::THREADS, RingShape::SMEM, st, early && !narrow.n, *b.ts, x.table, x.n);
     } else {
         auto go = [&](void (*k)(TankSet, const Tile *, unsigned, int)) {
             launch(k, dim3(x.grid), BULK_THREADS, 0, st, early, *b.ts, x.table, x.n, b.zb);
@@ -4559,7 +4563,7 @@ template <int S> struct BatchStep {
         batch_short<BkNbUpdate>(b, SH_LIST, LIST_THREADS, st, chain);
         mark();
         int n = 0;
-        const int shapes[] = {SH_TANK, SH_FORCE, SH_BULK, SH_GEN, SH_IFACE, SH_LIST, SH_LIST, SH_LIST, SH_LIST,
+        const int shapes[] = {SH_TANK, SH_FORCE, SH_BULK, SH_NARROW, SH_GEN, SH_IFACE, SH_LIST, SH_LIST, SH_LIST, SH_LIST,
                               SH_LIST, SH_LIST, SH_LIST, SH_BODY, SH_SCAN, SH_LIST, SH_ONE, SH_LIST};
         for (int sh : shapes) n += b.sh[sh].n ? 1 : 0;
         return n;
@@ -4567,8 +4571,8 @@ template <int S> struct BatchStep {
     static void bulk(const BatchLaunch &b, cudaStream_t st) { batch_bulk_launch<S>(b, st, false); }
     static int bulk_blocks_per_sm() {
         int nb = 0;
-        if (S == 2) return RING_CTAS;
-        if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k_batch<BkLiquid<S, 4>>, BULK_THREADS, 0) != cudaSuccess)
+        if constexpr (S == 2) nb = RING_CTAS;
+        else if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k_batch<BkLiquid<S, 4>>, BULK_THREADS, 0) != cudaSuccess)
             return 1;
         return nb > 0 ? nb : 1;
     }
