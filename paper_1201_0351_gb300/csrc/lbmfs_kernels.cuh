@@ -3404,12 +3404,17 @@ __device__ __forceinline__ void conv_excess_body(const Dev &d, const VB &vb) {
 template <int S>
 __global__ void k_conv_excess(const __grid_constant__ Dev d) { conv_excess_body<S>(d, vb_own()); }
 
-// marks are cleared (bit by bit: the remap may be marking covered cells by then)
+// marks are cleared (with several bodies bit by bit: the remap may be marking
+// covered cells by then; the atomics take 0.8 us longer)
 __device__ __forceinline__ void conv_finish_body(const Dev &d, const VB &vb) {
     const int lists[5] = {WL_FILLED, WL_EMPTIED, WL_NEWG, WL_NEWL, WL_RECV};
 #pragma unroll
     for (int k = 0; k < 5; ++k) {
-        LIST_LOOP(lists[k], a) mark_and(d, d.list[lists[k]][it_a], MK_FILLED | MK_EMPTIED | MK_NEWG | MK_NEWL | MK_RECV);
+        LIST_LOOP(lists[k], a) {
+            const long long i = d.list[lists[k]][it_a];
+            if (d.nb > 1) mark_and(d, i, MK_FILLED | MK_EMPTIED | MK_NEWG | MK_NEWL | MK_RECV);
+            else d.cmark[i] = 0;
+        }
     }
 }
 __global__ void k_conv_finish(const __grid_constant__ Dev d) { conv_finish_body(d, vb_own()); }
