@@ -273,8 +273,9 @@ lbm_fs_status lbm_fs_sync(lbm_fs *h);
 
 /* Runs nsteps steps without graphs, all kernels in one chain (a captured step
  * runs several of them beside the bulk kernel, so a step takes less than the
- * sum), timing every kernel with CUDA events on the handle's stream; ms[k] receives the summed milliseconds of kernel k over the
- * steps and names (may be NULL) a static name per kernel.  Returns the number
+ * sum), timing every kernel with CUDA events on the handle's stream; ms[k]
+ * receives the summed milliseconds of kernel k over the steps and names (may be
+ * NULL) a static name per kernel.  Returns the number
  * of kernels in *nk (at most cap entries are written). */
 lbm_fs_status lbm_fs_kernel_times(lbm_fs *h, int32_t nsteps, double *ms,
                                   const char **names, int32_t cap, int32_t *nk);
@@ -337,12 +338,12 @@ typedef struct {
 
 /* Times the batched bulk kernel over a set of candidate tilings (zb in
  * {1, 2, 4, 8}; persistent grids of 1, 2 and 4 times the resident blocks,
- * and one block per tile) on the current state and keeps the fastest;
+ * and one block per tile; FP16 storage: the three grids, zb as it is) on the
+ * current state and keeps the fastest;
  * *out (may be NULL) receives it.  The state is not advanced: the timed
  * launches write only the second population grid (rewritten by the next
  * step), and the worklist counters and mass ledger are restored.  Call it
- * between steps; the interface-cell count that lbm_fs_stats reports reads 0
- * until the next step. */
+ * between steps. */
 lbm_fs_status lbm_fs_batch_autotune(lbm_fs_batch *b, lbm_fs_batch_config_t *out);
 lbm_fs_status lbm_fs_batch_set_config(lbm_fs_batch *b, const lbm_fs_batch_config_t *c);
 lbm_fs_status lbm_fs_batch_get_config(lbm_fs_batch *b, lbm_fs_batch_config_t *c);

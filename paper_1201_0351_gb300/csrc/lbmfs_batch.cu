@@ -504,8 +504,10 @@ lbm_fs_status lbm_fs_batch_autotune(lbm_fs_batch *b, lbm_fs_batch_config_t *out)
     }
     const int keep_zb = b->zb, keep_blocks = b->bulk_blocks;
     const int per_sm = b->ks.bulk_blocks_per_sm();
-    const int zbs[] = {1, 2, 4, 8};
-    const int mults[] = {1, 2, 4, 0};
+    // (the FP16 storage's bulk kernels take no zb, and its grid is persistent)
+    const bool ring = b->tanks[0]->p.storage == LBM_FS_F16S;
+    const std::vector<int> zbs = ring ? std::vector<int>{keep_zb} : std::vector<int>{1, 2, 4, 8};
+    const std::vector<int> mults = ring ? std::vector<int>{1, 2, 4} : std::vector<int>{1, 2, 4, 0};
     cudaEvent_t e0, e1;
     CK(cudaEventCreate(&e0));
     CK(cudaEventCreate(&e1));
