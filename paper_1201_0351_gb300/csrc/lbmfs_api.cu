@@ -225,10 +225,9 @@ lbm_fs_status lbm_fs_create(const lbm_fs_params *p, lbm_fs **out) {
     d.force_mean = (p->readings & LBM_FS_READING_FORCE_MEAN) ? (p->force_mean != 0) : 1;
     d.nb_rule = (p->readings & LBM_FS_READING_NEIGHBOUR_RULE) ? (p->neighbour_rule != 0) : 1;
     d.pair_ok = p->nx % 2 == 0 && N % 2 == 0;
-    // row segments are 16-byte aligned when nx is a multiple of 16 / element size
-    // bulk-kernel variant (float storages): direct loads by default;
-    // LBMFS_BULK=pipe|tma selects the shared-memory staged variants (both
-    // measured slower on GB300; the TMA one needs rows of 16-byte multiples)
+    // bulk-kernel variant (float storages): LBMFS_BULK=pipe|tma selects the staged
+    // variants instead of the default (both measured slower on GB300; the TMA one
+    // needs rows of 16-byte multiples)
     d.bulk = BULK_PLAIN;
     if (const char *v = getenv("LBMFS_BULK")) {
         if (!strcmp(v, "pipe")) d.bulk = BULK_PIPE;

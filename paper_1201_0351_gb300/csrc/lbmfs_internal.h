@@ -120,7 +120,8 @@ struct Dev {
     int loose;         // obstacle cells came with the initial classes: they may lie away from every body
 };
 
-// bulk-kernel variants: direct loads, per-thread cp.async pipeline over z,
+// bulk-kernel variants: the default (FP64, FP32 and narrow FP16 grids one cell
+// per thread, other FP16 grids the ring), per-thread cp.async pipeline over z,
 // TMA-staged rows (needs 16-byte aligned rows)
 enum { BULK_PLAIN = 0, BULK_PIPE = 1, BULK_TMA = 2 };
 

@@ -65,7 +65,7 @@ __host__ __device__ __forceinline__ constexpr float wf(int q) {
 #define LBMFS_BULK_MINB 8  // resident blocks per SM asked of ptxas for the bulk kernel (64 registers)
 #endif
 #ifndef LBMFS_BULK_ZB
-#define LBMFS_BULK_ZB 8    // z-planes per bulk-kernel block (measured: 8 beat 4 by 2 % for FP32, 2 was far slower)
+#define LBMFS_BULK_ZB 8    // z-planes per block of the TMA-staged bulk kernel (those of the default kernel: bulk_planes)
 #endif
 #ifndef LBMFS_BULK_PIPE_ZB
 #define LBMFS_BULK_PIPE_ZB 16  // z-planes per block of the software-pipelined bulk kernel
@@ -538,15 +538,6 @@ __device__ __forceinline__ double feq_d(int q, double rho, const double *u) {
     double usq = (u[0] * u[0] + u[1] * u[1]) + u[2] * u[2];
     double t = ((1.0 + 3.0 * cu) + (4.5 * cu) * cu) - 1.5 * usq;
     return (wd(q) * rho) * t;
-}
-
-// Eq. forceterm (Luo): w rho [3 (c - u) + 9 (c.u) c] . a
-__device__ __forceinline__ double force_d(int q, double rho, const double *u, const double *a) {
-    double cu = (cx(q) * u[0] + cy(q) * u[1]) + cz(q) * u[2];
-    double tx = (3.0 * (cx(q) - u[0]) + (9.0 * cu) * cx(q)) * a[0];
-    double ty = (3.0 * (cy(q) - u[1]) + (9.0 * cu) * cy(q)) * a[1];
-    double tz = (3.0 * (cz(q) - u[2]) + (9.0 * cu) * cz(q)) * a[2];
-    return (wd(q) * rho) * ((tx + ty) + tz);
 }
 
 template <int S>
@@ -1172,7 +1163,6 @@ __device__ __forceinline__ void nb_update_body(const Dev &d, const VB &vb) {
         __syncwarp();
     }
 }
-__global__ void k_nb_update(const __grid_constant__ Dev d) { nb_update_body(d, vb_own()); }
 
 // ---- C4: momentum exchange at the links into body vb.y (state at t):
 // Sec. 2.3 Eqs. momentumexchange, netforce, torque; Sec. 2.4 Eq.
@@ -3173,7 +3163,6 @@ __device__ __forceinline__ void conv_filled_body(const Dev &d, const VB &vb) {
         mark_append(d, cls(d, yi) == CL_G, yi, MK_NEWG, WL_NEWG);
     }
 }
-__global__ void k_conv_filled(const __grid_constant__ Dev d) { conv_filled_body(d, vb_own()); }
 
 // an emptied cell next to a filled one is kept; liquid neighbours of the others
 // become interface
@@ -3192,7 +3181,6 @@ __device__ __forceinline__ void conv_emptied_body(const Dev &d, const VB &vb) {
         mark_append(d, c == CL_L, yi, MK_NEWL, WL_NEWL);
     }
 }
-__global__ void k_conv_emptied(const __grid_constant__ Dev d) { conv_emptied_body(d, vb_own()); }
 
 // density of a cell by a whole warp: lane q loads population q, the sum is
 // taken in q order (as cell_density takes it) on every lane
@@ -3283,8 +3271,6 @@ __device__ __forceinline__ void conv_init_body(const Dev &d, const VB &vb) {
         }
     }
 }
-template <int S>
-__global__ void k_conv_init(const __grid_constant__ Dev d) { conv_init_body<S>(d, vb_own()); }
 
 // the new classes
 __device__ __forceinline__ void conv_flags_body(const Dev &d, const VB &vb) {
@@ -3304,7 +3290,6 @@ __device__ __forceinline__ void conv_flags_body(const Dev &d, const VB &vb) {
         LIST_LOOP(WL_NEWL, e) set_cls(d, d.list[WL_NEWL][it_e], CL_I);
     }
 }
-__global__ void k_conv_flags(const __grid_constant__ Dev d) { conv_flags_body(d, vb_own()); }
 
 // the class a cell of class c has after the conversions, by its marks
 __device__ __forceinline__ int class_after(int c, int mk) {
@@ -3348,8 +3333,6 @@ __device__ __forceinline__ void conv_claim_body(const Dev &d, const VB &vb) {
         }
     }
 }
-template <int S>
-__global__ void k_conv_claim(const __grid_constant__ Dev d) { conv_claim_body<S>(d, vb_own()); }
 
 // Receivers gather e(x) / k(x) over their converted neighbours in q order: the
 // neighbours' marks, then the converted ones' shares (computed when the
@@ -3401,8 +3384,6 @@ __device__ __forceinline__ void conv_excess_body(const Dev &d, const VB &vb) {
         set_mass<S>(d, i, d.m[i] + acc, rho);
     }
 }
-template <int S>
-__global__ void k_conv_excess(const __grid_constant__ Dev d) { conv_excess_body<S>(d, vb_own()); }
 
 // marks are cleared (with several bodies bit by bit: the remap may be marking
 // covered cells by then; the atomics take 0.8 us longer)
@@ -3417,7 +3398,6 @@ __device__ __forceinline__ void conv_finish_body(const Dev &d, const VB &vb) {
         }
     }
 }
-__global__ void k_conv_finish(const __grid_constant__ Dev d) { conv_finish_body(d, vb_own()); }
 
 // ----------------------------------------------- C5: rigid-body update
 // (the role the paper gives the pe engine, Sec. 2.3: the body moves under the
@@ -3745,8 +3725,6 @@ __device__ __forceinline__ void remap_apply_body(const Dev &d, const VB &vb) {
         LIST_LOOP(WL_PEND, b) mark_or(d, d.list[WL_PEND][it_b], MK_PEND);
     }
 }
-template <int S>
-__global__ void k_remap_apply(const __grid_constant__ Dev d) { remap_apply_body<S>(d, vb_own()); }
 
 // What a pending cell becomes (Sec. 2.4), from its numbers of liquid, interface
 // and gas neighbours and their sums of density and fill level.
@@ -3955,8 +3933,6 @@ __device__ __forceinline__ void remap_resolve_body(const Dev &d, const VB &vb) {
         d.ledger[LG_UNCOVERED] += t;
     }
 }
-template <int S>
-__global__ void __launch_bounds__(REMAP_THREADS) k_remap_resolve(const __grid_constant__ Dev d) { remap_resolve_body<S>(d, vb_own()); }
 
 // ------------------------------------------- conversions and remap in one launch
 //
@@ -4214,7 +4190,7 @@ __global__ void __launch_bounds__(K::THREADS, K::MINB)
 }
 
 // The short kernels of a batch's step (counters, conversions, rigid bodies,
-// remap): the descriptors come from memory instead of the parameter space, 25 KB
+// remap): the descriptors come from memory instead of the parameter space, 32 KB
 // of which cost every launch a few us, and each launch is a programmatic
 // dependent of the one before it in the chain.
 template <class K>
@@ -4300,8 +4276,9 @@ template <class K> void batch_launch(const BatchLaunch &b, int sh, dim3 block, c
 // fill the GPU several times over; on smaller ones a few threads would walk 8
 // dependent cells while SMs idle.  Measured (bulk kernel, us at 8 / 4 / 2 / 1
 // planes): 32^3 FP64 111 / 60 / 34 / 21, 96^3 FP64 308 / 304 / 304 / 288;
-// 96x32x32 FP32 27 / 17 / 12 / 10, 128^3 FP32 42 / 39 / 39 / 49, 385x190x127
-// FP16S 141 / 124 / 136 / 199; the 768x384x256 tank 2 % faster at 8 than at 4.
+// 96x32x32 FP32 27 / 17 / 12 / 10, 128^3 FP32 42 / 39 / 39 / 49, 385x190x127 FP32
+// 138 / 135 / 156 / 246, 512x256x170 FP32 284 / 292 / 571 / 863; the 768x384x256
+// tank 2 % faster at 8 than at 4.
 inline int bulk_planes(int storage, unsigned gx, int nz) {
     auto blocks = [&](int zb) { return (long long)gx * ((nz + zb - 1) / zb); };
     if (storage == 0) return 1;  // bound by the double unit: the most even spread
