@@ -2129,8 +2129,8 @@ __global__ void __launch_bounds__(BULK_THREADS, LBMFS_BULK_MINB) k_liquid_tma(De
 // Fetching the x faces in the consumers too cost a global load's latency per
 // warp: 768x384x256 bulk kernel 763 us against 581 without any face work.
 // Measured, us, before (one cell per thread) and now: 768x384x256 856 and 593
-// (5.1 TB/s, 76 % of the copy bandwidth; on 384x192x128 issue is 58 % and the FMA
-// pipe 46 % active, so no unit alone is the bound),
+// (5.1 TB/s, 76 % of the copy bandwidth; on 384x192x128 issue is 59 % and the FMA
+// pipe 47 % active, so no unit alone is the bound),
 // 385x190x127 127 and 91, 64 tanks of edge 48..112 626 and 408.  On grids too
 // small to fill the GPU it is even (130x40x40 11 and 12).  The FP32 storage
 // keeps the other kernel: 944 us against 1021 in a ring, HBM-bound either way.
