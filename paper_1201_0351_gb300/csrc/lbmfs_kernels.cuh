@@ -3385,15 +3385,15 @@ __device__ __forceinline__ void conv_excess_body(const Dev &d, const VB &vb) {
     }
 }
 
-// marks are cleared (with several bodies bit by bit: the remap may be marking
-// covered cells by then; the atomics take 0.8 us longer)
-__device__ __forceinline__ void conv_finish_body(const Dev &d, const VB &vb) {
+// marks are cleared; bit by bit where the remap may be marking covered cells at
+// the same time (shared; the atomics take 0.8 us longer)
+__device__ __forceinline__ void conv_finish_body(const Dev &d, const VB &vb, bool shared) {
     const int lists[5] = {WL_FILLED, WL_EMPTIED, WL_NEWG, WL_NEWL, WL_RECV};
 #pragma unroll
     for (int k = 0; k < 5; ++k) {
         LIST_LOOP(lists[k], a) {
             const long long i = d.list[lists[k]][it_a];
-            if (d.nb > 1) mark_and(d, i, MK_FILLED | MK_EMPTIED | MK_NEWG | MK_NEWL | MK_RECV);
+            if (shared) mark_and(d, i, MK_FILLED | MK_EMPTIED | MK_NEWG | MK_NEWL | MK_RECV);
             else d.cmark[i] = 0;
         }
     }
@@ -4082,7 +4082,7 @@ __global__ void __launch_bounds__(tail_threads(CLUSTER)) k_tail(const __grid_con
         conv_flags_body(d, vb);
         conv_excess_body<S>(d, vb);
         if (!tail_barrier(d, vb, cluster)) return;
-        conv_finish_body(d, vb);
+        conv_finish_body(d, vb, nmoved > 0 && d.nb > 1);
     }
     if (nmoved) {
         remap_apply_body<S>(d, vb);
@@ -4238,7 +4238,7 @@ template <int S> LBMFS_BATCH_BODY(BkConvInit, LIST_THREADS, 1, conv_init_body<S>
 LBMFS_BATCH_BODY(BkConvFlags, LIST_THREADS, 1, conv_flags_body(d, vb))
 template <int S> LBMFS_BATCH_BODY(BkConvClaim, LIST_THREADS, 1, conv_claim_body<S>(d, vb))
 template <int S> LBMFS_BATCH_BODY(BkConvExcess, LIST_THREADS, 1, conv_excess_body<S>(d, vb))
-LBMFS_BATCH_BODY(BkConvFinish, LIST_THREADS, 1, conv_finish_body(d, vb))
+LBMFS_BATCH_BODY(BkConvFinish, LIST_THREADS, 1, conv_finish_body(d, vb, false))
 LBMFS_BATCH_BODY(BkBodies, 32, 1, bodies_body(d, vb))
 LBMFS_BATCH_BODY(BkRemapScan, SCAN_THREADS, 1, remap_scan_body(d, vb))
 template <int S> LBMFS_BATCH_BODY(BkRemapApply, LIST_THREADS, 1, remap_apply_body<S>(d, vb))
